@@ -4,7 +4,7 @@
 // quantised score q = round-half-even(s * 2^15) of each CSR entry breaks ties between equally
 // connected labels (larger score sum first) and orders admission after the gain.
 //
-// Features of entry (v,u), symmetric in v and u (rows of degree above 512 are spread over a CTA):
+// Features of entry (v,u), symmetric in v and u:
 //   0 log2(1 + min(d(v), d(u)))        1 log2(1 + max(d(v), d(u)))
 //   2 log2(1 + omega(v,u))             3 log2(1 + min(c(v), c(u)))
 //   4 log2(1 + max(c(v), c(u)))
@@ -42,152 +42,71 @@ __device__ __forceinline__ uint16_t float_to_bf16(float f) {
 
 __device__ __forceinline__ unsigned pack2(uint16_t lo, uint16_t hi) { return (unsigned)lo | ((unsigned)hi << 16); }
 
-__global__ void k_wdeg(DGraph g, float *wdeg) {
+// The CSR entries are taken in segments of kSeg by the warps, whatever rows they belong to: the longest
+// rows of a power-law graph are spread over as many warps as they have segments.
+constexpr int kSeg = 256;
+
+// The largest v with off[v] <= x (0 <= x < m), found by the whole warp: 32 pivots per step.
+__device__ __forceinline__ int64_t warp_row_of(const DGraph &g, int64_t x) {
   const int lane = threadIdx.x & 31;
+  int64_t lo = 0, hi = g.n;  // off[lo] <= x < off[hi]
+  while (hi - lo > 1) {
+    const int64_t step = (hi - lo + 31) / 32;
+    const int64_t p = lo + (lane + 1) * step;
+    const unsigned below = __ballot_sync(kFull, p < hi && g.row_begin(p) <= x);  // (a prefix of the lanes)
+    const int c = __popc(below);
+    const int64_t base = lo;
+    lo = base + c * step;
+    hi = min(hi, base + (c + 1) * step);
+  }
+  return lo;
+}
+
+// The rows of a segment, in order; lane l holds the end of row base + l.
+struct RowWindow {
+  int64_t base, first, ends;  // first: begin of row `base`
+  __device__ __forceinline__ void load(const DGraph &g, int64_t v) {
+    base = v;
+    first = g.row_begin(v);
+    const int64_t x = v + 1 + (threadIdx.x & 31);
+    ends = g.row_begin(x < g.n ? x : g.n);
+  }
+  // the row that holds entry e (at or after the window's start) and its bounds
+  __device__ __forceinline__ int64_t seek(const DGraph &g, int64_t e, int64_t *beg, int64_t *end) {
+    unsigned m;
+    while ((m = __ballot_sync(kFull, ends > e)) == 0) load(g, base + 32);
+    const int f = __ffs(m) - 1;
+    *end = __shfl_sync(kFull, ends, f);
+    const int64_t b = __shfl_sync(kFull, ends, f > 0 ? f - 1 : 0);
+    *beg = f > 0 ? b : first;
+    return base + f;
+  }
+};
+
+// Weighted degrees (graphs with edge weights; without, the degree serves). Exact integer sums: a row
+// inside one segment is stored, the parts of a row that spans segments are added (wsum is zero on entry).
+__global__ void __launch_bounds__(256) k_wdeg(DGraph g, unsigned long long *wsum) {
+  const int lane = threadIdx.x & 31;
+  const int64_t m = gp_min64(g.m, g.row_begin(g.n)), nseg = (m + kSeg - 1) / kSeg;
   const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t v = gw; v < g.n; v += nw) {
-    const int64_t b = g.row_begin(v), e = g.row_begin(v + 1);
-    double s = 0;
-    for (int64_t x = b + lane; x < e; x += 32) s += (double)g.eweight(x);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
-    if (lane == 0) wdeg[v] = (float)s;
-  }
-}
-
-// Features of entry e = (v,u) of v's row (called by one lane per entry; `has` false for the lanes past
-// the row's end). The shared-neighbour count: the lane takes the first 64 neighbours of u and looks
-// each up in `tab`, the set of v's first 64 neighbours (an open-addressing table of kTab slots in shared
-// memory, slot mix32(x) mod kTab, linear probing).
-constexpr int kTab = 128;  // set slots (at most 64 keys)
-constexpr int64_t kFeatSmall = 512;  // rows up to this degree: a half-warp per vertex; longer: a CTA
-
-template <bool BF16>
-__device__ __forceinline__ void feature_entry(const DGraph &g, const float *wdeg, int64_t e, bool has, int64_t dv,
-                                              float cv, float wv, const int *tab, float flevel, float *fout,
-                                              unsigned *bout) {
-  const int u = has ? g.adj[e] : 0;
-  const int64_t bu = has ? g.row_begin(u) : 0;
-  const int64_t eu = has ? g.row_begin(u + 1) : 0;
-  const int lenu = (int)gp_min64(eu - bu, 64);
-  // u's weight, its weighted degree and the entry's weight are loaded before the search
-  const float cu = has ? (float)g.vweight(u) : 0.0f;
-  const float wu = has ? wdeg[u] : 0.0f;
-  const float w = has ? (float)g.eweight(e) : 0.0f;
-  int mine = 0;
-  // eight of u's neighbours are loaded before any is searched (independent loads in flight)
-  constexpr int kBatch = 8;
-  for (int k0 = 0; k0 < lenu; k0 += kBatch) {
-    int xs[kBatch];
-#pragma unroll
-    for (int q = 0; q < kBatch; q++) xs[q] = k0 + q < lenu ? __ldg(g.adj + bu + k0 + q) : 0;
-#pragma unroll
-    for (int q = 0; q < kBatch; q++) {
-      if (k0 + q >= lenu) break;
-      const int x = xs[q];
-      unsigned sl = mix32((unsigned)x) & (kTab - 1);
-      while (true) {
-        const int k = tab[sl];
-        if (k == x) {
-          mine++;
-          break;
-        }
-        if (k == -1) break;
-        sl = (sl + 1) & (kTab - 1);
+  for (int64_t sg = gw; sg < nseg; sg += nw) {
+    const int64_t s1 = gp_min64(m, (sg + 1) * kSeg);
+    RowWindow W;
+    W.load(g, warp_row_of(g, sg * kSeg));
+    for (int64_t e = sg * kSeg; e < s1;) {
+      int64_t beg, end;
+      const int64_t v = W.seek(g, e, &beg, &end);
+      const int64_t stop = gp_min64(end, s1);
+      long long s = 0;
+      for (int64_t x = e + lane; x < stop; x += 32) s += g.eweight(x);
+      s = warp_sum64(s);
+      if (lane == 0) {
+        if (beg >= sg * kSeg && end <= s1) wsum[v] = (unsigned long long)s;
+        else atomicAdd(&wsum[v], (unsigned long long)s);
       }
+      e = stop;
     }
-  }
-  if (!has) return;
-  const float du = (float)(eu - bu);
-  const float dvf = (float)dv;
-  float f[kIn];
-  f[0] = log2f(1.0f + fminf(dvf, du));
-  f[1] = log2f(1.0f + fmaxf(dvf, du));
-  f[2] = log2f(1.0f + w);
-  f[3] = log2f(1.0f + fminf(cv, cu));
-  f[4] = log2f(1.0f + fmaxf(cv, cu));
-  f[5] = (float)mine / 64.0f;
-  f[6] = w / fmaxf(wv, wu);
-  f[7] = flevel;
-  if (BF16) {
-#pragma unroll
-    for (int i = 0; i < 4; i++) bout[e * 4 + i] = pack2(float_to_bf16(f[2 * i]), float_to_bf16(f[2 * i + 1]));
-  } else {
-#pragma unroll
-    for (int i = 0; i < kIn; i++) fout[e * kIn + i] = f[i];
-  }
-}
-
-// Rows of degree <= kFeatSmall: one half-warp (16 lanes) per vertex, each lane one entry of a 16-entry
-// step; the set of v's first 64 neighbours is the half-warp's own table.
-template <bool BF16>
-__global__ void __launch_bounds__(256, 6) k_features(DGraph g, int level, const float *wdeg, float *fout, unsigned *bout) {
-  constexpr int kH = 16;  // lanes per vertex
-  __shared__ int tab_s[8][2][kTab];
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, half = lane / kH, hl = lane % kH;
-  const unsigned hmask = 0xFFFFu << (kH * half);
-  int *tab = tab_s[wid][half];
-  const int64_t gh = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kH;
-  const int64_t nh = ((int64_t)gridDim.x * blockDim.x) / kH;
-  const float flevel = (float)level / 16.0f;
-  for (int64_t v = gh; v < g.n; v += nh) {
-    const int64_t beg = g.row_begin(v), end = g.row_begin(v + 1);
-    const int64_t dv = end - beg;
-    if (dv == 0 || dv > kFeatSmall) continue;  // (uniform over the half-warp)
-    const int lenv = (int)gp_min64(dv, 64);
-    __syncwarp(hmask);
-    for (int t = hl; t < kTab; t += kH) tab[t] = -1;
-    __syncwarp(hmask);
-    for (int t = hl; t < lenv; t += kH) {
-      const int x = g.adj[beg + t];
-      unsigned sl = mix32((unsigned)x) & (kTab - 1);
-      while (atomicCAS(&tab[sl], -1, x) != -1) sl = (sl + 1) & (kTab - 1);  // ids in a row are distinct
-    }
-    __syncwarp(hmask);
-    const float cv = (float)g.vweight(v);
-    const float wv = wdeg[v];
-    for (int64_t e0 = beg; e0 < end; e0 += kH) {
-      const int64_t e = e0 + hl;
-      feature_entry<BF16>(g, wdeg, e, e < end, dv, cv, wv, tab, flevel, fout, bout);
-    }
-  }
-}
-
-// Rows of degree > kFeatSmall (hubs of power-law graphs): one CTA per vertex, its 16 half-warps taking
-// 16-entry steps of the row in turn, one shared set of v's first 64 neighbours. A row is thus spread
-// over 256 lanes instead of 16, which keeps the longest rows from deciding the kernel's duration.
-__global__ void k_list_feat_big(DGraph g, int32_t *big, unsigned *nbig) {
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < g.n; v += (int64_t)gridDim.x * blockDim.x)
-    if (g.row_begin(v + 1) - g.row_begin(v) > kFeatSmall) big[atomicAdd(nbig, 1u)] = (int32_t)v;
-}
-
-template <bool BF16>
-__global__ void __launch_bounds__(256) k_features_big(DGraph g, int level, const float *wdeg, float *fout,
-                                                      unsigned *bout, const int32_t *big, const unsigned *nbig) {
-  __shared__ int tab[kTab];
-  const int hw = threadIdx.x >> 4, hl = threadIdx.x & 15;
-  const float flevel = (float)level / 16.0f;
-  const unsigned cnt = *nbig;
-  for (unsigned i = blockIdx.x; i < cnt; i += gridDim.x) {
-    const int v = big[i];
-    const int64_t beg = g.row_begin(v), end = g.row_begin(v + 1);
-    const int64_t dv = end - beg;
-    for (int t = threadIdx.x; t < kTab; t += blockDim.x) tab[t] = -1;
-    __syncthreads();
-    if (threadIdx.x < 64) {
-      const int x = g.adj[beg + threadIdx.x];  // (dv > 64)
-      unsigned sl = mix32((unsigned)x) & (kTab - 1);
-      while (atomicCAS(&tab[sl], -1, x) != -1) sl = (sl + 1) & (kTab - 1);
-    }
-    __syncthreads();
-    const float cv = (float)g.vweight(v);
-    const float wv = wdeg[v];
-    for (int64_t e0 = beg + hw * 16; e0 < end; e0 += 256) {
-      const int64_t e = e0 + hl;
-      feature_entry<BF16>(g, wdeg, e, e < end, dv, cv, wv, tab, flevel, fout, bout);
-    }
-    __syncthreads();
   }
 }
 
@@ -199,63 +118,188 @@ __device__ __forceinline__ void mma_16816(float c[4], const unsigned a[4], const
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-// One warp scores 16 entries per step: A = 16 entries x 16 features (8 used, 8 zero), B = W1^T in
-// four 16x8 slices (32 hidden units). Thread (g = lane/4, t = lane%4) holds features 2t, 2t+1 of
-// rows g and g+8, and C elements (rows g, g+8; hidden units 8nb + 2t, 8nb + 2t + 1).
-__global__ void __launch_bounds__(256) k_mlp_score(const unsigned *fb, int64_t m, const gp_mlp *mlp, float *s_out,
-                                                   int32_t *q_out) {
-  const int lane = threadIdx.x & 31, gq = lane >> 2, t = lane & 3;
-  unsigned bfrag[4][2];
-  float bias[4][2], w2v[4][2];
-#pragma unroll
-  for (int nb = 0; nb < 4; nb++) {
-    const int j = nb * 8 + gq;
-    bfrag[nb][0] = pack2(mlp->w1[j * kIn + 2 * t], mlp->w1[j * kIn + 2 * t + 1]);
-    bfrag[nb][1] = 0;  // features 8..15 are zero
-    bias[nb][0] = mlp->b1[nb * 8 + 2 * t];
-    bias[nb][1] = mlp->b1[nb * 8 + 2 * t + 1];
-    w2v[nb][0] = bf16_to_float(mlp->w2[nb * 8 + 2 * t]);
-    w2v[nb][1] = bf16_to_float(mlp->w2[nb * 8 + 2 * t + 1]);
-  }
-  const float b2 = mlp->b2;
-  const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t tiles = (m + 15) / 16;
-  for (int64_t tile = gw; tile < tiles; tile += nw) {
-    const int64_t r0 = tile * 16 + gq, r1 = r0 + 8;
-    unsigned a[4];
-    a[0] = r0 < m ? fb[r0 * 4 + t] : 0u;
-    a[1] = r1 < m ? fb[r1 * 4 + t] : 0u;
-    a[2] = 0u;
-    a[3] = 0u;
-    float z0 = 0.f, z1 = 0.f;
+// Features of every entry (SCORE false: written as floats) or their scores (SCORE true: the features go
+// straight into the network and never to memory).
+//
+// What bounds it: the shared-neighbour counts look up to 64 neighbours of u up for every entry (v,u), from
+// rows scattered over the adjacency. A warp takes a segment of kSeg entries; for each of its rows the set of
+// v's first 64 neighbours is a table in the warp's shared memory (kTab slots and no probing: the keys whose
+// slot was taken, two on average for a full set, are compared one by one), and lane l owns one entry of 32.
+// The neighbours of two entries are looked up together, each by a half-warp that reads them contiguously, up
+// to 64 per entry, with the loads of four entries issued before the first lookup. Half-warps serve short lists (mesh rows of 12 entries take one step) and long
+// ones (four steps) alike. A lane per entry, walking its list alone, read 32 separate rows per load and
+// waited for the warp's longest list and probe: 27.3 ms for inference on an R-MAT graph of scale 19 with
+// edge weights (15.5 M entries) against 2.7 ms now, at the same bits.
+//
+// Scores: 16 entries per tensor-core step, A = 16 entries x 16 features (8 used, 8 zero), B = W1^T in four
+// 16x8 slices (32 hidden units). Thread (g = lane/4, t = lane%4) holds features 2t, 2t+1 of rows g and
+// g+8, and C elements (rows g, g+8; hidden units 8nb + 2t, 8nb + 2t + 1).
+constexpr int kTab = 1024;
+constexpr int kEdgeWarps = 8;
+__device__ __forceinline__ unsigned tab_slot(int x) { return ((unsigned)x * 0x9E3779B1u) >> 22; }
+static_assert(kTab == 1 << 10, "tab_slot keeps ten bits");
+
+template <bool SCORE>
+__global__ void __launch_bounds__(kEdgeWarps * 32, 4) k_edges(DGraph g, int level, const unsigned long long *wsum,
+                                                           float *fout, const gp_mlp *mlp, float *s_out,
+                                                           int32_t *q_out) {
+  __shared__ int s_tab[kEdgeWarps][kTab], s_over[kEdgeWarps][64];
+  __shared__ uint4 s_x[SCORE ? kEdgeWarps : 1][32];
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, half = lane >> 4, hl = lane & 15;
+  const int gq = lane >> 2, t = lane & 3;
+  int *tab = s_tab[wid], *over = s_over[wid];
+  for (int x = lane; x < kTab; x += 32) tab[x] = -1;
+  unsigned bfrag[4];  // (features 8..15 are zero)
+  float bias[4][2], w2v[4][2], b2 = 0.f;
+  if (SCORE) {
 #pragma unroll
     for (int nb = 0; nb < 4; nb++) {
-      float c[4] = {bias[nb][0], bias[nb][1], bias[nb][0], bias[nb][1]};
-      mma_16816(c, a, bfrag[nb]);
-      // hidden activations are rounded to BF16 before the second layer
-      const float h0 = bf16_to_float(float_to_bf16(fmaxf(c[0], 0.f)));
-      const float h1 = bf16_to_float(float_to_bf16(fmaxf(c[1], 0.f)));
-      const float h2 = bf16_to_float(float_to_bf16(fmaxf(c[2], 0.f)));
-      const float h3 = bf16_to_float(float_to_bf16(fmaxf(c[3], 0.f)));
-      z0 = fmaf(h0, w2v[nb][0], fmaf(h1, w2v[nb][1], z0));
-      z1 = fmaf(h2, w2v[nb][0], fmaf(h3, w2v[nb][1], z1));
+      const int j = nb * 8 + gq;
+      bfrag[nb] = pack2(mlp->w1[j * kIn + 2 * t], mlp->w1[j * kIn + 2 * t + 1]);
+      bias[nb][0] = mlp->b1[nb * 8 + 2 * t];
+      bias[nb][1] = mlp->b1[nb * 8 + 2 * t + 1];
+      w2v[nb][0] = bf16_to_float(mlp->w2[nb * 8 + 2 * t]);
+      w2v[nb][1] = bf16_to_float(mlp->w2[nb * 8 + 2 * t + 1]);
     }
-    z0 += __shfl_xor_sync(kFull, z0, 1);
-    z0 += __shfl_xor_sync(kFull, z0, 2);
-    z1 += __shfl_xor_sync(kFull, z1, 1);
-    z1 += __shfl_xor_sync(kFull, z1, 2);
-    if (t == 0) {
-      if (r0 < m) {
-        const float s = 1.0f / (1.0f + expf(-(z0 + b2)));
-        if (s_out) s_out[r0] = s;
-        if (q_out) q_out[r0] = __float2int_rn(s * 32768.0f);
+    b2 = mlp->b2;
+  }
+  const float flevel = (float)level / 16.0f;
+  const int64_t m = gp_min64(g.m, g.row_begin(g.n)), nseg = (m + kSeg - 1) / kSeg;
+  const int64_t gw = blockIdx.x * (int64_t)kEdgeWarps + wid, nw = (int64_t)gridDim.x * kEdgeWarps;
+  for (int64_t sg = gw; sg < nseg; sg += nw) {
+    const int64_t s1 = gp_min64(m, (sg + 1) * kSeg);
+    RowWindow W;
+    W.load(g, warp_row_of(g, sg * kSeg));
+    for (int64_t e0 = sg * kSeg; e0 < s1;) {
+      int64_t beg, end;
+      const int64_t v = W.seek(g, e0, &beg, &end);
+      const int64_t stop = gp_min64(end, s1), dv = end - beg;
+      // v's first 64 neighbours (two per lane; the ids of a row are distinct) enter the table; a key whose
+      // slot is taken goes to the list instead
+      int own[2], nover = 0;
+#pragma unroll
+      for (int h = 0; h < 2; h++) {
+        own[h] = -1;
+        bool put = false;
+        int x = 0;
+        if (lane + 32 * h < dv) {
+          x = __ldg(g.adj + beg + lane + 32 * h);
+          const unsigned sl = tab_slot(x);
+          if (atomicCAS(&tab[sl], -1, x) == -1) own[h] = (int)sl;
+          else put = true;
+        }
+        const unsigned m = __ballot_sync(kFull, put);
+        if (put) over[nover + __popc(m & lanemask_lt())] = x;
+        nover += __popc(m);
       }
-      if (r1 < m) {
-        const float s = 1.0f / (1.0f + expf(-(z1 + b2)));
-        if (s_out) s_out[r1] = s;
-        if (q_out) q_out[r1] = __float2int_rn(s * 32768.0f);
+      __syncwarp();
+      const float cv = (float)g.vweight(v);
+      const float wv = wsum ? (float)(double)wsum[v] : (float)dv;
+      for (; e0 < stop; e0 += 32) {
+        const int64_t e = e0 + lane;
+        const bool has = e < stop;
+        const int u = has ? __ldg(g.adj + e) : 0;
+        const int64_t bu = has ? g.row_begin(u) : 0;
+        const int64_t du64 = has ? g.row_begin(u + 1) - bu : 0;
+        const int lenu = (int)gp_min64(du64, 64);
+        const float cu = has ? (float)g.vweight(u) : 0.0f;
+        const float wu = has ? (wsum ? (float)(double)wsum[u] : (float)du64) : 0.0f;
+        const float w = has ? (float)g.eweight(e) : 0.0f;
+        const int cnt = (int)gp_min64(stop - e0, 32);
+        int mine = 0;
+        for (int p = 0; p < cnt; p += 4) {
+          // entries p, p + 2 (lower half-warp) and p + 1, p + 3 (upper)
+          int xs[2][4], most[2];
+#pragma unroll
+          for (int y = 0; y < 2; y++) {
+            const int64_t b = __shfl_sync(kFull, bu, p + 2 * y + half);
+            const int len = __shfl_sync(kFull, lenu, p + 2 * y + half);
+            most[y] = max(len, __shfl_xor_sync(kFull, len, 16));
+#pragma unroll
+            for (int q = 0; q < 4; q++) xs[y][q] = hl + 16 * q < len ? __ldg(g.adj + b + hl + 16 * q) : -2;
+          }
+#pragma unroll
+          for (int y = 0; y < 2; y++) {
+            unsigned hits = 0;
+#pragma unroll
+            for (int q = 0; q < 4; q++)
+              if (16 * q < most[y]) hits += tab[tab_slot(xs[y][q])] == xs[y][q];
+            for (int o = 0; o < nover; o++) {
+              const int k = over[o];
+#pragma unroll
+              for (int q = 0; q < 4; q++) hits += k == xs[y][q];
+            }
+            const unsigned c = __reduce_add_sync(kFull, hits << (16 * half));  // both half-warps' counts
+            if (lane == p + 2 * y) mine = (int)(c & 0xffffu);
+            if (lane == p + 2 * y + 1) mine = (int)(c >> 16);
+          }
+        }
+        const float du = (float)du64, dvf = (float)dv;
+        float f[kIn];
+        f[0] = log2f(1.0f + fminf(dvf, du));
+        f[1] = log2f(1.0f + fmaxf(dvf, du));
+        f[2] = log2f(1.0f + w);
+        f[3] = log2f(1.0f + fminf(cv, cu));
+        f[4] = log2f(1.0f + fmaxf(cv, cu));
+        f[5] = (float)mine / 64.0f;
+        f[6] = w / fmaxf(wv, wu);
+        f[7] = flevel;
+        if (!SCORE) {
+          if (has) {
+#pragma unroll
+            for (int i = 0; i < kIn; i++) fout[e * kIn + i] = f[i];
+          }
+          continue;
+        }
+        uint4 pk;
+        pk.x = pack2(float_to_bf16(f[0]), float_to_bf16(f[1]));
+        pk.y = pack2(float_to_bf16(f[2]), float_to_bf16(f[3]));
+        pk.z = pack2(float_to_bf16(f[4]), float_to_bf16(f[5]));
+        pk.w = pack2(float_to_bf16(f[6]), float_to_bf16(f[7]));
+        __syncwarp();
+        s_x[SCORE ? wid : 0][lane] = pk;
+        __syncwarp();
+        const unsigned *xw = reinterpret_cast<const unsigned *>(s_x[SCORE ? wid : 0]);
+        float zmine = 0.f;
+#pragma unroll
+        for (int tile = 0; tile < 2; tile++) {
+          if (tile * 16 >= cnt) break;
+          const int r0 = tile * 16 + gq, r1 = r0 + 8;
+          const unsigned a[4] = {r0 < cnt ? xw[r0 * 4 + t] : 0u, r1 < cnt ? xw[r1 * 4 + t] : 0u, 0u, 0u};
+          float z0 = 0.f, z1 = 0.f;
+#pragma unroll
+          for (int nb = 0; nb < 4; nb++) {
+            float c[4] = {bias[nb][0], bias[nb][1], bias[nb][0], bias[nb][1]};
+            const unsigned bf[2] = {bfrag[nb], 0u};
+            mma_16816(c, a, bf);
+            // hidden activations are rounded to BF16 before the second layer
+            const float h0 = bf16_to_float(float_to_bf16(fmaxf(c[0], 0.f)));
+            const float h1 = bf16_to_float(float_to_bf16(fmaxf(c[1], 0.f)));
+            const float h2 = bf16_to_float(float_to_bf16(fmaxf(c[2], 0.f)));
+            const float h3 = bf16_to_float(float_to_bf16(fmaxf(c[3], 0.f)));
+            z0 = fmaf(h0, w2v[nb][0], fmaf(h1, w2v[nb][1], z0));
+            z1 = fmaf(h2, w2v[nb][0], fmaf(h3, w2v[nb][1], z1));
+          }
+          z0 += __shfl_xor_sync(kFull, z0, 1);
+          z0 += __shfl_xor_sync(kFull, z0, 2);
+          z1 += __shfl_xor_sync(kFull, z1, 1);
+          z1 += __shfl_xor_sync(kFull, z1, 2);
+          // back to the entries' lanes: entry 16 tile + x comes from lane 4 (x mod 8)
+          const float a0 = __shfl_sync(kFull, z0, (lane & 7) * 4), a1 = __shfl_sync(kFull, z1, (lane & 7) * 4);
+          if (half == tile) zmine = lane & 8 ? a1 : a0;
+        }
+        if (has) {
+          const float s = 1.0f / (1.0f + expf(-(zmine + b2)));
+          if (s_out) s_out[e] = s;
+          if (q_out) q_out[e] = __float2int_rn(s * 32768.0f);
+        }
       }
+      e0 = stop;
+      __syncwarp();
+#pragma unroll
+      for (int h = 0; h < 2; h++)
+        if (own[h] >= 0) tab[own[h]] = -1;
+      __syncwarp();
     }
   }
 }
@@ -380,27 +424,24 @@ int grid_for(int64_t items, int per_block, int limit) {
   return (int)std::max<int64_t>(1, std::min<int64_t>((items + per_block - 1) / per_block, limit));
 }
 
-int features(const DGraph &g, int level, float *fout, unsigned *bout, cudaStream_t s) {
+// The entry kernel of features (fout) or scores (mlp, s_out, q_out) after the weighted degrees.
+int run_edges(const DGraph &g, int level, float *fout, const gp_mlp *mlp, float *s_out, int32_t *q_out, cudaStream_t s) {
   if (g.m == 0) return GP_OK;
   Workspace ws(s);
-  float *wdeg;
-  GP_TRY(ws.get(&wdeg, (size_t)g.n));
   const int nsm = num_sms();
-  int32_t *big;
-  unsigned *nbig;
-  GP_TRY(ws.get(&big, (size_t)g.n));
-  GP_TRY(ws.zeros(&nbig, 1));
-  (::gp::count_launch(), k_wdeg<<<grid_for(g.n * 32, 256, nsm * 8), 256, 0, s>>>(g, wdeg));
-  (::gp::count_launch(), k_list_feat_big<<<grid_for(g.n, 256, nsm * 8), 256, 0, s>>>(g, big, nbig));
+  const int64_t warps = (g.m + kSeg - 1) / kSeg;
+  unsigned long long *wsum = nullptr;
+  if (g.ew) {
+    GP_TRY(ws.zeros(&wsum, (size_t)g.n));
+    (::gp::count_launch(), k_wdeg<<<grid_for(warps, 8, nsm * 8), 256, 0, s>>>(g, wsum));
+  }
   {
-    ProfScope ps("mlp_features", s);
-    if (bout) {
-      (::gp::count_launch(), k_features<true><<<grid_for(g.n * 16, 256, nsm * 6), 256, 0, s>>>(g, level, wdeg, nullptr, bout));
-      (::gp::count_launch(), k_features_big<true><<<nsm * 8, 256, 0, s>>>(g, level, wdeg, nullptr, bout, big, nbig));
-    } else {
-      (::gp::count_launch(), k_features<false><<<grid_for(g.n * 16, 256, nsm * 6), 256, 0, s>>>(g, level, wdeg, fout, nullptr));
-      (::gp::count_launch(), k_features_big<false><<<nsm * 8, 256, 0, s>>>(g, level, wdeg, fout, nullptr, big, nbig));
-    }
+    ProfScope ps(fout ? "mlp_features" : "mlp_score_mma", s);
+    const int grid = grid_for(warps, kEdgeWarps, nsm * 16);
+    if (fout)
+      (::gp::count_launch(), k_edges<false><<<grid, kEdgeWarps * 32, 0, s>>>(g, level, wsum, fout, nullptr, nullptr, nullptr));
+    else
+      (::gp::count_launch(), k_edges<true><<<grid, kEdgeWarps * 32, 0, s>>>(g, level, wsum, nullptr, mlp, s_out, q_out));
   }
   GP_LAUNCH_CHECK();
   return GP_OK;
@@ -410,16 +451,8 @@ int features(const DGraph &g, int level, float *fout, unsigned *bout, cudaStream
 
 int mlp_score(const DGraph &g, int level, const gp_mlp *mlp, float *s_out, int32_t *q_out, cudaStream_t s) {
   if (g.m == 0) return GP_OK;
-  Workspace ws(s);
-  unsigned *fb;
-  GP_TRY(ws.get(&fb, (size_t)g.m * 4));
-  GP_TRY(features(g, level, nullptr, fb, s));
-  {
-    ProfScope ps("mlp_score_mma", s);
-    (::gp::count_launch(), k_mlp_score<<<grid_for((g.m + 15) / 16, 8, num_sms() * 8), 256, 0, s>>>(fb, g.m, mlp, s_out, q_out));
-  }
-  GP_LAUNCH_CHECK();
-  prof_add_counts("mlp_score_mma", g.m, g.m, g.m * (16 + 4 + (s_out ? 4 : 0)));
+  GP_TRY(run_edges(g, level, nullptr, mlp, s_out, q_out, s));
+  prof_add_counts("mlp_score_mma", g.m, g.m, g.m * (4 + g.ew_bytes() + (q_out ? 4 : 0) + (s_out ? 4 : 0)));
   return GP_OK;
 }
 
@@ -480,7 +513,7 @@ int gp_edge_features(const gp_graph *g, int32_t level, float *feat_out, gp_strea
     return GP_ERR_INVALID_ARG;
   }
   cudaStream_t s = (cudaStream_t)stream;
-  GP_TRY(features(make_dgraph(g), level, feat_out, nullptr, s));
+  GP_TRY(run_edges(make_dgraph(g), level, feat_out, nullptr, nullptr, nullptr, s));
   GP_CUDA(cudaStreamSynchronize(s));
   return GP_OK;
 }

@@ -153,6 +153,9 @@ struct LpProblem {
   uint8_t *mv_adm;
   int32_t *mv_of_v;  // vertex -> its proposal index in the current sub-round
   int64_t *demand;
+  // block-owned problems (k_lp_own): label weights and demand in two copies, by sub-round parity (lw and
+  // demand above are the current ones); lw_next is the copy that admitted moves update at once
+  int64_t *lw2[2], *demand2[2], *lw_next;
   uint32_t *ct, *ct2;
   unsigned long long *ck, *ck2;  // packed contest keys (large contests)
   unsigned long long *big;       // marking items of the sub-round's admitted movers of degree > kBigDeg:
@@ -517,6 +520,11 @@ __device__ __forceinline__ unsigned apply_movers_pre(const LpProblem &P, SubCoun
   }
   const unsigned am = __ballot_sync(kFull, adm);
   if (!am) return 0;
+  if (P.lw_next) {
+    const long long c = adm ? P.g.vweight(v) : 0;
+    warp_add_by_key(P.lw_next, adm, T, c);
+    warp_add_by_key(P.lw_next, adm, L0, -c);
+  }
   const bool dl = hub_deltas_on(P);
   if (!act_next && !dl) return (unsigned)__popc(am);
   const bool big = adm && deg > (dl ? kBigDegKept : kBigDeg);
@@ -855,27 +863,44 @@ __device__ __forceinline__ int group_best_unit(unsigned long long K, int L, int 
   return L;
 }
 
-template <int EW, bool LQ>
-__device__ void choose_groups(const LpProblem &P, const SubCounters &V, int lb, int nb) {
+// Where the choice finds the active vertices of a degree bin and leaves its proposals: lists of the whole
+// problem in memory with one proposal slot per position (ListBins), or a block's own vertices in its shared
+// memory with the proposals appended (OwnBins, below).
+struct ListBins {
+  const LpProblem &P;
+  const SubCounters &V;
+  __device__ __forceinline__ unsigned count(int b) const { return V.bin_count[b]; }
+  __device__ __forceinline__ void row(int b, unsigned i, int *v, int64_t *beg, int64_t *d) const {
+    *v = P.bin[b][i];
+    const unsigned long long x = P.binx[b][i];
+    *beg = (int64_t)(x >> 6);
+    *d = (int64_t)(x & 63);
+  }
+  __device__ __forceinline__ void none(int b, unsigned i) const { P.mv_t[P.bin_base[b] + i] = -1; }
+  template <bool LQ>
+  __device__ __forceinline__ void put(int b, unsigned i, int v, const Best &x, long long c0) const {
+    write_slot<LQ>(P, P.bin_base[b] + i, v, x, c0);
+  }
+};
+
+template <int EW, bool LQ, class Bins>
+__device__ __forceinline__ void choose_groups(const LpProblem &P, const Bins &B, unsigned gw, unsigned nw) {
   constexpr int U = 2;
   unsigned pre[5];
   pre[0] = 0;
 #pragma unroll
   for (int b = 0; b < 4; b++) {
     const unsigned per = (32u >> (2 + b)) * U;
-    pre[b + 1] = pre[b] + (V.bin_count[b] + per - 1) / per;
+    pre[b + 1] = pre[b] + (B.count(b) + per - 1) / per;
   }
   const unsigned total = pre[4];
   if (total == 0) return;
   const int lane = threadIdx.x & 31;
-  const unsigned gw = (unsigned)lb * kWarps + (threadIdx.x >> 5), nw = (unsigned)nb * kWarps;
   for (unsigned j = gw; j < total; j += nw) {
     const int bin = (j >= pre[1]) + (j >= pre[2]) + (j >= pre[3]);
     const int G = 4 << bin;
     const unsigned gpw = 32u >> (2 + bin);
-    const unsigned cnt = V.bin_count[bin];
-    const int32_t *list = P.bin[bin];
-    const unsigned long long *listx = P.binx[bin];
+    const unsigned cnt = B.count(bin);
     const int gl = lane & (G - 1);
     const unsigned sub = (unsigned)lane / (unsigned)G;
     const unsigned base = (j - pre[bin]) * gpw * U;
@@ -891,12 +916,7 @@ __device__ void choose_groups(const LpProblem &P, const SubCounters &V, int lb, 
       v[u] = 0;
       beg[u] = 0;
       d[u] = 0;
-      if (valid[u]) {
-        v[u] = list[i];
-        const unsigned long long x = listx[i];
-        beg[u] = (int64_t)(x >> 6);
-        d[u] = (int64_t)(x & 63);
-      }
+      if (valid[u]) B.row(bin, i, &v[u], &beg[u], &d[u]);
     }
 #pragma unroll
     for (int u = 0; u < U; u++) {
@@ -958,7 +978,7 @@ __device__ void choose_groups(const LpProblem &P, const SubCounters &V, int lb, 
       if (!__any_sync(kFull, cand[u])) {
         // no lane of the warp has a candidate (every vertex keeps its label, the common case once
         // clusters or blocks settle): only the empty proposals are recorded
-        if (valid[u] && gl == 0) P.mv_t[P.bin_base[bin] + base + u * gpw + sub] = -1;
+        if (valid[u] && gl == 0) B.none(bin, base + u * gpw + sub);
         continue;
       }
       if constexpr (EW == 0 && !LQ) {
@@ -986,7 +1006,7 @@ __device__ void choose_groups(const LpProblem &P, const SubCounters &V, int lb, 
         b = group_best_rt<LQ>(b, G);
       }
       const bool mover = valid[u] && gl == 0 && b.L >= 0;
-      if (valid[u] && gl == 0) write_slot<LQ>(P, P.bin_base[bin] + base + u * gpw + sub, v[u], b, c0[u]);
+      if (valid[u] && gl == 0) B.template put<LQ>(bin, base + u * gpw + sub, v[u], b, c0[u]);
       // (at most one mover per group: equal targets within a warp are rare, so no aggregation)
       if (mover) atomicAdd(reinterpret_cast<unsigned long long *>(&P.demand[b.L]), (unsigned long long)cv[u]);
     }
@@ -2359,7 +2379,7 @@ __device__ bool lp_problem(const LpProblem *prob, unsigned char *dsm) {
         // while block 0 prepares the hub list, the other blocks take its share of the choice
         const int clb = (hubs_now && nb > 1) ? lb - 1 : lb, cnb = (hubs_now && nb > 1) ? nb - 1 : nb;
         if (clb >= 0) {
-          choose_groups<EW, LQ>(P, sV, clb, cnb);
+          choose_groups<EW, LQ>(P, ListBins{P, sV}, (unsigned)clb * kWarps + (threadIdx.x >> 5), (unsigned)cnb * kWarps);
           choose_warp<EW, TB>(P, sV, clb, cnb, dsm, direct);
           choose_cta<EW, TB>(P, sV, clb, cnb, dsm, sm, direct);
         }
@@ -2453,6 +2473,413 @@ __global__ void __launch_bounds__(kThreads, 4) k_lp(const LpProblem *probs, cons
   extern __shared__ __align__(16) unsigned char dsm[];
   for (int q = blk_start[blockIdx.x]; q < blk_start[blockIdx.x + 1]; q++)
     if (!lp_problem<EW, TB>(probs + blk_list[q], dsm)) return;
+}
+
+// ------------------------------------------------------------------------------------ block-owned problems
+// Graphs without a vertex of degree above kOwnDeg (meshes and their coarse levels, mostly) run without
+// problem-wide lists: a block owns a contiguous range of vertices, finds its active ones itself, chooses for
+// them at once, keeps its proposals and admits them. A sub-round then has two grid barriers instead of three
+//     replay + classify + choose | admit + apply (| contest)
+// and neither lists nor proposals of vertices without one travel through memory. What the third barrier
+// separated is kept apart by copies instead: the label weights exist twice. Sub-round t reads copy t & 1;
+// its admitted moves update the other copy at once and are replayed on the first one (by their block, in the
+// choice phase of t + 1, when nobody reads it). The demand counters alternate likewise.
+// These problems are bound by the dependent loads and the barriers of each phase: a sub-round of RGG 2^20 is
+// about 12 us of which half is work; the list form, which balances the work of unequal rows over all
+// blocks, stays for the graphs with longer rows.
+constexpr int kOwnDeg = 128;    // longest row (half of a warp's table)
+constexpr int kOwnTile = 2048;  // vertices classified at a time (kOwnPer per thread)
+constexpr int kOwnPer = kOwnTile / kThreads;
+constexpr int kOwnKeep = 512;   // proposals kept in shared memory beside their slots
+constexpr int kOwnCap = 2 * kOwnDeg;  // table slots per warp
+static_assert(kOwnPer == 8, "a thread's flags are one 64-bit word");
+template <bool LQ>
+constexpr int kOwnListOff = kWarps * kOwnCap * (LQ ? 16 : 12);
+template <bool LQ>
+constexpr size_t kOwnSmem = std::max<size_t>(kOwnListOff<LQ> + kOwnTile * 6, kContestSmall * 8);
+
+struct OwnProps {
+  int v[kOwnKeep], t[kOwnKeep];
+  unsigned n;
+};
+
+struct OwnBins {
+  const LpProblem &P;
+  OwnProps &O;
+  const unsigned *start;       // first list position of every bin (6 entries: G4..G32, WARP, end)
+  const unsigned short *list;  // vertices of the tile, by bin
+  const unsigned *rowx;        // per vertex of the tile: (row begin - tile's first row begin) << 8 | degree
+  int t0;                      // first vertex of the tile
+  int64_t r0;                  // its row begin
+  int64_t slot0;               // first proposal slot of the block
+  __device__ __forceinline__ unsigned count(int b) const { return start[b + 1] - start[b]; }
+  __device__ __forceinline__ void row(int b, unsigned i, int *v, int64_t *beg, int64_t *d) const {
+    const unsigned x = list[start[b] + i], y = rowx[x];
+    *v = t0 + (int)x;
+    *beg = r0 + (int64_t)(y >> 8);
+    *d = (int64_t)(y & 255u);
+  }
+  __device__ __forceinline__ void none(int, unsigned) const {}
+  template <bool LQ>
+  __device__ __forceinline__ void put(int, unsigned, int v, const Best &x, long long c0) const {
+    if (x.L < 0) return;
+    const unsigned pos = atomicAdd(&O.n, 1u);
+    if (pos < kOwnKeep) {
+      O.v[pos] = v;
+      O.t[pos] = x.L;
+    }
+    write_slot<LQ>(P, slot0 + pos, v, x, c0);
+  }
+};
+
+// One warp per vertex with 32 < d <= kOwnDeg, table in shared memory.
+template <int EW, bool LQ>
+__device__ __forceinline__ void choose_own_warp(const LpProblem &P, const OwnBins &B, unsigned char *dsm) {
+  const unsigned cnt = B.count(4);
+  if (cnt == 0) return;
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  unsigned long long *vals = reinterpret_cast<unsigned long long *>(dsm) + wid * kOwnCap;
+  int *keys = reinterpret_cast<int *>(dsm + kWarps * kOwnCap * 8) + wid * kOwnCap;
+  unsigned *qv = reinterpret_cast<unsigned *>(dsm + kWarps * kOwnCap * 12) + wid * kOwnCap;
+  for (int s = lane; s < kOwnCap; s += 32) {
+    keys[s] = -1;
+    vals[s] = 0;
+    if (LQ) qv[s] = 0;
+  }
+  __syncwarp();
+  for (unsigned i = wid; i < cnt; i += kWarps) {
+    int v;
+    int64_t beg, d;
+    B.row(4, i, &v, &beg, &d);
+    const unsigned cap = d <= 64 ? 128 : 256, mask = cap - 1;
+    const int L0 = P.labels[P.vbase + v];
+    long long c0 = 0;
+    bool other = false;
+    for (int64_t x0 = 0; x0 < d; x0 += 32) {
+      const int64_t e = beg + x0 + lane;
+      const bool in = x0 + lane < d;
+      const int L = in ? P.labels[__ldg(P.g.adj + e)] : -1;
+      const long long w = in ? load_ew<EW>(P.g.ew, e) : 0;
+      if (in && L == L0) c0 += w;
+      other |= in && L != L0;
+      warp_insert<EW, LQ>(keys, vals, qv, mask, in && L != L0, L, w, (LQ && in) ? (unsigned)__ldg(P.q + e) : 0u,
+                          P.ctr, 8);
+    }
+    if (!__any_sync(kFull, other)) continue;  // every neighbour carries the own label; the table is still empty
+    c0 = warp_sum64(c0);
+    __syncwarp();
+    const long long cv = P.g.vweight(v);
+    Best b = no_best();
+    for (unsigned s = lane; s < cap; s += 32) {
+      const int L = keys[s];
+      if (L >= 0) {
+        const Best x = make_cand(P, v, L, L0, (long long)vals[s], LQ ? (long long)qv[s] : 0, c0, cv);
+        if (better(x, b)) b = x;
+        keys[s] = -1;
+        vals[s] = 0;
+        if (LQ) qv[s] = 0;
+      }
+    }
+    __syncwarp();
+    b = group_best<LQ, 32>(b);
+    if (lane == 0 && b.L >= 0) {
+      B.template put<LQ>(4, i, v, b, c0);
+      atomicAdd(reinterpret_cast<unsigned long long *>(&P.demand[b.L]), (unsigned long long)cv);
+    }
+  }
+}
+
+// The block's moves of the previous sub-round on the label weights that sub-round read, and its demand
+// cleared.
+__device__ __forceinline__ void replay_own(const LpProblem &P, const OwnProps &O, int64_t *old_demand, int64_t slot0) {
+  for (unsigned base = 0; base < O.n; base += kThreads) {
+    const unsigned k = base + threadIdx.x;
+    int T = -1, v = 0, L0 = -1;
+    bool adm = false;
+    if (k < O.n) {
+      T = k < kOwnKeep ? O.t[k] : P.mv_t[slot0 + k];
+      v = k < kOwnKeep ? O.v[k] : P.mv_v[slot0 + k];
+      adm = P.mv_adm[slot0 + k] != 0;
+      L0 = P.mv_from[slot0 + k];
+      old_demand[T] = 0;
+    }
+    const long long c = adm ? P.g.vweight(v) : 0;
+    warp_add_by_key(P.lw_next, adm, T, c);
+    warp_add_by_key(P.lw_next, adm, adm ? L0 : -1, -c);
+  }
+}
+
+// The active vertices of one tile by degree bin. Returns the tile's active count (degree-0 ones, which take
+// no part in the choice, only count as visits).
+__device__ __forceinline__ unsigned classify_own(const LpProblem &P, const uint8_t *act, uint8_t *act_clear, int r, int s,
+                                                 uint64_t rmix, int t0, int t1, int64_t r0, unsigned *start,
+                                                 unsigned short *list, unsigned *rowx, Smem &sm) {
+  const int v0 = t0 + (int)threadIdx.x * kOwnPer;  // (act + vbase and t0 are multiples of 8 from the allocation)
+  unsigned flag = 0;
+  if (v0 < t1) {
+    if (r == 0) {
+      flag = 0xffu;
+    } else {
+      const uint64_t f = *reinterpret_cast<const uint64_t *>(act + P.vbase + v0);
+#pragma unroll
+      for (int i = 0; i < kOwnPer; i++) flag |= ((unsigned)(f >> (8 * i)) & 1u) << i;
+    }
+    if (s == 0) *reinterpret_cast<uint64_t *>(act_clear + P.vbase + v0) = 0;
+    if (t1 - v0 < kOwnPer) flag &= (1u << (t1 - v0)) - 1u;
+  }
+#pragma unroll
+  for (int i = 0; i < kOwnPer; i++)
+    if ((flag >> i & 1u) && (int)(mix64(rmix ^ (uint64_t)(v0 + i)) >> 63) != s) flag &= ~(1u << i);
+  int64_t rb[kOwnPer];
+  int dd[kOwnPer];
+#pragma unroll
+  for (int i = 0; i < kOwnPer; i++) {
+    rb[i] = 0;
+    dd[i] = 0;
+    if (flag >> i & 1u) {
+      rb[i] = P.g.row_begin(v0 + i);
+      dd[i] = (int)(P.g.row_begin(v0 + i + 1) - rb[i]);
+    }
+  }
+  // counts per bin, 12 bits each
+  unsigned long long mine = 0;
+  unsigned edges = 0;
+#pragma unroll
+  for (int i = 0; i < kOwnPer; i++) {
+    if (dd[i] > 0) {
+      mine += 1ull << (12 * bin_of(dd[i], kOwnDeg, kOwnDeg));
+      edges += (unsigned)dd[i];
+    }
+  }
+  const unsigned wact = warp_sum_u32((unsigned)__popc(flag)), wedg = warp_sum_u32(edges);
+  if ((threadIdx.x & 31) == 0 && wact) {
+    atomicAdd(&sm.vis[0], (unsigned long long)wact);
+    atomicAdd(&sm.edg[0], (unsigned long long)wedg);
+  }
+  long long total;
+  const unsigned long long at = (unsigned long long)block_excl_scan64((long long)mine, sm.tmp, &sm.tot);
+  total = sm.tot;
+  unsigned st[6];
+  st[0] = 0;
+#pragma unroll
+  for (int b = 0; b < 5; b++) st[b + 1] = st[b] + (unsigned)(total >> (12 * b) & 0xfff);
+  if (threadIdx.x < 6) start[threadIdx.x] = st[threadIdx.x];
+  unsigned long long pos = at;
+#pragma unroll
+  for (int i = 0; i < kOwnPer; i++) {
+    if (dd[i] > 0) {
+      const int b = bin_of(dd[i], kOwnDeg, kOwnDeg);
+      const unsigned x = threadIdx.x * kOwnPer + i;
+      unsigned sb = 0;
+#pragma unroll
+      for (int y = 1; y < 5; y++) sb = b == y ? st[y] : sb;
+      list[sb + (unsigned)(pos >> (12 * b) & 0xfff)] = (unsigned short)x;
+      rowx[x] = (unsigned)(rb[i] - r0) << 8 | (unsigned)dd[i];
+      pos += 1ull << (12 * b);
+    }
+  }
+  __syncthreads();
+  return st[5];
+}
+
+// Admission of the block's proposals; the ones whose target cannot take all of its demand are contested.
+template <bool LQ>
+__device__ __forceinline__ void admit_own(const LpProblem &P, SubCounters &C, const OwnProps &O, int r, int64_t slot0,
+                                          Smem &sm) {
+  unsigned long long mg = 0, mq = 0;
+  unsigned moved = 0;
+  uint8_t *act_next = r + 1 < P.rounds ? P.act[(r + 1) & 1] : nullptr;  // (no marks in the last round)
+  for (unsigned base = 0; base < O.n; base += kThreads) {
+    const unsigned k = base + threadIdx.x;
+    bool contested = false, adm = false;
+    int T = -1, v = 0, L0 = 0;
+    int64_t rb = 0, deg = 0;
+    const int64_t i = slot0 + k;
+    if (k < O.n) {
+      T = k < kOwnKeep ? O.t[k] : P.mv_t[i];
+      v = k < kOwnKeep ? O.v[k] : P.mv_v[i];
+      const long long lwT = P.lw[T], dT = P.demand[T];
+      L0 = P.labels[P.vbase + v];
+      rb = P.g.row_begin(v);
+      deg = P.g.row_begin(v + 1) - rb;
+      if (lwT + dT <= P.U) {
+        adm = true;
+        P.mv_adm[i] = 1;
+      } else {
+        contested = true;
+        mg = max(mg, (unsigned long long)P.mv_gain[i]);
+        if (LQ) mq = max(mq, (unsigned long long)P.mv_q[i]);
+      }
+    }
+    moved += apply_movers_pre(P, C, act_next, adm, i, v, T, L0, rb, deg);
+    const unsigned pos = warp_append(&C.n_contested, contested);
+    if (contested) P.ct[pos] = (unsigned)i;
+  }
+  if (O.n == 0) return;
+  if ((threadIdx.x & 31) == 0 && moved) atomicAdd(&sm.moves, (unsigned long long)moved);
+  for (int o = 16; o > 0; o >>= 1) {
+    mg = max(mg, __shfl_xor_sync(kFull, mg, o));
+    mq = max(mq, __shfl_xor_sync(kFull, mq, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    if (mg) atomicMax(&C.max_gain, mg);
+    if (LQ && mq) atomicMax(&C.max_q, mq);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    sm.movers += O.n;
+    if (sm.moves) {
+      atomicAdd(&P.ctr->moves_round[r & 1], sm.moves);
+      sm.moves = 0;
+    }
+  }
+}
+
+template <int EW, bool LQ>
+__device__ bool lp_problem_own(const LpProblem *prob, unsigned char *dsm) {
+  __shared__ __align__(16) unsigned char p_raw[sizeof(LpProblem)];
+  __shared__ Smem sm;
+  __shared__ OwnProps O;
+  __shared__ unsigned s_start[6];
+  __shared__ SubCounters sV;
+  __shared__ unsigned long long s_mr;
+  LpProblem &P = *reinterpret_cast<LpProblem *>(p_raw);
+  unsigned short *const list = reinterpret_cast<unsigned short *>(dsm + kOwnListOff<LQ> + kOwnTile * 4);
+  unsigned *const rowx = reinterpret_cast<unsigned *>(dsm + kOwnListOff<LQ>);
+  __syncthreads();  // the block's previous problem is done with the shared state
+  {
+    const unsigned *src = reinterpret_cast<const unsigned *>(prob);
+    unsigned *dst = reinterpret_cast<unsigned *>(p_raw);
+    for (unsigned i = threadIdx.x; i < sizeof(LpProblem) / 4; i += kThreads) dst[i] = src[i];
+  }
+  if (threadIdx.x < 8) {
+    sm.vis[threadIdx.x] = 0;
+    sm.edg[threadIdx.x] = 0;
+  }
+  if (threadIdx.x == 0) {
+    sm.moves = 0;
+    sm.movers = 0;
+    O.n = 0;
+  }
+  __syncthreads();
+  const int lb = (int)blockIdx.x - P.block_begin, nb = P.block_count;
+  LpCounters *ctr = P.ctr;
+#define bar (GridBarrier{P.bar, &P.ctr->err, (unsigned)nb, (unsigned)lb, P.wait_us})
+  __shared__ unsigned long long pacc[8];
+  if (threadIdx.x < 8) pacc[threadIdx.x] = 0;
+  unsigned long long tmark = 0;
+  auto tick = [&](int phase) {
+    if (lb == 0 && threadIdx.x == 0) {
+      const unsigned long long now = global_ns();
+      if (phase >= 0) pacc[phase] += now - tmark;
+      tmark = now;
+    }
+  };
+  const int64_t n = P.g.n;
+  const int64_t chunk = ((n + nb - 1) / nb + kOwnPer - 1) / kOwnPer * kOwnPer;
+  const int64_t lo = min(n, (int64_t)lb * chunk), hi = min(n, lo + chunk);
+  // the second copies start as the first (label weights) and as zero (demand)
+  for (int64_t x = P.lbase + (int64_t)lb * kThreads + threadIdx.x; x < P.lbase + P.nl; x += (int64_t)nb * kThreads) {
+    P.lw2[1][x] = P.lw2[0][x];
+    P.demand2[1][x] = 0;
+  }
+  tick(-1);
+  int t_last = -1;
+  for (int r = 0; r < P.rounds; r++) {
+    const uint64_t rmix = mix64(P.smix ^ (uint64_t)r);
+    for (int s = 0; s < 2; s++) {
+      const int t = 2 * r + s;
+      SubCounters &C = ctr->sc[t % 3];
+      SubCounters &Cn = ctr->sc[(t + 1) % 3];
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        P.lw = P.lw2[t & 1];
+        P.lw_next = P.lw2[(t + 1) & 1];
+        P.demand = P.demand2[t & 1];
+        P.sub_t = t;
+        if (lb == 0) {
+          // counter set t+1 was last used by sub-round t-2, which every block has finished
+          Cn.n_contested = 0;
+          Cn.n_big = 0;
+          Cn.max_gain = 0;
+          Cn.max_q = 0;
+        }
+      }
+      __syncthreads();
+      if (t > 0) {
+        replay_own(P, O, P.demand2[(t + 1) & 1], lo);
+        __syncthreads();
+        if (threadIdx.x == 0) O.n = 0;
+      }
+      t_last = t;
+      for (int64_t t0 = lo; t0 < hi; t0 += kOwnTile) {
+        const int64_t r0 = P.g.row_begin(t0);
+        const unsigned na = classify_own(P, P.act[r & 1], P.act[(r + 1) & 1], r, s, rmix, (int)t0,
+                                         (int)min(hi, t0 + kOwnTile), r0, s_start, list, rowx, sm);
+        if (na == 0) continue;
+        const OwnBins B{P, O, s_start, list, rowx, (int)t0, r0, lo};
+        choose_groups<EW, LQ>(P, B, threadIdx.x >> 5, kWarps);
+        choose_own_warp<EW, LQ>(P, B, dsm);
+        __syncthreads();
+      }
+      if (!grid_sync(bar)) return false;
+      tick(1);
+      if (lb == 0 && threadIdx.x == 0 && s == 0) ctr->moves_round[(r + 1) & 1] = 0;
+      admit_own<LQ>(P, C, O, r, lo, sm);
+      if (!grid_sync(bar)) return false;
+      // contested count and key ranges; the round's move count
+      if (threadIdx.x < sizeof(SubCounters) / 4)
+        reinterpret_cast<unsigned *>(&sV)[threadIdx.x] = reinterpret_cast<const volatile unsigned *>(&C)[threadIdx.x];
+      if (threadIdx.x == kThreads - 1) s_mr = *(volatile unsigned long long *)&ctr->moves_round[r & 1];
+      __syncthreads();
+      tick(3);
+      const unsigned nc = sV.n_contested;
+      if (nc > 0) {
+        if (nc <= kContestSmall) {
+          if (lb == 0) contest_small<LQ>(P, sV, &C, nc, r, dsm, sm);
+        } else {
+          if (!contest_large<LQ>(P, sV, &C, nc, r, lb, nb, bar, sm, dsm)) return false;
+        }
+        if (!grid_sync(bar)) return false;
+        if (threadIdx.x == 0) s_mr = *(volatile unsigned long long *)&ctr->moves_round[r & 1];
+        __syncthreads();
+        tick(4);
+      }
+    }
+    const unsigned long long mr = s_mr;
+    if (lb == 0 && threadIdx.x == 0) {
+      ctr->rounds += 1;
+      ctr->moves += mr;
+    }
+    if (mr == 0) break;
+  }
+  // the last sub-round's moves on the copy it read: both copies are final then
+  if (t_last >= 0) {
+    __syncthreads();
+    if (threadIdx.x == 0) P.lw_next = P.lw2[t_last & 1];
+    __syncthreads();
+    replay_own(P, O, P.demand2[t_last & 1], lo);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (sm.vis[0]) atomicAdd(&ctr->bin_visits[0], sm.vis[0]);
+    if (sm.edg[0]) atomicAdd(&ctr->bin_edges[0], sm.edg[0]);
+    if (sm.movers) atomicAdd(&ctr->movers, sm.movers);
+  }
+  tick(5);
+  if (lb == 0 && threadIdx.x == 0)
+    for (int k = 0; k < 8; k++) ctr->phase_ns[k] = pacc[k];
+  return true;
+}
+
+#undef bar
+
+template <int EW, bool LQ>
+__global__ void __launch_bounds__(kThreads, 4) k_lp_own(const LpProblem *probs, const int *blk_start,
+                                                        const int *blk_list) {
+  extern __shared__ __align__(16) unsigned char dsm[];
+  for (int q = blk_start[blockIdx.x]; q < blk_start[blockIdx.x + 1]; q++)
+    if (!lp_problem_own<EW, LQ>(probs + blk_list[q], dsm)) return;
 }
 
 // ------------------------------------------------------------------------------------ host helpers
@@ -2583,6 +3010,34 @@ int max_coop_blocks(int *out) {
     cached[EW][TB] = std::max(1, per_sm);
   }
   *out = cached[EW][TB] * num_sms();
+  return GP_OK;
+}
+
+template <int EW, bool LQ>
+int max_coop_blocks_own(int *out) {
+  static int cached[3][2] = {{0, 0}, {0, 0}, {0, 0}};
+  if (!cached[EW][LQ]) {
+    GP_CUDA(cudaFuncSetAttribute(k_lp_own<EW, LQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOwnSmem<LQ>));
+    int per_sm = 0;
+    GP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lp_own<EW, LQ>, kThreads, kOwnSmem<LQ>));
+    cached[EW][LQ] = std::max(1, per_sm);
+  }
+  *out = cached[EW][LQ] * num_sms();
+  return GP_OK;
+}
+
+template <bool LQ>
+int coop_capacity_own(int ew, int *out) {
+  return ew == 0 ? max_coop_blocks_own<0, LQ>(out) : ew == 1 ? max_coop_blocks_own<1, LQ>(out) : max_coop_blocks_own<2, LQ>(out);
+}
+
+template <bool LQ>
+int launch_lp_own(int ew, const LpProblem *probs_dev, const int *blk_start_dev, const int *blk_list_dev, int grid,
+                  cudaStream_t s) {
+  count_launch();
+  void *args[] = {(void *)&probs_dev, (void *)&blk_start_dev, (void *)&blk_list_dev};
+  void *k = ew == 0 ? (void *)k_lp_own<0, LQ> : ew == 1 ? (void *)k_lp_own<1, LQ> : (void *)k_lp_own<2, LQ>;
+  GP_CUDA(cudaLaunchCooperativeKernel(k, grid, kThreads, args, kOwnSmem<LQ>, s));
   return GP_OK;
 }
 
@@ -2868,8 +3323,14 @@ int run_lp_multi(const LpJob *jobs, int njobs, cudaStream_t s, const LpConfig &c
   for (int j = 0; j < njobs; j++) wide = wide || hhub[3 * (size_t)j + 2] > 0;
   const int tb = lq ? 0 : (wide ? 2 : 1);
   if (tb == 1) cfg.deg_cta = std::max(cfg.deg_warp, std::min(cfg.deg_cta, kCtaCapT<1> / 2));
+  // Block-owned form (see k_lp_own): every row of the launch fits a warp's table, so that a block's share of
+  // vertices is about its share of work. One longer row and the list form takes the launch: it spreads long
+  // rows over blocks.
+  bool own = cfg.deg_warp <= kOwnDeg;
+  for (int j = 0; j < njobs; j++) own = own && hcls[9 * (size_t)j + 5] == 0 && hcls[9 * (size_t)j + 6] == 0;
   int cap_blocks = 0;
-  GP_TRY(coop_capacity(ew, tb, &cap_blocks));
+  GP_TRY(own ? (lq ? coop_capacity_own<true>(ew, &cap_blocks) : coop_capacity_own<false>(ew, &cap_blocks))
+             : coop_capacity(ew, tb, &cap_blocks));
   // Blocks: a job gets at most one block per cfg.verts_per_block vertices. When all jobs fit the co-resident
   // capacity that way, they do; otherwise work is balanced by a cost model (entries + 4 per vertex
   // + a fixed per-problem latency term): jobs above twice the mean block load get several blocks,
@@ -2970,6 +3431,13 @@ int run_lp_multi(const LpJob *jobs, int njobs, cudaStream_t s, const LpConfig &c
     for (int j = 0; j < njobs; j++) total += (size_t)std::max<int64_t>(jobs[j].nl, 1);
     GP_TRY(ws.zeros(&demand_all, total));
   }
+  int64_t *lw2_all = nullptr, *demand2_all = nullptr;
+  if (own) {
+    size_t total = 0;
+    for (int j = 0; j < njobs; j++) total += (size_t)std::max<int64_t>(jobs[j].nl, 1);
+    GP_TRY(ws.get(&lw2_all, total));
+    GP_TRY(ws.get(&demand2_all, total));
+  }
   size_t demand_off = 0;
   int64_t keep_total = 0;  // slots of the kept hub tables of the launch
   for (int j = 0; j < njobs; j++) {
@@ -3000,7 +3468,7 @@ int run_lp_multi(const LpJob *jobs, int njobs, cudaStream_t s, const LpConfig &c
     P.block_count = nblk[j];
     const size_t n = (size_t)std::max<int64_t>(jb.g.n, 1);
     int64_t slots_total = 0;
-    for (int b = 0; b < kBins; b++) {
+    for (int b = 0; b < kBins && !own; b++) {
       GP_TRY(ws.get(&P.bin[b], (size_t)std::max<unsigned>(hcls[9 * j + b], 1)));
       if (b < 4) GP_TRY(ws.get(&P.binx[b], (size_t)std::max<unsigned>(hcls[9 * j + b], 1)));
       P.bin_base[b] = slots_total;
@@ -3014,6 +3482,12 @@ int run_lp_multi(const LpJob *jobs, int njobs, cudaStream_t s, const LpConfig &c
     GP_TRY(ws.get(&P.mv_adm, n));
     GP_TRY(ws.get(&P.mv_of_v, n));
     P.demand = demand_all + demand_off - jb.lbase;  // indexed by global label
+    if (own) {
+      P.lw2[0] = jb.lw;
+      P.lw2[1] = lw2_all + demand_off - jb.lbase;
+      P.demand2[0] = P.demand;
+      P.demand2[1] = demand2_all + demand_off - jb.lbase;
+    }
     demand_off += (size_t)std::max<int64_t>(jb.nl, 1);
     GP_TRY(ws.get(&P.ct, n));
     GP_TRY(ws.get(&P.ct2, n));
@@ -3025,8 +3499,9 @@ int run_lp_multi(const LpJob *jobs, int njobs, cudaStream_t s, const LpConfig &c
     static_assert(kBigChunkKept <= kBigChunk, "the kept-table items bound the others");
     GP_TRY(ws.get(&P.big,
                   (size_t)(hent[j] / kBigChunkKept + hcls[9 * j + 4] + hcls[9 * j + 5] + hcls[9 * j + 6] + 1)));
-    GP_TRY(ws.get(&P.act[0], n));
-    GP_TRY(ws.get(&P.act[1], n));
+    // (the block-owned form reads the flags eight at a time)
+    GP_TRY(ws.get(&P.act[0], (n + 7) & ~(size_t)7));
+    GP_TRY(ws.get(&P.act[1], (n + 7) & ~(size_t)7));
     P.act[0] -= jb.vbase;  // indexed by global vertex id
     P.act[1] -= jb.vbase;
     GP_TRY(ws.get(&P.hist, (size_t)nblk[j] * 256 + 16));
@@ -3098,7 +3573,9 @@ int run_lp_multi(const LpJob *jobs, int njobs, cudaStream_t s, const LpConfig &c
   {
     ProfScope ps(jobs[0].prof, s);
     int st;
-    if (tb == 0) st = launch_lp_tb<0>(ew, probs_dev, bs_dev, bl_dev, grid, s);
+    if (own) st = lq ? launch_lp_own<true>(ew, probs_dev, bs_dev, bl_dev, grid, s)
+                     : launch_lp_own<false>(ew, probs_dev, bs_dev, bl_dev, grid, s);
+    else if (tb == 0) st = launch_lp_tb<0>(ew, probs_dev, bs_dev, bl_dev, grid, s);
     else if (tb == 1) st = launch_lp_tb<1>(ew, probs_dev, bs_dev, bl_dev, grid, s);
     else st = launch_lp_tb<2>(ew, probs_dev, bs_dev, bl_dev, grid, s);
     GP_TRY(st);

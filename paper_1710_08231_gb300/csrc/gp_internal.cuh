@@ -264,7 +264,7 @@ __device__ __forceinline__ T block_excl_scan64(T x, T *tmp, T *total) {
 // global timer (or that sees another block's timeout) stores GP_ERR_TIMEOUT in `err` and returns false,
 // and so does every other waiting block once it sees the flag, so the kernel ends with every block
 // returned and the host reads the status.
-constexpr unsigned kBarrierStride = 32;
+constexpr unsigned kBarrierStride = 64;
 inline unsigned barrier_words(unsigned) { return kBarrierStride; }
 constexpr unsigned long long kDefaultWaitNs = 20ull * 1000 * 1000 * 1000;  // 20 s
 // Process-wide limit of every bounded device wait (host setting, copied into each launch's arguments).

@@ -2496,25 +2496,41 @@ static_assert(kOwnPer == 8, "a thread's flags are one 64-bit word");
 template <bool LQ>
 constexpr int kOwnListOff = kWarps * kOwnCap * (LQ ? 16 : 12);
 template <bool LQ>
-constexpr size_t kOwnSmem = std::max<size_t>(kOwnListOff<LQ> + kOwnTile * 6, kContestSmall * 8);
+constexpr int kOwnRowOff = kOwnListOff<LQ> + kOwnTile * 4;  // (the rows outlive a contest, which takes 32 KB)
+template <bool LQ>
+constexpr size_t kOwnSmem = kOwnRowOff<LQ> + kOwnTile * 4;
+static_assert(kOwnRowOff<false> >= kContestSmall * 8, "the rows lie behind the contest's keys");
+// A bin of up to this many vertices goes to lane groups, a longer one to a thread per vertex: the groups take
+// one vertex through in the least time (four steps of 16 vertices at most here), the threads take many through
+// with fewer instructions and more loads in flight.
+constexpr unsigned kOwnRowsMin = 64;
 
 struct OwnProps {
   int v[kOwnKeep], t[kOwnKeep];
-  unsigned n;
+  unsigned n[2];  // proposals by sub-round parity
+  unsigned cur;   // parity of the running sub-round
 };
 
+// The active vertices of a tile. Four bins: 1: d <= 8, 2: d <= 16, 3: d <= 32, 4: d <= kOwnDeg (bin 0 is part
+// of bin 1 here); bins 1 and 2 grow towards each other in the first half of the list, 3 and 4 in the second.
 struct OwnBins {
   const LpProblem &P;
   OwnProps &O;
-  const unsigned *start;       // first list position of every bin (6 entries: G4..G32, WARP, end)
-  const unsigned short *list;  // vertices of the tile, by bin
-  const unsigned *rowx;        // per vertex of the tile: (row begin - tile's first row begin) << 8 | degree
+  unsigned long long counts;   // 16 bits per bin from bin 1 on
+  unsigned short *list;        // vertices of the tile, 2 kOwnTile entries
+  unsigned *rowx;              // per vertex of the tile: (row begin - tile's first row begin) << 8 | degree
   int t0;                      // first vertex of the tile
   int64_t r0;                  // its row begin
   int64_t slot0;               // first proposal slot of the block
-  __device__ __forceinline__ unsigned count(int b) const { return start[b + 1] - start[b]; }
+  __device__ __forceinline__ static int bin(int d) { return d <= 8 ? 1 : d <= 16 ? 2 : d <= 32 ? 3 : 4; }
+  __device__ __forceinline__ static unsigned at(int b, unsigned i) {
+    return (b < 3 ? 0u : (unsigned)kOwnTile) + (b & 1 ? i : (unsigned)kOwnTile - 1u - i);
+  }
+  __device__ __forceinline__ unsigned count(int b) const {
+    return b ? (unsigned)(counts >> (16 * (b - 1))) & 0xffffu : 0u;
+  }
   __device__ __forceinline__ void row(int b, unsigned i, int *v, int64_t *beg, int64_t *d) const {
-    const unsigned x = list[start[b] + i], y = rowx[x];
+    const unsigned x = list[at(b, i)], y = rowx[x];
     *v = t0 + (int)x;
     *beg = r0 + (int64_t)(y >> 8);
     *d = (int64_t)(y & 255u);
@@ -2523,7 +2539,7 @@ struct OwnBins {
   template <bool LQ>
   __device__ __forceinline__ void put(int, unsigned, int v, const Best &x, long long c0) const {
     if (x.L < 0) return;
-    const unsigned pos = atomicAdd(&O.n, 1u);
+    const unsigned pos = atomicAdd(&O.n[O.cur], 1u);
     if (pos < kOwnKeep) {
       O.v[pos] = v;
       O.t[pos] = x.L;
@@ -2531,6 +2547,125 @@ struct OwnBins {
     write_slot<LQ>(P, slot0 + pos, v, x, c0);
   }
 };
+
+// One thread per vertex with any weights (the sums of choose_own_rows are 32 bits wide): the row is read again
+// for every neighbour.
+template <int EW>
+__device__ __noinline__ void choose_own_wide(const LpProblem &P, const OwnBins &B, int v, int64_t beg, int d, int L0,
+                                             long long cv) {
+  long long c0 = 0;
+  for (int i = 0; i < d; i++)
+    if (P.labels[__ldg(P.g.adj + beg + i)] == L0) c0 += load_ew<EW>(P.g.ew, beg + i);
+  Best b = no_best();
+  for (int i = 0; i < d; i++) {
+    const int L = P.labels[__ldg(P.g.adj + beg + i)];
+    if (L == L0) continue;
+    long long c = 0;
+    for (int j = 0; j < d; j++)
+      if (P.labels[__ldg(P.g.adj + beg + j)] == L) c += load_ew<EW>(P.g.ew, beg + j);
+    const Best x = make_cand(P, v, L, L0, c, 0, c0, cv);
+    if (better(x, b)) b = x;
+  }
+  if (b.L < 0) return;
+  B.template put<false>(0, 0, v, b, c0);
+  atomicAdd(reinterpret_cast<unsigned long long *>(&P.demand[b.L]), (unsigned long long)cv);
+}
+
+// One thread per vertex with at most D neighbours (bin `bin`), all of their labels in registers. A thread has
+// up to D label gathers in flight (a lane group has one per lane), which is what hides their latency, and the
+// connections take D^2 compares of registers for 32 vertices at a time instead of a match, reductions and
+// votes for two. Only the label that wins is looked up in the label weights; when it has no room, it is taken
+// out and the next one wins.
+template <int EW, int D>
+__device__ __forceinline__ void choose_own_rows(const LpProblem &P, const OwnBins &B, int bin) {
+  const unsigned cnt = B.count(bin);
+  for (unsigned i = threadIdx.x; i < cnt; i += kThreads) {
+    int v;
+    int64_t beg, d64;
+    B.row(bin, i, &v, &beg, &d64);
+    const int d = (int)d64;
+    int L[D];
+    unsigned w[EW ? D : 1];
+#pragma unroll
+    for (int j = 0; j < D; j++) L[j] = j < d ? __ldg(P.g.adj + beg + j) : -1;
+    const int L0 = P.labels[P.vbase + v];
+    const long long cv = P.g.vweight(v);
+#pragma unroll
+    for (int j = 0; j < D; j++) L[j] = j < d ? P.labels[L[j]] : -1;
+    bool other = false;
+#pragma unroll
+    for (int j = 0; j < D; j++) other |= L[j] >= 0 && L[j] != L0;
+    if (!other) continue;  // (the weights of an inner vertex are not read)
+    if (EW) {
+      bool wide = false;
+#pragma unroll
+      for (int j = 0; j < D; j++) {
+        const long long x = j < d ? load_ew<EW>(P.g.ew, beg + j) : 0;
+        wide |= (unsigned long long)x >> 26 != 0;
+        w[EW ? j : 0] = (unsigned)x;
+      }
+      if (wide) {
+        choose_own_wide<EW>(P, B, v, beg, d, L0, cv);
+        continue;
+      }
+    }
+    unsigned c0 = 0;
+#pragma unroll
+    for (int j = 0; j < D; j++) {
+      if (L[j] == L0) {
+        c0 += EW ? w[EW ? j : 0] : 1u;
+        L[j] = -1;
+      }
+    }
+    const uint64_t hv = mix64(P.smix ^ (uint64_t)(uint32_t)v);
+    while (other) {
+      // the labels of largest connection, as positions; equal ones share all their positions
+      unsigned most = c0, pos = 0;
+#pragma unroll
+      for (int x = 0; x < D; x++) {
+        unsigned c = 0;
+#pragma unroll
+        for (int y = 0; y < D; y++) c += L[y] == L[x] ? (EW ? w[EW ? y : 0] : 1u) : 0u;
+        if (L[x] < 0) c = 0;
+        if (c > most) {
+          most = c;
+          pos = 1u << x;
+        } else if (c == most && pos) {
+          pos |= 1u << x;
+        }
+      }
+      if (!pos) break;
+      uint64_t bh = 0;
+      int bL = -1;
+#pragma unroll
+      for (int x = 0; x < D; x++) {
+        if ((pos >> x & 1u) && L[x] != bL) {
+          const uint64_t h = mix64(hv ^ (uint64_t)(L[x] - P.lbase));
+          if (bL < 0 || h > bh || (h == bh && L[x] < bL)) {
+            bh = h;
+            bL = L[x];
+          }
+        }
+      }
+      if (P.lw[bL] + cv <= P.U) {
+        Best b;
+        b.L = bL;
+        b.conn = most;
+        b.qs = 0;
+        b.h = bh;
+        B.template put<false>(bin, i, v, b, c0);
+        atomicAdd(reinterpret_cast<unsigned long long *>(&P.demand[bL]), (unsigned long long)cv);
+        break;
+      }
+      other = false;
+#pragma unroll
+      for (int x = 0; x < D; x++) {
+        if (L[x] == bL) L[x] = -1;
+        other |= L[x] >= 0;
+      }
+    }
+  }
+}
 
 // One warp per vertex with 32 < d <= kOwnDeg, table in shared memory.
 template <int EW, bool LQ>
@@ -2591,12 +2726,13 @@ __device__ __forceinline__ void choose_own_warp(const LpProblem &P, const OwnBin
 
 // The block's moves of the previous sub-round on the label weights that sub-round read, and its demand
 // cleared.
-__device__ __forceinline__ void replay_own(const LpProblem &P, const OwnProps &O, int64_t *old_demand, int64_t slot0) {
-  for (unsigned base = 0; base < O.n; base += kThreads) {
+__device__ __forceinline__ void replay_own(const LpProblem &P, const OwnProps &O, int64_t *weights, int64_t *old_demand,
+                                           int64_t slot0, unsigned np) {
+  for (unsigned base = 0; base < np; base += kThreads) {
     const unsigned k = base + threadIdx.x;
     int T = -1, v = 0, L0 = -1;
     bool adm = false;
-    if (k < O.n) {
+    if (k < np) {
       T = k < kOwnKeep ? O.t[k] : P.mv_t[slot0 + k];
       v = k < kOwnKeep ? O.v[k] : P.mv_v[slot0 + k];
       adm = P.mv_adm[slot0 + k] != 0;
@@ -2604,98 +2740,113 @@ __device__ __forceinline__ void replay_own(const LpProblem &P, const OwnProps &O
       old_demand[T] = 0;
     }
     const long long c = adm ? P.g.vweight(v) : 0;
-    warp_add_by_key(P.lw_next, adm, T, c);
-    warp_add_by_key(P.lw_next, adm, adm ? L0 : -1, -c);
+    warp_add_by_key(weights, adm, T, c);
+    warp_add_by_key(weights, adm, adm ? L0 : -1, -c);
   }
 }
 
-// The active vertices of one tile by degree bin. Returns the tile's active count (degree-0 ones, which take
-// no part in the choice, only count as visits).
-__device__ __forceinline__ unsigned classify_own(const LpProblem &P, const uint8_t *act, uint8_t *act_clear, int r, int s,
-                                                 uint64_t rmix, int t0, int t1, int64_t r0, unsigned *start,
-                                                 unsigned short *list, unsigned *rowx, Smem &sm) {
-  const int v0 = t0 + (int)threadIdx.x * kOwnPer;  // (act + vbase and t0 are multiples of 8 from the allocation)
+// The marks of the calling thread's eight vertices (the vertices of a block start at a multiple of eight from
+// the allocation, whose end is padded).
+__device__ __forceinline__ uint64_t marks_own(const LpProblem &P, int r, int64_t v0, int64_t t1) {
+  if (v0 >= t1) return 0;
+  return r == 0 ? ~0ull : *reinterpret_cast<const uint64_t *>(P.act[r & 1] + P.vbase + v0);
+}
+
+// The active vertices of one tile by degree bin (degree-0 ones, which take no part in the choice, only count as
+// visits). known: rowx holds the rows already (a block of one tile reads them once per call). *packed must be
+// zero on entry; returns the bins' counts, 16 bits each.
+__device__ __forceinline__ unsigned long long classify_own(const LpProblem &P, uint8_t *act_clear,
+                                                           int s, uint64_t rmix, int t0, int t1, int64_t r0,
+                                                           uint64_t marks, bool known, unsigned short *list,
+                                                           unsigned *rowx, unsigned long long *packed, Smem &sm) {
+  const int v0 = t0 + (int)threadIdx.x * kOwnPer;
   unsigned flag = 0;
   if (v0 < t1) {
-    if (r == 0) {
-      flag = 0xffu;
-    } else {
-      const uint64_t f = *reinterpret_cast<const uint64_t *>(act + P.vbase + v0);
-#pragma unroll
-      for (int i = 0; i < kOwnPer; i++) flag |= ((unsigned)(f >> (8 * i)) & 1u) << i;
-    }
+    // the marks' lowest bits, gathered into one byte
+    flag = (unsigned)((marks & 0x0101010101010101ull) * 0x0102040810204080ull >> 56);
     if (s == 0) *reinterpret_cast<uint64_t *>(act_clear + P.vbase + v0) = 0;
     if (t1 - v0 < kOwnPer) flag &= (1u << (t1 - v0)) - 1u;
   }
+  if (__any_sync(kFull, flag)) {
 #pragma unroll
-  for (int i = 0; i < kOwnPer; i++)
-    if ((flag >> i & 1u) && (int)(mix64(rmix ^ (uint64_t)(v0 + i)) >> 63) != s) flag &= ~(1u << i);
-  int64_t rb[kOwnPer];
-  int dd[kOwnPer];
+    for (int i = 0; i < kOwnPer; i++)
+      if ((flag >> i & 1u) && (int)(mix64(rmix ^ (uint64_t)(v0 + i)) >> 63) != s) flag &= ~(1u << i);
+    unsigned *const rx = rowx + threadIdx.x * kOwnPer;
+    int dd[kOwnPer];
+    if (known) {
 #pragma unroll
-  for (int i = 0; i < kOwnPer; i++) {
-    rb[i] = 0;
-    dd[i] = 0;
-    if (flag >> i & 1u) {
-      rb[i] = P.g.row_begin(v0 + i);
-      dd[i] = (int)(P.g.row_begin(v0 + i + 1) - rb[i]);
+      for (int i = 0; i < kOwnPer; i++) dd[i] = flag >> i & 1u ? (int)(rx[i] & 255u) : 0;
+    } else {
+      int rel[kOwnPer];
+#pragma unroll
+      for (int i = 0; i < kOwnPer; i++) {
+        rel[i] = 0;
+        dd[i] = 0;
+        if (flag >> i & 1u) {
+          const int64_t rb = P.g.row_begin(v0 + i);
+          dd[i] = (int)(P.g.row_begin(v0 + i + 1) - rb);
+          rel[i] = (int)(rb - r0);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < kOwnPer; i++)
+        if (dd[i] > 0) rx[i] = (unsigned)rel[i] << 8 | (unsigned)dd[i];
     }
-  }
-  // counts per bin, 12 bits each
-  unsigned long long mine = 0;
-  unsigned edges = 0;
+    unsigned long long mine = 0;
+    unsigned edges = 0;
 #pragma unroll
-  for (int i = 0; i < kOwnPer; i++) {
-    if (dd[i] > 0) {
-      mine += 1ull << (12 * bin_of(dd[i], kOwnDeg, kOwnDeg));
-      edges += (unsigned)dd[i];
+    for (int i = 0; i < kOwnPer; i++) {
+      if (dd[i] > 0) {
+        mine += 1ull << (16 * (OwnBins::bin(dd[i]) - 1));
+        edges += (unsigned)dd[i];
+      }
     }
-  }
-  const unsigned wact = warp_sum_u32((unsigned)__popc(flag)), wedg = warp_sum_u32(edges);
-  if ((threadIdx.x & 31) == 0 && wact) {
-    atomicAdd(&sm.vis[0], (unsigned long long)wact);
-    atomicAdd(&sm.edg[0], (unsigned long long)wedg);
-  }
-  long long total;
-  const unsigned long long at = (unsigned long long)block_excl_scan64((long long)mine, sm.tmp, &sm.tot);
-  total = sm.tot;
-  unsigned st[6];
-  st[0] = 0;
+    // places: the lane's share of the warp's, the warp's share of the tile's (the order is of no account)
+    const int lane = threadIdx.x & 31;
+    unsigned long long incl = mine;
 #pragma unroll
-  for (int b = 0; b < 5; b++) st[b + 1] = st[b] + (unsigned)(total >> (12 * b) & 0xfff);
-  if (threadIdx.x < 6) start[threadIdx.x] = st[threadIdx.x];
-  unsigned long long pos = at;
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long y = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += y;
+    }
+    unsigned long long pos = 0;
+    if (lane == 31 && incl) pos = atomicAdd(packed, incl);
+    pos = __shfl_sync(kFull, pos, 31) + incl - mine;
+    const unsigned wact = warp_sum_u32((unsigned)__popc(flag)), wedg = warp_sum_u32(edges);
+    if (lane == 0 && wact) {
+      atomicAdd(&sm.vis[0], (unsigned long long)wact);
+      atomicAdd(&sm.edg[0], (unsigned long long)wedg);
+    }
 #pragma unroll
-  for (int i = 0; i < kOwnPer; i++) {
-    if (dd[i] > 0) {
-      const int b = bin_of(dd[i], kOwnDeg, kOwnDeg);
-      const unsigned x = threadIdx.x * kOwnPer + i;
-      unsigned sb = 0;
-#pragma unroll
-      for (int y = 1; y < 5; y++) sb = b == y ? st[y] : sb;
-      list[sb + (unsigned)(pos >> (12 * b) & 0xfff)] = (unsigned short)x;
-      rowx[x] = (unsigned)(rb[i] - r0) << 8 | (unsigned)dd[i];
-      pos += 1ull << (12 * b);
+    for (int i = 0; i < kOwnPer; i++) {
+      if (dd[i] > 0) {
+        const int b = OwnBins::bin(dd[i]);
+        const unsigned x = threadIdx.x * kOwnPer + i;
+        list[OwnBins::at(b, (unsigned)(pos >> (16 * (b - 1))) & 0xffffu)] = (unsigned short)x;
+        pos += 1ull << (16 * (b - 1));
+      }
     }
   }
   __syncthreads();
-  return st[5];
+  return *packed;
 }
 
 // Admission of the block's proposals; the ones whose target cannot take all of its demand are contested.
+// Adds the block's moves to sm.moves and sets *any when it has contested ones.
 template <bool LQ>
 __device__ __forceinline__ void admit_own(const LpProblem &P, SubCounters &C, const OwnProps &O, int r, int64_t slot0,
-                                          Smem &sm) {
+                                          unsigned np, unsigned *any, Smem &sm) {
   unsigned long long mg = 0, mq = 0;
   unsigned moved = 0;
   uint8_t *act_next = r + 1 < P.rounds ? P.act[(r + 1) & 1] : nullptr;  // (no marks in the last round)
-  for (unsigned base = 0; base < O.n; base += kThreads) {
+  for (unsigned base = 0; base < np; base += kThreads) {
     const unsigned k = base + threadIdx.x;
+    if (!__any_sync(kFull, k < np)) break;
     bool contested = false, adm = false;
     int T = -1, v = 0, L0 = 0;
     int64_t rb = 0, deg = 0;
     const int64_t i = slot0 + k;
-    if (k < O.n) {
+    if (k < np) {
       T = k < kOwnKeep ? O.t[k] : P.mv_t[i];
       v = k < kOwnKeep ? O.v[k] : P.mv_v[i];
       const long long lwT = P.lw[T], dT = P.demand[T];
@@ -2712,27 +2863,59 @@ __device__ __forceinline__ void admit_own(const LpProblem &P, SubCounters &C, co
       }
     }
     moved += apply_movers_pre(P, C, act_next, adm, i, v, T, L0, rb, deg);
-    const unsigned pos = warp_append(&C.n_contested, contested);
-    if (contested) P.ct[pos] = (unsigned)i;
-  }
-  if (O.n == 0) return;
-  if ((threadIdx.x & 31) == 0 && moved) atomicAdd(&sm.moves, (unsigned long long)moved);
-  for (int o = 16; o > 0; o >>= 1) {
-    mg = max(mg, __shfl_xor_sync(kFull, mg, o));
-    mq = max(mq, __shfl_xor_sync(kFull, mq, o));
-  }
-  if ((threadIdx.x & 31) == 0) {
-    if (mg) atomicMax(&C.max_gain, mg);
-    if (LQ && mq) atomicMax(&C.max_q, mq);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    sm.movers += O.n;
-    if (sm.moves) {
-      atomicAdd(&P.ctr->moves_round[r & 1], sm.moves);
-      sm.moves = 0;
+    if (__any_sync(kFull, contested)) {
+      const unsigned pos = warp_append(&C.n_contested, contested);
+      if (contested) P.ct[pos] = (unsigned)i;
+      *any = 1;
     }
   }
+  if ((threadIdx.x & 31) == 0 && moved) atomicAdd(&sm.moves, (unsigned long long)moved);
+  if (__any_sync(kFull, mg | mq)) {
+    for (int o = 16; o > 0; o >>= 1) {
+      mg = max(mg, __shfl_xor_sync(kFull, mg, o));
+      mq = max(mq, __shfl_xor_sync(kFull, mq, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+      if (mg) atomicMax(&C.max_gain, mg);
+      if (LQ && mq) atomicMax(&C.max_q, mq);
+    }
+  }
+}
+
+// Barrier over a problem's blocks that also sums what the blocks have to tell one another: `add` (thread 0's;
+// 1 in the low 16 bits, what else above) of all blocks. Two words alternate, so that a word's value is final
+// when the last block has arrived: nobody adds to it again before everybody has met at the other word. `prev`
+// is the word's value after its last use. Thread 0 adds without waiting for the old value and polls with
+// acquire loads; the wait is bounded like grid_sync's. Returns false when it gave up.
+constexpr unsigned kOwnBarWord = 16;  // 32-bit words from P.bar: words 16 and 32 (grid_sync's is word 0)
+static_assert(2 * kOwnBarWord + 2 <= kBarrierStride, "the barrier words of a problem");
+
+struct OwnMeet {
+  unsigned long long prev[2], sum;
+  int ok;
+};
+
+__device__ __forceinline__ void own_meet(const LpProblem &P, OwnMeet &M, int which, unsigned long long add, unsigned nb) {
+  // (thread 0, after a block barrier; the caller's next block barrier publishes M.sum and M.ok)
+  if (nb <= 1) {
+    M.sum = add;
+    return;
+  }
+  unsigned long long *w = reinterpret_cast<unsigned long long *>(P.bar + kOwnBarWord * (which + 1));
+  asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(w), "l"(add) : "memory");
+  const unsigned long long before = M.prev[which], t0 = global_ns();
+  unsigned long long now;
+  for (;;) {
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(now) : "l"(w) : "memory");
+    if (((now - before) & 0xffffu) == nb) break;
+    if (global_ns() - t0 > 1000ull * P.wait_us || *(volatile int *)&P.ctr->err == GP_ERR_TIMEOUT) {
+      atomicExch(&P.ctr->err, GP_ERR_TIMEOUT);
+      M.ok = 0;
+      break;
+    }
+  }
+  M.prev[which] = now;
+  M.sum = now - before;
 }
 
 template <int EW, bool LQ>
@@ -2740,12 +2923,13 @@ __device__ bool lp_problem_own(const LpProblem *prob, unsigned char *dsm) {
   __shared__ __align__(16) unsigned char p_raw[sizeof(LpProblem)];
   __shared__ Smem sm;
   __shared__ OwnProps O;
-  __shared__ unsigned s_start[6];
+  __shared__ OwnMeet M;
+  __shared__ unsigned long long s_packed[2];
+  __shared__ unsigned s_contested;
   __shared__ SubCounters sV;
-  __shared__ unsigned long long s_mr;
   LpProblem &P = *reinterpret_cast<LpProblem *>(p_raw);
-  unsigned short *const list = reinterpret_cast<unsigned short *>(dsm + kOwnListOff<LQ> + kOwnTile * 4);
-  unsigned *const rowx = reinterpret_cast<unsigned *>(dsm + kOwnListOff<LQ>);
+  unsigned short *const list = reinterpret_cast<unsigned short *>(dsm + kOwnListOff<LQ>);
+  unsigned *const rowx = reinterpret_cast<unsigned *>(dsm + kOwnRowOff<LQ>);
   __syncthreads();  // the block's previous problem is done with the shared state
   {
     const unsigned *src = reinterpret_cast<const unsigned *>(prob);
@@ -2759,7 +2943,11 @@ __device__ bool lp_problem_own(const LpProblem *prob, unsigned char *dsm) {
   if (threadIdx.x == 0) {
     sm.moves = 0;
     sm.movers = 0;
-    O.n = 0;
+    O.n[0] = O.n[1] = 0;
+    M.prev[0] = M.prev[1] = 0;
+    M.ok = 1;
+    s_packed[0] = s_packed[1] = 0;
+    s_contested = 0;
   }
   __syncthreads();
   const int lb = (int)blockIdx.x - P.block_begin, nb = P.block_count;
@@ -2767,7 +2955,7 @@ __device__ bool lp_problem_own(const LpProblem *prob, unsigned char *dsm) {
 #define bar (GridBarrier{P.bar, &P.ctr->err, (unsigned)nb, (unsigned)lb, P.wait_us})
   __shared__ unsigned long long pacc[8];
   if (threadIdx.x < 8) pacc[threadIdx.x] = 0;
-  unsigned long long tmark = 0;
+  unsigned long long tmark = 0, moves = 0;  // (thread 0's)
   auto tick = [&](int phase) {
     if (lb == 0 && threadIdx.x == 0) {
       const unsigned long long now = global_ns();
@@ -2778,93 +2966,138 @@ __device__ bool lp_problem_own(const LpProblem *prob, unsigned char *dsm) {
   const int64_t n = P.g.n;
   const int64_t chunk = ((n + nb - 1) / nb + kOwnPer - 1) / kOwnPer * kOwnPer;
   const int64_t lo = min(n, (int64_t)lb * chunk), hi = min(n, lo + chunk);
+  const int64_t r_lo = P.g.row_begin(lo);
+  const bool one_tile = hi - lo <= kOwnTile;
   // the second copies start as the first (label weights) and as zero (demand)
   for (int64_t x = P.lbase + (int64_t)lb * kThreads + threadIdx.x; x < P.lbase + P.nl; x += (int64_t)nb * kThreads) {
     P.lw2[1][x] = P.lw2[0][x];
     P.demand2[1][x] = 0;
   }
+  if (one_tile) {
+#pragma unroll
+    for (int i = 0; i < kOwnPer; i++) {
+      const int64_t v = lo + threadIdx.x * kOwnPer + i;
+      if (v < hi) {
+        const int64_t rb = P.g.row_begin(v);
+        rowx[threadIdx.x * kOwnPer + i] = (unsigned)(rb - r_lo) << 8 | (unsigned)(P.g.row_begin(v + 1) - rb);
+      }
+    }
+  }
   tick(-1);
   int t_last = -1;
+  unsigned tile = 0;  // classified tiles so far (their counts alternate between the two words)
   for (int r = 0; r < P.rounds; r++) {
     const uint64_t rmix = mix64(P.smix ^ (uint64_t)r);
+    bool round_moved = false, round_contest = false;
     for (int s = 0; s < 2; s++) {
       const int t = 2 * r + s;
       SubCounters &C = ctr->sc[t % 3];
-      SubCounters &Cn = ctr->sc[(t + 1) % 3];
-      __syncthreads();
+      // (every thread of the block has passed the last sub-round's final barrier)
       if (threadIdx.x == 0) {
         P.lw = P.lw2[t & 1];
         P.lw_next = P.lw2[(t + 1) & 1];
         P.demand = P.demand2[t & 1];
-        P.sub_t = t;
+        O.cur = t & 1;
         if (lb == 0) {
           // counter set t+1 was last used by sub-round t-2, which every block has finished
+          SubCounters &Cn = ctr->sc[(t + 1) % 3];
           Cn.n_contested = 0;
           Cn.n_big = 0;
           Cn.max_gain = 0;
           Cn.max_q = 0;
         }
       }
-      __syncthreads();
-      if (t > 0) {
-        replay_own(P, O, P.demand2[(t + 1) & 1], lo);
-        __syncthreads();
-        if (threadIdx.x == 0) O.n = 0;
-      }
       t_last = t;
-      for (int64_t t0 = lo; t0 < hi; t0 += kOwnTile) {
-        const int64_t r0 = P.g.row_begin(t0);
-        const unsigned na = classify_own(P, P.act[r & 1], P.act[(r + 1) & 1], r, s, rmix, (int)t0,
-                                         (int)min(hi, t0 + kOwnTile), r0, s_start, list, rowx, sm);
-        if (na == 0) continue;
-        const OwnBins B{P, O, s_start, list, rowx, (int)t0, r0, lo};
-        choose_groups<EW, LQ>(P, B, threadIdx.x >> 5, kWarps);
-        choose_own_warp<EW, LQ>(P, B, dsm);
-        __syncthreads();
+      uint64_t marks = marks_own(P, r, lo + threadIdx.x * kOwnPer, hi);  // (loaded while the replay runs)
+      replay_own(P, O, P.lw2[(t + 1) & 1], P.demand2[(t + 1) & 1], lo, O.n[(t + 1) & 1]);
+      for (int64_t t0 = lo; t0 < hi; t0 += kOwnTile, tile++) {
+        const int64_t r0 = one_tile ? r_lo : P.g.row_begin(t0);
+        if (t0 > lo) marks = marks_own(P, r, t0 + threadIdx.x * kOwnPer, hi);
+        const unsigned long long counts =
+            classify_own(P, P.act[(r + 1) & 1], s, rmix, (int)t0, (int)min(hi, t0 + kOwnTile), r0, marks, one_tile, list,
+                         rowx, &s_packed[tile & 1], sm);
+        if (threadIdx.x == 0) s_packed[(tile + 1) & 1] = 0;  // (read by all before the barrier in classify_own)
+        if (counts) {
+          unsigned long long grouped = counts;
+          if constexpr (!LQ) {
+            const OwnBins B{P, O, counts, list, rowx, (int)t0, r0, lo};
+            if (B.count(1) > kOwnRowsMin) {
+              choose_own_rows<EW, 8>(P, B, 1);
+              grouped &= ~0xffffull;
+            }
+            if (B.count(2) > kOwnRowsMin) {
+              choose_own_rows<EW, 16>(P, B, 2);
+              grouped &= ~(0xffffull << 16);
+            }
+          }
+          const OwnBins B{P, O, grouped, list, rowx, (int)t0, r0, lo};
+          choose_groups<EW, LQ>(P, B, threadIdx.x >> 5, kWarps);
+          choose_own_warp<EW, LQ>(P, B, dsm);
+        }
+        if (t0 + kOwnTile < hi) __syncthreads();  // (the next tile writes the lists and their counts)
       }
-      if (!grid_sync(bar)) return false;
-      tick(1);
-      if (lb == 0 && threadIdx.x == 0 && s == 0) ctr->moves_round[(r + 1) & 1] = 0;
-      admit_own<LQ>(P, C, O, r, lo, sm);
-      if (!grid_sync(bar)) return false;
-      // contested count and key ranges; the round's move count
-      if (threadIdx.x < sizeof(SubCounters) / 4)
-        reinterpret_cast<unsigned *>(&sV)[threadIdx.x] = reinterpret_cast<const volatile unsigned *>(&C)[threadIdx.x];
-      if (threadIdx.x == kThreads - 1) s_mr = *(volatile unsigned long long *)&ctr->moves_round[r & 1];
       __syncthreads();
+      if (threadIdx.x == 0) own_meet(P, M, 0, 1, (unsigned)nb);
+      __syncthreads();
+      if (!M.ok) return false;
+      tick(1);
+      const unsigned np = O.n[t & 1];
+      if (threadIdx.x == 0) {
+        if (lb == 0 && s == 0) ctr->moves_round[(r + 1) & 1] = 0;
+        O.n[(t + 1) & 1] = 0;  // (the replay is done)
+        sm.movers += np;
+      }
+      admit_own<LQ>(P, C, O, r, lo, np, &s_contested, sm);
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        const unsigned long long mv = sm.moves;
+        own_meet(P, M, 1, 1 | (s_contested ? 1ull << 16 : 0) | (mv ? 1ull << 32 : 0), (unsigned)nb);
+        moves += mv;
+        sm.moves = 0;
+        s_contested = 0;
+      }
+      __syncthreads();
+      if (!M.ok) return false;
       tick(3);
-      const unsigned nc = sV.n_contested;
-      if (nc > 0) {
+      round_moved |= M.sum >> 32 != 0;
+      if (M.sum >> 16 & 0xffffu) {
+        // contested count and key ranges
+        if (threadIdx.x < sizeof(SubCounters) / 4)
+          reinterpret_cast<unsigned *>(&sV)[threadIdx.x] = reinterpret_cast<const volatile unsigned *>(&C)[threadIdx.x];
+        __syncthreads();
+        const unsigned nc = sV.n_contested;
         if (nc <= kContestSmall) {
           if (lb == 0) contest_small<LQ>(P, sV, &C, nc, r, dsm, sm);
         } else {
           if (!contest_large<LQ>(P, sV, &C, nc, r, lb, nb, bar, sm, dsm)) return false;
         }
         if (!grid_sync(bar)) return false;
-        if (threadIdx.x == 0) s_mr = *(volatile unsigned long long *)&ctr->moves_round[r & 1];
-        __syncthreads();
+        round_contest = true;
         tick(4);
       }
     }
-    const unsigned long long mr = s_mr;
-    if (lb == 0 && threadIdx.x == 0) {
-      ctr->rounds += 1;
-      ctr->moves += mr;
+    if (round_contest) {
+      // moves of the contests (final after the last barrier)
+      __shared__ unsigned long long s_mr;
+      if (threadIdx.x == 0) {
+        s_mr = *(volatile unsigned long long *)&ctr->moves_round[r & 1];
+        if (lb == 0) moves += s_mr;
+      }
+      __syncthreads();
+      round_moved |= s_mr != 0;
+      __syncthreads();
     }
-    if (mr == 0) break;
+    if (lb == 0 && threadIdx.x == 0) ctr->rounds += 1;
+    if (!round_moved) break;
   }
   // the last sub-round's moves on the copy it read: both copies are final then
-  if (t_last >= 0) {
-    __syncthreads();
-    if (threadIdx.x == 0) P.lw_next = P.lw2[t_last & 1];
-    __syncthreads();
-    replay_own(P, O, P.demand2[t_last & 1], lo);
-  }
+  if (t_last >= 0) replay_own(P, O, P.lw2[t_last & 1], P.demand2[t_last & 1], lo, O.n[t_last & 1]);
   __syncthreads();
   if (threadIdx.x == 0) {
     if (sm.vis[0]) atomicAdd(&ctr->bin_visits[0], sm.vis[0]);
     if (sm.edg[0]) atomicAdd(&ctr->bin_edges[0], sm.edg[0]);
     if (sm.movers) atomicAdd(&ctr->movers, sm.movers);
+    if (moves) atomicAdd(&ctr->moves, moves);
   }
   tick(5);
   if (lb == 0 && threadIdx.x == 0)
@@ -2875,7 +3108,7 @@ __device__ bool lp_problem_own(const LpProblem *prob, unsigned char *dsm) {
 #undef bar
 
 template <int EW, bool LQ>
-__global__ void __launch_bounds__(kThreads, 4) k_lp_own(const LpProblem *probs, const int *blk_start,
+__global__ void __launch_bounds__(kThreads, EW ? 3 : 4) k_lp_own(const LpProblem *probs, const int *blk_start,
                                                         const int *blk_list) {
   extern __shared__ __align__(16) unsigned char dsm[];
   for (int q = blk_start[blockIdx.x]; q < blk_start[blockIdx.x + 1]; q++)

@@ -5,15 +5,15 @@
 // sum of its members; each coarse edge (a, b), a != b, weighs the sum of the fine edges between
 // clusters a and b.
 //
-// GPU design: instead of the paper's concurrent hash table, the (cv, cu, omega) pairs are sorted
-// and reduced in two levels. Fine vertices are bucketed by coarse id (a counting sort), which sorts
-// the pairs by cv; within one coarse row the pairs are sorted by cu and equal keys are summed:
-// in registers by one warp (<= 32 pairs), in shared memory by one CTA (<= 4096 pairs), or by a
-// CTA-wide LSD radix sort in global memory for larger rows. Rows come out sorted by neighbour id,
-// so the coarse CSR is canonical and independent of scheduling.
+// GPU design: instead of the paper's concurrent hash table, one stable sort of the (cv, cu, omega) pairs and a
+// segmented sum. Fine vertices are bucketed by coarse id (a counting sort). Walking their rows in that order
+// lists the pairs in ascending order of the walking side cu; because the graph is symmetric, each entry can
+// stand for its reverse, row = the cluster of its other end cv, so only a stable sort by cv is left: two or
+// three radix passes over the bits of n' where sorting by (cv, cu) would take twice as many. Pairs inside a
+// cluster are dropped before the first pass. The sorted pairs are the coarse rows, sorted by neighbour id;
+// equal pairs are adjacent and summed. Rows of every length take the same path, so neither a hub row nor the
+// mix of lengths decides the time.
 #include <algorithm>
-#include <climits>
-#include <type_traits>
 
 #include "contract.cuh"
 #include "lp.cuh"
@@ -22,14 +22,6 @@
 namespace gp {
 
 namespace {
-
-constexpr int kRowSmall = 32;     // <= 32 pairs: one warp, registers
-constexpr int kRowWarp = 256;     // <= 256 pairs: one warp, shared-memory hash of 512 slots
-constexpr int kRowWarpBig = 1024; // <= 1024 pairs: one warp, shared-memory hash of 2048 slots
-constexpr int kRowMedium = 4096;  // <= 4096 pairs: one CTA, shared-memory hash
-constexpr int kRowThreads = 256;
-constexpr int kWarpSlots = 2 * kRowWarp;
-constexpr int kCtaSlots = 2 * kRowMedium;
 
 __global__ void k_mark_used(const int32_t *labels, int64_t n, int64_t nl, uint32_t *used, int *bad) {
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
@@ -42,17 +34,17 @@ __global__ void k_mark_used(const int32_t *labels, int64_t n, int64_t nl, uint32
   }
 }
 
-// Fine -> coarse map and, per coarse vertex, member count, weight and degree sum. Members of one
-// cluster are mostly neighbours in id order, so the warp combines equal coarse ids before its atomics.
+// Fine -> coarse map and, per coarse vertex, member count and weight. Members of one cluster are mostly
+// neighbours in id order, so the warp combines equal coarse ids before its atomics.
 // A label outside [0, nl) sets *bad and maps its vertex to 0 (the caller reports the error).
 __global__ void k_f2c(DGraph g, const int32_t *labels, int64_t nl, const int32_t *newid, int32_t *f2c, int64_t *cnt,
-                      int64_t *cw, int64_t *dsum, int *bad) {
+                      int64_t *cw, int *bad) {
   const int lane = threadIdx.x & 31;
   for (int64_t v0 = blockIdx.x * (int64_t)blockDim.x; v0 < g.n; v0 += (int64_t)gridDim.x * blockDim.x) {
     const int64_t v = v0 + threadIdx.x;
     bool ok = v < g.n;
     int cv = 0;
-    long long c = 0, d = 0;
+    long long c = 0;
     if (ok) {
       const int L = labels[v];
       if (L < 0 || L >= nl) {
@@ -63,581 +55,273 @@ __global__ void k_f2c(DGraph g, const int32_t *labels, int64_t nl, const int32_t
         cv = newid[L];
         f2c[v] = cv;
         c = g.vweight(v);
-        d = g.row_begin(v + 1) - g.row_begin(v);
       }
     }
     const unsigned peers = __match_any_sync(kFull, ok ? cv : -1);
     if (!ok) continue;
-    long long cs = 0, ds = 0;
-    for (unsigned m = peers; m; m &= m - 1) {
-      const int src = __ffs(m) - 1;
-      cs += __shfl_sync(peers, c, src);
-      ds += __shfl_sync(peers, d, src);
-    }
+    long long cs = 0;
+    for (unsigned m = peers; m; m &= m - 1) cs += __shfl_sync(peers, c, __ffs(m) - 1);
     if (lane == __ffs(peers) - 1) {
       atomicAdd(reinterpret_cast<unsigned long long *>(&cnt[cv]), (unsigned long long)__popc(peers));
       atomicAdd(reinterpret_cast<unsigned long long *>(&cw[cv]), (unsigned long long)cs);
-      atomicAdd(reinterpret_cast<unsigned long long *>(&dsum[cv]), (unsigned long long)ds);
     }
   }
 }
 
-__global__ void k_members(int64_t n, const int32_t *f2c, const int64_t *mstart, unsigned *fill, int32_t *members) {
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
+// Members bucketed by coarse id (in any order within a cluster) with their degrees; largest coarse weight.
+__global__ void k_members(DGraph g, const int32_t *f2c, const int64_t *mstart, unsigned *fill, int32_t *members,
+                          int64_t *mdeg, const int64_t *cw, int64_t ncb, unsigned long long *maxcw) {
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < g.n; v += (int64_t)gridDim.x * blockDim.x) {
     const int cv = f2c[v];
-    const unsigned pos = atomicAdd(&fill[cv], 1u);
-    members[mstart[cv] + pos] = (int32_t)v;
+    const int64_t pos = mstart[cv] + atomicAdd(&fill[cv], 1u);
+    members[pos] = (int32_t)v;
+    mdeg[pos] = g.row_begin(v + 1) - g.row_begin(v);
   }
-}
-
-__global__ void k_max_i64(const int64_t *x, int64_t n, unsigned long long *out) {
   unsigned long long m = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    m = max(m, (unsigned long long)x[i]);
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ncb; i += (int64_t)gridDim.x * blockDim.x)
+    m = max(m, (unsigned long long)cw[i]);
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(kFull, m, o));
-  if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
+  if ((threadIdx.x & 31) == 0 && m) atomicMax(maxcw, m);
 }
 
-// nc_dev: the number of coarse vertices (device; the grid is sized for an upper bound)
-__global__ void k_row_classify(const int64_t *nc_dev, const int64_t *dsum, int32_t *l0, int32_t *l1, int32_t *l2,
-                               int32_t *l3, int32_t *l4, unsigned *counts) {
-  const int64_t nc = *nc_dev;
-  for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < nc; base += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t c = base + threadIdx.x;
-    int b = -1;
-    if (c < nc) {
-      const int64_t D = dsum[c];
-      b = D <= kRowSmall ? 0 : (D <= kRowWarp ? 3 : (D <= kRowWarpBig ? 4 : (D <= kRowMedium ? 1 : 2)));
-    }
-    int32_t *lists[5] = {l0, l1, l2, l3, l4};
-    for (int bb = 0; bb < 5; bb++) {
-      const unsigned m = __ballot_sync(kFull, b == bb);
-      if (!m) continue;
-      const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
-      unsigned pos = 0;
-      if (lane == leader) pos = atomicAdd(&counts[bb], (unsigned)__popc(m));
-      pos = __shfl_sync(kFull, pos, leader) + __popc(m & lanemask_lt());
-      if (b == bb) lists[bb][pos] = (int32_t)c;
-    }
+// Edge-weight values that travel with the pairs: none (unit weights), 32 or 64 bits.
+template <int EW>
+constexpr int kValBytes = EW == 0 ? 0 : (EW == 1 ? 4 : 8);
+
+// The largest i with pre[i] <= x (0 <= x < pre[n]), found by the whole warp: 32 pivots per step.
+__device__ __forceinline__ int64_t warp_owner(const int64_t *pre, int64_t n, int64_t x) {
+  const int lane = threadIdx.x & 31;
+  int64_t lo = 0, hi = n;
+  while (hi - lo > 1) {
+    const int64_t step = (hi - lo + 31) / 32;
+    const int64_t p = lo + (lane + 1) * step;
+    const int c = __popc(__ballot_sync(kFull, p < hi && pre[p] <= x));  // (a prefix of the lanes)
+    hi = min(hi, lo + (c + 1) * step);
+    lo += c * step;
   }
+  return lo;
 }
 
-struct RowArgs {
-  DGraph g;
-  const int32_t *f2c;
-  const int64_t *mstart;
-  const int32_t *members;
-  const int64_t *tstart;
-  int32_t *okey;
-  int64_t *oval;
-  int64_t *rowcnt;
-  const int32_t *list;
-  const unsigned *count;
-  const int64_t *dsum;
-  int key_bits;
-};
-
-// Rows with at most 32 pairs: one warp gathers them into shared memory, sorts them in registers
-// (bitonic network over the lanes) and sums runs of equal neighbour ids.
+// The pairs in walking order, keys (cv << 32 | cu) and values omega, and the digit counts of the sort's first
+// pass. Position p of the walk belongs to the member row with mpre[i] <= p < mpre[i + 1]; a warp takes 256
+// consecutive positions, eight per lane, whatever rows they lie in: 32 rows at a time are held by the lanes
+// and searched by shuffles. All positions are resolved first, then their adjacency entries are loaded, then
+// the coarse ids of those are gathered, so that eight gathers per lane are in flight: the gathers bound it.
 template <int EW>
-__global__ void __launch_bounds__(256) k_row_warp(RowArgs a) {
-  __shared__ int skey[8][32];
-  __shared__ long long sval[8][32];
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const unsigned cnt = *a.count;
-  const unsigned gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
-  for (unsigned i = gw; i < cnt; i += nw) {
-    const int cv = a.list[i];
-    const int64_t mb = a.mstart[cv], me = a.mstart[cv + 1];
-    int P = 0;
-    for (int64_t m = mb; m < me; m++) {
-      const int v = a.members[m];
-      const int64_t b = a.g.row_begin(v), e = a.g.row_begin(v + 1);
-      for (int64_t x = b; x < e; x += 32) {
-        const int64_t j = x + lane;
-        const bool valid = j < e;
-        const int cu = valid ? a.f2c[__ldg(a.g.adj + j)] : -1;
-        const bool keep = valid && cu != cv;
-        const unsigned mask = __ballot_sync(kFull, keep);
-        if (keep) {
-          const int pos = P + __popc(mask & lanemask_lt());
-          skey[wid][pos] = cu;
-          sval[wid][pos] = load_ew<EW>(a.g.ew, j);
+__global__ void __launch_bounds__(kSortThreads) k_pairs(DGraph g, const int32_t *members, const int64_t *mpre,
+                                                        const int32_t *f2c, unsigned long long *keys, void *vals,
+                                                        int bits, int64_t ntiles, int64_t *hist) {
+  __shared__ unsigned h[1 << kSortBits];
+  static_assert(kSortThreads == 1 << kSortBits, "one thread per digit");
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const unsigned mask = (1u << bits) - 1u;
+  const int64_t m = mpre[g.n];
+  h[threadIdx.x] = 0;
+  __syncthreads();
+  const int64_t s0 = (int64_t)blockIdx.x * kSortTile + (int64_t)wid * (32 * kSortItems);
+  if (s0 < m) {
+    int64_t x[kSortItems];
+    int cu[kSortItems];
+    int64_t base = 0, ends = 0, delta = 0;
+    int own = 0;
+    auto window = [&](int64_t i0) {  // lane l: row i0 + l (rows past the last one end where the walk ends)
+      base = i0;
+      const int64_t i = i0 + lane;
+      ends = mpre[i < g.n ? i + 1 : g.n];
+      if (i < g.n) {
+        const int v = members[i];
+        delta = g.row_begin(v) - mpre[i];
+        own = f2c[v];
+      }
+    };
+    window(warp_owner(mpre, g.n, s0));
+#pragma unroll
+    for (int k = 0; k < kSortItems; k++) {
+      const int64_t p = s0 + 32 * k + lane;
+      bool open = p < m;
+      x[k] = -1;
+      cu[k] = 0;
+      while (true) {
+        int j = 0;  // rows of the window that end at or before p (31 at most)
+#pragma unroll
+        for (int step = 16; step > 0; step >>= 1)
+          if (__shfl_sync(kFull, ends, j + step - 1) <= p) j += step;
+        const int64_t ej = __shfl_sync(kFull, ends, j), dj = __shfl_sync(kFull, delta, j);
+        const int cj = __shfl_sync(kFull, own, j);
+        if (open && ej > p) {
+          x[k] = p + dj;
+          cu[k] = cj;
+          open = false;
         }
-        P += __popc(mask);
+        const unsigned left = __ballot_sync(kFull, open);
+        if (!left) break;
+        // the next 32 rows, or past a stretch without entries the first open position's row
+        const int64_t want = s0 + 32 * k + (__ffs(left) - 1);
+        const int64_t after = base + 64 < g.n ? mpre[base + 64] : mpre[g.n];
+        window(after > want ? base + 32 : warp_owner(mpre, g.n, want));
       }
     }
-    __syncwarp();
-    int key = lane < P ? skey[wid][lane] : INT_MAX;
-    long long val = lane < P ? sval[wid][lane] : 0;
-    __syncwarp();
+    int cv[kSortItems];
 #pragma unroll
-    for (int k = 2; k <= 32; k <<= 1) {
+    for (int k = 0; k < kSortItems; k++) cv[k] = x[k] >= 0 ? __ldg(g.adj + x[k]) : 0;
 #pragma unroll
-      for (int j = k >> 1; j > 0; j >>= 1) {
-        const int ok = __shfl_xor_sync(kFull, key, j);
-        const long long ov = __shfl_xor_sync(kFull, val, j);
-        const bool up = (lane & k) == 0;
-        const bool lower = (lane & j) == 0;
-        const bool take = lower ? (up ? ok < key : ok > key) : (up ? ok > key : ok < key);
-        if (take) {
-          key = ok;
-          val = ov;
-        }
-      }
-    }
-    long long sum = 0;
+    for (int k = 0; k < kSortItems; k++) cv[k] = x[k] >= 0 ? f2c[cv[k]] : 0;
 #pragma unroll
-    for (int j = 0; j < 32; j++) {
-      const int kj = __shfl_sync(kFull, key, j);
-      const long long vj = __shfl_sync(kFull, val, j);
-      if (kj == key) sum += vj;
+    for (int k = 0; k < kSortItems; k++) {
+      if (x[k] < 0) continue;
+      const int64_t p = s0 + 32 * k + lane;
+      const bool out = cv[k] != cu[k];
+      keys[p] = out ? ((unsigned long long)(unsigned)cv[k] << 32) | (unsigned)cu[k] : kSortDropped;
+      if (EW == 1) static_cast<int32_t *>(vals)[p] = __ldg(static_cast<const int32_t *>(g.ew) + x[k]);
+      if (EW == 2) static_cast<long long *>(vals)[p] = __ldg(static_cast<const long long *>(g.ew) + x[k]);
+      if (out) atomicAdd(&h[(unsigned)cv[k] & mask], 1u);
     }
-    const int prev = __shfl_up_sync(kFull, key, 1);
-    const bool head = lane < P && (lane == 0 || prev != key);
-    const unsigned hm = __ballot_sync(kFull, head);
-    if (head) {
-      const int64_t pos = a.tstart[cv] + __popc(hm & lanemask_lt());
-      a.okey[pos] = key;
-      a.oval[pos] = sum;
-    }
-    if (lane == 0) a.rowcnt[cv] = __popc(hm);
-  }
-}
-
-
-
-__device__ __forceinline__ unsigned row_slot(int cu) { return mix32((unsigned)cu); }
-
-// Rows with 32 < pairs <= 256: one warp sums the pairs by neighbour id in a shared-memory hash
-// table, compacts the distinct ids and sorts them (bitonic) before writing the row.
-// Rows of up to S/2 pairs: one warp per row, an S-slot hash table per warp in shared memory (the
-// CTA's warps are laid out one table after another). The warp walks the concatenated rows of 32
-// members at a time, 64 entries per step (all lanes busy whatever the members' degrees, adjacency
-// read contiguously); equal coarse neighbours of one step are combined in the warp before they touch
-// the table.
-// Table values: 32-bit counts with unit edge weights (a coarse entry counts at most the fine entries,
-// fewer than 2^32), else 64-bit sums.
-template <int EW>
-using RowVal = typename std::conditional<EW == 0, unsigned, unsigned long long>::type;
-template <int EW>
-constexpr int row_slot_bytes() { return 4 + (int)sizeof(RowVal<EW>); }
-
-template <int EW, int S>
-__global__ void __launch_bounds__(kRowThreads) k_row_whash(RowArgs a) {
-  using V = RowVal<EW>;
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, nwb = blockDim.x >> 5;
-  V *vals = reinterpret_cast<V *>(smem) + wid * S;
-  int *keys = reinterpret_cast<int *>(smem + (size_t)nwb * S * sizeof(V)) + wid * S;
-  for (int t = lane; t < S; t += 32) {
-    keys[t] = -1;
-    vals[t] = 0;
-  }
-  __syncwarp();
-  const unsigned cnt = *a.count;
-  const unsigned gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
-  for (unsigned i = gw; i < cnt; i += nw) {
-    const int cv = a.list[i];
-    const int64_t mb = a.mstart[cv], me = a.mstart[cv + 1];
-    int cap = 64;
-    while (cap < 2 * a.dsum[cv]) cap <<= 1;
-    const unsigned mask = (unsigned)cap - 1;
-    for (int64_t m0 = mb; m0 < me; m0 += 32) {
-      // the warp walks the concatenation of the rows of members m0 .. m0+31, 64 entries per step
-      const int64_t m = m0 + lane;
-      int64_t rb = 0, deg = 0;
-      if (m < me) {
-        const int v = a.members[m];
-        rb = a.g.row_begin(v);
-        deg = a.g.row_begin(v + 1) - rb;
-      }
-      int64_t incl = deg;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int64_t y = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += y;
-      }
-      const int64_t excl = incl - deg;
-      const int64_t total = __shfl_sync(kFull, incl, 31);
-      for (int64_t t0 = 0; t0 < total; t0 += 64) {
-        int cu[2];
-        long long w[2];
-        bool on[2];
-#pragma unroll
-        for (int h = 0; h < 2; h++) {
-          const int64_t t = t0 + h * 32 + lane;
-          int j = 0;  // owner: the largest lane j with excl_j <= t
-#pragma unroll
-          for (int step = 16; step > 0; step >>= 1) {
-            const int64_t ex = __shfl_sync(kFull, excl, j + step);
-            if (j + step < 32 && ex <= t) j += step;
-          }
-          const int64_t x = __shfl_sync(kFull, rb, j) + (t - __shfl_sync(kFull, excl, j));
-          on[h] = t < total;
-          cu[h] = on[h] ? a.f2c[__ldg(a.g.adj + x)] : -1;
-          w[h] = on[h] ? load_ew<EW>(a.g.ew, x) : 0;
-        }
-#pragma unroll
-        for (int h = 0; h < 2; h++) {
-          const bool ok = on[h] && cu[h] != cv;
-          const unsigned peers = __match_any_sync(kFull, ok ? cu[h] : -1);
-          // weights below 2^26 sum exactly in 32 bits over at most 32 lanes: one warp reduction
-          const bool wide = EW != 0 && __any_sync(kFull, ok && (w[h] >= (1ll << 26) || w[h] < 0));
-          if (!ok) continue;
-          long long sum = 0;
-          if constexpr (EW == 0) {
-            sum = __popc(peers);
-          } else if (!wide) {
-            sum = (long long)__reduce_add_sync(peers, (unsigned)w[h]);
-          } else {
-            for (unsigned pm = peers; pm; pm &= pm - 1) sum += __shfl_sync(peers, w[h], __ffs(pm) - 1);
-          }
-          if (lane != __ffs(peers) - 1) continue;
-          unsigned sl = row_slot(cu[h]) & mask;
-          while (true) {
-            const int k = atomicCAS(&keys[sl], -1, cu[h]);
-            if (k == -1 || k == cu[h]) {
-              atomicAdd(&vals[sl], (V)sum);
-              break;
-            }
-            sl = (sl + 1) & mask;
-          }
-        }
-      }
-    }
-    __syncwarp();
-    // compact the used slots to the front (every lane reads its slot before anyone writes)
-    int u = 0;
-    for (int c0 = 0; c0 < cap; c0 += 32) {
-      const int k = keys[c0 + lane];
-      const V val = vals[c0 + lane];
-      const unsigned hm = __ballot_sync(kFull, k >= 0);
-      __syncwarp();
-      if (k >= 0) {
-        const int pos = u + __popc(hm & lanemask_lt());
-        keys[pos] = k;
-        vals[pos] = val;
-      }
-      u += __popc(hm);
-      __syncwarp();
-    }
-    int Pp = 1;
-    while (Pp < u) Pp <<= 1;
-    for (int t = u + lane; t < cap; t += 32) {
-      keys[t] = t < Pp ? INT_MAX : -1;
-      vals[t] = 0;
-    }
-    __syncwarp();
-    for (int k = 2; k <= Pp; k <<= 1) {
-      for (int j = k >> 1; j > 0; j >>= 1) {
-        for (int t = lane; t < Pp / 2; t += 32) {
-          const int lo = 2 * j * (t / j) + (t % j), hi = lo + j;
-          const bool up = (lo & k) == 0;
-          const int x = keys[lo], y = keys[hi];
-          if ((x > y) == up && x != y) {
-            keys[lo] = y;
-            keys[hi] = x;
-            const V vx = vals[lo];
-            vals[lo] = vals[hi];
-            vals[hi] = vx;
-          }
-        }
-        __syncwarp();
-      }
-    }
-    const int64_t dst = a.tstart[cv];
-    for (int t = lane; t < u; t += 32) {
-      a.okey[dst + t] = keys[t];
-      a.oval[dst + t] = (int64_t)vals[t];
-    }
-    if (lane == 0) a.rowcnt[cv] = u;
-    __syncwarp();
-    for (int t = lane; t < Pp; t += 32) {
-      keys[t] = -1;
-      vals[t] = 0;
-    }
-    __syncwarp();
-  }
-}
-
-// Rows with 256 < pairs <= 4096: the same with one CTA and a larger table.
-template <int EW>
-__global__ void __launch_bounds__(kRowThreads) k_row_cta(RowArgs a) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  long long *vals = reinterpret_cast<long long *>(smem);
-  int *keys = reinterpret_cast<int *>(smem + kCtaSlots * 8);
-  __shared__ long long tmp[32];
-  __shared__ long long tot_s, carry_s;
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-  for (int t = threadIdx.x; t < kCtaSlots; t += blockDim.x) {
-    keys[t] = -1;
-    vals[t] = 0;
   }
   __syncthreads();
-  const unsigned cnt = *a.count;
-  for (unsigned i = blockIdx.x; i < cnt; i += gridDim.x) {
-    const int cv = a.list[i];
-    const int64_t mb = a.mstart[cv], me = a.mstart[cv + 1];
-    int cap = 64;
-    while (cap < 2 * a.dsum[cv]) cap <<= 1;
-    const unsigned mask = (unsigned)cap - 1;
-    for (int64_t m = mb + wid; m < me; m += nwarps) {
-      const int v = a.members[m];
-      const int64_t b = a.g.row_begin(v), e = a.g.row_begin(v + 1);
-      for (int64_t x = b + lane; x < e; x += 32) {
-        const int cu = a.f2c[__ldg(a.g.adj + x)];
-        if (cu == cv) continue;
-        const long long w = load_ew<EW>(a.g.ew, x);
-        unsigned sl = row_slot(cu) & mask;
-        while (true) {
-          const int k = atomicCAS(&keys[sl], -1, cu);
-          if (k == -1 || k == cu) {
-            atomicAdd(reinterpret_cast<unsigned long long *>(&vals[sl]), (unsigned long long)w);
-            break;
-          }
-          sl = (sl + 1) & mask;
-        }
-      }
+  if (threadIdx.x <= mask) hist[(int64_t)threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
+}
+
+// Sorted pairs: the first of equal ones is a head. Heads per tile and per coarse row.
+constexpr int kHeadThreads = 256;
+constexpr int kHeadItems = 8;  // per lane
+constexpr int64_t kHeadTile = (int64_t)kHeadThreads * kHeadItems;
+
+__global__ void __launch_bounds__(kHeadThreads) k_heads(const unsigned long long *keys, const int64_t *n_dev,
+                                                        int64_t *tile_heads, int64_t *rowcnt) {
+  __shared__ unsigned s_heads;
+  const int64_t n = *n_dev;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t base = (int64_t)blockIdx.x * kHeadTile + (int64_t)wid * (32 * kHeadItems);
+  if (threadIdx.x == 0) s_heads = 0;
+  __syncthreads();
+  if (base < n) {
+    unsigned long long key[kHeadItems];
+#pragma unroll
+    for (int k = 0; k < kHeadItems; k++) {
+      const int64_t i = base + 32 * k + lane;
+      key[k] = i < n ? keys[i] : kSortDropped;
     }
-    if (threadIdx.x == 0) carry_s = 0;
-    __syncthreads();
-    for (int c0 = 0; c0 < cap; c0 += blockDim.x) {
-      const int t = c0 + threadIdx.x;
-      const int k = t < cap ? keys[t] : -1;
-      const long long val = t < cap ? vals[t] : 0;
-      const long long ex = block_excl_scan64((long long)(k >= 0 ? 1 : 0), tmp, &tot_s);
-      if (k >= 0) {
-        keys[carry_s + ex] = k;
-        vals[carry_s + ex] = val;
-      }
-      __syncthreads();
-      if (threadIdx.x == 0) carry_s += tot_s;
-      __syncthreads();
+    unsigned long long before = base > 0 ? keys[base - 1] : kSortDropped;
+    unsigned total = 0;
+#pragma unroll
+    for (int k = 0; k < kHeadItems; k++) {
+      unsigned long long prev = __shfl_up_sync(kFull, key[k], 1);
+      if (lane == 0) prev = before;
+      before = __shfl_sync(kFull, key[k], 31);
+      const bool head = base + 32 * k + lane < n && key[k] != prev;
+      const unsigned heads = __ballot_sync(kFull, head);
+      total += (unsigned)__popc(heads);
+      const int row = (int)(key[k] >> 32);
+      const unsigned peers = __match_any_sync(kFull, head ? row : -1);
+      if (head && lane == __ffs(peers) - 1)
+        atomicAdd(reinterpret_cast<unsigned long long *>(&rowcnt[row]), (unsigned long long)__popc(peers));
     }
-    const int u = (int)carry_s;
-    int Pp = 1;
-    while (Pp < u) Pp <<= 1;
-    for (int t = u + threadIdx.x; t < cap; t += blockDim.x) {
-      keys[t] = t < Pp ? INT_MAX : -1;
-      vals[t] = 0;
-    }
-    __syncthreads();
-    for (int k = 2; k <= Pp; k <<= 1) {
-      for (int j = k >> 1; j > 0; j >>= 1) {
-        for (int t = threadIdx.x; t < Pp / 2; t += blockDim.x) {
-          const int lo = 2 * j * (t / j) + (t % j), hi = lo + j;
-          const bool up = (lo & k) == 0;
-          const int x = keys[lo], y = keys[hi];
-          if ((x > y) == up && x != y) {
-            keys[lo] = y;
-            keys[hi] = x;
-            const long long vx = vals[lo];
-            vals[lo] = vals[hi];
-            vals[hi] = vx;
-          }
-        }
-        __syncthreads();
-      }
-    }
-    const int64_t dst = a.tstart[cv];
-    for (int t = threadIdx.x; t < u; t += blockDim.x) {
-      a.okey[dst + t] = keys[t];
-      a.oval[dst + t] = vals[t];
-    }
-    if (threadIdx.x == 0) a.rowcnt[cv] = u;
-    __syncthreads();
-    for (int t = threadIdx.x; t < Pp; t += blockDim.x) {
-      keys[t] = -1;
-      vals[t] = 0;
-    }
-    __syncthreads();
+    if (lane == 0) atomicAdd(&s_heads, total);
   }
+  __syncthreads();
+  if (threadIdx.x == 0) tile_heads[blockIdx.x] = s_heads;
 }
 
-// Rows with more than 4096 pairs: the pairs of all such rows are gathered into one array keyed by
-// (row index, neighbour id), sorted together by a device-wide radix sort and reduced by key.
-__global__ void k_large_index(const int32_t *list, const unsigned *count, int32_t *large_idx) {
-  const unsigned cnt = *count;
-  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x)
-    large_idx[list[i]] = (int32_t)i;
-}
-
+// Sorted pairs to coarse entries: a run of equal pairs becomes one entry at the run's rank. A run inside one
+// step of 32 is stored; the parts of a run that crosses steps are added (ew must be zero on entry).
 template <int EW>
-__global__ void k_large_gather(DGraph g, const int32_t *f2c, const int32_t *large_idx, const int64_t *lofs,
-                               unsigned long long *lfill, int kb, unsigned long long *keys,
-                               unsigned long long *vals) {
-  const int lane = threadIdx.x & 31;
-  const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t v = gw; v < g.n; v += nw) {
-    const int i = large_idx[f2c[v]];
-    if (i < 0) continue;
-    const int64_t b = g.row_begin(v), e = g.row_begin(v + 1);
-    unsigned long long pos = 0;
-    if (lane == 0) pos = atomicAdd(&lfill[i], (unsigned long long)(e - b));
-    pos = __shfl_sync(kFull, pos, 0) + (unsigned long long)lofs[i];
-    for (int64_t x = b + lane; x < e; x += 32) {
-      const int cu = f2c[__ldg(g.adj + x)];
-      keys[pos + (x - b)] = ((unsigned long long)i << kb) | (unsigned long long)(unsigned)cu;
-      vals[pos + (x - b)] = (unsigned long long)load_ew<EW>(g.ew, x);
-    }
+__global__ void __launch_bounds__(kHeadThreads) k_entries(const unsigned long long *keys, const void *vals,
+                                                          const int64_t *n_dev, const int64_t *tile_first, int32_t *adj,
+                                                          int64_t *ew) {
+  __shared__ unsigned s_warp[kHeadThreads / 32];
+  const int64_t n = *n_dev;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t tbase = (int64_t)blockIdx.x * kHeadTile;
+  if (tbase >= n) return;
+  const int64_t base = tbase + (int64_t)wid * (32 * kHeadItems);
+  unsigned long long key[kHeadItems], before = kSortDropped, after = kSortDropped;
+  long long w[kHeadItems];
+#pragma unroll
+  for (int k = 0; k < kHeadItems; k++) {
+    const int64_t i = base + 32 * k + lane;
+    key[k] = i < n ? keys[i] : kSortDropped;
+    w[k] = 0;
+    if (i < n) w[k] = EW == 0 ? 1 : EW == 1 ? (long long)static_cast<const int32_t *>(vals)[i] : static_cast<const long long *>(vals)[i];
   }
-}
-
-__global__ void k_large_heads(const unsigned long long *keys, int64_t N, int kb, const int32_t *list, int64_t *flag) {
-  const unsigned long long mask = (1ull << kb) - 1;
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < N; j += (int64_t)gridDim.x * blockDim.x) {
-    const unsigned long long k = keys[j];
-    const int cv = list[k >> kb];
-    const bool head = (int)(k & mask) != cv && (j == 0 || keys[j - 1] != k);
-    flag[j] = head ? 1 : 0;
+  if (base < n && base > 0) before = keys[base - 1];
+  if (base + 32 * kHeadItems < n) after = keys[base + 32 * kHeadItems];
+  unsigned heads[kHeadItems], total = 0;
+#pragma unroll
+  for (int k = 0; k < kHeadItems; k++) {
+    unsigned long long prev = __shfl_up_sync(kFull, key[k], 1);
+    if (lane == 0) prev = before;
+    before = __shfl_sync(kFull, key[k], 31);
+    heads[k] = __ballot_sync(kFull, base + 32 * k + lane < n && key[k] != prev);
+    total += (unsigned)__popc(heads[k]);
   }
-}
-
-// Sorted large-row pairs to coarse entries: every pair of a non-self run adds its weight to the run's
-// output slot (the run's rank among its row's runs, from the head scan), a warp adding once per run it
-// holds; the run's head writes the neighbour id. oval must be zero on entry.
-__global__ void k_large_write(const unsigned long long *keys, const unsigned long long *vals, int64_t N, int kb,
-                              const int32_t *list, const int64_t *uidx, const int64_t *lofs, const int64_t *tstart,
-                              int32_t *okey, int64_t *oval) {
-  const unsigned long long mask = (1ull << kb) - 1;
-  const int lane = threadIdx.x & 31;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t j0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); j0 < N; j0 += stride) {
-    const int64_t j = j0 + lane;
-    bool on = false;
-    unsigned long long out = ~0ull;
-    long long v = 0;
-    if (j < N) {
-      const unsigned long long k = keys[j];
-      const int64_t i = (int64_t)(k >> kb);
-      const int cu = (int)(k & mask), cv = list[i];
-      if (cu != cv) {
-        on = true;
-        const int64_t u1 = uidx[j + 1];
-        out = (unsigned long long)(tstart[cv] + (u1 - 1 - uidx[lofs[i]]));
-        v = (long long)vals[j];
-        if (u1 != uidx[j]) okey[out] = cu;
+  if (lane == 0) s_warp[wid] = total;
+  __syncthreads();
+  int64_t at = tile_first[blockIdx.x] - 1;  // rank of the run open before the warp's first item
+  for (int x = 0; x < wid; x++) at += s_warp[x];
+#pragma unroll
+  for (int k = 0; k < kHeadItems; k++) {
+    if (base + 32 * k >= n) break;  // (uniform over the warp)
+    const bool on = base + 32 * k + lane < n;
+    const int64_t run = at + __popc(heads[k] & (lanemask_lt() | 1u << lane));
+    const unsigned long long next = k + 1 < kHeadItems ? __shfl_sync(kFull, key[k + 1 < kHeadItems ? k + 1 : k], 0) : after;
+    const unsigned peers = __match_any_sync(kFull, on ? (unsigned)(run - at) : 64u);
+    long long sum = EW == 0 ? (long long)__popc(peers) : 0;
+    if (EW) {
+      // weights below 2^26 sum exactly in 32 bits over at most 32 lanes: one warp reduction
+      if (!__any_sync(kFull, w[k] >= (1ll << 26) || w[k] < 0)) {
+        sum = (long long)__reduce_add_sync(peers, (unsigned)w[k]);
+      } else {
+        for (unsigned pm = peers; pm; pm &= pm - 1) sum += __shfl_sync(peers, w[k], __ffs(pm) - 1);
       }
     }
-    const unsigned peers = __match_any_sync(kFull, out);
-    if (on) {
-      long long sum = 0;
-      for (unsigned m = peers; m; m &= m - 1) sum += __shfl_sync(peers, v, __ffs(m) - 1);
-      if (lane == __ffs(peers) - 1) atomicAdd(reinterpret_cast<unsigned long long *>(&oval[out]), (unsigned long long)sum);
+    if (on && lane == __ffs(peers) - 1) {
+      const bool starts = heads[k] >> lane & 1u;
+      const int last = 31 - __clz(peers);
+      const bool ends = last < 31 || next != key[k];
+      if (starts) adj[run] = (int32_t)(key[k] & 0xffffffffull);
+      if (starts && ends) ew[run] = sum;
+      else atomicAdd(reinterpret_cast<unsigned long long *>(&ew[run]), (unsigned long long)sum);
     }
+    at += __popc(heads[k]);
   }
 }
 
-__global__ void k_large_counts(const int32_t *list, const unsigned *count, const int64_t *uidx, const int64_t *lofs,
-                               int64_t *rowcnt) {
-  const unsigned cnt = *count;
-  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x)
-    rowcnt[list[i]] = uidx[lofs[i + 1]] - uidx[lofs[i]];
-}
-
-__global__ void k_large_sizes(const int32_t *list, const unsigned *count, const int64_t *dsum, int64_t *sz) {
-  const unsigned cnt = *count;
-  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x)
-    sz[i] = dsum[list[i]];
-}
-
-// Compaction of the rows into the coarse CSR: a warp per row of at most kCompactLong entries; longer
-// rows (the large clusters of power-law graphs) are cut into items of kCompactLong entries that the
-// CTAs take in turn, so that no single warp copies a row of millions of entries.
-constexpr int64_t kCompactLong = 4096;
-
-__global__ void k_compact_rows(int64_t nc, const int64_t *tstart, const int64_t *rowcnt, const int64_t *off,
-                               const int32_t *okey, const int64_t *oval, int32_t *adj, int64_t *ew) {
-  const int lane = threadIdx.x & 31;
-  const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t c = gw; c < nc; c += nw) {
-    const int64_t src = tstart[c], dst = off[c], len = rowcnt[c];
-    if (len > kCompactLong) continue;
-    for (int64_t t = lane; t < len; t += 32) {
-      adj[dst + t] = okey[src + t];
-      ew[dst + t] = oval[src + t];
-    }
-  }
-}
-
-// the long rows among the large ones: (coarse id << 32) | item, at most cap items
-__global__ void k_compact_list(const int32_t *list, const unsigned *count, const int64_t *rowcnt,
-                               unsigned long long *items, unsigned long long cap, unsigned long long *nitems) {
-  const unsigned cnt = *count;
-  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x) {
-    const int c = list[i];
-    const int64_t len = rowcnt[c];
-    if (len <= kCompactLong) continue;
-    const unsigned long long nch = (unsigned long long)((len + kCompactLong - 1) / kCompactLong);
-    const unsigned long long base = atomicAdd(nitems, nch);
-    for (unsigned long long x = 0; x < nch && base + x < cap; x++) items[base + x] = ((unsigned long long)c << 32) | x;
-  }
-}
-
-__global__ void k_compact_items(const unsigned long long *items, unsigned long long cap, const unsigned long long *nitems,
-                                const int64_t *tstart, const int64_t *rowcnt, const int64_t *off, const int32_t *okey,
-                                const int64_t *oval, int32_t *adj, int64_t *ew) {
-  const unsigned long long nit = min(*nitems, cap);
-  for (unsigned long long it = blockIdx.x; it < nit; it += gridDim.x) {
-    const int64_t c = (int64_t)(items[it] >> 32);
-    const int64_t b = (int64_t)(items[it] & 0xffffffffull) * kCompactLong;
-    const int64_t e = min(rowcnt[c], b + kCompactLong);
-    const int64_t src = tstart[c], dst = off[c];
-    for (int64_t t = b + threadIdx.x; t < e; t += blockDim.x) {
-      adj[dst + t] = okey[src + t];
-      ew[dst + t] = oval[src + t];
-    }
-  }
-}
-
-template <class K>
-void set_smem(K kernel, int bytes) {
-  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-}
-
+// The pairs of g, sorted by (cv, cu): keys and values end in *keys_out / *vals_out, their number on the device at
+// *count_out.
 template <int EW>
-int build_rows(RowArgs a, const unsigned *counts_dev, const unsigned counts[5], int32_t *lists[5], cudaStream_t s) {
-  const int nsm = num_sms();
-  auto grid_for = [&](int64_t items, int per_block, int limit) {
-    int64_t g = (items + per_block - 1) / per_block;
-    return (int)std::max<int64_t>(1, std::min<int64_t>(g, limit));
-  };
+int sorted_pairs(const DGraph &g, const int32_t *members, const int64_t *mpre, const int32_t *f2c, int kb,
+                 unsigned long long **keys_out, void **vals_out, int64_t **count_out, Workspace &ws) {
+  cudaStream_t s = ws.stream();
+  const size_t m = (size_t)g.m;
+  unsigned long long *k0, *k1;
+  unsigned char *v0 = nullptr, *v1 = nullptr;
+  GP_TRY(ws.get(&k0, m));
+  GP_TRY(ws.get(&k1, m));
+  if (kValBytes<EW>) {
+    GP_TRY(ws.get(&v0, m * kValBytes<EW>));
+    GP_TRY(ws.get(&v1, m * kValBytes<EW>));
+  }
+  const int passes = sort_passes(kb), width = std::max(1, (kb + passes - 1) / passes);
+  const int64_t ntiles = sort_tiles(g.m), cells = ntiles << width;
+  int64_t *hist, *count;
+  GP_TRY(ws.get(&hist, (size_t)cells + 1));
+  GP_TRY(ws.get(&count, 1));
   ProfScope ps("contract_rows", s);
-  if (counts[0]) {
-    RowArgs b = a;
-    b.list = lists[0];
-    b.count = counts_dev + 0;
-    (::gp::count_launch(), k_row_warp<EW><<<grid_for(counts[0], 8, nsm * 16), 256, 0, s>>>(b));
-  }
-  if (counts[3]) {
-    RowArgs b = a;
-    b.list = lists[3];
-    b.count = counts_dev + 3;
-    const int sm = (kRowThreads / 32) * kWarpSlots * row_slot_bytes<EW>();
-    set_smem(k_row_whash<EW, kWarpSlots>, sm);
-    (::gp::count_launch(), k_row_whash<EW, kWarpSlots><<<grid_for(counts[3], 8, nsm * (EW == 0 ? 6 : 4)), kRowThreads, sm, s>>>(b));
-  }
-  if (counts[4]) {
-    RowArgs b = a;
-    b.list = lists[4];
-    b.count = counts_dev + 4;
-    constexpr int kBigSlots = 2 * kRowWarpBig;
-    const int sm = 4 * kBigSlots * row_slot_bytes<EW>();  // 4 warps per CTA
-    set_smem(k_row_whash<EW, kBigSlots>, sm);
-    (::gp::count_launch(), k_row_whash<EW, kBigSlots><<<grid_for(counts[4], 4, nsm * (EW == 0 ? 3 : 2)), 128, sm, s>>>(b));
-  }
-  if (counts[1]) {
-    RowArgs b = a;
-    b.list = lists[1];
-    b.count = counts_dev + 1;
-    const int sm = kCtaSlots * 12;
-    set_smem(k_row_cta<EW>, sm);
-    (::gp::count_launch(), k_row_cta<EW><<<grid_for(counts[1], 1, nsm * 2), kRowThreads, sm, s>>>(b));
-  }
+  (::gp::count_launch(), k_pairs<EW><<<(unsigned)ntiles, kSortThreads, 0, s>>>(g, members, mpre, f2c, k0, v0, width, ntiles, hist));
   GP_LAUNCH_CHECK();
+  for (int p = 0; p < passes; p++) {
+    const int shift = 32 + p * width, w = std::max(1, std::min(width, kb - p * width));
+    if (p > 0) GP_TRY(radix_hist(k0, count, g.m, shift, w, hist, s));
+    GP_TRY(radix_offsets(hist, g.m, w, ws));
+    if (p == 0)  // the number of pairs that are not inside a cluster
+      GP_CUDA(cudaMemcpyAsync(count, hist + (ntiles << w), sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
+    GP_TRY(radix_scatter(k0, v0, k1, v1, kValBytes<EW>, p > 0 ? count : mpre + g.n, g.m, shift, w, hist, p == 0, s));
+    std::swap(k0, k1);
+    std::swap(v0, v1);
+  }
+  *keys_out = k0;
+  *vals_out = v0;
+  *count_out = count;
   return GP_OK;
 }
 
@@ -691,37 +375,29 @@ int contract_graph(const DGraph &g, const int32_t *labels, int64_t nl, OwnedGrap
   // arrays indexed by coarse vertex are sized for the bound min(n, nl) (zero beyond nc, so the scans
   // over the bound equal the scans over nc) and the row classification reads nc on the device.
   const int64_t ncb = std::max<int64_t>(1, std::min<int64_t>(n, nl));
-  // 2. fine -> coarse map, member counts, coarse vertex weights, degree sums
+  // 2. fine -> coarse map, member counts, coarse vertex weights
   int32_t *f2c = f2c_user;
   if (!f2c) GP_TRY(ws.get(&f2c, (size_t)n));
-  int64_t *cnt, *dsum, *mstart, *tstart, *cw;
+  int64_t *cnt, *mstart, *cw;
   GP_TRY(ws.zeros(&cnt, (size_t)ncb + 1));
-  GP_TRY(ws.zeros(&dsum, (size_t)ncb + 1));
   GP_TRY(ws.zeros(&cw, (size_t)ncb));
   GP_TRY(ws.get(&mstart, (size_t)ncb + 1));
-  GP_TRY(ws.get(&tstart, (size_t)ncb + 1));
-  (::gp::count_launch(), k_f2c<<<grid_n(n), 256, 0, s>>>(g, labels, nl, newid, f2c, cnt, cw, dsum, bad));
+  (::gp::count_launch(), k_f2c<<<grid_n(n), 256, 0, s>>>(g, labels, nl, newid, f2c, cnt, cw, bad));
   GP_LAUNCH_CHECK();
   GP_TRY(scan_excl_i64(cnt, mstart, ncb, mstart + ncb, ws));
-  GP_TRY(scan_excl_i64(dsum, tstart, ncb, tstart + ncb, ws));
-  // 3. members bucketed by coarse id
+  // 3. members bucketed by coarse id, and where their rows start in the walk over them
   unsigned *fill;
   int32_t *members;
+  int64_t *mpre;
+  unsigned long long *maxvw_dev;
   GP_TRY(ws.zeros(&fill, (size_t)ncb));
   GP_TRY(ws.get(&members, (size_t)n));
-  (::gp::count_launch(), k_members<<<grid_n(n), 256, 0, s>>>(n, f2c, mstart, fill, members));
-  // 4. rows binned by pair count
-  int32_t *lists[5];
-  unsigned *counts_dev;
-  for (int b = 0; b < 5; b++) GP_TRY(ws.get(&lists[b], (size_t)ncb));
-  GP_TRY(ws.zeros(&counts_dev, 5));
-  (::gp::count_launch(), k_row_classify<<<grid_n(ncb), 256, 0, s>>>(hdr, dsum, lists[0], lists[1], lists[2],
-                                                                     lists[3], lists[4], counts_dev));
-  GP_LAUNCH_CHECK();
-  unsigned long long *maxvw_dev;
+  GP_TRY(ws.get(&mpre, (size_t)n + 1));
   GP_TRY(ws.zeros(&maxvw_dev, 1));
-  (::gp::count_launch(), k_max_i64<<<grid_n(ncb), 256, 0, s>>>(cw, ncb, maxvw_dev));
-  unsigned counts[5];
+  (::gp::count_launch(),
+   k_members<<<grid_n(n), 256, 0, s>>>(g, f2c, mstart, fill, members, mpre, cw, ncb, maxvw_dev));
+  GP_LAUNCH_CHECK();
+  GP_TRY(scan_excl_i64(mpre, mpre, n, mpre + n, ws));
   unsigned long long maxvw = 0;
   int64_t hh[4];
   int hbad = 0;
@@ -729,7 +405,6 @@ int contract_graph(const DGraph &g, const int32_t *labels, int64_t nl, OwnedGrap
     Readback rb;
     rb.add(hh, hdr, sizeof(hh));
     rb.add(&hbad, bad, sizeof(int));
-    rb.add(counts, counts_dev, sizeof(counts));
     rb.add(&maxvw, maxvw_dev, sizeof(maxvw));
     GP_TRY(rb.run(s));
   }
@@ -738,75 +413,27 @@ int contract_graph(const DGraph &g, const int32_t *labels, int64_t nl, OwnedGrap
     return GP_ERR_INVALID_ARG;
   }
   const int64_t nc = hh[0];
-  RowArgs a;
-  a.g = g;
-  a.f2c = f2c;
-  a.mstart = mstart;
-  a.members = members;
-  a.tstart = tstart;
-  a.dsum = dsum;
   int kb = 0;
   while (kb < 31 && ((int64_t)1 << kb) < nc) kb++;
-  a.key_bits = kb;
-  GP_TRY(ws.get(&a.okey, (size_t)std::max<int64_t>(g.m, 1)));
-  GP_TRY(ws.get(&a.oval, (size_t)std::max<int64_t>(g.m, 1)));
-  GP_TRY(ws.get(&a.rowcnt, (size_t)nc + 1));
+  // 4. sorted pairs, heads per coarse row, coarse offsets
   const int ew = g.ew_mode();
-  if (counts[2]) {
-    // very large rows: gather, sort by (row, neighbour), reduce
-    ProfScope ps("contract_large_rows", s);
-    const unsigned R = counts[2];
-    int64_t *sz, *lofs;
-    GP_TRY(ws.get(&sz, (size_t)R));
-    GP_TRY(ws.get(&lofs, (size_t)R + 1));
-    (::gp::count_launch(), k_large_sizes<<<grid_n(R), 256, 0, s>>>(lists[2], counts_dev + 2, dsum, sz));
-    GP_TRY(scan_excl_i64(sz, lofs, R, lofs + R, ws));
-    int64_t N = 0;
-    GP_CUDA(cudaMemcpyAsync(&N, lofs + R, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    GP_CUDA(cudaStreamSynchronize(s));
-    int32_t *large_idx;
-    unsigned long long *lfill, *k0, *v0, *k1, *v1;
-    GP_TRY(ws.get(&large_idx, (size_t)nc));
-    GP_CUDA(cudaMemsetAsync(large_idx, 0xff, sizeof(int32_t) * (size_t)nc, s));
-    GP_TRY(ws.zeros(&lfill, (size_t)R));
-    GP_TRY(ws.get(&k0, (size_t)N));
-    GP_TRY(ws.get(&v0, (size_t)N));
-    GP_TRY(ws.get(&k1, (size_t)N));
-    GP_TRY(ws.get(&v1, (size_t)N));
-    (::gp::count_launch(), k_large_index<<<grid_n(R), 256, 0, s>>>(lists[2], counts_dev + 2, large_idx));
-    int rb = 0;
-    while (rb < 31 && ((int64_t)1 << rb) < (int64_t)R) rb++;
-    const int kbits = std::max(kb, 1);
-    if (ew == 0)
-      (::gp::count_launch(), k_large_gather<0><<<grid_n(n * 32), 256, 0, s>>>(g, f2c, large_idx, lofs, lfill, kbits, k0, v0));
-    else if (ew == 1)
-      (::gp::count_launch(), k_large_gather<1><<<grid_n(n * 32), 256, 0, s>>>(g, f2c, large_idx, lofs, lfill, kbits, k0, v0));
-    else
-      (::gp::count_launch(), k_large_gather<2><<<grid_n(n * 32), 256, 0, s>>>(g, f2c, large_idx, lofs, lfill, kbits, k0, v0));
-    GP_LAUNCH_CHECK();
-    bool in_tmp = false;
-    GP_TRY(radix_sort_pairs(k0, v0, k1, v1, N, rb + kbits, &in_tmp, ws));
-    unsigned long long *ks = in_tmp ? k1 : k0, *vs = in_tmp ? v1 : v0;
-    int64_t *flag, *uidx;
-    GP_TRY(ws.get(&flag, (size_t)N));
-    GP_TRY(ws.get(&uidx, (size_t)N + 1));
-    (::gp::count_launch(), k_large_heads<<<grid_n(N), 256, 0, s>>>(ks, N, kbits, lists[2], flag));
-    GP_TRY(scan_excl_i64(flag, uidx, N, uidx + N, ws));
-    // (the large rows' weights are summed into zeroed slots)
-    GP_CUDA(cudaMemsetAsync(a.oval, 0, sizeof(int64_t) * (size_t)std::max<int64_t>(g.m, 1), s));
-    (::gp::count_launch(), k_large_write<<<grid_n(N), 256, 0, s>>>(ks, vs, N, kbits, lists[2], uidx, lofs, tstart,
-                                                                   a.okey, a.oval));
-    (::gp::count_launch(), k_large_counts<<<grid_n(R), 256, 0, s>>>(lists[2], counts_dev + 2, uidx, lofs, a.rowcnt));
-    GP_LAUNCH_CHECK();
-  }
-  GP_TRY(ew == 0 ? build_rows<0>(a, counts_dev, counts, lists, s)
-       : ew == 1 ? build_rows<1>(a, counts_dev, counts, lists, s)
-                 : build_rows<2>(a, counts_dev, counts, lists, s));
-  // 5. coarse offsets from the unique counts, then compaction of the rows
-  int64_t mc = 0;
-  int64_t *off_tmp;
+  unsigned long long *keys = nullptr;
+  void *vals = nullptr;
+  int64_t *npairs = nullptr, *rowcnt, *off_tmp, *tile_heads = nullptr;
+  GP_TRY(ws.zeros(&rowcnt, (size_t)nc + 1));
   GP_TRY(ws.get(&off_tmp, (size_t)nc + 1));
-  GP_TRY(scan_excl_i64(a.rowcnt, off_tmp, nc, off_tmp + nc, ws));
+  const int64_t htiles = (g.m + kHeadTile - 1) / kHeadTile;
+  if (g.m > 0) {
+    GP_TRY(ew == 0   ? sorted_pairs<0>(g, members, mpre, f2c, kb, &keys, &vals, &npairs, ws)
+           : ew == 1 ? sorted_pairs<1>(g, members, mpre, f2c, kb, &keys, &vals, &npairs, ws)
+                     : sorted_pairs<2>(g, members, mpre, f2c, kb, &keys, &vals, &npairs, ws));
+    GP_TRY(ws.get(&tile_heads, (size_t)htiles));
+    (::gp::count_launch(), k_heads<<<(unsigned)htiles, kHeadThreads, 0, s>>>(keys, npairs, tile_heads, rowcnt));
+    GP_LAUNCH_CHECK();
+    GP_TRY(scan_excl_i64(tile_heads, tile_heads, htiles, nullptr, ws));
+  }
+  int64_t mc = 0;
+  GP_TRY(scan_excl_i64(rowcnt, off_tmp, nc, off_tmp + nc, ws));
   // the next level's LP degree classes need only the coarse offsets: computed here and read back
   // with the coarse entry count
   unsigned long long *cls_dev = nullptr;
@@ -830,22 +457,18 @@ int contract_graph(const DGraph &g, const int32_t *labels, int64_t nl, OwnedGrap
   out->max_vw = (int64_t)maxvw;
   GP_CUDA(cudaMemcpyAsync(out->off, off_tmp, sizeof(int64_t) * (size_t)(nc + 1), cudaMemcpyDeviceToDevice, s));
   GP_CUDA(cudaMemcpyAsync(out->vw, cw, sizeof(int64_t) * (size_t)nc, cudaMemcpyDeviceToDevice, s));
-  {
+  // 5. equal pairs summed into the coarse entries
+  if (mc > 0) {
     ProfScope ps("contract_compact", s);
-    (::gp::count_launch(), k_compact_rows<<<grid_n(nc * 32), 256, 0, s>>>(nc, tstart, a.rowcnt, out->off, a.okey, a.oval, out->adj, out->ew));
-    if (counts[2]) {
-      // items: at most one per kCompactLong coarse entries plus one per large row
-      const unsigned long long cap = (unsigned long long)(mc / kCompactLong + counts[2] + 1);
-      unsigned long long *items, *nitems;
-      GP_TRY(ws.get(&items, (size_t)cap));
-      GP_TRY(ws.zeros(&nitems, 1));
-      (::gp::count_launch(), k_compact_list<<<grid_n(counts[2]), 256, 0, s>>>(lists[2], counts_dev + 2, a.rowcnt, items,
-                                                                              cap, nitems));
-      (::gp::count_launch(), k_compact_items<<<num_sms() * 8, 256, 0, s>>>(items, cap, nitems, tstart, a.rowcnt,
-                                                                         out->off, a.okey, a.oval, out->adj, out->ew));
-    }
+    GP_CUDA(cudaMemsetAsync(out->ew, 0, sizeof(int64_t) * (size_t)mc, s));
+    if (ew == 0)
+      (::gp::count_launch(), k_entries<0><<<(unsigned)htiles, kHeadThreads, 0, s>>>(keys, vals, npairs, tile_heads, out->adj, out->ew));
+    else if (ew == 1)
+      (::gp::count_launch(), k_entries<1><<<(unsigned)htiles, kHeadThreads, 0, s>>>(keys, vals, npairs, tile_heads, out->adj, out->ew));
+    else
+      (::gp::count_launch(), k_entries<2><<<(unsigned)htiles, kHeadThreads, 0, s>>>(keys, vals, npairs, tile_heads, out->adj, out->ew));
+    GP_LAUNCH_CHECK();
   }
-  GP_LAUNCH_CHECK();
   if (profiling()) {
     const int64_t rb = n * 2 * g.offset_bytes() + g.m * (4 + g.ew_bytes()) + g.m * 4;
     prof_add_counts("contract_rows", nc, g.m, rb);

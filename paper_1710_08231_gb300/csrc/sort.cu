@@ -1,11 +1,11 @@
-// sort.cu -- device-wide stable LSD radix sort of (uint64 key, uint64 value) pairs.
+// sort.cu -- device-wide stable LSD radix sort of (uint64 key, value) pairs.
 //
-// Each pass handles 8 key bits with three kernels: per-tile digit histograms (digit-major), an
-// exclusive scan of the histograms, and a stable scatter in which every tile ranks its items per
-// digit in order (warp match + per-warp counts), stages them in shared memory in digit order and
-// writes each digit's run contiguously. Used where many independent rows must be sorted at
-// once (the contraction of very large clusters).
+// Each pass takes up to nine key bits with three kernels: per-tile digit counts (digit-major), an exclusive scan
+// of the counts, and a stable scatter in which every tile ranks its items per digit in order (one warp match
+// per 32 items, per-warp counts), stages them in shared memory in digit order and writes each digit's run
+// contiguously. Used where many independent rows must be sorted at once (contraction) and for vertex orders.
 #include <algorithm>
+#include <type_traits>
 
 #include "sort.cuh"
 
@@ -13,57 +13,99 @@ namespace gp {
 
 namespace {
 
-constexpr int kSortThreads = 256;
-constexpr int kSortItems = 8;
-constexpr int64_t kSortTile = (int64_t)kSortThreads * kSortItems;
+constexpr int kSortWarps = kSortThreads / 32;
+constexpr int kMaxDigits = 1 << kSortBits;
+static_assert(kSortThreads == kMaxDigits, "one thread per digit");
 
-__global__ void __launch_bounds__(kSortThreads) k_radix_hist(const unsigned long long *keys, int64_t n, int shift,
-                                                             int64_t ntiles, int64_t *hist) {
-  __shared__ unsigned h[256];
-  for (int t = threadIdx.x; t < 256; t += kSortThreads) h[t] = 0;
-  __syncthreads();
+__global__ void __launch_bounds__(kSortThreads) k_radix_hist(const unsigned long long *keys, const int64_t *n_dev,
+                                                             int64_t n_max, int shift, int bits, int64_t ntiles,
+                                                             int64_t *hist) {
+  __shared__ unsigned h[kMaxDigits];
+  const int64_t n = n_dev ? *n_dev : n_max;
   const int64_t base = (int64_t)blockIdx.x * kSortTile;
-  for (int k = 0; k < kSortItems; k++) {
-    const int64_t i = base + (int64_t)k * kSortThreads + threadIdx.x;
-    if (i < n) atomicAdd(&h[(keys[i] >> shift) & 255], 1u);
+  const unsigned mask = (1u << bits) - 1u;
+  h[threadIdx.x] = 0;
+  __syncthreads();
+  if (base < n) {
+    unsigned long long key[kSortItems];
+#pragma unroll
+    for (int k = 0; k < kSortItems; k++) {
+      const int64_t i = base + (int64_t)k * kSortThreads + threadIdx.x;
+      key[k] = i < n ? keys[i] : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < kSortItems; k++)
+      if (base + (int64_t)k * kSortThreads + threadIdx.x < n) atomicAdd(&h[(unsigned)(key[k] >> shift) & mask], 1u);
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < 256; t += kSortThreads) hist[(int64_t)t * ntiles + blockIdx.x] = h[t];
+  if (threadIdx.x <= mask) hist[(int64_t)threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
 }
 
-// Stable scatter of one pass. Warp w of a tile owns its items [w, w + 1) * 32 kSortItems (the tile's
-// order is warp, then round, then lane). The warps count their digits first; the counts become each
-// warp's starting positions inside the tile's digit runs; the warps then place their items in order
-// in shared memory, and the tile leaves run by run: consecutive threads write consecutive addresses.
-__global__ void __launch_bounds__(kSortThreads) k_radix_scatter(const unsigned long long *kin,
-                                                                const unsigned long long *vin,
-                                                                unsigned long long *kout, unsigned long long *vout,
-                                                                int64_t n, int shift, int64_t ntiles,
-                                                                const int64_t *offs) {
-  extern __shared__ unsigned long long s_items[];  // kSortTile keys, then kSortTile values
-  constexpr int kW = kSortThreads / 32;
-  static_assert(kSortThreads == 256, "one thread per digit");
-  __shared__ unsigned wpos[kW][256];
-  __shared__ unsigned loc[256];
-  __shared__ int64_t gbase[256];
-  __shared__ unsigned wsum[kW];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+// Stable scatter of one pass. Warp w of a tile owns its items [w, w + 1) * 32 kSortItems (the tile's order is
+// warp, then round, then lane). Bound by memory: an item is read once and written once; its key stays in a
+// register between ranking and staging. Two blocks per SM hold 8192 items of 16 bytes in shared memory.
+struct NoVal {};
+
+template <class V>
+__global__ void __launch_bounds__(kSortThreads, 2) k_radix_scatter(const unsigned long long *kin, const V *vin,
+                                                                   unsigned long long *kout, V *vout,
+                                                                   const int64_t *n_dev, int64_t n_max, int shift,
+                                                                   int bits, int64_t ntiles, const int64_t *offs,
+                                                                   bool drop) {
+  constexpr bool kVals = !std::is_same<V, NoVal>::value;
+  extern __shared__ unsigned long long s_key[];  // kSortTile keys, then kSortTile values
+  V *const s_val = reinterpret_cast<V *>(s_key + kSortTile);
+  __shared__ unsigned short wcnt[kSortWarps][kMaxDigits];
+  __shared__ unsigned loc[kMaxDigits];
+  __shared__ int64_t gbase[kMaxDigits];
+  __shared__ unsigned wsum[kSortWarps];
+  const int64_t n = n_dev ? *n_dev : n_max;
   const int64_t tbase = (int64_t)blockIdx.x * kSortTile;
-  const int64_t wbase = tbase + (int64_t)wid * (32 * kSortItems);
-  for (int d = lane; d < 256; d += 32) wpos[wid][d] = 0;
-  __syncwarp();
+  if (tbase >= n) return;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const unsigned mask = (1u << bits) - 1u;
+  const int64_t wbase = tbase + (int64_t)wid * (32 * kSortItems) + lane;
+  unsigned long long key[kSortItems];
+#pragma unroll
+  for (int k = 0; k < kSortItems; k++) key[k] = wbase + 32 * k < n ? kin[wbase + 32 * k] : kSortDropped;
+  // this thread's digit's first output position (loaded while the items are ranked)
+  const int64_t first = threadIdx.x <= mask ? offs[(int64_t)threadIdx.x * ntiles + blockIdx.x] : 0;
+  V val[kVals ? kSortItems : 1];
+  if constexpr (kVals) {
+#pragma unroll
+    for (int k = 0; k < kSortItems; k++) val[k] = wbase + 32 * k < n ? vin[wbase + 32 * k] : (V)0;
+  }
+  for (int t = threadIdx.x; t < kSortWarps * kMaxDigits / 2; t += kSortThreads) reinterpret_cast<unsigned *>(wcnt)[t] = 0;
+  __syncthreads();
+  unsigned live = 0;
+  unsigned short rank[kSortItems];
+#pragma unroll
   for (int k = 0; k < kSortItems; k++) {
-    const int64_t i = wbase + k * 32 + lane;
-    const int dg = i < n ? (int)((kin[i] >> shift) & 255) : 256;
+    const bool on = wbase + 32 * k < n && !(drop && key[k] == kSortDropped);
+    const unsigned dg = on ? (unsigned)(key[k] >> shift) & mask : (unsigned)kMaxDigits;
     const unsigned peers = __match_any_sync(kFull, dg);
-    if (dg < 256 && lane == __ffs(peers) - 1) wpos[wid][dg] += (unsigned)__popc(peers);
+    const unsigned lt = (unsigned)__popc(peers & lanemask_lt());
+    unsigned old = 0;
+    if (on) {
+      old = wcnt[wid][dg];
+      live |= 1u << k;
+    }
     __syncwarp();
+    if (on && lt == 0) wcnt[wid][dg] = (unsigned short)(old + __popc(peers));
+    __syncwarp();
+    rank[k] = (unsigned short)(old + lt);
   }
   __syncthreads();
   {
+    // thread d: the warps' starts inside digit d's run, and the run's start in the tile
     const int d = threadIdx.x;
     unsigned tot = 0;
-    for (int w = 0; w < kW; w++) tot += wpos[w][d];
+#pragma unroll
+    for (int w = 0; w < kSortWarps; w++) {
+      const unsigned c = wcnt[w][d];
+      wcnt[w][d] = (unsigned short)tot;
+      tot += c;
+    }
     unsigned x = tot;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -75,64 +117,84 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(const unsigned l
     unsigned run = x - tot;
     for (int w = 0; w < wid; w++) run += wsum[w];
     loc[d] = run;
-    for (int w = 0; w < kW; w++) {
-      const unsigned c = wpos[w][d];
-      wpos[w][d] = run;
-      run += c;
-    }
-    gbase[d] = offs[(int64_t)d * ntiles + blockIdx.x];
+    gbase[d] = first - (int64_t)run;
   }
   __syncthreads();
+#pragma unroll
   for (int k = 0; k < kSortItems; k++) {
-    const int64_t i = wbase + k * 32 + lane;
-    const bool valid = i < n;
-    const unsigned long long key = valid ? kin[i] : 0, val = valid ? vin[i] : 0;
-    const int dg = valid ? (int)((key >> shift) & 255) : 256;
-    const unsigned peers = __match_any_sync(kFull, dg);
-    const unsigned rank = (unsigned)__popc(peers & lanemask_lt());
-    if (valid) {
-      const unsigned p = wpos[wid][dg] + rank;
-      s_items[p] = key;
-      s_items[kSortTile + p] = val;
+    if (live >> k & 1u) {
+      const unsigned dg = (unsigned)(key[k] >> shift) & mask;
+      const unsigned p = loc[dg] + wcnt[wid][dg] + rank[k];
+      s_key[p] = key[k];
+      if constexpr (kVals) s_val[p] = val[k];
     }
-    __syncwarp();
-    if (valid && rank == 0) wpos[wid][dg] += (unsigned)__popc(peers);
-    __syncwarp();
   }
   __syncthreads();
-  const int tn = (int)min((int64_t)kSortTile, n - tbase);
-  for (int p = threadIdx.x; p < tn; p += kSortThreads) {
-    const unsigned long long key = s_items[p];
-    const int dg = (int)((key >> shift) & 255);
-    const int64_t out = gbase[dg] + (int64_t)(p - (int)loc[dg]);
-    kout[out] = key;
-    vout[out] = s_items[kSortTile + p];
+  unsigned tn = 0;
+#pragma unroll
+  for (int w = 0; w < kSortWarps; w++) tn += wsum[w];
+  for (unsigned p = threadIdx.x; p < tn; p += kSortThreads) {
+    const unsigned long long x = s_key[p];
+    const int64_t out = gbase[(unsigned)(x >> shift) & mask] + (int64_t)p;
+    kout[out] = x;
+    if constexpr (kVals) vout[out] = s_val[p];
   }
 }
 
+template <class V>
+int scatter_as(const unsigned long long *kin, const void *vin, unsigned long long *kout, void *vout,
+               const int64_t *n_dev, int64_t n_max, int shift, int bits, const int64_t *offs, bool drop,
+               cudaStream_t s) {
+  constexpr int kBytes = (int)(kSortTile * (8 + (std::is_same<V, NoVal>::value ? 0 : sizeof(V))));
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(k_radix_scatter<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
+  GP_CUDA(attr);
+  const int64_t ntiles = sort_tiles(n_max);
+  (::gp::count_launch(), k_radix_scatter<V><<<(unsigned)ntiles, kSortThreads, kBytes, s>>>(
+                             kin, static_cast<const V *>(vin), kout, static_cast<V *>(vout), n_dev, n_max, shift, bits,
+                             ntiles, offs, drop));
+  GP_LAUNCH_CHECK();
+  return GP_OK;
+}
+
 }  // namespace
+
+int radix_hist(const unsigned long long *keys, const int64_t *n_dev, int64_t n_max, int shift, int bits, int64_t *hist,
+               cudaStream_t s) {
+  const int64_t ntiles = sort_tiles(n_max);
+  (::gp::count_launch(),
+   k_radix_hist<<<(unsigned)ntiles, kSortThreads, 0, s>>>(keys, n_dev, n_max, shift, bits, ntiles, hist));
+  GP_LAUNCH_CHECK();
+  return GP_OK;
+}
+
+int radix_offsets(int64_t *hist, int64_t n_max, int bits, Workspace &ws) {
+  const int64_t cells = sort_tiles(n_max) << bits;
+  return scan_excl_i64(hist, hist, cells, hist + cells, ws);
+}
+
+int radix_scatter(const unsigned long long *kin, const void *vin, unsigned long long *kout, void *vout, int val_bytes,
+                  const int64_t *n_dev, int64_t n_max, int shift, int bits, const int64_t *offs, bool drop,
+                  cudaStream_t s) {
+  if (val_bytes == 0) return scatter_as<NoVal>(kin, vin, kout, vout, n_dev, n_max, shift, bits, offs, drop, s);
+  if (val_bytes == 4) return scatter_as<unsigned>(kin, vin, kout, vout, n_dev, n_max, shift, bits, offs, drop, s);
+  return scatter_as<unsigned long long>(kin, vin, kout, vout, n_dev, n_max, shift, bits, offs, drop, s);
+}
 
 int radix_sort_pairs(unsigned long long *keys, unsigned long long *vals, unsigned long long *keys_tmp,
                      unsigned long long *vals_tmp, int64_t n, int bits, bool *result_in_tmp, Workspace &ws) {
   cudaStream_t s = ws.stream();
   *result_in_tmp = false;
   if (n <= 1 || bits <= 0) return GP_OK;
-  const int64_t ntiles = (n + kSortTile - 1) / kSortTile;
-  constexpr int kScatterSmem = (int)(2 * kSortTile * sizeof(unsigned long long));
-  static bool smem_set = false;
-  if (!smem_set) {
-    GP_CUDA(cudaFuncSetAttribute(k_radix_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, kScatterSmem));
-    smem_set = true;
-  }
-  int64_t *hist, *offs;
-  GP_TRY(ws.get(&hist, (size_t)(256 * ntiles)));
-  GP_TRY(ws.get(&offs, (size_t)(256 * ntiles + 1)));
+  const int passes = sort_passes(bits), width = (bits + passes - 1) / passes;
+  int64_t *hist;
+  GP_TRY(ws.get(&hist, (size_t)((sort_tiles(n) << width) + 1)));
   unsigned long long *ks = keys, *vs = vals, *kd = keys_tmp, *vd = vals_tmp;
-  for (int shift = 0; shift < bits; shift += 8) {
-    (::gp::count_launch(), k_radix_hist<<<(unsigned)ntiles, kSortThreads, 0, s>>>(ks, n, shift, ntiles, hist));
-    GP_TRY(scan_excl_i64(hist, offs, 256 * ntiles, offs + 256 * ntiles, ws));
-    (::gp::count_launch(), k_radix_scatter<<<(unsigned)ntiles, kSortThreads, kScatterSmem, s>>>(ks, vs, kd, vd, n, shift, ntiles, offs));
-    GP_LAUNCH_CHECK();
+  for (int shift = 0; shift < bits; shift += width) {
+    const int w = std::min(width, bits - shift);
+    GP_TRY(radix_hist(ks, nullptr, n, shift, w, hist, s));
+    GP_TRY(radix_offsets(hist, n, w, ws));
+    GP_TRY(radix_scatter(ks, vs, kd, vd, 8, nullptr, n, shift, w, hist, false, s));
     std::swap(ks, kd);
     std::swap(vs, vd);
     *result_in_tmp = !*result_in_tmp;

@@ -148,6 +148,8 @@ def lib():
         L.gp_coarse_graph.argtypes = [VP]
         L.gp_coarse_free.restype = None
         L.gp_coarse_free.argtypes = [VP, VP]
+        L.gp_coarse_drop.restype = None
+        L.gp_coarse_drop.argtypes = [VP, VP]
         L.gp_partition.restype = ctypes.c_int
         L.gp_partition.argtypes = [ctypes.POINTER(GpGraph), I32, DBL, U64, ctypes.POINTER(GpParams), VP,
                                    ctypes.POINTER(GpResult), VP]
@@ -359,7 +361,8 @@ def lp_refine(dg: DeviceGraph, part, k: int, lmax_: int, rounds: int, seed: int,
 
 
 class CoarseGraph:
-    """Library-owned coarse graph returned by ``contract``; freed with ``free()`` or on collection."""
+    """Library-owned coarse graph returned by ``contract``; freed with ``free()``, or with the library's next
+    allocation after it was collected."""
 
     def __init__(self, handle, stream):
         self.handle = handle
@@ -383,8 +386,12 @@ class CoarseGraph:
             self.handle = None
 
     def __del__(self):
+        # (tensors that view the arrays may outlive their owner by a few statements: the memory goes back
+        # with the library's next allocation, not to torch's next tensor)
         try:
-            self.free()
+            if self.handle:
+                lib().gp_coarse_drop(self.handle, self._stream)
+                self.handle = None
         except Exception:
             pass
 

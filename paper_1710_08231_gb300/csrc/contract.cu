@@ -17,76 +17,64 @@
 
 #include "contract.cuh"
 #include "lp.cuh"
-#include "sort.cuh"
+#include "sort_tile.cuh"
 
 namespace gp {
 
 namespace {
 
-__global__ void k_mark_used(const int32_t *labels, int64_t n, int64_t nl, uint32_t *used, int *bad) {
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-    const int L = labels[v];
-    if (L < 0 || L >= nl) {
-      atomicExch(bad, 1);
-      continue;
-    }
-    used[L] = 1;
-  }
-}
-
-// Fine -> coarse map and, per coarse vertex, member count and weight. Members of one cluster are mostly
-// neighbours in id order, so the warp combines equal coarse ids before its atomics.
-// A label outside [0, nl) sets *bad and maps its vertex to 0 (the caller reports the error).
-__global__ void k_f2c(DGraph g, const int32_t *labels, int64_t nl, const int32_t *newid, int32_t *f2c, int64_t *cnt,
-                      int64_t *cw, int *bad) {
-  const int lane = threadIdx.x & 31;
-  for (int64_t v0 = blockIdx.x * (int64_t)blockDim.x; v0 < g.n; v0 += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t v = v0 + threadIdx.x;
-    bool ok = v < g.n;
-    int cv = 0;
-    long long c = 0;
-    if (ok) {
-      const int L = labels[v];
-      if (L < 0 || L >= nl) {
-        atomicExch(bad, 1);
-        f2c[v] = 0;
-        ok = false;
-      } else {
-        cv = newid[L];
-        f2c[v] = cv;
-        c = g.vweight(v);
-      }
-    }
-    const unsigned peers = __match_any_sync(kFull, ok ? cv : -1);
-    if (!ok) continue;
-    long long cs = 0;
-    for (unsigned m = peers; m; m &= m - 1) cs += __shfl_sync(peers, c, __ffs(m) - 1);
-    if (lane == __ffs(peers) - 1) {
-      atomicAdd(reinterpret_cast<unsigned long long *>(&cnt[cv]), (unsigned long long)__popc(peers));
-      atomicAdd(reinterpret_cast<unsigned long long *>(&cw[cv]), (unsigned long long)cs);
-    }
-  }
-}
-
-// Members bucketed by coarse id (in any order within a cluster) with their degrees; largest coarse weight.
-__global__ void k_members(DGraph g, const int32_t *f2c, const int64_t *mstart, unsigned *fill, int32_t *members,
-                          int64_t *mdeg, const int64_t *cw, int64_t ncb, unsigned long long *maxcw) {
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < g.n; v += (int64_t)gridDim.x * blockDim.x) {
-    const int cv = f2c[v];
-    const int64_t pos = mstart[cv] + atomicAdd(&fill[cv], 1u);
-    members[pos] = (int32_t)v;
-    mdeg[pos] = g.row_begin(v + 1) - g.row_begin(v);
-  }
-  unsigned long long m = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ncb; i += (int64_t)gridDim.x * blockDim.x)
-    m = max(m, (unsigned long long)cw[i]);
-  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(kFull, m, o));
-  if ((threadIdx.x & 31) == 0 && m) atomicMax(maxcw, m);
-}
+constexpr int kMaxContractBlocks = 1024;  // (per-block partial sums)
 
 // Edge-weight values that travel with the pairs: none (unit weights), 32 or 64 bits.
 template <int EW>
-constexpr int kValBytes = EW == 0 ? 0 : (EW == 1 ? 4 : 8);
+struct PairVal {
+  using T = NoVal;
+};
+template <>
+struct PairVal<1> {
+  using T = unsigned;
+};
+template <>
+struct PairVal<2> {
+  using T = unsigned long long;
+};
+
+constexpr int kThreads = kSortThreads;
+constexpr int kHeadThreads = 256;
+constexpr int kHeadItems = 8;  // per lane
+constexpr int64_t kHeadTile = (int64_t)kHeadThreads * kHeadItems;
+
+// What the host reads back.
+struct ContractHead {
+  int64_t nc, mc, pairs;
+  unsigned long long maxcw;
+  unsigned long long classes[kLpClassWords];
+  int bad, err;
+};
+
+struct ContractArgs {
+  DGraph g;
+  const int32_t *labels;
+  int64_t nl;
+  uint32_t *used;    // zeroed (used, cnt, cw, rowcnt, head, bar)
+  int32_t *newid, *f2c, *members;
+  int64_t *cnt, *mstart, *cw, *mpre, *hist, *tile_heads, *rowcnt, *off, *part;
+  unsigned long long *k0, *k1;
+  void *v0, *v1;
+  int *tile_n;
+  ContractHead *head;
+  unsigned *bar;
+  unsigned wait_us;
+  int want_classes, deg_warp, deg_cta;
+};
+
+struct ContractSmem {
+  RadixSmem radix;
+  unsigned h[kMaxDigits];
+  unsigned wbase[kSortWarps + 1];
+  long long tmp[32], tot;
+  unsigned heads[2];
+};
 
 // The largest i with pre[i] <= x (0 <= x < pre[n]), found by the whole warp: 32 pivots per step.
 __device__ __forceinline__ int64_t warp_owner(const int64_t *pre, int64_t n, int64_t x) {
@@ -102,26 +90,79 @@ __device__ __forceinline__ int64_t warp_owner(const int64_t *pre, int64_t n, int
   return lo;
 }
 
-// The pairs in walking order, keys (cv << 32 | cu) and values omega, and the digit counts of the sort's first
-// pass. Position p of the walk belongs to the member row with mpre[i] <= p < mpre[i + 1]; a warp takes 256
-// consecutive positions, eight per lane, whatever rows they lie in: 32 rows at a time are held by the lanes
-// and searched by shuffles. All positions are resolved first, then their adjacency entries are loaded, then
-// the coarse ids of those are gathered, so that eight gathers per lane are in flight: the gathers bound it.
+// A scan over all blocks in two halves with a meeting between them: every block sums a contiguous chunk (the sum
+// goes to part[block]); then it adds up the chunks before its own and writes its exclusive sums. Four
+// consecutive items per thread.
+__device__ __forceinline__ int64_t scan_chunk(int64_t n) {
+  const int64_t step = 4 * kThreads;
+  return ((n + gridDim.x - 1) / gridDim.x + step - 1) / step * step;
+}
+
+template <class In>
+__device__ __forceinline__ void scan_sums(int64_t n, In in, int64_t *part, ContractSmem &sm) {
+  const int64_t per = scan_chunk(n), lo = min(n, (int64_t)blockIdx.x * per), hi = min(n, lo + per);
+  long long s = 0;
+  for (int64_t i = lo + threadIdx.x; i < hi; i += kThreads) s += in(i);
+  block_excl_scan64(s, sm.tmp, &sm.tot);
+  if (threadIdx.x == 0) part[blockIdx.x] = sm.tot;
+}
+
+// Returns the sum of all items. out(i, sum of the items before i) may overwrite item i.
+template <class In, class Out>
+__device__ __forceinline__ int64_t scan_write(int64_t n, In in, Out out, const int64_t *part, ContractSmem &sm) {
+  const int64_t per = scan_chunk(n), lo = min(n, (int64_t)blockIdx.x * per), hi = min(n, lo + per);
+  __syncthreads();
+  long long before = 0, all = 0;
+  for (unsigned x = threadIdx.x; x < gridDim.x; x += kThreads) {
+    const long long p = part[x];
+    all += p;
+    if (x < blockIdx.x) before += p;
+  }
+  block_excl_scan64(all, sm.tmp, &sm.tot);
+  const long long total = sm.tot;
+  block_excl_scan64(before, sm.tmp, &sm.tot);
+  long long run = sm.tot;
+  for (int64_t base = lo; base < hi; base += 4 * kThreads) {
+    const int64_t i = base + 4 * (int64_t)threadIdx.x;
+    long long x[4], s = 0;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      x[k] = i + k < hi ? (long long)in(i + k) : 0;
+      s += x[k];
+    }
+    long long at = run + block_excl_scan64(s, sm.tmp, &sm.tot);
+    run += sm.tot;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      if (i + k < hi) out(i + k, at);
+      at += x[k];
+    }
+  }
+  return total;
+}
+
+// The pairs of tile `tile` of the walk, keys (cv << 32 | cu) and values omega, compacted to the tile's front, and
+// the digit counts of the sort's first pass. Position p of the walk belongs to the member row with
+// mpre[i] <= p < mpre[i + 1]; a warp takes 256 consecutive positions, eight per lane, whatever rows they lie in:
+// 32 rows at a time are held by the lanes and searched by shuffles. All positions are resolved first, then
+// their adjacency entries are loaded, then the coarse ids of those are gathered, so that eight gathers per lane
+// are in flight: the gathers bound it.
 template <int EW>
-__global__ void __launch_bounds__(kSortThreads) k_pairs(DGraph g, const int32_t *members, const int64_t *mpre,
-                                                        const int32_t *f2c, unsigned long long *keys, void *vals,
-                                                        int bits, int64_t ntiles, int64_t *hist) {
-  __shared__ unsigned h[1 << kSortBits];
-  static_assert(kSortThreads == 1 << kSortBits, "one thread per digit");
+__device__ __forceinline__ void pairs_tile(const ContractArgs &a, int64_t tile, int64_t m, int bits, int64_t ntiles,
+                                           ContractSmem &sm) {
+  using V = typename PairVal<EW>::T;
+  const DGraph &g = a.g;
+  const int64_t *const mpre = a.mpre;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const unsigned mask = (1u << bits) - 1u;
-  const int64_t m = mpre[g.n];
-  h[threadIdx.x] = 0;
+  const int64_t s0 = tile * kSortTile + (int64_t)wid * (32 * kSortItems);
   __syncthreads();
-  const int64_t s0 = (int64_t)blockIdx.x * kSortTile + (int64_t)wid * (32 * kSortItems);
+  sm.h[threadIdx.x] = 0;
+  int64_t x[kSortItems];
+  int cu[kSortItems], cv[kSortItems];
+#pragma unroll
+  for (int k = 0; k < kSortItems; k++) x[k] = -1;
   if (s0 < m) {
-    int64_t x[kSortItems];
-    int cu[kSortItems];
     int64_t base = 0, ends = 0, delta = 0;
     int own = 0;
     auto window = [&](int64_t i0) {  // lane l: row i0 + l (rows past the last one end where the walk ends)
@@ -129,9 +170,9 @@ __global__ void __launch_bounds__(kSortThreads) k_pairs(DGraph g, const int32_t 
       const int64_t i = i0 + lane;
       ends = mpre[i < g.n ? i + 1 : g.n];
       if (i < g.n) {
-        const int v = members[i];
+        const int v = a.members[i];
         delta = g.row_begin(v) - mpre[i];
-        own = f2c[v];
+        own = a.f2c[v];
       }
     };
     window(warp_owner(mpre, g.n, s0));
@@ -139,7 +180,6 @@ __global__ void __launch_bounds__(kSortThreads) k_pairs(DGraph g, const int32_t 
     for (int k = 0; k < kSortItems; k++) {
       const int64_t p = s0 + 32 * k + lane;
       bool open = p < m;
-      x[k] = -1;
       cu[k] = 0;
       while (true) {
         int j = 0;  // rows of the window that end at or before p (31 at most)
@@ -157,51 +197,60 @@ __global__ void __launch_bounds__(kSortThreads) k_pairs(DGraph g, const int32_t 
         if (!left) break;
         // the next 32 rows, or past a stretch without entries the first open position's row
         const int64_t want = s0 + 32 * k + (__ffs(left) - 1);
-        const int64_t after = base + 64 < g.n ? mpre[base + 64] : mpre[g.n];
+        const int64_t after = mpre[base + 64 < g.n ? base + 64 : g.n];
         window(after > want ? base + 32 : warp_owner(mpre, g.n, want));
       }
     }
-    int cv[kSortItems];
+  }
 #pragma unroll
-    for (int k = 0; k < kSortItems; k++) cv[k] = x[k] >= 0 ? __ldg(g.adj + x[k]) : 0;
+  for (int k = 0; k < kSortItems; k++) cv[k] = x[k] >= 0 ? __ldg(g.adj + x[k]) : -1;
 #pragma unroll
-    for (int k = 0; k < kSortItems; k++) cv[k] = x[k] >= 0 ? f2c[cv[k]] : 0;
+  for (int k = 0; k < kSortItems; k++) cv[k] = x[k] >= 0 ? a.f2c[cv[k]] : -1;
+  unsigned kept = 0;
 #pragma unroll
-    for (int k = 0; k < kSortItems; k++) {
-      if (x[k] < 0) continue;
-      const int64_t p = s0 + 32 * k + lane;
-      const bool out = cv[k] != cu[k];
-      keys[p] = out ? ((unsigned long long)(unsigned)cv[k] << 32) | (unsigned)cu[k] : kSortDropped;
-      if (EW == 1) static_cast<int32_t *>(vals)[p] = __ldg(static_cast<const int32_t *>(g.ew) + x[k]);
-      if (EW == 2) static_cast<long long *>(vals)[p] = __ldg(static_cast<const long long *>(g.ew) + x[k]);
-      if (out) atomicAdd(&h[(unsigned)cv[k] & mask], 1u);
+  for (int k = 0; k < kSortItems; k++) kept += (unsigned)__popc(__ballot_sync(kFull, x[k] >= 0 && cv[k] != cu[k]));
+  if (lane == 0) sm.wbase[wid] = kept;
+  __syncthreads();
+  int64_t at = tile * kSortTile;
+  unsigned all = 0;
+#pragma unroll
+  for (int w = 0; w < kSortWarps; w++) {
+    if (w < wid) at += sm.wbase[w];
+    all += sm.wbase[w];
+  }
+#pragma unroll
+  for (int k = 0; k < kSortItems; k++) {
+    const bool out = x[k] >= 0 && cv[k] != cu[k];
+    const unsigned outs = __ballot_sync(kFull, out);
+    if (out) {
+      const int64_t to = at + __popc(outs & lanemask_lt());
+      a.k0[to] = ((unsigned long long)(unsigned)cv[k] << 32) | (unsigned)cu[k];
+      if constexpr (EW != 0) static_cast<V *>(a.v0)[to] = __ldg(static_cast<const V *>(g.ew) + x[k]);
+      atomicAdd(&sm.h[(unsigned)cv[k] & mask], 1u);
     }
+    at += __popc(outs);
   }
   __syncthreads();
-  if (threadIdx.x <= mask) hist[(int64_t)threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
+  if (threadIdx.x <= mask) a.hist[(int64_t)threadIdx.x * ntiles + tile] = sm.h[threadIdx.x];
+  if (threadIdx.x == 0) a.tile_n[tile] = (int)all;
 }
 
-// Sorted pairs: the first of equal ones is a head. Heads per tile and per coarse row.
-constexpr int kHeadThreads = 256;
-constexpr int kHeadItems = 8;  // per lane
-constexpr int64_t kHeadTile = (int64_t)kHeadThreads * kHeadItems;
-
-__global__ void __launch_bounds__(kHeadThreads) k_heads(const unsigned long long *keys, const int64_t *n_dev,
-                                                        int64_t *tile_heads, int64_t *rowcnt) {
-  __shared__ unsigned s_heads;
-  const int64_t n = *n_dev;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int64_t base = (int64_t)blockIdx.x * kHeadTile + (int64_t)wid * (32 * kHeadItems);
-  if (threadIdx.x == 0) s_heads = 0;
+// Heads (first of equal sorted pairs) of two head tiles, half a block each, and per coarse row.
+__device__ __forceinline__ void heads_tiles(const unsigned long long *keys, int64_t n, int64_t pair, int64_t *tile_heads,
+                                            int64_t htiles, int64_t *rowcnt, ContractSmem &sm) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, half = wid / (kHeadThreads / 32);
+  const int64_t base = 2 * pair * kHeadTile + (int64_t)wid * (32 * kHeadItems);
+  __syncthreads();
+  if (threadIdx.x < 2) sm.heads[threadIdx.x] = 0;
   __syncthreads();
   if (base < n) {
     unsigned long long key[kHeadItems];
 #pragma unroll
     for (int k = 0; k < kHeadItems; k++) {
       const int64_t i = base + 32 * k + lane;
-      key[k] = i < n ? keys[i] : kSortDropped;
+      key[k] = i < n ? keys[i] : ~0ull;
     }
-    unsigned long long before = base > 0 ? keys[base - 1] : kSortDropped;
+    unsigned long long before = base > 0 ? keys[base - 1] : ~0ull;
     unsigned total = 0;
 #pragma unroll
     for (int k = 0; k < kHeadItems; k++) {
@@ -216,30 +265,211 @@ __global__ void __launch_bounds__(kHeadThreads) k_heads(const unsigned long long
       if (head && lane == __ffs(peers) - 1)
         atomicAdd(reinterpret_cast<unsigned long long *>(&rowcnt[row]), (unsigned long long)__popc(peers));
     }
-    if (lane == 0) atomicAdd(&s_heads, total);
+    if (lane == 0) atomicAdd(&sm.heads[half], total);
   }
   __syncthreads();
-  if (threadIdx.x == 0) tile_heads[blockIdx.x] = s_heads;
+  if (threadIdx.x < 2 && 2 * pair + threadIdx.x < htiles) tile_heads[2 * pair + threadIdx.x] = sm.heads[threadIdx.x];
 }
 
-// Sorted pairs to coarse entries: a run of equal pairs becomes one entry at the run's rank. A run inside one
-// step of 32 is stored; the parts of a run that crosses steps are added (ew must be zero on entry).
+// Everything up to the coarse offsets in one cooperative launch: the steps follow one another by grid meetings
+// (about 2 us each) instead of kernel launches, and the sizes that the later steps need (n', the number of pairs)
+// never go to the host. Small levels are bound by these steps one after another: 17 launches and 9 memsets took
+// 250 us for a few thousand vertices. Large ones are bound by the sort's passes over memory.
 template <int EW>
-__global__ void __launch_bounds__(kHeadThreads) k_entries(const unsigned long long *keys, const void *vals,
-                                                          const int64_t *n_dev, const int64_t *tile_first, int32_t *adj,
-                                                          int64_t *ew) {
+__global__ void __launch_bounds__(kThreads, 2) k_contract(ContractArgs a) {
+  using V = typename PairVal<EW>::T;
+  extern __shared__ unsigned long long dsm[];
+  __shared__ ContractSmem sm;
+  const GridBarrier bar{a.bar, &a.head->err, gridDim.x, blockIdx.x, a.wait_us};
+  unsigned met = 0;
+#define MEET() \
+  if (!grid_meet(bar, met)) return
+  const DGraph &g = a.g;
+  const int64_t n = g.n;
+  const int lane = threadIdx.x & 31;
+  const int64_t tid = (int64_t)blockIdx.x * kThreads + threadIdx.x, stride = (int64_t)gridDim.x * kThreads;
+  // 1. used labels (a label outside [0, nl) is an error of the call: nothing more is done)
+  for (int64_t v = tid; v < n; v += stride) {
+    const int L = a.labels[v];
+    if (L < 0 || L >= a.nl) atomicExch(&a.head->bad, 1);
+    else a.used[L] = 1;
+  }
+  MEET();
+  if (*(volatile int *)&a.head->bad) return;
+  // 2. new ids by a prefix sum
+  scan_sums(a.nl, [&](int64_t i) { return (long long)a.used[i]; }, a.part, sm);
+  MEET();
+  const int64_t nc = scan_write(a.nl, [&](int64_t i) { return (long long)a.used[i]; },
+                                [&](int64_t i, long long x) { a.newid[i] = (int32_t)x; }, a.part, sm);
+  MEET();
+  // 3. fine -> coarse map and, per coarse vertex, member count and weight. Members of one cluster are mostly
+  // neighbours in id order, so the warp combines equal coarse ids before its atomics.
+  for (int64_t v0 = (int64_t)blockIdx.x * kThreads; v0 < n; v0 += stride) {
+    const int64_t v = v0 + threadIdx.x;
+    const bool ok = v < n;
+    int cv = -1;
+    long long c = 0;
+    if (ok) {
+      cv = a.newid[a.labels[v]];
+      a.f2c[v] = cv;
+      c = g.vweight(v);
+    }
+    const unsigned peers = __match_any_sync(kFull, cv);
+    if (!ok) continue;
+    long long cs = 0;
+    for (unsigned m = peers; m; m &= m - 1) cs += __shfl_sync(peers, c, __ffs(m) - 1);
+    if (lane == __ffs(peers) - 1) {
+      atomicAdd(reinterpret_cast<unsigned long long *>(&a.cnt[cv]), (unsigned long long)__popc(peers));
+      atomicAdd(reinterpret_cast<unsigned long long *>(&a.cw[cv]), (unsigned long long)cs);
+    }
+  }
+  MEET();
+  // 4. members bucketed by coarse id (in any order within a cluster) with their degrees; largest coarse weight
+  scan_sums(nc, [&](int64_t i) { return (long long)a.cnt[i]; }, a.part, sm);
+  MEET();
+  scan_write(nc, [&](int64_t i) { return (long long)a.cnt[i]; }, [&](int64_t i, long long x) { a.mstart[i] = x; }, a.part,
+             sm);
+  {
+    unsigned long long m = 0;
+    for (int64_t i = tid; i < nc; i += stride) m = max(m, (unsigned long long)a.cw[i]);
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(kFull, m, o));
+    if (lane == 0 && m) atomicMax(&a.head->maxcw, m);
+  }
+  MEET();
+  for (int64_t v = tid; v < n; v += stride) {
+    const int cv = a.f2c[v];
+    const int64_t pos =
+        a.mstart[cv] + (int64_t)atomicAdd(reinterpret_cast<unsigned long long *>(&a.cnt[cv]), ~0ull) - 1;
+    a.members[pos] = (int32_t)v;
+    a.mpre[pos] = g.row_begin(v + 1) - g.row_begin(v);
+  }
+  MEET();
+  // 5. where the members' rows start in the walk over them
+  scan_sums(n, [&](int64_t i) { return (long long)a.mpre[i]; }, a.part, sm);
+  MEET();
+  const int64_t m = min(g.m, scan_write(n, [&](int64_t i) { return (long long)a.mpre[i]; },
+                                        [&](int64_t i, long long x) { a.mpre[i] = x; }, a.part, sm));
+  if (tid == 0) {
+    a.mpre[n] = m;
+    a.head->nc = nc;
+  }
+  MEET();
+  // 6. pairs, sorted by row
+  int kb = 0;
+  while (kb < 31 && ((int64_t)1 << kb) < nc) kb++;
+  const int passes = sort_passes(kb), width = max(1, (kb + passes - 1) / passes);
+  int64_t ntiles = sort_tiles(m);
+  for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) pairs_tile<EW>(a, t, m, width, ntiles, sm);
+  MEET();
+  unsigned long long *ki = a.k0, *ko = a.k1;
+  V *vi = static_cast<V *>(a.v0), *vo = static_cast<V *>(a.v1);
+  int64_t pairs = 0;
+  for (int p = 0; p < passes; p++) {
+    const int shift = 32 + p * width, w = max(1, min(width, kb - p * width));
+    if (p > 0) {
+      ntiles = sort_tiles(pairs);
+      for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x)
+        radix_tile_hist(ki, t * kSortTile, pairs, shift, w, a.hist + t, ntiles, sm.h);
+      MEET();
+    }
+    const int64_t cells = ntiles << w;
+    scan_sums(cells, [&](int64_t i) { return (long long)a.hist[i]; }, a.part, sm);
+    MEET();
+    pairs = scan_write(cells, [&](int64_t i) { return (long long)a.hist[i]; },
+                       [&](int64_t i, long long x) { a.hist[i] = x; }, a.part, sm);
+    MEET();
+    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+      const int tn = p == 0 ? a.tile_n[t] : (int)min(kSortTile, pairs - t * kSortTile);
+      radix_tile_scatter<V>(ki, vi, ko, vo, t * kSortTile, tn, shift, w, a.hist + t, ntiles, dsm, sm.radix);
+    }
+    MEET();
+    unsigned long long *tk = ki;
+    ki = ko;
+    ko = tk;
+    V *tv = vi;
+    vi = vo;
+    vo = tv;
+  }
+  // 7. heads, coarse offsets
+  const int64_t htiles = (pairs + kHeadTile - 1) / kHeadTile;
+  for (int64_t t = blockIdx.x; 2 * t < htiles; t += gridDim.x)
+    heads_tiles(ki, pairs, t, a.tile_heads, htiles, a.rowcnt, sm);
+  MEET();
+  scan_sums(htiles, [&](int64_t i) { return (long long)a.tile_heads[i]; }, a.part, sm);
+  scan_sums(nc, [&](int64_t i) { return (long long)a.rowcnt[i]; }, a.part + gridDim.x, sm);
+  MEET();
+  const int64_t mc = scan_write(htiles, [&](int64_t i) { return (long long)a.tile_heads[i]; },
+                                [&](int64_t i, long long x) { a.tile_heads[i] = x; }, a.part, sm);
+  scan_write(nc, [&](int64_t i) { return (long long)a.rowcnt[i]; }, [&](int64_t i, long long x) { a.off[i] = x; },
+             a.part + gridDim.x, sm);
+  if (tid == 0) {
+    a.off[nc] = mc;
+    a.head->mc = mc;
+    a.head->pairs = pairs;
+  }
+  // 8. LP degree classes of the coarse graph, from the row lengths (words as lp_classes_from reads them)
+  if (a.want_classes) {
+    unsigned *const cls = sm.h;
+    __syncthreads();
+    if (threadIdx.x < 16) cls[threadIdx.x] = 0;
+    __syncthreads();
+    unsigned long long ent = 0, hub_max = 0, hub_sum = 0, wide = 0;
+    for (int64_t c = tid; c < nc; c += stride) {
+      const int64_t d = a.rowcnt[c];
+      if (d == 0) continue;
+      const int b = lp_bin_of(d, a.deg_warp, a.deg_cta);
+      atomicAdd(&cls[b], 1u);
+      ent += (unsigned long long)d;
+      if (b == 6) {
+        hub_max = max(hub_max, (unsigned long long)hub_cap(d));
+        hub_sum += (unsigned long long)hub_cap(d);
+      }
+      if (d > kWideDeg) wide++;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      ent += __shfl_xor_sync(kFull, ent, o);
+      hub_max = max(hub_max, __shfl_xor_sync(kFull, hub_max, o));
+      hub_sum += __shfl_xor_sync(kFull, hub_sum, o);
+      wide += __shfl_xor_sync(kFull, wide, o);
+    }
+    unsigned long long *const words = a.head->classes;
+    if (lane == 0 && ent) {
+      atomicAdd(&words[5], ent);
+      if (hub_max) atomicMax(&words[6], hub_max);
+      if (hub_sum) atomicAdd(&words[7], hub_sum);
+      if (wide) atomicAdd(&words[8], wide);
+    }
+    __syncthreads();
+    if (threadIdx.x < 9 && cls[threadIdx.x]) atomicAdd(reinterpret_cast<unsigned *>(words) + threadIdx.x, cls[threadIdx.x]);
+  }
+#undef MEET
+}
+
+// Sorted pairs to coarse entries: a run of equal pairs becomes one entry at the run's rank, written by its last
+// lane. A run inside one step of 32 is stored; the parts of a run that crosses steps are added (ew must be zero on
+// entry). Bound by memory: the pairs are read once and the entries written once (the run sums are five shuffle
+// steps; a reduction per run of a step took four times as long on rows of distinct neighbours). Also copies the
+// coarse offsets and vertex weights.
+template <int EW>
+__global__ void __launch_bounds__(kHeadThreads) k_entries(const unsigned long long *keys, const void *vals, int64_t n,
+                                                          const int64_t *tile_first, int32_t *adj, int64_t *ew,
+                                                          int64_t nc, const int64_t *off_in, int64_t *off,
+                                                          const int64_t *vw_in, int64_t *vw) {
   __shared__ unsigned s_warp[kHeadThreads / 32];
-  const int64_t n = *n_dev;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int64_t i = (int64_t)blockIdx.x * kHeadThreads + threadIdx.x; i <= nc; i += (int64_t)gridDim.x * kHeadThreads) {
+    off[i] = off_in[i];
+    if (i < nc) vw[i] = vw_in[i];
+  }
   const int64_t tbase = (int64_t)blockIdx.x * kHeadTile;
   if (tbase >= n) return;
   const int64_t base = tbase + (int64_t)wid * (32 * kHeadItems);
-  unsigned long long key[kHeadItems], before = kSortDropped, after = kSortDropped;
+  unsigned long long key[kHeadItems], before = ~0ull, after = ~0ull;
   long long w[kHeadItems];
 #pragma unroll
   for (int k = 0; k < kHeadItems; k++) {
     const int64_t i = base + 32 * k + lane;
-    key[k] = i < n ? keys[i] : kSortDropped;
+    key[k] = i < n ? keys[i] : ~0ull;
     w[k] = 0;
     if (i < n) w[k] = EW == 0 ? 1 : EW == 1 ? (long long)static_cast<const int32_t *>(vals)[i] : static_cast<const long long *>(vals)[i];
   }
@@ -262,22 +492,34 @@ __global__ void __launch_bounds__(kHeadThreads) k_entries(const unsigned long lo
   for (int k = 0; k < kHeadItems; k++) {
     if (base + 32 * k >= n) break;  // (uniform over the warp)
     const bool on = base + 32 * k + lane < n;
-    const int64_t run = at + __popc(heads[k] & (lanemask_lt() | 1u << lane));
+    const unsigned upto = heads[k] & (lanemask_lt() | 1u << lane);
+    const int64_t run = at + __popc(upto);
+    const int first = upto ? 31 - __clz(upto) : 0;  // the run's first lane in this step
     const unsigned long long next = k + 1 < kHeadItems ? __shfl_sync(kFull, key[k + 1 < kHeadItems ? k + 1 : k], 0) : after;
-    const unsigned peers = __match_any_sync(kFull, on ? (unsigned)(run - at) : 64u);
-    long long sum = EW == 0 ? (long long)__popc(peers) : 0;
-    if (EW) {
-      // weights below 2^26 sum exactly in 32 bits over at most 32 lanes: one warp reduction
-      if (!__any_sync(kFull, w[k] >= (1ll << 26) || w[k] < 0)) {
-        sum = (long long)__reduce_add_sync(peers, (unsigned)w[k]);
-      } else {
-        for (unsigned pm = peers; pm; pm &= pm - 1) sum += __shfl_sync(peers, w[k], __ffs(pm) - 1);
+    unsigned long long mine_next = __shfl_down_sync(kFull, key[k], 1);
+    if (lane == 31) mine_next = next;
+    long long sum;
+    if (EW == 0) {
+      sum = on ? lane - first + 1 : 0;
+    } else if (!__any_sync(kFull, w[k] >= (1ll << 26) || w[k] < 0)) {  // (32 of them fit 32 bits)
+      unsigned x = (unsigned)w[k];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(kFull, x, o);
+        if (lane - o >= first) x += y;
+      }
+      sum = x;
+    } else {
+      sum = w[k];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const long long y = __shfl_up_sync(kFull, sum, o);
+        if (lane - o >= first) sum += y;
       }
     }
-    if (on && lane == __ffs(peers) - 1) {
-      const bool starts = heads[k] >> lane & 1u;
-      const int last = 31 - __clz(peers);
-      const bool ends = last < 31 || next != key[k];
+    const bool ends = mine_next != key[k];  // the run ends with this lane (past n the keys differ from any pair)
+    if (on && (ends || lane == 31)) {
+      const bool starts = upto != 0;
       if (starts) adj[run] = (int32_t)(key[k] & 0xffffffffull);
       if (starts && ends) ew[run] = sum;
       else atomicAdd(reinterpret_cast<unsigned long long *>(&ew[run]), (unsigned long long)sum);
@@ -286,42 +528,22 @@ __global__ void __launch_bounds__(kHeadThreads) k_entries(const unsigned long lo
   }
 }
 
-// The pairs of g, sorted by (cv, cu): keys and values end in *keys_out / *vals_out, their number on the device at
-// *count_out.
 template <int EW>
-int sorted_pairs(const DGraph &g, const int32_t *members, const int64_t *mpre, const int32_t *f2c, int kb,
-                 unsigned long long **keys_out, void **vals_out, int64_t **count_out, Workspace &ws) {
-  cudaStream_t s = ws.stream();
-  const size_t m = (size_t)g.m;
-  unsigned long long *k0, *k1;
-  unsigned char *v0 = nullptr, *v1 = nullptr;
-  GP_TRY(ws.get(&k0, m));
-  GP_TRY(ws.get(&k1, m));
-  if (kValBytes<EW>) {
-    GP_TRY(ws.get(&v0, m * kValBytes<EW>));
-    GP_TRY(ws.get(&v1, m * kValBytes<EW>));
+int launch_contract(ContractArgs &a, cudaStream_t s) {
+  using V = typename PairVal<EW>::T;
+  static int per_sm = 0;
+  if (!per_sm) {
+    GP_CUDA(cudaFuncSetAttribute(k_contract<EW>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSortSmem<V>));
+    int x = 0;
+    GP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x, k_contract<EW>, kThreads, kSortSmem<V>));
+    per_sm = std::max(1, x);
   }
-  const int passes = sort_passes(kb), width = std::max(1, (kb + passes - 1) / passes);
-  const int64_t ntiles = sort_tiles(g.m), cells = ntiles << width;
-  int64_t *hist, *count;
-  GP_TRY(ws.get(&hist, (size_t)cells + 1));
-  GP_TRY(ws.get(&count, 1));
-  ProfScope ps("contract_rows", s);
-  (::gp::count_launch(), k_pairs<EW><<<(unsigned)ntiles, kSortThreads, 0, s>>>(g, members, mpre, f2c, k0, v0, width, ntiles, hist));
-  GP_LAUNCH_CHECK();
-  for (int p = 0; p < passes; p++) {
-    const int shift = 32 + p * width, w = std::max(1, std::min(width, kb - p * width));
-    if (p > 0) GP_TRY(radix_hist(k0, count, g.m, shift, w, hist, s));
-    GP_TRY(radix_offsets(hist, g.m, w, ws));
-    if (p == 0)  // the number of pairs that are not inside a cluster
-      GP_CUDA(cudaMemcpyAsync(count, hist + (ntiles << w), sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
-    GP_TRY(radix_scatter(k0, v0, k1, v1, kValBytes<EW>, p > 0 ? count : mpre + g.n, g.m, shift, w, hist, p == 0, s));
-    std::swap(k0, k1);
-    std::swap(v0, v1);
-  }
-  *keys_out = k0;
-  *vals_out = v0;
-  *count_out = count;
+  // a block per sort tile or per 2048 vertices, up to what is resident: fewer blocks meet sooner
+  const int64_t want = std::max<int64_t>(sort_tiles(a.g.m), (std::max(a.g.n, a.nl) + 2047) / 2048);
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, std::min<int64_t>((int64_t)per_sm * num_sms(), kMaxContractBlocks)));
+  count_launch();
+  void *args[] = {(void *)&a};
+  GP_CUDA(cudaLaunchCooperativeKernel((void *)k_contract<EW>, grid, kThreads, args, kSortSmem<V>, s));
   return GP_OK;
 }
 
@@ -349,130 +571,107 @@ int alloc_graph(OwnedGraph *g, int64_t n, int64_t m, cudaStream_t s) {
 int contract_graph(const DGraph &g, const int32_t *labels, int64_t nl, OwnedGraph *out, int32_t *f2c_user,
                    cudaStream_t s, const LpConfig *cfg, LpClassInfo *cls) {
   Workspace ws(s);
-  const int nsm = num_sms();
   const int64_t n = g.n;
-  auto grid_n = [&](int64_t items) {
-    return (int)std::max<int64_t>(1, std::min<int64_t>((items + 255) / 256, nsm * 8));
-  };
   if (n == 0) {
     GP_TRY(alloc_graph(out, 0, 0, s));
     GP_CUDA(cudaMemsetAsync(out->off, 0, sizeof(int64_t), s));
     return GP_OK;
   }
-  // 1. used flags -> new ids by an exclusive prefix sum
-  uint32_t *used;
-  int32_t *newid;
-  int *bad;
-  int64_t *hdr;  // [0] = n', [1] = m'
-  GP_TRY(ws.zeros(&used, (size_t)nl));
-  GP_TRY(ws.get(&newid, (size_t)nl));
-  GP_TRY(ws.zeros(&bad, 1));
-  GP_TRY(ws.zeros(&hdr, 4));
-  (::gp::count_launch(), k_mark_used<<<grid_n(n), 256, 0, s>>>(labels, n, nl, used, bad));
-  GP_LAUNCH_CHECK();
-  GP_TRY(scan_excl_u32(used, newid, nl, hdr, ws));
-  // The coarse vertex count nc = hdr[0] stays on the device until the read back after step 4: the
-  // arrays indexed by coarse vertex are sized for the bound min(n, nl) (zero beyond nc, so the scans
-  // over the bound equal the scans over nc) and the row classification reads nc on the device.
-  const int64_t ncb = std::max<int64_t>(1, std::min<int64_t>(n, nl));
-  // 2. fine -> coarse map, member counts, coarse vertex weights
-  int32_t *f2c = f2c_user;
-  if (!f2c) GP_TRY(ws.get(&f2c, (size_t)n));
-  int64_t *cnt, *mstart, *cw;
-  GP_TRY(ws.zeros(&cnt, (size_t)ncb + 1));
-  GP_TRY(ws.zeros(&cw, (size_t)ncb));
-  GP_TRY(ws.get(&mstart, (size_t)ncb + 1));
-  (::gp::count_launch(), k_f2c<<<grid_n(n), 256, 0, s>>>(g, labels, nl, newid, f2c, cnt, cw, bad));
-  GP_LAUNCH_CHECK();
-  GP_TRY(scan_excl_i64(cnt, mstart, ncb, mstart + ncb, ws));
-  // 3. members bucketed by coarse id, and where their rows start in the walk over them
-  unsigned *fill;
-  int32_t *members;
-  int64_t *mpre;
-  unsigned long long *maxvw_dev;
-  GP_TRY(ws.zeros(&fill, (size_t)ncb));
-  GP_TRY(ws.get(&members, (size_t)n));
-  GP_TRY(ws.get(&mpre, (size_t)n + 1));
-  GP_TRY(ws.zeros(&maxvw_dev, 1));
-  (::gp::count_launch(),
-   k_members<<<grid_n(n), 256, 0, s>>>(g, f2c, mstart, fill, members, mpre, cw, ncb, maxvw_dev));
-  GP_LAUNCH_CHECK();
-  GP_TRY(scan_excl_i64(mpre, mpre, n, mpre + n, ws));
-  unsigned long long maxvw = 0;
-  int64_t hh[4];
-  int hbad = 0;
+  // Arrays indexed by coarse vertex are sized for the bound min(n, nl); what must start at zero is one
+  // allocation and one memset.
+  const size_t ncb = (size_t)std::max<int64_t>(1, std::min<int64_t>(n, nl)), m = (size_t)g.m;
+  const int ew = g.ew_mode();
+  ContractArgs a;
+  a.g = g;
+  a.labels = labels;
+  a.nl = nl;
+  {
+    auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
+    const size_t b_head = up(sizeof(ContractHead)), b_bar = up(sizeof(unsigned) * kBarrierStride),
+                 b_used = up(sizeof(uint32_t) * (size_t)nl), b_cnt = up(sizeof(int64_t) * (ncb + 1));
+    unsigned char *z;
+    GP_TRY(ws.zeros(&z, b_head + b_bar + b_used + 3 * b_cnt));
+    a.head = reinterpret_cast<ContractHead *>(z);
+    a.bar = reinterpret_cast<unsigned *>(z + b_head);
+    a.used = reinterpret_cast<uint32_t *>(z + b_head + b_bar);
+    z += b_head + b_bar + b_used;
+    a.cnt = reinterpret_cast<int64_t *>(z);
+    a.cw = reinterpret_cast<int64_t *>(z + b_cnt);
+    a.rowcnt = reinterpret_cast<int64_t *>(z + 2 * b_cnt);
+  }
+  GP_TRY(ws.get(&a.newid, (size_t)nl));
+  a.f2c = f2c_user;
+  if (!a.f2c) GP_TRY(ws.get(&a.f2c, (size_t)n));
+  GP_TRY(ws.get(&a.members, (size_t)n));
+  GP_TRY(ws.get(&a.mstart, ncb + 1));
+  GP_TRY(ws.get(&a.mpre, (size_t)n + 1));
+  GP_TRY(ws.get(&a.off, ncb + 1));
+  GP_TRY(ws.get(&a.part, (size_t)2 * kMaxContractBlocks));
+  GP_TRY(ws.get(&a.k0, m));
+  GP_TRY(ws.get(&a.k1, m));
+  const size_t vb = ew == 0 ? 0 : ew == 1 ? 4 : 8;
+  unsigned char *v0 = nullptr, *v1 = nullptr;
+  if (vb) {
+    GP_TRY(ws.get(&v0, m * vb));
+    GP_TRY(ws.get(&v1, m * vb));
+  }
+  a.v0 = v0;
+  a.v1 = v1;
+  const size_t ntiles = (size_t)sort_tiles(g.m);
+  int kbound = 0;  // bits of the largest n' possible: the widest digit the kernel can choose
+  while (kbound < 31 && ((int64_t)1 << kbound) < (int64_t)ncb) kbound++;
+  GP_TRY(ws.get(&a.tile_n, ntiles));
+  GP_TRY(ws.get(&a.hist, ntiles << std::min(std::max(kbound, 1), kSortBits)));
+  GP_TRY(ws.get(&a.tile_heads, m / (size_t)kHeadTile + 1));
+  a.wait_us = (unsigned)std::min<unsigned long long>(wait_limit_ns() / 1000, 0xffffffffull);
+  a.want_classes = cfg && cls;
+  a.deg_warp = cfg ? cfg->deg_warp : 0;
+  a.deg_cta = cfg ? cfg->deg_cta : 0;
+  {
+    ProfScope ps("contract_rows", s);
+    GP_TRY(ew == 0 ? launch_contract<0>(a, s) : ew == 1 ? launch_contract<1>(a, s) : launch_contract<2>(a, s));
+  }
+  ContractHead h;
   {
     Readback rb;
-    rb.add(hh, hdr, sizeof(hh));
-    rb.add(&hbad, bad, sizeof(int));
-    rb.add(&maxvw, maxvw_dev, sizeof(maxvw));
+    rb.add(&h, a.head, sizeof(h));
     GP_TRY(rb.run(s));
   }
-  if (hbad) {
+  if (h.bad) {
     set_error("contract: a label is outside [0, n)");
     return GP_ERR_INVALID_ARG;
   }
-  const int64_t nc = hh[0];
-  int kb = 0;
-  while (kb < 31 && ((int64_t)1 << kb) < nc) kb++;
-  // 4. sorted pairs, heads per coarse row, coarse offsets
-  const int ew = g.ew_mode();
-  unsigned long long *keys = nullptr;
-  void *vals = nullptr;
-  int64_t *npairs = nullptr, *rowcnt, *off_tmp, *tile_heads = nullptr;
-  GP_TRY(ws.zeros(&rowcnt, (size_t)nc + 1));
-  GP_TRY(ws.get(&off_tmp, (size_t)nc + 1));
-  const int64_t htiles = (g.m + kHeadTile - 1) / kHeadTile;
-  if (g.m > 0) {
-    GP_TRY(ew == 0   ? sorted_pairs<0>(g, members, mpre, f2c, kb, &keys, &vals, &npairs, ws)
-           : ew == 1 ? sorted_pairs<1>(g, members, mpre, f2c, kb, &keys, &vals, &npairs, ws)
-                     : sorted_pairs<2>(g, members, mpre, f2c, kb, &keys, &vals, &npairs, ws));
-    GP_TRY(ws.get(&tile_heads, (size_t)htiles));
-    (::gp::count_launch(), k_heads<<<(unsigned)htiles, kHeadThreads, 0, s>>>(keys, npairs, tile_heads, rowcnt));
-    GP_LAUNCH_CHECK();
-    GP_TRY(scan_excl_i64(tile_heads, tile_heads, htiles, nullptr, ws));
+  if (h.err) {
+    set_error("contraction: a bounded device barrier gave up");
+    return GP_ERR_TIMEOUT;
   }
-  int64_t mc = 0;
-  GP_TRY(scan_excl_i64(rowcnt, off_tmp, nc, off_tmp + nc, ws));
-  // the next level's LP degree classes need only the coarse offsets: computed here and read back
-  // with the coarse entry count
-  unsigned long long *cls_dev = nullptr;
-  unsigned long long cls_words[kLpClassWords];
-  if (cfg && cls) {
-    GP_TRY(ws.get(&cls_dev, (size_t)kLpClassWords));
-    DGraph cg;
-    cg.n = nc;
-    cg.off = off_tmp;
-    cg.off64 = 1;
-    GP_TRY(lp_classes_launch(cg, *cfg, cls_dev, ws));
-  }
+  if (cfg && cls) lp_classes_from(h.classes, *cfg, cls);
+  GP_TRY(alloc_graph(out, h.nc, h.mc, s));
+  out->max_vw = (int64_t)h.maxcw;
   {
-    Readback rb;
-    rb.add(&mc, off_tmp + nc, sizeof(int64_t));
-    if (cls_dev) rb.add(cls_words, cls_dev, sizeof(cls_words));
-    GP_TRY(rb.run(s));
-  }
-  if (cls_dev) lp_classes_from(cls_words, *cfg, cls);
-  GP_TRY(alloc_graph(out, nc, mc, s));
-  out->max_vw = (int64_t)maxvw;
-  GP_CUDA(cudaMemcpyAsync(out->off, off_tmp, sizeof(int64_t) * (size_t)(nc + 1), cudaMemcpyDeviceToDevice, s));
-  GP_CUDA(cudaMemcpyAsync(out->vw, cw, sizeof(int64_t) * (size_t)nc, cudaMemcpyDeviceToDevice, s));
-  // 5. equal pairs summed into the coarse entries
-  if (mc > 0) {
+    // equal pairs summed into the coarse entries; the sorted pairs lie where the last pass left them
+    int kb = 0;
+    while (kb < 31 && ((int64_t)1 << kb) < h.nc) kb++;
+    const bool odd = sort_passes(kb) & 1;
+    const unsigned long long *keys = odd ? a.k1 : a.k0;
+    const void *vals = odd ? a.v1 : a.v0;
     ProfScope ps("contract_compact", s);
-    GP_CUDA(cudaMemsetAsync(out->ew, 0, sizeof(int64_t) * (size_t)mc, s));
-    if (ew == 0)
-      (::gp::count_launch(), k_entries<0><<<(unsigned)htiles, kHeadThreads, 0, s>>>(keys, vals, npairs, tile_heads, out->adj, out->ew));
-    else if (ew == 1)
-      (::gp::count_launch(), k_entries<1><<<(unsigned)htiles, kHeadThreads, 0, s>>>(keys, vals, npairs, tile_heads, out->adj, out->ew));
-    else
-      (::gp::count_launch(), k_entries<2><<<(unsigned)htiles, kHeadThreads, 0, s>>>(keys, vals, npairs, tile_heads, out->adj, out->ew));
+    if (h.mc > 0) GP_CUDA(cudaMemsetAsync(out->ew, 0, sizeof(int64_t) * (size_t)h.mc, s));
+    const unsigned grid = (unsigned)std::max<int64_t>((h.pairs + kHeadTile - 1) / kHeadTile,
+                                                      std::min<int64_t>(h.nc / kHeadThreads + 1, (int64_t)num_sms() * 8));
+    auto run = [&](auto kernel) {
+      (::gp::count_launch(), kernel<<<grid, kHeadThreads, 0, s>>>(keys, vals, h.pairs, a.tile_heads, out->adj, out->ew,
+                                                                  h.nc, a.off, out->off, a.cw, out->vw));
+    };
+    if (ew == 0) run(k_entries<0>);
+    else if (ew == 1) run(k_entries<1>);
+    else run(k_entries<2>);
     GP_LAUNCH_CHECK();
   }
   if (profiling()) {
     const int64_t rb = n * 2 * g.offset_bytes() + g.m * (4 + g.ew_bytes()) + g.m * 4;
-    prof_add_counts("contract_rows", nc, g.m, rb);
-    prof_add_counts("contract_compact", nc, mc, mc * 12 + nc * 8);
+    prof_add_counts("contract_rows", h.nc, g.m, rb);
+    prof_add_counts("contract_compact", h.nc, h.mc, h.mc * 12 + h.nc * 8);
   }
   return GP_OK;  // stream-ordered: the temporary buffers are released on s after the kernels
 }

@@ -43,6 +43,8 @@ void set_thread_arena(ScratchArena *a);
 bool arena_active();
 void *dev_alloc(size_t bytes, cudaStream_t s);
 void dev_free(void *p, size_t bytes, cudaStream_t s);
+void dev_drop(void *p, size_t bytes, cudaStream_t s);  // dev_free at the next dev_alloc (see gp_coarse_drop)
+void release_dropped(size_t keep);  // dropped blocks back until at most `keep` bytes are held
 void free_cached();  // returns the blocks the library keeps for reuse to the allocator
 long long pinned_stage_allocs();  // pinned host staging allocations made by Readback so far
 
@@ -314,6 +316,30 @@ __device__ __forceinline__ bool grid_sync(const GridBarrier &b) {
   }
   __syncthreads();
   return s_ok != 0;
+}
+
+// Bounded barrier over all blocks of a cooperative launch that is met a known number of times: the word counts
+// arrivals, and the k-th meeting is over when it holds k * nblocks. A block adds without waiting for the old
+// value and polls; a wait that runs out ends as in grid_sync. `met` (thread 0's) counts the meetings so far.
+__device__ __forceinline__ bool grid_meet(const GridBarrier &b, unsigned &met) {
+  __shared__ int s_met_ok;
+  __syncthreads();
+  if (b.nblocks <= 1) return true;
+  if (threadIdx.x == 0) {
+    s_met_ok = 1;
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(b.count), "r"(1u) : "memory");
+    const unsigned want = ++met * b.nblocks;
+    const unsigned long long t0 = global_ns();
+    while ((int)(ld_acquire_u32(b.count) - want) < 0) {
+      if (global_ns() - t0 > 1000ull * b.wait_us || *(volatile int *)b.err == GP_ERR_TIMEOUT) {
+        atomicExch(b.err, GP_ERR_TIMEOUT);
+        s_met_ok = 0;
+        break;
+      }
+    }
+  }
+  __syncthreads();
+  return s_met_ok != 0;
 }
 
 // ------------------------------------------------------------------------------------------ scans

@@ -35,6 +35,21 @@ struct LpClassInfo {
   unsigned long long wide = 0;  // vertices of degree above 1024 (they need the larger shared tables)
 };
 
+// Degree bins of the LP kernels: lane groups of 4/8/16/32, a warp, a CTA, several CTAs (hubs).
+__device__ __forceinline__ int lp_bin_of(int64_t d, int deg_warp, int deg_cta) {
+  if (d <= 4) return 0;
+  if (d <= 8) return 1;
+  if (d <= 16) return 2;
+  if (d <= 32) return 3;
+  if (d <= deg_warp) return 4;
+  if (d <= deg_cta) return 5;
+  return 6;
+}
+// Hub tables: round_up(2 x, 64) slots for x = min(d, number of labels) (a hub row has at most that many
+// distinct labels, so the load stays at or below 1/2).
+__host__ __device__ __forceinline__ int64_t hub_cap(int64_t d) { return ((2 * d + 63) / 64) * 64; }
+constexpr int kWideDeg = 1024;  // degrees above this need the larger shared-memory tables
+
 // Degree classes of one graph computed without a read back: lp_classes_launch writes kLpClassWords
 // words into words_dev (device, caller-owned) on the workspace's stream; after the caller has read
 // them to the host, lp_classes_from fills the LpClassInfo.

@@ -716,6 +716,12 @@ void gp_coarse_free(gp_coarse *c, gp_stream stream) {
   delete c;
 }
 
+void gp_coarse_drop(gp_coarse *c, gp_stream stream) {
+  if (!c) return;
+  c->g.drop((cudaStream_t)stream);
+  delete c;
+}
+
 int gp_partition(const gp_graph *g, int32_t k, double eps, uint64_t seed, const gp_params *params, int32_t *part_out,
                  gp_result *res, gp_stream stream) {
   const int st = partition_device(g, k, eps, seed, params, part_out, res, (cudaStream_t)stream);

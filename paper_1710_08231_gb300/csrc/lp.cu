@@ -65,7 +65,6 @@ constexpr int kHubCap = 2048;
 constexpr int kStageOff = kHubCap * 12, kStageAdj = 4096, kStageBuf = 4096 + 8192;
 static_assert(kStageOff + 2 * kStageBuf <= (int)kDynSmemT<2>, "staging buffers fit the larger class");
 static_assert(kHubCap * 16 <= (int)kDynSmemT<0> && kHubCap * 12 <= (int)kDynSmemT<1>, "hub tables fit every class");
-constexpr int kWideDeg = 1024;          // degrees above this need the larger tables
 constexpr int kSlotChunk = 8192;                      // hub table slots per choice work item
 constexpr int kContestSmall = 4096;
 // Hub table slots per batch and the fewest vertices per block come from LpConfig (tile sizes picked by
@@ -192,16 +191,6 @@ struct LpProblem {
   LpCounters *ctr;
 };
 
-__device__ __forceinline__ int bin_of(int64_t d, int deg_warp, int deg_cta) {
-  if (d <= 4) return 0;
-  if (d <= 8) return 1;
-  if (d <= 16) return 2;
-  if (d <= 32) return 3;
-  if (d <= deg_warp) return 4;
-  if (d <= deg_cta) return 5;
-  return 6;
-}
-
 __device__ __forceinline__ unsigned warp_append(unsigned int *counter, bool pred) {
   const unsigned m = __ballot_sync(kFull, pred);
   if (!m) return 0;
@@ -314,10 +303,7 @@ __device__ __forceinline__ void write_slot(const LpProblem &P, int64_t idx, int 
 
 __device__ __forceinline__ unsigned slot_hash(int L) { return mix32((unsigned)L); }
 
-// Hub tables: round_up(2 x, 64) slots for x = min(d, number of labels) (a hub row has at most that many
-// distinct labels, so the load stays at or below 1/2), indexed by a multiply-shift range reduction of
-// the mixed label.
-__host__ __device__ __forceinline__ int64_t hub_cap(int64_t d) { return ((2 * d + 63) / 64) * 64; }
+// Hub tables (hub_cap slots) are indexed by a multiply-shift range reduction of the mixed label.
 __device__ __forceinline__ uint64_t hub_slot(int L, uint64_t cap) {
   return ((uint64_t)slot_hash(L) * cap) >> 32;
 }
@@ -688,7 +674,7 @@ __device__ __forceinline__ int active_bin(const LpProblem &P, int64_t v, const u
   if (!((r == 0 || act[P.vbase + v]) && (int)(mix64(rmix ^ (uint64_t)v) >> 63) == s)) return -1;
   const int64_t d = P.g.row_begin(v + 1) - P.g.row_begin(v);
   *deg = d;
-  return d == 0 ? kBinZero : bin_of(d, P.deg_warp, P.deg_cta);
+  return d == 0 ? kBinZero : lp_bin_of(d, P.deg_warp, P.deg_cta);
 }
 
 __device__ void phase_classify(const LpProblem &P, SubCounters &C, const SubCounters *Vp, int r, int s, uint64_t rmix,
@@ -739,7 +725,7 @@ __device__ void phase_classify(const LpProblem &P, SubCounters &C, const SubCoun
     for (int it = 0; it < kCls; it++) {
       if (it >= niter) break;
       int b = -1;
-      if (flag >> it & 1) b = dd[it] == 0 ? kBinZero : bin_of(dd[it], P.deg_warp, P.deg_cta);
+      if (flag >> it & 1) b = dd[it] == 0 ? kBinZero : lp_bin_of(dd[it], P.deg_warp, P.deg_cta);
       if (b >= 0) codes = (codes & ~(15u << (4 * it))) | ((unsigned)b << (4 * it));
       const unsigned peers = __match_any_sync(kFull, b);
       // entries of the lanes in the same bin summed in the warp (at most 2^31 in all): one shared
@@ -3152,7 +3138,7 @@ __global__ void k_degree_classes(const DGraph *gs, const int64_t *pre, int njobs
       const DGraph &g = gs[j];
       const int64_t v = x - pre[j];
       d = g.row_begin(v + 1) - g.row_begin(v);
-      if (d > 0) bin = bin_of(d, deg_warp, deg_cta);
+      if (d > 0) bin = lp_bin_of(d, deg_warp, deg_cta);
     }
     // one atomic per distinct (job, bin) and per distinct job in the warp
     const unsigned pk = __match_any_sync(kFull, (j << 3) | (bin & 7));

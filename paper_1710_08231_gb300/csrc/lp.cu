@@ -24,6 +24,7 @@
 //     target fit, no order is needed; otherwise the contested proposals are sorted (one CTA in shared
 //     memory up to 4096, else a cooperative LSD radix sort) and admitted by a segmented prefix sum.
 #include <algorithm>
+#include <climits>
 #include <cstddef>
 #include <cstring>
 #include <vector>
@@ -849,13 +850,19 @@ __device__ __forceinline__ int group_best_unit(unsigned long long K, int L, int 
   return L;
 }
 
+// A bin of up to this many vertices per block goes to lane groups, a longer one to a thread per vertex: the groups take
+// one vertex through in the least time (four steps of 16 vertices at most here), the threads take many through
+// with fewer instructions and more loads in flight.
+constexpr unsigned kRowsMin = 64;
+
 // Where the choice finds the active vertices of a degree bin and leaves its proposals: lists of the whole
 // problem in memory with one proposal slot per position (ListBins), or a block's own vertices in its shared
 // memory with the proposals appended (OwnBins, below).
 struct ListBins {
   const LpProblem &P;
   const SubCounters &V;
-  __device__ __forceinline__ unsigned count(int b) const { return V.bin_count[b]; }
+  unsigned which;  // bins that take part
+  __device__ __forceinline__ unsigned count(int b) const { return which >> b & 1u ? V.bin_count[b] : 0u; }
   __device__ __forceinline__ void row(int b, unsigned i, int *v, int64_t *beg, int64_t *d) const {
     *v = P.bin[b][i];
     const unsigned long long x = P.binx[b][i];
@@ -934,28 +941,47 @@ __device__ __forceinline__ void choose_groups(const LpProblem &P, const Bins &B,
 #pragma unroll
     for (int u = 0; u < U; u++) {
       const bool has = gl < d[u];
-      const unsigned peers = __match_any_sync(kFull, (unsigned)Lu[u]) & gmask;
-      if constexpr (EW == 0) {
+      bool first = true;  // the lowest lane of the group with this label
+      unsigned qsum = 0;
+      if constexpr (EW == 0 && !LQ) {
+        const unsigned peers = __match_any_sync(kFull, (unsigned)Lu[u]) & gmask;
         conn[u] = __popc(peers);
+        first = lane == __ffs(peers) - 1;
+        c0[u] = __popc(__ballot_sync(kFull, has && Lu[u] == L0[u]) & gmask);
       } else {
-        if (!__any_sync(kFull, w[u] >= (1ll << 26))) {
-          conn[u] = (long long)__reduce_add_sync(peers, (unsigned)w[u]);
-        } else {
-          conn[u] = 0;
-          for (unsigned m = peers; m; m &= m - 1) conn[u] += __shfl_sync(peers, w[u], __ffs(m) - 1);
+        // each lane compares its label with those of the group's lanes, four at a time (a match and a
+        // reduction over each set of equal labels would take a step per distinct label of the warp, twice)
+        long long c = 0, own = 0;
+        const bool narrow = !__any_sync(kFull, w[u] >= (1ll << 26) || w[u] < 0);
+        for (int j0 = 0; j0 < G; j0 += 4) {
+          int Lj[4];
+          long long wj[4];
+          unsigned qj[4];
+#pragma unroll
+          for (int x = 0; x < 4; x++) {
+            Lj[x] = __shfl_sync(kFull, Lu[u], j0 + x, G);
+            wj[x] = EW == 0 ? 1 : (long long)__shfl_sync(kFull, (unsigned)w[u], j0 + x, G);
+            qj[x] = LQ ? __shfl_sync(kFull, (unsigned)qq[u], j0 + x, G) : 0u;
+          }
+          if (EW == 2 && !narrow) {  // (the high halves of wide weights)
+#pragma unroll
+            for (int x = 0; x < 4; x++)
+              wj[x] |= (long long)((unsigned long long)__shfl_sync(kFull, (unsigned)((unsigned long long)w[u] >> 32), j0 + x, G) << 32);
+          }
+#pragma unroll
+          for (int x = 0; x < 4; x++) {
+            const bool eq = Lj[x] == Lu[u];
+            c += eq ? wj[x] : 0;
+            own += Lj[x] >= 0 && Lj[x] == L0[u] ? wj[x] : 0;
+            qsum += LQ && eq ? qj[x] : 0u;
+            first = first && !(eq && j0 + x < gl);
+          }
         }
+        conn[u] = c;
+        c0[u] = own;
       }
-      qs[u] = 0;
-      if constexpr (LQ) qs[u] = (long long)__reduce_add_sync(peers, (unsigned)qq[u]);
-      // the own-label connection is the connection of the group's lanes that carry the own label
-      const unsigned own = __ballot_sync(kFull, has && Lu[u] == L0[u]) & gmask;
-      if constexpr (EW == 0) {
-        c0[u] = __popc(own);
-      } else {
-        const long long cown = __shfl_sync(kFull, conn[u], own ? __ffs(own) - 1 : lane);
-        c0[u] = own ? cown : 0;
-      }
-      cand[u] = has && lane == __ffs(peers) - 1 && Lu[u] != L0[u] && conn[u] > c0[u];
+      qs[u] = LQ ? (long long)qsum : 0;
+      cand[u] = has && first && Lu[u] != L0[u] && conn[u] > c0[u];
       lwL[u] = cand[u] ? P.lw[Lu[u]] : 0;
     }
 #pragma unroll
@@ -999,10 +1025,147 @@ __device__ __forceinline__ void choose_groups(const LpProblem &P, const Bins &B,
   }
 }
 
-// Warp-cooperative insert of (label L, weight w, score q) into an open-addressing table in shared
-// memory (slots keys/vals/qv, `mask` = slots - 1). Lanes are grouped by label first, so each distinct
-// label of the warp costs one insert however many neighbours carry it. All lanes call; lanes with
-// `on` false contribute nothing.
+// One thread per vertex with any weights (the sums of choose_rows are 32 bits wide): the row is read again for
+// every neighbour.
+template <int EW>
+__device__ __noinline__ Best choose_row_wide(const LpProblem &P, int v, int64_t beg, int d, int L0, long long cv,
+                                             long long *c0_out) {
+  long long c0 = 0;
+  for (int i = 0; i < d; i++)
+    if (P.labels[__ldg(P.g.adj + beg + i)] == L0) c0 += load_ew<EW>(P.g.ew, beg + i);
+  Best b = no_best();
+  for (int i = 0; i < d; i++) {
+    const int L = P.labels[__ldg(P.g.adj + beg + i)];
+    if (L == L0) continue;
+    long long c = 0;
+    for (int j = 0; j < d; j++)
+      if (P.labels[__ldg(P.g.adj + beg + j)] == L) c += load_ew<EW>(P.g.ew, beg + j);
+    const Best x = make_cand(P, v, L, L0, c, 0, c0, cv);
+    if (better(x, b)) b = x;
+  }
+  *c0_out = c0;
+  return b;
+}
+
+// One thread per vertex with at most D neighbours (positions i0, i0 + step, ... of bin `bin`), all of their labels in
+// registers. A thread has up to D label gathers in flight (a lane group has one per lane), which is what hides
+// their latency, and the connections take D^2 compares of registers for 32 vertices at a time where a lane group
+// spends that on two or four. Only the label that wins is looked up in the label weights; when it has no room, it
+// is taken out and the next one wins. direct: the first sub-round of a clustering from singletons, where vertex u
+// carries the label lbase + u - vbase and all labels of a row differ.
+template <int EW, int D, class Bins>
+__device__ __forceinline__ void choose_rows(const LpProblem &P, const Bins &B, int bin, unsigned i0, unsigned step,
+                                            bool direct) {
+  const unsigned cnt = B.count(bin);
+  for (unsigned i = i0; i < cnt; i += step) {
+    int v;
+    int64_t beg, d64;
+    B.row(bin, i, &v, &beg, &d64);
+    const int d = (int)d64;
+    int L[D];
+    unsigned w[EW ? D : 1];
+#pragma unroll
+    for (int j = 0; j < D; j++) L[j] = j < d ? __ldg(P.g.adj + beg + j) : -1;
+    const int L0 = P.labels[P.vbase + v];
+    const long long cv = P.g.vweight(v);
+    if (direct) {
+      const int shift = (int)(P.lbase - P.vbase);
+#pragma unroll
+      for (int j = 0; j < D; j++) L[j] = j < d ? L[j] + shift : -1;
+    } else {
+#pragma unroll
+      for (int j = 0; j < D; j++) L[j] = j < d ? P.labels[L[j]] : -1;
+    }
+    bool other = false, wide = false;
+#pragma unroll
+    for (int j = 0; j < D; j++) other |= L[j] >= 0 && L[j] != L0;
+    Best b = no_best();
+    long long c0 = 0;
+    if (EW && other) {  // (the weights of an inner vertex are not read)
+#pragma unroll
+      for (int j = 0; j < D; j++) {
+        const long long x = j < d ? load_ew<EW>(P.g.ew, beg + j) : 0;
+        wide |= (unsigned long long)x >> 26 != 0;
+        w[EW ? j : 0] = (unsigned)x;
+      }
+      if (wide) {
+        b = choose_row_wide<EW>(P, v, beg, d, L0, cv, &c0);
+        other = false;
+      }
+    }
+    if (other) {
+      unsigned own = 0;
+#pragma unroll
+      for (int j = 0; j < D; j++) {
+        if (L[j] == L0) {
+          own += EW ? w[EW ? j : 0] : 1u;
+          L[j] = -1;
+        }
+      }
+      c0 = own;
+      const uint64_t hv = mix64(P.smix ^ (uint64_t)(uint32_t)v);
+      while (other) {
+        // the labels of largest connection, as positions; equal ones share all their positions
+        unsigned most = own, pos = 0;
+        if (direct && EW == 0) {
+          most = 1;
+#pragma unroll
+          for (int x = 0; x < D; x++) pos |= L[x] >= 0 ? 1u << x : 0u;
+        } else {
+#pragma unroll
+          for (int x = 0; x < D; x++) {
+            unsigned c = 0;
+            if (direct) {
+              c = EW ? w[EW ? x : 0] : 1u;
+            } else {
+#pragma unroll
+              for (int y = 0; y < D; y++) c += L[y] == L[x] ? (EW ? w[EW ? y : 0] : 1u) : 0u;
+            }
+            if (L[x] < 0) c = 0;
+            if (c > most) {
+              most = c;
+              pos = 1u << x;
+            } else if (c == most && pos) {
+              pos |= 1u << x;
+            }
+          }
+        }
+        if (!pos) break;
+        uint64_t bh = 0;
+        int bL = -1;
+#pragma unroll
+        for (int x = 0; x < D; x++) {
+          if ((pos >> x & 1u) && L[x] != bL) {
+            const uint64_t h = mix64(hv ^ (uint64_t)(L[x] - P.lbase));
+            if (bL < 0 || h > bh || (h == bh && L[x] < bL)) {
+              bh = h;
+              bL = L[x];
+            }
+          }
+        }
+        if (P.lw[bL] + cv <= P.U) {
+          b.L = bL;
+          b.conn = most;
+          b.h = bh;
+          break;
+        }
+        other = false;
+#pragma unroll
+        for (int x = 0; x < D; x++) {
+          if (L[x] == bL) L[x] = -1;
+          other |= L[x] >= 0;
+        }
+      }
+    }
+    if (b.L < 0) {
+      B.none(bin, i);
+      continue;
+    }
+    B.template put<false>(bin, i, v, b, c0);
+    atomicAdd(reinterpret_cast<unsigned long long *>(&P.demand[b.L]), (unsigned long long)cv);
+  }
+}
+
 // A table that is full (an invariant of the sizing broken) ends the probe after one pass over the table,
 // records GP_ERR_INTERNAL with the site in the problem's counters, and drops the label.
 __device__ __forceinline__ void table_full(LpCounters *ctr, int site) {
@@ -1010,119 +1173,217 @@ __device__ __forceinline__ void table_full(LpCounters *ctr, int site) {
   atomicExch(&ctr->pad, site);
 }
 
-template <int EW, bool LQ>
-__device__ __forceinline__ void warp_insert(int *keys, unsigned long long *vals, unsigned *qv, unsigned mask, bool on,
-                                            int L, long long w, unsigned q, LpCounters *ctr, int site) {
-  const unsigned peers = __match_any_sync(kFull, on ? L : -1);
-  // weights below 2^26 sum exactly in 32 bits over at most 32 lanes: one warp reduction
-  const bool wide = EW != 0 && __any_sync(kFull, on && (w >= (1ll << 26) || w < 0));
-  if (!on) return;
-  long long sum;
-  if constexpr (EW == 0) {
-    sum = __popc(peers);
-  } else if (!wide) {
-    sum = (long long)__reduce_add_sync(peers, (unsigned)w);
-  } else {
-    sum = 0;
-    for (unsigned m = peers; m; m &= m - 1) sum += __shfl_sync(peers, w, __ffs(m) - 1);
-  }
-  unsigned qs = 0;
-  if constexpr (LQ) qs = __reduce_add_sync(peers, q);
-  if ((int)(threadIdx.x & 31) != __ffs(peers) - 1) return;
-  unsigned sl = slot_hash(L) & mask;
-  for (unsigned probe = 0; probe <= mask; probe++) {
-    const int k = atomicCAS(&keys[sl], -1, L);
-    if (k == -1 || k == L) {
-      atomicAdd(&vals[sl], (unsigned long long)sum);
-      if (LQ) atomicAdd(&qv[sl], qs);
-      return;
-    }
-    sl = (sl + 1) & mask;
-  }
-  table_full(ctr, site);
+// 64-bit sum in two 32-bit words of shared memory: one 32-bit atomic as long as neither the weight nor the sum
+// passes 2^32 (a 64-bit shared atomic is a loop of compare-and-swaps). Exact modulo 2^64 in any order.
+__device__ __forceinline__ void add_wide(unsigned *lo, unsigned *hi, long long w) {
+  const unsigned wl = (unsigned)w;
+  const unsigned old = atomicAdd(lo, wl);
+  const unsigned up = (unsigned)((unsigned long long)w >> 32) + (old + wl < old ? 1u : 0u);
+  if (up) atomicAdd(hi, up);
 }
 
-// One warp per vertex (32 < d <= deg_warp), open-addressing table in shared memory.
+// Open-addressing table of labels in shared memory: per slot the label, its connection (a count with unit weights,
+// else 64 bits in two words) and with scores its score sum. Lanes insert one by one: a slot is read before it is
+// claimed, and lanes with equal labels meet in the atomics. (Combining equal labels in the warp first takes a step
+// per distinct label for the match and another for each reduction: per warp and SM 46 ns for 32 different labels
+// with unit weights and 104 ns with others, against 18 ns; 10 ns when only two labels occur, against 12 and 16.)
+template <int EW, bool LQ>
+struct LabelTable {
+  int *keys;
+  unsigned *lo, *hi, *qv;
+  // Slots [first, ...) of a table of `all` slots at `base`: the block's one table and the shares of it that its teams
+  // and warps use lie in the same arrays, so that each finds them as the others left them, cleared.
+  __device__ __forceinline__ LabelTable(unsigned char *base, int all, int first) {
+    keys = reinterpret_cast<int *>(base) + first;
+    lo = reinterpret_cast<unsigned *>(base) + all + first;
+    hi = lo + all;
+    qv = hi + all;
+  }
+  __device__ __forceinline__ void clear(int s) const {
+    keys[s] = -1;
+    lo[s] = 0;
+    if (EW) hi[s] = 0;
+    if (LQ) qv[s] = 0;
+  }
+  __device__ __forceinline__ long long sum(int s) const {
+    return EW == 0 ? (long long)lo[s] : (long long)((unsigned long long)hi[s] << 32 | lo[s]);
+  }
+  // Returns the slot when the label took a new one, else -1: whoever claimed a slot later reads and clears it, so that
+  // a table is never scanned and may be as sparse as there is room for.
+  __device__ __forceinline__ int add(unsigned mask, int L, long long w, unsigned q, LpCounters *ctr, int site) const {
+    unsigned sl = slot_hash(L) & mask;
+    for (unsigned probe = 0; probe <= mask; probe++) {
+      int k = *(volatile int *)&keys[sl];
+      if (k == -1) k = atomicCAS(&keys[sl], -1, L);
+      if (k == -1 || k == L) {
+        if (EW == 0) atomicAdd(&lo[sl], 1u);
+        else add_wide(&lo[sl], &hi[sl], w);
+        if (LQ) atomicAdd(&qv[sl], q);
+        return k == -1 ? (int)sl : -1;
+      }
+      sl = (sl + 1) & mask;
+    }
+    table_full(ctr, site);
+    return -1;
+  }
+};
+
+// One row in a table: thread tt of kN enters the entries tt, tt + kN, ... (at most 4 * B of them) of row [beg, end)
+// that do not carry the own label L0, and keeps the labels whose slots it claimed.
+template <int EW, bool LQ, int B>
+struct RowLabels {
+  int L[4 * B], sl[4 * B];
+  // returns the thread's part of the own label's connection
+  __device__ __forceinline__ long long enter(const LpProblem &P, const LabelTable<EW, LQ> &T, unsigned mask,
+                                             int64_t beg, int64_t end, int tt, int kN, int L0, int site) {
+    long long c0 = 0;
+#pragma unroll
+    for (int b = 0; b < B; b++) {
+      long long w[4];
+      unsigned q[4];
+#pragma unroll
+      for (int x = 0; x < 4; x++) {
+        const int64_t e = beg + tt + (int64_t)kN * (4 * b + x);
+        L[4 * b + x] = e < end ? __ldg(P.g.adj + e) : -1;
+        w[x] = e < end ? load_ew<EW>(P.g.ew, e) : 0;
+        q[x] = (LQ && e < end) ? (unsigned)__ldg(P.q + e) : 0u;
+      }
+#pragma unroll
+      for (int x = 0; x < 4; x++) L[4 * b + x] = L[4 * b + x] >= 0 ? P.labels[L[4 * b + x]] : -1;
+#pragma unroll
+      for (int x = 0; x < 4; x++) {
+        const int k = L[4 * b + x];
+        sl[4 * b + x] = -1;
+        if (k == L0) c0 += w[x];
+        else if (k >= 0) sl[4 * b + x] = T.add(mask, k, w[x], q[x], P.ctr, site);
+      }
+      if (beg + (int64_t)kN * 4 * (b + 1) >= end) {  // (uniform: nothing left for any thread)
+#pragma unroll
+        for (int x = 4 * (b + 1); x < 4 * B; x++) sl[x] = -1;
+        break;
+      }
+    }
+    return c0;
+  }
+  __device__ __forceinline__ bool any() const {
+    bool a = false;
+#pragma unroll
+    for (int x = 0; x < 4 * B; x++) a |= sl[x] >= 0;
+    return a;
+  }
+  // the best eligible one of the thread's labels (the row is complete), whose slots are cleared; the label weights are
+  // loaded four at a time
+  __device__ __forceinline__ Best best(const LpProblem &P, const LabelTable<EW, LQ> &T, int v, long long c0,
+                                       long long cv) const {
+    Best r = no_best();
+    const uint64_t hv = mix64(P.smix ^ (uint64_t)(uint32_t)v);
+#pragma unroll
+    for (int b = 0; b < B; b++) {
+      long long c[4], room[4];
+      unsigned qs[4];
+#pragma unroll
+      for (int x = 0; x < 4; x++) {
+        const int s = sl[4 * b + x];
+        c[x] = s >= 0 ? T.sum(s) : 0;
+        qs[x] = LQ && s >= 0 ? T.qv[s] : 0u;
+        if (s >= 0) T.clear(s);
+        if (c[x] <= c0 || (r.L >= 0 && c[x] < r.conn)) c[x] = -1;
+      }
+#pragma unroll
+      for (int x = 0; x < 4; x++) room[x] = c[x] >= 0 ? P.lw[L[4 * b + x]] : 0;
+#pragma unroll
+      for (int x = 0; x < 4; x++) {
+        if (c[x] < 0 || room[x] + cv > P.U || (r.L >= 0 && c[x] < r.conn)) continue;
+        Best y;
+        y.conn = c[x];
+        y.qs = qs[x];
+        y.L = L[4 * b + x];
+        y.h = mix64(hv ^ (uint64_t)(y.L - P.lbase));
+        if (better(y, r)) r = y;
+      }
+    }
+    return r;
+  }
+};
+
+// The same over row entries e0, e0 + step, ... below end in the first sub-round of a clustering from singletons:
+// every entry's label is its own candidate, the label of vertex u being lbase + u - vbase.
+template <int EW, bool LQ>
+__device__ __forceinline__ Best direct_best(const LpProblem &P, int64_t e0, int64_t step, int64_t end, int v,
+                                            long long cv) {
+  const uint64_t hv = mix64(P.smix ^ (uint64_t)(uint32_t)v);
+  Best lim = no_best();
+  while (true) {
+    Best b = no_best();
+    for (int64_t e = e0; e < end; e += step) {
+      Best x;
+      x.L = (int)(__ldg(P.g.adj + e) - P.vbase + P.lbase);
+      x.conn = load_ew<EW>(P.g.ew, e);
+      if (b.L >= 0 && x.conn < b.conn) continue;
+      x.qs = LQ ? (long long)__ldg(P.q + e) : 0;
+      x.h = mix64(hv ^ (uint64_t)(x.L - P.lbase));
+      if (lim.L >= 0 && !better(lim, x)) continue;
+      if (better(x, b)) b = x;
+    }
+    if (b.L < 0 || P.lw[b.L] + cv <= P.U) return b;
+    lim = b;
+  }
+}
+
+// One warp per vertex (32 < d <= deg_warp), open-addressing table in shared memory. Bound by the latency of a
+// vertex (row, adjacency, labels, label weight, one after another): the next vertex's row is read while this one
+// is resolved, and four entries per lane are in flight.
 template <int EW, int TB>
-__device__ void choose_warp(const LpProblem &P, const SubCounters &V, int lb, int nb, unsigned char *dsm, bool direct) {
+__device__ __forceinline__ void choose_warp(const LpProblem &P, const SubCounters &V, int lb, int nb,
+                                            unsigned char *dsm, bool direct) {
   constexpr bool LQ = TB == 0;
   const unsigned cnt = V.bin_count[4];
   if (cnt == 0) return;
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr int kCap = kWarpCapT<TB>;
-  unsigned long long *vals = reinterpret_cast<unsigned long long *>(dsm) + wid * kCap;
-  int *keys = reinterpret_cast<int *>(dsm + kWarps * kCap * 8) + wid * kCap;
-  unsigned *qv = reinterpret_cast<unsigned *>(dsm + kWarps * kCap * 12) + wid * kCap;
-  for (int s = lane; s < kCap; s += 32) {
-    keys[s] = -1;
-    vals[s] = 0;
-    if (LQ) qv[s] = 0;
-  }
+  static_assert(kCap * kWarps == kCtaCapT<TB>, "the warps' tables are shares of the block's");
+  static_assert(kCap == 256 || kCap == 512, "a lane enters kCap / 64 entries at most");
+  const LabelTable<EW, LQ> T(dsm, kCtaCapT<TB>, wid * kCap);
+  for (int s = lane; s < kCap; s += 32) T.clear(s);
   __syncwarp();
   const int32_t *list = P.bin[4];
   const unsigned gw = (unsigned)lb * kWarps + wid, nw = (unsigned)nb * kWarps;
-  if (direct) {
-    // distinct singleton labels: the connection to a label is the weight of its one entry
-    for (unsigned i = gw; i < cnt; i += nw) {
-      const int v = list[i];
-      const int64_t beg = P.g.row_begin(v), end = P.g.row_begin(v + 1);
-      const int L0 = P.labels[P.vbase + v];
-      const long long cv = P.g.vweight(v);
-      Best b = no_best();
-      for (int64_t e = beg + lane; e < end; e += 32) {
-        const Best x = make_cand(P, v, P.labels[__ldg(P.g.adj + e)], L0, load_ew<EW>(P.g.ew, e),
-                                 LQ ? (long long)__ldg(P.q + e) : 0, 0, cv);
-        if (better(x, b)) b = x;
-      }
-      b = group_best<LQ, 32>(b);
+  int vn = 0;
+  int64_t begn = 0, endn = 0;
+  if (gw < cnt) {
+    vn = list[gw];
+    begn = P.g.row_begin(vn);
+    endn = P.g.row_begin(vn + 1);
+  }
+  for (unsigned i = gw; i < cnt; i += nw) {
+    const int v = vn;
+    const int64_t beg = begn, end = endn;
+    if (i + nw < cnt) {
+      vn = list[i + nw];
+      begn = P.g.row_begin(vn);
+      endn = P.g.row_begin(vn + 1);
+    }
+    const long long cv = P.g.vweight(v);
+    if (direct) {
+      const Best b = group_best<LQ, 32>(direct_best<EW, LQ>(P, beg + lane, 32, end, v, cv));
       if (lane == 0) {
         write_slot<LQ>(P, P.bin_base[4] + i, v, b, 0);
         if (b.L >= 0) atomicAdd(reinterpret_cast<unsigned long long *>(&P.demand[b.L]), (unsigned long long)cv);
       }
+      continue;
     }
-    return;
-  }
-  for (unsigned i = gw; i < cnt; i += nw) {
-    const int v = list[i];
-    const int64_t beg = P.g.row_begin(v), end = P.g.row_begin(v + 1);
-    const int d = (int)(end - beg);
-    int cap = 64;
-    while (cap < 2 * d) cap <<= 1;
-    const unsigned mask = (unsigned)cap - 1;
     const int L0 = P.labels[P.vbase + v];
-    long long c0 = 0;
-    bool other = false;  // some neighbour carries another label
-    for (int64_t e0 = beg; e0 < end; e0 += 32) {
-      const int64_t e = e0 + lane;
-      const bool in = e < end;
-      const int L = in ? P.labels[__ldg(P.g.adj + e)] : -1;
-      const long long w = in ? load_ew<EW>(P.g.ew, e) : 0;
-      if (in && L == L0) c0 += w;
-      other |= in && L != L0;
-      warp_insert<EW, LQ>(keys, vals, qv, mask, in && L != L0, L, w, (LQ && in) ? (unsigned)__ldg(P.q + e) : 0u,
-                          P.ctr, 1);
-    }
-    if (!__any_sync(kFull, other)) {
+    RowLabels<EW, LQ, kCap / 256> R;
+    long long c0 = R.enter(P, T, kCap - 1, beg, end, lane, 32, L0, 1);
+    if (!__any_sync(kFull, R.any())) {
       // every neighbour carries the own label: no candidate, the table is still empty
       if (lane == 0) P.mv_t[P.bin_base[4] + i] = -1;
       continue;
     }
-    c0 = warp_sum64(c0);
+    c0 = EW == 0 ? (long long)warp_sum_u32((unsigned)c0) : warp_sum64(c0);
     __syncwarp();
-    const long long cv = P.g.vweight(v);
-    Best b = no_best();
-    for (int s = lane; s < cap; s += 32) {
-      const int L = keys[s];
-      if (L >= 0) {
-        const Best x = make_cand(P, v, L, L0, (long long)vals[s], LQ ? (long long)qv[s] : 0, c0, cv);
-        if (better(x, b)) b = x;
-        keys[s] = -1;
-        vals[s] = 0;
-        if (LQ) qv[s] = 0;
-      }
-    }
+    const Best b = group_best<LQ, 32>(R.best(P, T, v, c0, cv));
     __syncwarp();
-    b = group_best<LQ, 32>(b);
     if (lane == 0) {
       write_slot<LQ>(P, P.bin_base[4] + i, v, b, c0);
       if (b.L >= 0) atomicAdd(reinterpret_cast<unsigned long long *>(&P.demand[b.L]), (unsigned long long)cv);
@@ -1130,84 +1391,123 @@ __device__ void choose_warp(const LpProblem &P, const SubCounters &V, int lb, in
   }
 }
 
-// One CTA per vertex (deg_warp < d <= deg_cta), table in shared memory.
+// Teams of NW warps inside a block (NW = kWarps: the block itself).
+template <int NW>
+__device__ __forceinline__ void team_sync(int team) {
+  if constexpr (NW == kWarps) __syncthreads();
+  else asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(NW * 32) : "memory");
+}
+
+template <int NW>
+__device__ __forceinline__ long long team_sum(long long x, Smem &sm, int team) {
+  x = warp_sum64(x);
+  if ((threadIdx.x & 31) == 0) sm.sum[threadIdx.x >> 5] = x;
+  team_sync<NW>(team);
+  long long r = 0;
+#pragma unroll
+  for (int w = 0; w < NW; w++) r += sm.sum[team * NW + w];
+  return r;  // (the caller's next team_sync precedes the next write)
+}
+
+template <bool LQ, int NW>
+__device__ __forceinline__ Best team_best(Best b, Smem &sm, int team) {
+  b = group_best<LQ, 32>(b);
+  if ((threadIdx.x & 31) == 0) sm.best[threadIdx.x >> 5] = b;
+  team_sync<NW>(team);
+  Best r = sm.best[team * NW];
+#pragma unroll
+  for (int w = 1; w < NW; w++)
+    if (better(sm.best[team * NW + w], r)) r = sm.best[team * NW + w];
+  return r;
+}
+
+// One vertex by a team: position i of bin 5, row [beg, end) of at most half as many entries as table T has slots.
+template <int EW, bool LQ, int NW, int kCap>
+__device__ __forceinline__ void team_vertex(const LpProblem &P, const LabelTable<EW, LQ> &T, Smem &sm, int team,
+                                            unsigned i, int v, int64_t beg, int64_t end, bool direct) {
+  constexpr int kN = NW * 32;
+  const int tt = (int)threadIdx.x - team * kN;
+  const long long cv = P.g.vweight(v);
+  long long c0 = 0;
+  Best b;
+  if (direct) {
+    b = direct_best<EW, LQ>(P, beg + tt, kN, end, v, cv);
+    team_sync<NW>(team);  // (sm.best of the team's last vertex has been read)
+  } else {
+    static_assert(kCap % (8 * kN) == 0, "rows of kCap / 2 entries, four per thread and step");
+    RowLabels<EW, LQ, kCap / (8 * kN)> R;
+    c0 = team_sum<NW>(R.enter(P, T, kCap - 1, beg, end, tt, kN, P.labels[P.vbase + v], 2), sm, team);
+    b = R.best(P, T, v, c0, cv);  // (the sum completed the table)
+  }
+  b = team_best<LQ, NW>(b, sm, team);  // (and completes the clearing)
+  if (tt == 0) {
+    write_slot<LQ>(P, P.bin_base[5] + i, v, b, c0);
+    if (b.L >= 0) atomicAdd(reinterpret_cast<unsigned long long *>(&P.demand[b.L]), (unsigned long long)cv);
+  }
+}
+
+// Bin 5 (deg_warp < d <= deg_cta). Bound by the latency of a vertex (row, adjacency, labels, label weights, and the
+// meetings of the threads that share it), so what counts is how many vertices are in hand: teams of kTeamWarps warps
+// take the rows that a team's share of the block's table holds, the next vertex's row being read while one is
+// resolved; the longer ones are left to the whole block after every kTeamBatch vertices per team. (A block per vertex
+// took 6.5 us for a row of 500 entries on R-MAT 21; one warp per vertex overflowed its table too often and was slower
+// still.)
+constexpr int kTeamWarps = 4;
+constexpr int kTeams = kWarps / kTeamWarps;
+constexpr int kTeamBatch = 16;
+
 template <int EW, int TB>
-__device__ void choose_cta(const LpProblem &P, const SubCounters &V, int lb, int nb, unsigned char *dsm, Smem &sm,
-                           bool direct) {
+__device__ __forceinline__ void choose_cta(const LpProblem &P, const SubCounters &V, int lb, int nb,
+                                           unsigned char *dsm, Smem &sm, bool direct) {
   const unsigned cnt = V.bin_count[5];
   if (cnt == 0) return;
   constexpr bool LQ = TB == 0;
-  constexpr int kCap = kCtaCapT<TB>;
-  unsigned long long *vals = reinterpret_cast<unsigned long long *>(dsm);
-  int *keys = reinterpret_cast<int *>(dsm + kCap * 8);
-  unsigned *qv = reinterpret_cast<unsigned *>(dsm + kCap * 12);
+  constexpr int kAll = kCtaCapT<TB>, kCap = kAll / kTeams;
+  __shared__ unsigned s_left[kTeams * kTeamBatch], s_nleft;
+  const int team = (int)(threadIdx.x >> 5) / kTeamWarps;
+  const LabelTable<EW, LQ> A(dsm, kAll, 0), T(dsm, kAll, team * kCap);
   __syncthreads();
-  for (int s = threadIdx.x; s < kCap; s += kThreads) {
-    keys[s] = -1;
-    vals[s] = 0;
-    if (LQ) qv[s] = 0;
-  }
+  for (int s = threadIdx.x; s < kAll; s += kThreads) A.clear(s);
+  if (threadIdx.x == 0) s_nleft = 0;
   __syncthreads();
   const int32_t *list = P.bin[5];
-  if (direct) {
-    for (unsigned i = lb; i < cnt; i += nb) {
-      const int v = list[i];
-      const int64_t beg = P.g.row_begin(v), end = P.g.row_begin(v + 1);
-      const int L0 = P.labels[P.vbase + v];
-      const long long cv = P.g.vweight(v);
-      Best b = no_best();
-      for (int64_t e = beg + threadIdx.x; e < end; e += kThreads) {
-        const Best x = make_cand(P, v, P.labels[__ldg(P.g.adj + e)], L0, load_ew<EW>(P.g.ew, e),
-                                 LQ ? (long long)__ldg(P.q + e) : 0, 0, cv);
-        if (better(x, b)) b = x;
+  const unsigned gt = (unsigned)lb * kTeams + (unsigned)team, nt = (unsigned)nb * kTeams;
+  const unsigned rounds = (cnt + nt - 1) / nt;  // (the same for every team of the block)
+  int vn = 0;
+  int64_t begn = 0, endn = 0;
+  if (gt < cnt) {
+    vn = list[gt];
+    begn = P.g.row_begin(vn);
+    endn = P.g.row_begin(vn + 1);
+  }
+  for (unsigned r = 0; r < rounds; r++) {
+    const unsigned i = gt + r * nt;
+    const int v = vn;
+    const int64_t beg = begn, end = endn;
+    if (i < cnt && i + nt < cnt) {
+      vn = list[i + nt];
+      begn = P.g.row_begin(vn);
+      endn = P.g.row_begin(vn + 1);
+    }
+    if (i < cnt) {
+      if (direct || 2 * (end - beg) <= kCap) {
+        team_vertex<EW, LQ, kTeamWarps, kCap>(P, T, sm, team, i, v, beg, end, direct);
+      } else if (threadIdx.x % (kTeamWarps * 32) == 0) {
+        s_left[atomicAdd(&s_nleft, 1u)] = i;  // (at most one per team and round of a batch)
       }
-      b = block_best_of<LQ>(b, sm);
-      if (threadIdx.x == 0) {
-        write_slot<LQ>(P, P.bin_base[5] + i, v, b, 0);
-        if (b.L >= 0) atomicAdd(reinterpret_cast<unsigned long long *>(&P.demand[b.L]), (unsigned long long)cv);
-      }
+    }
+    if (r % kTeamBatch != kTeamBatch - 1 && r + 1 < rounds) continue;
+    __syncthreads();
+    const unsigned left = s_nleft;
+    for (unsigned y = 0; y < left; y++) {
+      const unsigned ic = s_left[y];
+      const int vc = list[ic];
+      team_vertex<EW, LQ, kWarps, kAll>(P, A, sm, 0, ic, vc, P.g.row_begin(vc), P.g.row_begin(vc + 1), false);
     }
     __syncthreads();
-    return;
+    if (threadIdx.x == 0) s_nleft = 0;
+    __syncthreads();
   }
-  for (unsigned i = lb; i < cnt; i += nb) {
-    const int v = list[i];
-    const int64_t beg = P.g.row_begin(v), end = P.g.row_begin(v + 1);
-    const int d = (int)(end - beg);
-    int cap = 64;
-    while (cap < 2 * d) cap <<= 1;
-    const unsigned mask = (unsigned)cap - 1;
-    const int L0 = P.labels[P.vbase + v];
-    long long c0 = 0;
-    for (int64_t e0 = beg + (threadIdx.x & ~31); e0 < end; e0 += kThreads) {
-      const int64_t e = e0 + (threadIdx.x & 31);
-      const bool in = e < end;
-      const int L = in ? P.labels[__ldg(P.g.adj + e)] : -1;
-      const long long w = in ? load_ew<EW>(P.g.ew, e) : 0;
-      if (in && L == L0) c0 += w;
-      warp_insert<EW, LQ>(keys, vals, qv, mask, in && L != L0, L, w, (LQ && in) ? (unsigned)__ldg(P.q + e) : 0u,
-                          P.ctr, 2);
-    }
-    c0 = block_sum_of(c0, sm);  // also completes the table
-    const long long cv = P.g.vweight(v);
-    Best b = no_best();
-    for (int s = threadIdx.x; s < cap; s += kThreads) {
-      const int L = keys[s];
-      if (L >= 0) {
-        const Best x = make_cand(P, v, L, L0, (long long)vals[s], LQ ? (long long)qv[s] : 0, c0, cv);
-        if (better(x, b)) b = x;
-        keys[s] = -1;
-        vals[s] = 0;
-        if (LQ) qv[s] = 0;
-      }
-    }
-    b = block_best_of<LQ>(b, sm);
-    if (threadIdx.x == 0) {
-      write_slot<LQ>(P, P.bin_base[5] + i, v, b, c0);
-      if (b.L >= 0) atomicAdd(reinterpret_cast<unsigned long long *>(&P.demand[b.L]), (unsigned long long)cv);
-    }
-  }
-  __syncthreads();
 }
 
 // Hubs (d > deg_cta), done by block 0 for the sub-round's hub list: prefixes of work chunks (P.hub_chunk
@@ -1458,17 +1758,11 @@ __device__ __noinline__ void hub_accum(const LpProblem &P, unsigned h0, unsigned
   constexpr bool kStage = TB == 2;
   constexpr int kCap = kHubCap;
   constexpr int kChunk = kHubChunkT<TB>;
-  unsigned long long *svals = reinterpret_cast<unsigned long long *>(dsm);
-  int *skeys = reinterpret_cast<int *>(dsm + kCap * 8);
-  unsigned *sq = reinterpret_cast<unsigned *>(dsm + kCap * 12);
+  const LabelTable<EW, LQ> T(dsm, kCap, 0);
   unsigned char *stage = dsm + kStageOff;
   __shared__ __align__(8) unsigned long long s_bar[2];
   __shared__ int s_to;
-  for (int t = threadIdx.x; t < kCap; t += kThreads) {
-    skeys[t] = -1;
-    svals[t] = 0;
-    if (LQ) sq[t] = 0;
-  }
+  for (int t = threadIdx.x; t < kCap; t += kThreads) T.clear(t);
   const unsigned c_lo = P.hub_prefix[h0], c_hi = P.hub_prefix[h1];
   // chunk c of the batch: its hub position and entries
   auto chunk_of = [&](unsigned c, unsigned *ip, int64_t *bp, int64_t *ep) {
@@ -1566,13 +1860,11 @@ __device__ __noinline__ void hub_accum(const LpProblem &P, unsigned h0, unsigned
 #pragma unroll
         for (int u = 0; u < 4; u++) {
           if (in[u] && L[u] == L0) c0 += w[u];
-          const bool on = in[u] && (P.hub_keep || L[u] != L0);  // kept tables hold the own label too
-          const unsigned peers = __match_any_sync(kFull, on ? L[u] : -1);
-          long long sum = 0;
-          if (on)
-            for (unsigned m = peers; m; m &= m - 1) sum += __shfl_sync(peers, w[u], __ffs(m) - 1);
-          if (on && (int)(threadIdx.x & 31) == __ffs(peers) - 1)
-            atomicAdd(&svals[L[u] - P.lbase], (unsigned long long)sum);
+          if (in[u] && (P.hub_keep || L[u] != L0)) {  // kept tables hold the own label too
+            const int t = (int)(L[u] - P.lbase);
+            if (EW == 0) atomicAdd(&T.lo[t], 1u);
+            else add_wide(&T.lo[t], &T.hi[t], w[u]);
+          }
         }
       }
       c0 = block_sum_of(c0, sm);  // also completes the counters (and makes s_to visible)
@@ -1582,10 +1874,10 @@ __device__ __noinline__ void hub_accum(const LpProblem &P, unsigned h0, unsigned
       }
       if (P.hub_keep) c0 = 0;  // (kept tables: the choice looks the own label up)
       for (int t = threadIdx.x; t < nl; t += kThreads) {
-        const unsigned long long x = svals[t];
+        const unsigned long long x = (unsigned long long)T.sum(t);
         if (x) {
           atomicAdd(&P.hub_vals[tb + t], x);
-          svals[t] = 0;
+          T.clear(t);
         }
       }
       if (kStage) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // (the buffer is refilled next)
@@ -1609,29 +1901,28 @@ __device__ __noinline__ void hub_accum(const LpProblem &P, unsigned h0, unsigned
     HubChunk<EW> hc;
     if (kStage) hc.view(P, beg, end, stage + (j & 1) * kStageBuf);
     long long c0 = 0;
-    // steps of 4 * kThreads entries: each thread takes four, loads first
-    static_assert(kChunk % (4 * kThreads) == 0 && 2 * kChunk <= kCap, "a chunk fills at most half the table");
-    for (int64_t s0 = beg; s0 < end; s0 += 4 * kThreads) {
-      int64_t e[4];
-      int L[4];
+    // each thread takes four entries, loads first, and keeps the labels whose slots it claimed
+    static_assert(kChunk == 4 * kThreads && 2 * kChunk <= kCap, "a chunk fills at most half the table");
+    int Ls[4], sl[4];
+    {
       long long w[4];
       unsigned q4[4];
       bool in[4];
 #pragma unroll
       for (int u = 0; u < 4; u++) {
-        e[u] = s0 + u * kThreads + threadIdx.x;
-        in[u] = ok && e[u] < end;
-        L[u] = in[u] ? (kStage ? hc.adj(P, e[u]) : __ldg(P.g.adj + e[u])) : 0;
-        w[u] = in[u] ? (kStage ? hc.ew(P, e[u]) : load_ew<EW>(P.g.ew, e[u])) : 0;
-        q4[u] = (LQ && in[u]) ? (unsigned)__ldg(P.q + e[u]) : 0u;
+        const int64_t e = beg + u * kThreads + threadIdx.x;
+        in[u] = ok && e < end;
+        Ls[u] = in[u] ? (kStage ? hc.adj(P, e) : __ldg(P.g.adj + e)) : 0;
+        w[u] = in[u] ? (kStage ? hc.ew(P, e) : load_ew<EW>(P.g.ew, e)) : 0;
+        q4[u] = (LQ && in[u]) ? (unsigned)__ldg(P.q + e) : 0u;
       }
 #pragma unroll
-      for (int u = 0; u < 4; u++) L[u] = in[u] ? P.labels[L[u]] : -1;
+      for (int u = 0; u < 4; u++) Ls[u] = in[u] ? P.labels[Ls[u]] : -1;
 #pragma unroll
       for (int u = 0; u < 4; u++) {
-        if (in[u] && L[u] == L0) c0 += w[u];
-        warp_insert<EW, LQ>(skeys, svals, sq, kCap - 1, in[u] && (P.hub_keep || L[u] != L0), L[u], w[u], q4[u], P.ctr,
-                            3);
+        sl[u] = -1;
+        if (in[u] && Ls[u] == L0) c0 += w[u];
+        if (in[u] && (P.hub_keep || Ls[u] != L0)) sl[u] = T.add(kCap - 1, Ls[u], w[u], q4[u], P.ctr, 3);
       }
     }
     c0 = block_sum_of(c0, sm);  // also completes the shared table (and makes s_to visible)
@@ -1639,17 +1930,14 @@ __device__ __noinline__ void hub_accum(const LpProblem &P, unsigned h0, unsigned
       stage_abort(j, c);
       return;
     }
-    // flush into the hub's table: each thread claims the slots of four of its labels at once (the
-    // claims are in flight together), then retries the ones that met another label
-    static_assert(kCap % (4 * kThreads) == 0, "the flush takes four table slots per thread per step");
-    for (int t0 = threadIdx.x; t0 < kCap; t0 += 4 * kThreads) {
-      int Ls[4];
+    // flush into the hub's table: each thread claims the slots of its labels at once (the claims are in flight
+    // together), then retries the ones that met another label
+    {
       uint64_t sg[4];
       bool pend[4];
 #pragma unroll
       for (int q = 0; q < 4; q++) {
-        Ls[q] = skeys[t0 + q * kThreads];
-        pend[q] = Ls[q] >= 0;
+        pend[q] = sl[q] >= 0;
         sg[q] = pend[q] ? hub_slot(Ls[q], cap) : 0;
       }
       uint64_t probes = 0;
@@ -1665,9 +1953,8 @@ __device__ __noinline__ void hub_accum(const LpProblem &P, unsigned h0, unsigned
         for (int q = 0; q < 4; q++) {
           if (!pend[q]) continue;
           if (ks[q] == -1 || ks[q] == Ls[q]) {
-            const int t = t0 + q * kThreads;
-            atomicAdd(&P.hub_vals[tb + sg[q]], svals[t]);
-            if (LQ) atomicAdd(&P.hub_qv[tb + sg[q]], (unsigned long long)sq[t]);
+            atomicAdd(&P.hub_vals[tb + sg[q]], (unsigned long long)T.sum(sl[q]));
+            if (LQ) atomicAdd(&P.hub_qv[tb + sg[q]], (unsigned long long)T.qv[sl[q]]);
             pend[q] = false;
           } else {
             sg[q] = sg[q] + 1 == cap ? 0 : sg[q] + 1;
@@ -1675,12 +1962,8 @@ __device__ __noinline__ void hub_accum(const LpProblem &P, unsigned h0, unsigned
         }
       }
 #pragma unroll
-      for (int q = 0; q < 4; q++) {
-        const int t = t0 + q * kThreads;
-        skeys[t] = -1;
-        svals[t] = 0;
-        if (LQ) sq[t] = 0;
-      }
+      for (int q = 0; q < 4; q++)
+        if (sl[q] >= 0) T.clear(sl[q]);
     }
     if (kStage) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // (the buffer is refilled next)
     __syncthreads();
@@ -1696,7 +1979,7 @@ template <bool LQ>
 __device__ __noinline__ void hub_choose_part(const LpProblem &P, unsigned h0, unsigned h1, int lb, int nb, Smem &sm) {
   const unsigned s_lo = P.hub_scx[h0], s_hi = P.hub_scx[h1];
   Best *part = reinterpret_cast<Best *>(P.hub_part);
-  constexpr int kU = 2;  // slots per thread in flight
+  constexpr int kU = LQ ? 2 : 4;  // slots per thread in flight
   for (unsigned it = s_lo + lb; it < s_hi; it += nb) {
     const unsigned i = search_prefix(P.hub_scx, h0, h1, it);
     const int v = P.bin[6][i];
@@ -1716,33 +1999,45 @@ __device__ __noinline__ void hub_choose_part(const LpProblem &P, unsigned h0, un
       c0 = s_c0;
     }
     const long long cv = P.g.vweight(v);
+    const uint64_t hv = mix64(P.smix ^ (uint64_t)(uint32_t)v);
     Best b = no_best();
     for (int64_t base = s0; base < s1; base += kU * kThreads) {
       int L[kU];
       long long cw[kU], lwL[kU];
-      unsigned long long qq[kU];
+      unsigned long long qq[kU], hh[kU];
 #pragma unroll
       for (int u = 0; u < kU; u++) {
         const int64_t sl = base + u * kThreads + threadIdx.x;
-        if (P.hub_dense) L[u] = (sl < s1 && P.hub_vals[tb + sl] != 0) ? (int)(P.lbase + sl) : -1;
+        cw[u] = sl < s1 ? (long long)P.hub_vals[tb + sl] : 0;
+        if (P.hub_dense) L[u] = cw[u] != 0 ? (int)(P.lbase + sl) : -1;
         else L[u] = sl < s1 ? P.hub_keys[tb + sl] : -1;
       }
 #pragma unroll
       for (int u = 0; u < kU; u++) {
         const int64_t sl = base + u * kThreads + threadIdx.x;
-        cw[u] = L[u] >= 0 ? (long long)P.hub_vals[tb + sl] : 0;
         qq[u] = (LQ && L[u] >= 0) ? P.hub_qv[tb + sl] : 0ull;
+        // label weights only of labels that would win (more connection than the own label, better than the
+        // best one so far)
+        Best x;
+        x.L = L[u] >= 0 && L[u] != L0 && cw[u] > c0 && (b.L < 0 || cw[u] >= b.conn) ? L[u] : -1;
+        x.conn = cw[u];
+        x.qs = (long long)qq[u];
+        x.h = x.L >= 0 ? mix64(hv ^ (uint64_t)(L[u] - P.lbase)) : 0;
+        hh[u] = x.h;
+        lwL[u] = better(x, b) ? P.lw[L[u]] : LLONG_MAX;
       }
-      // label weights only of labels that could win (more connection than the own label)
-#pragma unroll
-      for (int u = 0; u < kU; u++) lwL[u] = (L[u] >= 0 && L[u] != L0 && cw[u] > c0) ? P.lw[L[u]] : 0;
 #pragma unroll
       for (int u = 0; u < kU; u++) {
-        if (L[u] < 0) continue;
+        if (lwL[u] != LLONG_MAX && lwL[u] + cv <= P.U) {
+          Best x;
+          x.L = L[u];
+          x.conn = cw[u];
+          x.qs = (long long)qq[u];
+          x.h = hh[u];
+          if (better(x, b)) b = x;
+        }
+        if (P.hub_keep || L[u] < 0) continue;  // kept tables stay
         const int64_t sl = base + u * kThreads + threadIdx.x;
-        const Best x = make_cand_lw(P, v, L[u], L0, cw[u], (long long)qq[u], c0, cv, lwL[u]);
-        if (better(x, b)) b = x;
-        if (P.hub_keep) continue;  // kept tables stay
         if (!P.hub_dense) P.hub_keys[tb + sl] = -1;
         P.hub_vals[tb + sl] = 0;
         if (LQ) P.hub_qv[tb + sl] = 0;
@@ -1779,15 +2074,8 @@ __device__ void hub_direct_part(const LpProblem &P, unsigned cnt, unsigned chunk
     const int64_t rb = P.g.row_begin(v), re = P.g.row_begin(v + 1);
     const int64_t beg = rb + (int64_t)(c - P.hub_prefix[i]) * P.hub_chunk;
     const int64_t end = min(re, beg + P.hub_chunk);
-    const int L0 = P.labels[P.vbase + v];
     const long long cv = P.g.vweight(v);
-    Best b = no_best();
-    for (int64_t e = beg + threadIdx.x; e < end; e += kThreads) {
-      const Best x = make_cand(P, v, P.labels[__ldg(P.g.adj + e)], L0, load_ew<EW>(P.g.ew, e),
-                               LQ ? (long long)__ldg(P.q + e) : 0, 0, cv);
-      if (better(x, b)) b = x;
-    }
-    b = block_best_of<LQ>(b, sm);
+    const Best b = block_best_of<LQ>(direct_best<EW, LQ>(P, beg + threadIdx.x, kThreads, end, v, cv), sm);
     if (threadIdx.x == 0) part[c] = b;
   }
 }
@@ -2365,7 +2653,23 @@ __device__ bool lp_problem(const LpProblem *prob, unsigned char *dsm) {
         // while block 0 prepares the hub list, the other blocks take its share of the choice
         const int clb = (hubs_now && nb > 1) ? lb - 1 : lb, cnb = (hubs_now && nb > 1) ? nb - 1 : nb;
         if (clb >= 0) {
-          choose_groups<EW, LQ>(P, ListBins{P, sV}, (unsigned)clb * kWarps + (threadIdx.x >> 5), (unsigned)cnb * kWarps);
+          unsigned grouped = 0xfu;
+          if constexpr (!LQ) {
+            // bins long enough to give every block more than kRowsMin vertices: a thread per vertex
+            const ListBins B{P, sV, 0xfu};
+            const unsigned i0 = (unsigned)clb * kThreads + threadIdx.x, step = (unsigned)cnb * kThreads;
+            for (int b = 0; b < 2; b++) {
+              if (B.count(b) > kRowsMin * (unsigned)cnb) {
+                choose_rows<EW, 8>(P, B, b, i0, step, direct);
+                grouped &= ~(1u << b);
+              }
+            }
+            if (B.count(2) > kRowsMin * (unsigned)cnb) {
+              choose_rows<EW, 16>(P, B, 2, i0, step, direct);
+              grouped &= ~4u;
+            }
+          }
+          choose_groups<EW, LQ>(P, ListBins{P, sV, grouped}, (unsigned)clb * kWarps + (threadIdx.x >> 5), (unsigned)cnb * kWarps);
           choose_warp<EW, TB>(P, sV, clb, cnb, dsm, direct);
           choose_cta<EW, TB>(P, sV, clb, cnb, dsm, sm, direct);
         }
@@ -2486,10 +2790,6 @@ constexpr int kOwnRowOff = kOwnListOff<LQ> + kOwnTile * 4;  // (the rows outlive
 template <bool LQ>
 constexpr size_t kOwnSmem = kOwnRowOff<LQ> + kOwnTile * 4;
 static_assert(kOwnRowOff<false> >= kContestSmall * 8, "the rows lie behind the contest's keys");
-// A bin of up to this many vertices goes to lane groups, a longer one to a thread per vertex: the groups take
-// one vertex through in the least time (four steps of 16 vertices at most here), the threads take many through
-// with fewer instructions and more loads in flight.
-constexpr unsigned kOwnRowsMin = 64;
 
 struct OwnProps {
   int v[kOwnKeep], t[kOwnKeep];
@@ -2534,175 +2834,28 @@ struct OwnBins {
   }
 };
 
-// One thread per vertex with any weights (the sums of choose_own_rows are 32 bits wide): the row is read again
-// for every neighbour.
-template <int EW>
-__device__ __noinline__ void choose_own_wide(const LpProblem &P, const OwnBins &B, int v, int64_t beg, int d, int L0,
-                                             long long cv) {
-  long long c0 = 0;
-  for (int i = 0; i < d; i++)
-    if (P.labels[__ldg(P.g.adj + beg + i)] == L0) c0 += load_ew<EW>(P.g.ew, beg + i);
-  Best b = no_best();
-  for (int i = 0; i < d; i++) {
-    const int L = P.labels[__ldg(P.g.adj + beg + i)];
-    if (L == L0) continue;
-    long long c = 0;
-    for (int j = 0; j < d; j++)
-      if (P.labels[__ldg(P.g.adj + beg + j)] == L) c += load_ew<EW>(P.g.ew, beg + j);
-    const Best x = make_cand(P, v, L, L0, c, 0, c0, cv);
-    if (better(x, b)) b = x;
-  }
-  if (b.L < 0) return;
-  B.template put<false>(0, 0, v, b, c0);
-  atomicAdd(reinterpret_cast<unsigned long long *>(&P.demand[b.L]), (unsigned long long)cv);
-}
-
-// One thread per vertex with at most D neighbours (bin `bin`), all of their labels in registers. A thread has
-// up to D label gathers in flight (a lane group has one per lane), which is what hides their latency, and the
-// connections take D^2 compares of registers for 32 vertices at a time instead of a match, reductions and
-// votes for two. Only the label that wins is looked up in the label weights; when it has no room, it is taken
-// out and the next one wins.
-template <int EW, int D>
-__device__ __forceinline__ void choose_own_rows(const LpProblem &P, const OwnBins &B, int bin) {
-  const unsigned cnt = B.count(bin);
-  for (unsigned i = threadIdx.x; i < cnt; i += kThreads) {
-    int v;
-    int64_t beg, d64;
-    B.row(bin, i, &v, &beg, &d64);
-    const int d = (int)d64;
-    int L[D];
-    unsigned w[EW ? D : 1];
-#pragma unroll
-    for (int j = 0; j < D; j++) L[j] = j < d ? __ldg(P.g.adj + beg + j) : -1;
-    const int L0 = P.labels[P.vbase + v];
-    const long long cv = P.g.vweight(v);
-#pragma unroll
-    for (int j = 0; j < D; j++) L[j] = j < d ? P.labels[L[j]] : -1;
-    bool other = false;
-#pragma unroll
-    for (int j = 0; j < D; j++) other |= L[j] >= 0 && L[j] != L0;
-    if (!other) continue;  // (the weights of an inner vertex are not read)
-    if (EW) {
-      bool wide = false;
-#pragma unroll
-      for (int j = 0; j < D; j++) {
-        const long long x = j < d ? load_ew<EW>(P.g.ew, beg + j) : 0;
-        wide |= (unsigned long long)x >> 26 != 0;
-        w[EW ? j : 0] = (unsigned)x;
-      }
-      if (wide) {
-        choose_own_wide<EW>(P, B, v, beg, d, L0, cv);
-        continue;
-      }
-    }
-    unsigned c0 = 0;
-#pragma unroll
-    for (int j = 0; j < D; j++) {
-      if (L[j] == L0) {
-        c0 += EW ? w[EW ? j : 0] : 1u;
-        L[j] = -1;
-      }
-    }
-    const uint64_t hv = mix64(P.smix ^ (uint64_t)(uint32_t)v);
-    while (other) {
-      // the labels of largest connection, as positions; equal ones share all their positions
-      unsigned most = c0, pos = 0;
-#pragma unroll
-      for (int x = 0; x < D; x++) {
-        unsigned c = 0;
-#pragma unroll
-        for (int y = 0; y < D; y++) c += L[y] == L[x] ? (EW ? w[EW ? y : 0] : 1u) : 0u;
-        if (L[x] < 0) c = 0;
-        if (c > most) {
-          most = c;
-          pos = 1u << x;
-        } else if (c == most && pos) {
-          pos |= 1u << x;
-        }
-      }
-      if (!pos) break;
-      uint64_t bh = 0;
-      int bL = -1;
-#pragma unroll
-      for (int x = 0; x < D; x++) {
-        if ((pos >> x & 1u) && L[x] != bL) {
-          const uint64_t h = mix64(hv ^ (uint64_t)(L[x] - P.lbase));
-          if (bL < 0 || h > bh || (h == bh && L[x] < bL)) {
-            bh = h;
-            bL = L[x];
-          }
-        }
-      }
-      if (P.lw[bL] + cv <= P.U) {
-        Best b;
-        b.L = bL;
-        b.conn = most;
-        b.qs = 0;
-        b.h = bh;
-        B.template put<false>(bin, i, v, b, c0);
-        atomicAdd(reinterpret_cast<unsigned long long *>(&P.demand[bL]), (unsigned long long)cv);
-        break;
-      }
-      other = false;
-#pragma unroll
-      for (int x = 0; x < D; x++) {
-        if (L[x] == bL) L[x] = -1;
-        other |= L[x] >= 0;
-      }
-    }
-  }
-}
-
 // One warp per vertex with 32 < d <= kOwnDeg, table in shared memory.
 template <int EW, bool LQ>
 __device__ __forceinline__ void choose_own_warp(const LpProblem &P, const OwnBins &B, unsigned char *dsm) {
   const unsigned cnt = B.count(4);
   if (cnt == 0) return;
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  unsigned long long *vals = reinterpret_cast<unsigned long long *>(dsm) + wid * kOwnCap;
-  int *keys = reinterpret_cast<int *>(dsm + kWarps * kOwnCap * 8) + wid * kOwnCap;
-  unsigned *qv = reinterpret_cast<unsigned *>(dsm + kWarps * kOwnCap * 12) + wid * kOwnCap;
-  for (int s = lane; s < kOwnCap; s += 32) {
-    keys[s] = -1;
-    vals[s] = 0;
-    if (LQ) qv[s] = 0;
-  }
+  const LabelTable<EW, LQ> T(dsm, kWarps * kOwnCap, wid * kOwnCap);
+  for (int s = lane; s < kOwnCap; s += 32) T.clear(s);
   __syncwarp();
   for (unsigned i = wid; i < cnt; i += kWarps) {
     int v;
     int64_t beg, d;
     B.row(4, i, &v, &beg, &d);
-    const unsigned cap = d <= 64 ? 128 : 256, mask = cap - 1;
     const int L0 = P.labels[P.vbase + v];
-    long long c0 = 0;
-    bool other = false;
-    for (int64_t x0 = 0; x0 < d; x0 += 32) {
-      const int64_t e = beg + x0 + lane;
-      const bool in = x0 + lane < d;
-      const int L = in ? P.labels[__ldg(P.g.adj + e)] : -1;
-      const long long w = in ? load_ew<EW>(P.g.ew, e) : 0;
-      if (in && L == L0) c0 += w;
-      other |= in && L != L0;
-      warp_insert<EW, LQ>(keys, vals, qv, mask, in && L != L0, L, w, (LQ && in) ? (unsigned)__ldg(P.q + e) : 0u,
-                          P.ctr, 8);
-    }
-    if (!__any_sync(kFull, other)) continue;  // every neighbour carries the own label; the table is still empty
+    RowLabels<EW, LQ, kOwnCap / 256> R;
+    long long c0 = R.enter(P, T, kOwnCap - 1, beg, beg + d, lane, 32, L0, 8);
+    if (!__any_sync(kFull, R.any())) continue;  // every neighbour carries the own label; the table is still empty
     c0 = warp_sum64(c0);
     __syncwarp();
     const long long cv = P.g.vweight(v);
-    Best b = no_best();
-    for (unsigned s = lane; s < cap; s += 32) {
-      const int L = keys[s];
-      if (L >= 0) {
-        const Best x = make_cand(P, v, L, L0, (long long)vals[s], LQ ? (long long)qv[s] : 0, c0, cv);
-        if (better(x, b)) b = x;
-        keys[s] = -1;
-        vals[s] = 0;
-        if (LQ) qv[s] = 0;
-      }
-    }
+    const Best b = group_best<LQ, 32>(R.best(P, T, v, c0, cv));
     __syncwarp();
-    b = group_best<LQ, 32>(b);
     if (lane == 0 && b.L >= 0) {
       B.template put<LQ>(4, i, v, b, c0);
       atomicAdd(reinterpret_cast<unsigned long long *>(&P.demand[b.L]), (unsigned long long)cv);
@@ -3007,12 +3160,13 @@ __device__ bool lp_problem_own(const LpProblem *prob, unsigned char *dsm) {
           unsigned long long grouped = counts;
           if constexpr (!LQ) {
             const OwnBins B{P, O, counts, list, rowx, (int)t0, r0, lo};
-            if (B.count(1) > kOwnRowsMin) {
-              choose_own_rows<EW, 8>(P, B, 1);
+            const bool direct = P.singletons && t == 0;
+            if (B.count(1) > kRowsMin) {
+              choose_rows<EW, 8>(P, B, 1, threadIdx.x, kThreads, direct);
               grouped &= ~0xffffull;
             }
-            if (B.count(2) > kOwnRowsMin) {
-              choose_own_rows<EW, 16>(P, B, 2);
+            if (B.count(2) > kRowsMin) {
+              choose_rows<EW, 16>(P, B, 2, threadIdx.x, kThreads, direct);
               grouped &= ~(0xffffull << 16);
             }
           }

@@ -22,6 +22,7 @@
 #include <vector>
 
 #include "mlp.cuh"
+#include "row_walk.cuh"
 
 namespace gp {
 
@@ -42,59 +43,18 @@ __device__ __forceinline__ uint16_t float_to_bf16(float f) {
 
 __device__ __forceinline__ unsigned pack2(uint16_t lo, uint16_t hi) { return (unsigned)lo | ((unsigned)hi << 16); }
 
-// The CSR entries are taken in segments of kSeg by the warps, whatever rows they belong to: the longest
-// rows of a power-law graph are spread over as many warps as they have segments.
-constexpr int kSeg = 256;
-
-// The largest v with off[v] <= x (0 <= x < m), found by the whole warp: 32 pivots per step.
-__device__ __forceinline__ int64_t warp_row_of(const DGraph &g, int64_t x) {
-  const int lane = threadIdx.x & 31;
-  int64_t lo = 0, hi = g.n;  // off[lo] <= x < off[hi]
-  while (hi - lo > 1) {
-    const int64_t step = (hi - lo + 31) / 32;
-    const int64_t p = lo + (lane + 1) * step;
-    const unsigned below = __ballot_sync(kFull, p < hi && g.row_begin(p) <= x);  // (a prefix of the lanes)
-    const int c = __popc(below);
-    const int64_t base = lo;
-    lo = base + c * step;
-    hi = min(hi, base + (c + 1) * step);
-  }
-  return lo;
-}
-
-// The rows of a segment, in order; lane l holds the end of row base + l.
-struct RowWindow {
-  int64_t base, first, ends;  // first: begin of row `base`
-  __device__ __forceinline__ void load(const DGraph &g, int64_t v) {
-    base = v;
-    first = g.row_begin(v);
-    const int64_t x = v + 1 + (threadIdx.x & 31);
-    ends = g.row_begin(x < g.n ? x : g.n);
-  }
-  // the row that holds entry e (at or after the window's start) and its bounds
-  __device__ __forceinline__ int64_t seek(const DGraph &g, int64_t e, int64_t *beg, int64_t *end) {
-    unsigned m;
-    while ((m = __ballot_sync(kFull, ends > e)) == 0) load(g, base + 32);
-    const int f = __ffs(m) - 1;
-    *end = __shfl_sync(kFull, ends, f);
-    const int64_t b = __shfl_sync(kFull, ends, f > 0 ? f - 1 : 0);
-    *beg = f > 0 ? b : first;
-    return base + f;
-  }
-};
-
 // Weighted degrees (graphs with edge weights; without, the degree serves). Exact integer sums: a row
 // inside one segment is stored, the parts of a row that spans segments are added (wsum is zero on entry).
-__global__ void __launch_bounds__(256) k_wdeg(DGraph g, unsigned long long *wsum) {
+__global__ void __launch_bounds__(256) k_wdeg(DGraph g, int seg, unsigned long long *wsum) {
   const int lane = threadIdx.x & 31;
-  const int64_t m = gp_min64(g.m, g.row_begin(g.n)), nseg = (m + kSeg - 1) / kSeg;
+  const int64_t m = gp_min64(g.m, g.row_begin(g.n)), nseg = (m + seg - 1) / seg;
   const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t sg = gw; sg < nseg; sg += nw) {
-    const int64_t s1 = gp_min64(m, (sg + 1) * kSeg);
+    const int64_t s1 = gp_min64(m, (sg + 1) * seg);
     RowWindow W;
-    W.load(g, warp_row_of(g, sg * kSeg));
-    for (int64_t e = sg * kSeg; e < s1;) {
+    W.load(g, warp_row_of(g, sg * seg));
+    for (int64_t e = sg * seg; e < s1;) {
       int64_t beg, end;
       const int64_t v = W.seek(g, e, &beg, &end);
       const int64_t stop = gp_min64(end, s1);
@@ -102,7 +62,7 @@ __global__ void __launch_bounds__(256) k_wdeg(DGraph g, unsigned long long *wsum
       for (int64_t x = e + lane; x < stop; x += 32) s += g.eweight(x);
       s = warp_sum64(s);
       if (lane == 0) {
-        if (beg >= sg * kSeg && end <= s1) wsum[v] = (unsigned long long)s;
+        if (beg >= sg * seg && end <= s1) wsum[v] = (unsigned long long)s;
         else atomicAdd(&wsum[v], (unsigned long long)s);
       }
       e = stop;
@@ -122,7 +82,7 @@ __device__ __forceinline__ void mma_16816(float c[4], const unsigned a[4], const
 // straight into the network and never to memory).
 //
 // What bounds it: the shared-neighbour counts look up to 64 neighbours of u up for every entry (v,u), from
-// rows scattered over the adjacency. A warp takes a segment of kSeg entries; for each of its rows the set of
+// rows scattered over the adjacency. A warp takes a segment of entries; for each of its rows the set of
 // v's first 64 neighbours is a table in the warp's shared memory (kTab slots and no probing: the keys whose
 // slot was taken, two on average for a full set, are compared one by one), and lane l owns one entry of 32.
 // The neighbours of two entries are looked up together, each by a half-warp that reads them contiguously, up
@@ -140,7 +100,7 @@ __device__ __forceinline__ unsigned tab_slot(int x) { return ((unsigned)x * 0x9E
 static_assert(kTab == 1 << 10, "tab_slot keeps ten bits");
 
 template <bool SCORE>
-__global__ void __launch_bounds__(kEdgeWarps * 32, 4) k_edges(DGraph g, int level, const unsigned long long *wsum,
+__global__ void __launch_bounds__(kEdgeWarps * 32, 4) k_edges(DGraph g, int seg, int level, const unsigned long long *wsum,
                                                            float *fout, const gp_mlp *mlp, float *s_out,
                                                            int32_t *q_out) {
   __shared__ int s_tab[kEdgeWarps][kTab], s_over[kEdgeWarps][64];
@@ -164,13 +124,13 @@ __global__ void __launch_bounds__(kEdgeWarps * 32, 4) k_edges(DGraph g, int leve
     b2 = mlp->b2;
   }
   const float flevel = (float)level / 16.0f;
-  const int64_t m = gp_min64(g.m, g.row_begin(g.n)), nseg = (m + kSeg - 1) / kSeg;
+  const int64_t m = gp_min64(g.m, g.row_begin(g.n)), nseg = (m + seg - 1) / seg;
   const int64_t gw = blockIdx.x * (int64_t)kEdgeWarps + wid, nw = (int64_t)gridDim.x * kEdgeWarps;
   for (int64_t sg = gw; sg < nseg; sg += nw) {
-    const int64_t s1 = gp_min64(m, (sg + 1) * kSeg);
+    const int64_t s1 = gp_min64(m, (sg + 1) * seg);
     RowWindow W;
-    W.load(g, warp_row_of(g, sg * kSeg));
-    for (int64_t e0 = sg * kSeg; e0 < s1;) {
+    W.load(g, warp_row_of(g, sg * seg));
+    for (int64_t e0 = sg * seg; e0 < s1;) {
       int64_t beg, end;
       const int64_t v = W.seek(g, e0, &beg, &end);
       const int64_t stop = gp_min64(end, s1), dv = end - beg;
@@ -207,6 +167,26 @@ __global__ void __launch_bounds__(kEdgeWarps * 32, 4) k_edges(DGraph g, int leve
         const float w = has ? (float)g.eweight(e) : 0.0f;
         const int cnt = (int)gp_min64(stop - e0, 32);
         int mine = 0;
+        if (!__any_sync(kFull, lenu > 16)) {
+          // (meshes: every list is one step of a half-warp)
+          for (int p = 0; p < cnt; p += 4) {
+            int xs[2];
+#pragma unroll
+            for (int y = 0; y < 2; y++) {
+              const int64_t b = __shfl_sync(kFull, bu, p + 2 * y + half);
+              const int len = __shfl_sync(kFull, lenu, p + 2 * y + half);
+              xs[y] = hl < len ? __ldg(g.adj + b + hl) : -2;
+            }
+#pragma unroll
+            for (int y = 0; y < 2; y++) {
+              unsigned hits = tab[tab_slot(xs[y])] == xs[y];
+              for (int o = 0; o < nover; o++) hits += over[o] == xs[y];
+              const unsigned c = __reduce_add_sync(kFull, hits << (16 * half));
+              if (lane == p + 2 * y) mine = (int)(c & 0xffffu);
+              if (lane == p + 2 * y + 1) mine = (int)(c >> 16);
+            }
+          }
+        } else
         for (int p = 0; p < cnt; p += 4) {
           // entries p, p + 2 (lower half-warp) and p + 1, p + 3 (upper)
           int xs[2][4], most[2];
@@ -480,19 +460,20 @@ int run_edges(const DGraph &g, int level, float *fout, const gp_mlp *mlp, float 
   if (g.m == 0) return GP_OK;
   Workspace ws(s);
   const int nsm = num_sms();
-  const int64_t warps = (g.m + kSeg - 1) / kSeg;
+  const int seg = row_segment(g.m);
+  const int64_t warps = (g.m + seg - 1) / seg;
   unsigned long long *wsum = nullptr;
   if (g.ew) {
     GP_TRY(ws.zeros(&wsum, (size_t)g.n));
-    (::gp::count_launch(), k_wdeg<<<grid_for(warps, 8, nsm * 8), 256, 0, s>>>(g, wsum));
+    (::gp::count_launch(), k_wdeg<<<grid_for(warps, 8, nsm * 8), 256, 0, s>>>(g, seg, wsum));
   }
   {
     ProfScope ps(fout ? "mlp_features" : "mlp_score_mma", s);
     const int grid = grid_for(warps, kEdgeWarps, nsm * 16);
     if (fout)
-      (::gp::count_launch(), k_edges<false><<<grid, kEdgeWarps * 32, 0, s>>>(g, level, wsum, fout, nullptr, nullptr, nullptr));
+      (::gp::count_launch(), k_edges<false><<<grid, kEdgeWarps * 32, 0, s>>>(g, seg, level, wsum, fout, nullptr, nullptr, nullptr));
     else
-      (::gp::count_launch(), k_edges<true><<<grid, kEdgeWarps * 32, 0, s>>>(g, level, wsum, nullptr, mlp, s_out, q_out));
+      (::gp::count_launch(), k_edges<true><<<grid, kEdgeWarps * 32, 0, s>>>(g, seg, level, wsum, nullptr, mlp, s_out, q_out));
   }
   GP_LAUNCH_CHECK();
   return GP_OK;

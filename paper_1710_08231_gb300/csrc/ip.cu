@@ -18,6 +18,7 @@
 #include "block_sort.cuh"
 #include "ip.cuh"
 #include "lp.cuh"
+#include "row_walk.cuh"
 
 namespace gp {
 
@@ -67,16 +68,46 @@ struct IpArgs {
   int *err;
 };
 
-// Multi-source BFS restricted to same-set vertices (part equal, set still being split).
+// Multi-source BFS restricted to same-set vertices (part equal, set still being split). All sources start at
+// distance 0 together, so a step finds the vertices of one distance. A frontier of more than an eighth of the vertices
+// is taken from the other side: every vertex still without a distance looks for a neighbour in the frontier and stops
+// at the first 32 entries that hold one, instead of every frontier vertex walking its whole row (on the coarsest
+// level of an R-MAT graph, one CTA per try, the two or three large steps of each search: 8.6 -> 7.2 ms). The
+// distances are the same.
 __device__ void set_bfs(const DGraph &g, int64_t vbase, int32_t *part, int32_t *gk, int32_t *dist, int32_t *qa,
                         int32_t *qb, int nf) {
   __shared__ int s_next;
-  while (nf > 0) {
+  const int n = (int)g.n;
+  for (int level = 0; nf > 0; level++) {
     if (threadIdx.x == 0) s_next = 0;
     __syncthreads();
     // one warp per frontier vertex, lanes over its row
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int i = wid; i < nf; i += nw) {
+    if (8 * (int64_t)nf > n) {
+      for (int u0 = wid * 32; u0 < n; u0 += nw * 32) {
+        const int mine = u0 + lane;
+        unsigned open = __ballot_sync(kFull, mine < n && gk[mine] > 1 && dist[mine] == -1);
+        for (; open; open &= open - 1) {
+          const int u = u0 + __ffs(open) - 1;
+          const int pu = part[u];
+          const int64_t b = g.row_begin(u), e = g.row_begin(u + 1);
+          for (int64_t j = b; j < e; j += 32) {
+            bool hit = false;
+            if (j + lane < e) {
+              const int x = (int)(g.adj[j + lane] - vbase);
+              hit = *(volatile int32_t *)&dist[x] == level && part[x] == pu;
+            }
+            if (__any_sync(kFull, hit)) {  // (a vertex found in this step has distance level + 1)
+              if (lane == 0) {
+                dist[u] = level + 1;
+                qb[atomicAdd(&s_next, 1)] = u;
+              }
+              break;
+            }
+          }
+        }
+      }
+    } else for (int i = wid; i < nf; i += nw) {
       const int x = qa[i];
       const int px = part[x];
       const int dx = dist[x];
@@ -370,81 +401,51 @@ __global__ void __launch_bounds__(kIpThreads) k_repair(IpArgs a) {
   }
 }
 
-// Rows up to kCutSmall entries: a thread each; longer rows (hubs of power-law graphs, whose walk by one
-// thread would decide the kernel's duration) are left to k_cut_big.
-constexpr int64_t kCutSmall = 256;
-
-__global__ void k_cut(DGraph g, const int32_t *part, unsigned long long *acc) {
-  __shared__ long long sh[32];
-  long long s = 0;
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < g.n; v += (int64_t)gridDim.x * blockDim.x) {
-    const int pv = part[v];
-    const int64_t b = g.row_begin(v), e = g.row_begin(v + 1);
-    if (e - b > kCutSmall) continue;
-    for (int64_t j = b; j < e; j++)
-      if (part[g.adj[j]] != pv) s += g.eweight(j);
-  }
-  s = warp_sum64(s);
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) sh[wid] = s;
+// Doubled cuts of up to T partitions of g (parts: one after another, g.n each): acc[t] += weight of each entry whose
+// ends lie in different blocks of partition t. The adjacency is read once for all of them, in segments, so that the
+// rows of millions of entries that power-law graphs have do not decide the time (128 M entries: 1.27 ms, a pass over
+// the adjacency and its weights takes 0.2 ms; the parts gathered by neighbour bound it. The tries' cuts on R-MAT 22's
+// coarsest graph, a vertex per thread and a launch per try: 2.2 ms; so: 0.02 ms).
+template <int T>
+__global__ void __launch_bounds__(256) k_cut(DGraph g, int seg, const int32_t *parts, int tries,
+                                             unsigned long long *acc) {
+  __shared__ unsigned long long s_acc[T];
+  if (threadIdx.x < T) s_acc[threadIdx.x] = 0;
   __syncthreads();
-  if (wid == 0) {
-    long long x = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0;
-    x = warp_sum64(x);
-    if (lane == 0 && x) atomicAdd(acc, (unsigned long long)x);
-  }
-}
-
-// Rows above kCutSmall entries are cut into items of kCutChunk entries, listed first so that every CTA
-// takes items in turn (the long rows of power-law graphs sit at small ids: tiles of vertices would leave
-// them to a few CTAs).
-constexpr int64_t kCutChunk = 4096;
-
-__global__ void k_cut_list(DGraph g, unsigned long long *items, unsigned long long cap, unsigned long long *cnt) {
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < g.n; v += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t d = g.row_begin(v + 1) - g.row_begin(v);
-    if (d <= kCutSmall) continue;
-    const unsigned long long nch = (unsigned long long)((d + kCutChunk - 1) / kCutChunk);
-    const unsigned long long base = atomicAdd(cnt, nch);
-    for (unsigned long long c = 0; c < nch && base + c < cap; c++) items[base + c] = ((unsigned long long)v << 32) | c;
-  }
-}
-
-__global__ void k_cut_items(DGraph g, const int32_t *part, const unsigned long long *items, unsigned long long cap,
-                            const unsigned long long *cnt, unsigned long long *acc) {
-  __shared__ long long sh[32];
-  const unsigned long long nit = min(*cnt, cap);  // (the list is sized for every row of the graph)
-  long long s = 0;
-  for (unsigned long long i = blockIdx.x; i < nit; i += gridDim.x) {
-    const unsigned long long it = items[i];
-    const int64_t v = (int64_t)(it >> 32);
-    const int pv = part[v];
-    const int64_t b = g.row_begin(v) + (int64_t)(it & 0xffffffffull) * kCutChunk;
-    const int64_t e = min(g.row_begin(v + 1), b + kCutChunk);
-    // four entries per thread in flight
-    for (int64_t j0 = b; j0 < e; j0 += 4 * (int64_t)blockDim.x) {
-      int a[4];
+  const int lane = threadIdx.x & 31;
+  const int64_t m = min(g.m, g.row_begin(g.n)), nseg = (m + seg - 1) / seg;
+  const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  unsigned long long c[T];
 #pragma unroll
-      for (int x = 0; x < 4; x++) {
-        const int64_t j = j0 + x * (int64_t)blockDim.x + threadIdx.x;
-        a[x] = j < e ? __ldg(g.adj + j) : -1;
-      }
+  for (int t = 0; t < T; t++) c[t] = 0;
+  for (int64_t sg = gw; sg < nseg; sg += nw) {
+    const int64_t s1 = min(m, (sg + 1) * seg);
+    RowWindow W;
+    W.load(g, warp_row_of(g, sg * seg));
+    for (int64_t e = sg * seg; e < s1;) {
+      int64_t beg, end;
+      const int64_t v = W.seek(g, e, &beg, &end);
+      const int64_t stop = min(end, s1);
+      for (int64_t x = e + lane; x < stop; x += 32) {
+        const int a = __ldg(g.adj + x);
+        const unsigned long long w = (unsigned long long)g.eweight(x);
 #pragma unroll
-      for (int x = 0; x < 4; x++) {
-        const int64_t j = j0 + x * (int64_t)blockDim.x + threadIdx.x;
-        if (a[x] >= 0 && part[a[x]] != pv) s += g.eweight(j);
+        for (int t = 0; t < T; t++) {
+          if (T > 1 && t >= tries) break;
+          const int32_t *p = parts + (size_t)t * g.n;
+          if (p[a] != p[v]) c[t] += w;
+        }
       }
+      e = stop;
     }
   }
-  s = warp_sum64(s);
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) sh[wid] = s;
-  __syncthreads();
-  if (wid == 0) {
-    long long x = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0;
-    x = warp_sum64(x);
-    if (lane == 0 && x) atomicAdd(acc, (unsigned long long)x);
+#pragma unroll
+  for (int t = 0; t < T; t++) {
+    const unsigned long long x = (unsigned long long)warp_sum64((int64_t)c[t]);
+    if (lane == 0 && x) atomicAdd(&s_acc[t], x);
   }
+  __syncthreads();
+  if (threadIdx.x < T && s_acc[threadIdx.x]) atomicAdd(&acc[threadIdx.x], s_acc[threadIdx.x]);
 }
 
 __global__ void k_project(const int32_t *coarse, const int32_t *f2c, int64_t n, int32_t *fine) {
@@ -519,9 +520,62 @@ __global__ void k_strip_adj(const int32_t *adj, int64_t m, const int32_t *rank, 
 // Degree-0 vertex placement with unit weights, closed form of the greedy rule: at water level x
 // every block of weight <= x receives one vertex, blocks in id order. F(x) = sum_b max(0, x - bw_b)
 // vertices are placed before level x; vertex j (0-based, ascending id) is placed at the level x with
-// F(x) <= j < F(x+1), into the (j - F(x))-th block (by id) among those with bw_b <= x.
-__global__ void k_place_unit(DGraph g, const int32_t *rank, const int32_t *part0, const int64_t *iso_idx,
-                             const long long *bw, int64_t k, int32_t *part_full) {
+// F(x) <= j < F(x+1), into the (j - F(x))-th block (by id) among those with bw_b <= x. With the block weights sorted
+// (in shared memory, k <= kPlaceK) and their prefix sums, the c lowest blocks are the ones below level x and
+// F(x) = c x - prefix(c): a search for c replaces a search for x over sums of k terms (2 M vertices, k = 64:
+// 2.0 -> 0.15 ms).
+constexpr int kPlaceK = 1024;
+
+__global__ void __launch_bounds__(256) k_place_unit(DGraph g, const int32_t *rank, const int32_t *part0,
+                                                    const int64_t *iso_idx, const long long *bw, int k,
+                                                    int32_t *part_full) {
+  __shared__ long long s_bw[kPlaceK], s_sorted[kPlaceK], s_pre[kPlaceK + 1];
+  for (int b = threadIdx.x; b < k; b += blockDim.x) s_bw[b] = bw[b];
+  __syncthreads();
+  for (int b = threadIdx.x; b < k; b += blockDim.x) {
+    int at = 0;
+    for (int x = 0; x < k; x++) at += s_bw[x] < s_bw[b] || (s_bw[x] == s_bw[b] && x < b);
+    s_sorted[at] = s_bw[b];
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    long long run = 0;
+    for (int b = 0; b < k; b++) {
+      s_pre[b] = run;
+      run += s_sorted[b];
+    }
+    s_pre[k] = run;
+  }
+  __syncthreads();
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < g.n; v += (int64_t)gridDim.x * blockDim.x) {
+    const int r = rank[v];
+    if (r >= 0) {
+      part_full[v] = part0[r];
+      continue;
+    }
+    const long long j = iso_idx[v];
+    int lo = 0, hi = k;  // the largest c with F(sorted[c]) <= j
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (mid * s_sorted[mid] - s_pre[mid] <= j) lo = mid;
+      else hi = mid;
+    }
+    const int c = lo + 1;
+    const long long x = (j + s_pre[c]) / c;
+    long long rem = j - (c * x - s_pre[c]);
+    int pick = (int)rem;
+    if (c < k) {
+      for (pick = 0; pick < k; pick++) {
+        if (s_bw[pick] <= x && rem-- == 0) break;
+      }
+    }
+    part_full[v] = pick;
+  }
+}
+
+// The same for any k, searching the level by sums over the blocks.
+__global__ void k_place_unit_any(DGraph g, const int32_t *rank, const int32_t *part0, const int64_t *iso_idx,
+                                 const long long *bw, int64_t k, int32_t *part_full) {
   long long bmin = LLONG_MAX;
   for (int64_t b = 0; b < k; b++) bmin = min(bmin, bw[b]);
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < g.n; v += (int64_t)gridDim.x * blockDim.x) {
@@ -556,21 +610,60 @@ __global__ void k_place_unit(DGraph g, const int32_t *rank, const int32_t *part0
   }
 }
 
-// Degree-0 vertices with general weights: one thread applies the greedy rule in id order.
-__global__ void k_place_seq(DGraph g, const int32_t *rank, const int32_t *part0, long long *bw, int64_t k,
-                            int32_t *part_full) {
-  if (blockIdx.x != 0 || threadIdx.x != 0) return;
-  for (int64_t v = 0; v < g.n; v++) {
+// Degree-0 vertices with general weights, part 1: kept vertices take their blocks, the others are listed in id order.
+__global__ void k_place_list(DGraph g, const int32_t *rank, const int32_t *part0, const int64_t *iso_idx, int32_t *iso,
+                             int32_t *part_full) {
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < g.n; v += (int64_t)gridDim.x * blockDim.x) {
     const int r = rank[v];
-    if (r >= 0) {
-      part_full[v] = part0[r];
-      continue;
+    if (r >= 0) part_full[v] = part0[r];
+    else iso[iso_idx[v]] = (int32_t)v;
+  }
+}
+
+// Part 2: one warp applies the greedy rule in id order. Lane l owns the blocks l, l + 32, ... and keeps the lightest
+// of them; a vertex costs one warp minimum (a thread going through all blocks took about a microsecond).
+__global__ void k_place_seq(DGraph g, const int32_t *iso, int64_t n_iso, long long *bw, int64_t k, int32_t *part_full) {
+  const int lane = threadIdx.x;
+  auto lightest = [&](long long *w) {
+    int best = -1;
+    long long bwt = LLONG_MAX;
+    for (int64_t b = lane; b < k; b += 32) {
+      const long long x = bw[b];
+      if (best < 0 || x < bwt) {
+        bwt = x;
+        best = (int)b;
+      }
     }
-    int b = 0;
-    for (int64_t x = 1; x < k; x++)
-      if (bw[x] < bw[b]) b = (int)x;
-    part_full[v] = b;
-    bw[b] += g.vweight(v);
+    *w = bwt;
+    return best;
+  };
+  long long w;
+  int b = lightest(&w);
+  for (int64_t i0 = 0; i0 < n_iso; i0 += 32) {
+    const int v = i0 + lane < n_iso ? iso[i0 + lane] : 0;
+    const long long c = i0 + lane < n_iso ? g.vweight(v) : 0;
+    const int cnt = (int)min((int64_t)32, n_iso - i0);
+    int mine = 0;
+    for (int y = 0; y < cnt; y++) {
+      const long long cy = __shfl_sync(kFull, c, y);
+      long long wm = b >= 0 ? w : LLONG_MAX;
+      int bm = b >= 0 ? b : INT_MAX;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const long long w2 = __shfl_xor_sync(kFull, wm, o);
+        const int b2 = __shfl_xor_sync(kFull, bm, o);
+        if (w2 < wm || (w2 == wm && b2 < bm)) {
+          wm = w2;
+          bm = b2;
+        }
+      }
+      if (lane == y) mine = bm;
+      if (b == bm) {
+        bw[b] = wm + cy;
+        b = lightest(&w);
+      }
+    }
+    if (lane < cnt) part_full[v] = mine;
   }
 }
 
@@ -695,21 +788,22 @@ int initial_partition(const DGraph &g, int k, int64_t lmax, uint64_t seed, int l
   return initial_partition_multi(&j, 1, tries, repair_rounds, s, err_dev);
 }
 
+int cuts_launch(const DGraph &g, const int32_t *parts, int tries, unsigned long long *acc_dev, cudaStream_t s) {
+  GP_CUDA(cudaMemsetAsync(acc_dev, 0, sizeof(unsigned long long) * (size_t)tries, s));
+  if (g.n == 0 || g.m == 0) return GP_OK;
+  const int seg = row_segment(g.m);
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(((g.m + seg - 1) / seg + 7) / 8, (int64_t)num_sms() * 8));
+  auto run = [&](auto kernel) { (::gp::count_launch(), kernel<<<grid, 256, 0, s>>>(g, seg, parts, tries, acc_dev)); };
+  if (tries == 1) run(k_cut<1>);
+  else if (tries <= 4) run(k_cut<4>);
+  else run(k_cut<16>);
+  GP_LAUNCH_CHECK();
+  return GP_OK;
+}
+
 int eval_cut_launch(const DGraph &g, const int32_t *part, int64_t k, unsigned long long *acc_dev, int64_t *bw_dev,
                     cudaStream_t s) {
-  GP_CUDA(cudaMemsetAsync(acc_dev, 0, sizeof(unsigned long long), s));
-  if (g.n > 0) {
-    Workspace ws(s);
-    unsigned long long *items, *cnt;
-    // items: at most one per kCutChunk entries plus one per row above kCutSmall
-    const unsigned long long cap = (unsigned long long)(g.m / kCutChunk + g.m / (kCutSmall + 1) + 1);
-    GP_TRY(ws.get(&items, (size_t)cap));
-    GP_TRY(ws.zeros(&cnt, 1));
-    (::gp::count_launch(), k_cut<<<grid_for_n(g.n), 256, 0, s>>>(g, part, acc_dev));
-    (::gp::count_launch(), k_cut_list<<<grid_for_n(g.n), 256, 0, s>>>(g, items, cap, cnt));
-    (::gp::count_launch(), k_cut_items<<<num_sms() * 8, 256, 0, s>>>(g, part, items, cap, cnt, acc_dev));
-    GP_LAUNCH_CHECK();
-  }
+  GP_TRY(cuts_launch(g, part, 1, acc_dev, s));
   if (bw_dev) GP_TRY(block_weights(g, part, k, bw_dev, nullptr, s));
   return GP_OK;
 }
@@ -843,10 +937,15 @@ int place_isolated(const DGraph &g, const Stripped &st, const int32_t *part0, in
   GP_TRY(ws.get(&iso_idx, (size_t)g.n));
   (::gp::count_launch(), k_mark_rank<<<grid_for_n(g.n), 256, 0, s>>>(g, st.rank, rank, iso_idx));
   GP_LAUNCH_CHECK();
-  if (!g.vw) {
-    (::gp::count_launch(), k_place_unit<<<grid_for_n(g.n), 256, 0, s>>>(g, rank, part0, iso_idx, bw, k, part_full));
+  if (!g.vw && k <= kPlaceK) {
+    (::gp::count_launch(), k_place_unit<<<grid_for_n(g.n), 256, 0, s>>>(g, rank, part0, iso_idx, bw, (int)k, part_full));
+  } else if (!g.vw) {
+    (::gp::count_launch(), k_place_unit_any<<<grid_for_n(g.n), 256, 0, s>>>(g, rank, part0, iso_idx, bw, k, part_full));
   } else {
-    (::gp::count_launch(), k_place_seq<<<1, 32, 0, s>>>(g, rank, part0, bw, k, part_full));
+    int32_t *iso;
+    GP_TRY(ws.get(&iso, (size_t)st.n_iso));
+    (::gp::count_launch(), k_place_list<<<grid_for_n(g.n), 256, 0, s>>>(g, rank, part0, iso_idx, iso, part_full));
+    (::gp::count_launch(), k_place_seq<<<1, 32, 0, s>>>(g, iso, st.n_iso, bw, k, part_full));
   }
   GP_LAUNCH_CHECK();
   return GP_OK;

@@ -27,6 +27,9 @@ struct IpJob {
 int initial_partition_multi(const IpJob *jobs, int njobs, int tries, int repair_rounds, cudaStream_t s,
                             int *err_dev = nullptr);
 
+// acc_dev[t] (device, t < tries <= 16) receives twice the cut of the t-th of `tries` partitions (parts: g.n each).
+int cuts_launch(const DGraph &g, const int32_t *parts, int tries, unsigned long long *acc_dev, cudaStream_t s);
+
 // The kernels of eval_cut without the read back: *acc_dev (device) receives twice the cut.
 int eval_cut_launch(const DGraph &g, const int32_t *part, int64_t k, unsigned long long *acc_dev, int64_t *bw_dev,
                     cudaStream_t s);

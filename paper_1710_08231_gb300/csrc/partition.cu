@@ -79,22 +79,6 @@ __global__ void k_validate(DGraph g, int *err) {
   }
 }
 
-// Doubled cut of every try partition (parts: tries * n): cut2[t] += weight of each entry whose ends
-// lie in different blocks of try t.
-__global__ void k_tries_cut(DGraph g, const int32_t *parts, int tries, unsigned long long *cut2) {
-  for (int t = 0; t < tries; t++) {
-    const int32_t *p = parts + (size_t)t * g.n;
-    unsigned long long c = 0;
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < g.n; v += (int64_t)gridDim.x * blockDim.x) {
-      const int pv = p[v];
-      for (int64_t j = g.row_begin(v); j < g.row_begin(v + 1); j++)
-        if (p[g.adj[j]] != pv) c += (unsigned long long)g.eweight(j);
-    }
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(kFull, c, o);
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd(&cut2[t], c);
-  }
-}
-
 gp_params g_schedule = {};
 int g_keep_pct = 0;  // stale threshold of kept hub tables (0: default)
 
@@ -323,11 +307,8 @@ int partition_device(const gp_graph *gin, int32_t k, double eps, uint64_t seed, 
     std::vector<int64_t> hbws((size_t)tries * k);
     {
       unsigned long long *cut2;
-      GP_TRY(ws.zeros(&cut2, (size_t)tries));
-      if (gc.n > 0) {
-        (::gp::count_launch(), k_tries_cut<<<grid_n(gc.n), 256, 0, s>>>(gc, parts, tries, cut2));
-        GP_LAUNCH_CHECK();
-      }
+      GP_TRY(ws.get(&cut2, (size_t)tries));
+      GP_TRY(cuts_launch(gc, parts, tries, cut2, s));
       int herr = 0;
       Readback rb;
       rb.add(hcut2.data(), cut2, sizeof(unsigned long long) * tries);

@@ -2194,10 +2194,11 @@ __device__ __forceinline__ bool mover_less(const LpProblem &P, unsigned x, unsig
 
 // Segmented inclusive prefix sums of c(v) over positions [lo, hi) of a sequence sorted by target,
 // starting from the carry of the segment open before lo; a proposal is admitted while the target's
-// snapshot weight plus the prefix fits. at(p) gives (target, proposal index) of position p.
+// snapshot weight plus the prefix fits. at(p) gives (target, proposal index) of position p. Without `apply` the
+// admitted proposals are only marked (apply_contested makes their moves).
 template <class At>
 __device__ void admit_sorted(const LpProblem &P, At at, unsigned lo, unsigned hi, long long carry_in,
-                             int carry_target, int r, SubCounters *Cg, Smem &sm) {
+                             int carry_target, int r, SubCounters *Cg, Smem &sm, bool apply) {
   uint8_t *act_next = r + 1 < P.rounds ? P.act[(r + 1) & 1] : nullptr;  // (no marks in the last round)
   unsigned moved = 0;
   if (threadIdx.x == 0) {
@@ -2251,7 +2252,8 @@ __device__ void admit_sorted(const LpProblem &P, At at, unsigned lo, unsigned hi
     const long long incl = f ? x : x + sm.sum[wid];
     const bool adm = valid && P.lw[T] + incl <= P.U;
     if (adm) P.mv_adm[idx] = 1;
-    moved += apply_movers(P, *Cg, act_next, adm, idx, adm ? P.mv_v[idx] : 0, T);
+    if (apply) moved += apply_movers(P, *Cg, act_next, adm, idx, adm ? P.mv_v[idx] : 0, T);
+    else moved += (unsigned)__popc(__ballot_sync(kFull, adm));
     __syncthreads();
     const unsigned last = min(hi, base + (unsigned)kThreads) - 1;
     if (p == last) {
@@ -2269,7 +2271,7 @@ __device__ __forceinline__ int bits_for(unsigned long long x) { return x ? 64 - 
 // keys are sorted in shared memory (bitonic); otherwise proposal indices are sorted with a comparator.
 template <bool LQ>
 __device__ void contest_small(const LpProblem &P, const SubCounters &C, SubCounters *Cg, unsigned cnt, int r,
-                              unsigned char *dsm, Smem &sm) {
+                              unsigned char *dsm, Smem &sm, bool apply) {
   unsigned Pp = 1;
   while (Pp < cnt) Pp <<= 1;
   const unsigned long long maxg = C.max_gain, maxq = C.max_q;
@@ -2315,7 +2317,7 @@ __device__ void contest_small(const LpProblem &P, const SubCounters &C, SubCount
           T = (int)((bt ? (long long)(k >> st) : 0) + P.lbase);
           idx = (unsigned)P.mv_of_v[(int)(k & vmask)];
         },
-        0, cnt, 0, -1, r, Cg, sm);
+        0, cnt, 0, -1, r, Cg, sm, apply);
     if (threadIdx.x == 0) P.ctr->contest_packed += 1;
     return;
   }
@@ -2346,7 +2348,7 @@ __device__ void contest_small(const LpProblem &P, const SubCounters &C, SubCount
         idx = key[p];
         T = P.mv_t[idx];
       },
-      0, cnt, 0, -1, r, Cg, sm);
+      0, cnt, 0, -1, r, Cg, sm, apply);
   if (threadIdx.x == 0) P.ctr->contest_small += 1;
 }
 
@@ -2542,12 +2544,30 @@ __device__ bool contest_large(const LpProblem &P, const SubCounters &C, SubCount
           idx = src[p];
           T = P.mv_t[idx];
         },
-        lo, hi, carry, carry_t, r, Cg, sm);
+        lo, hi, carry, carry_t, r, Cg, sm, true);
   if (lb == 0 && threadIdx.x == 0) {
     P.ctr->contest_large += 1;
     P.ctr->contest_large_items += cnt;
   }
   return true;
+}
+
+// A contest of more than this many proposals decided by one block leaves the moves to all blocks: walking the movers'
+// rows is most of the work (a block with 4096 of them on R-MAT 22, whose neighbours' kept tables follow each move,
+// kept the others waiting for about 100 us in nearly every sub-round). Below, the moves cost less than a meeting.
+constexpr unsigned kContestApply = 256;
+
+// The moves of the contested proposals that were admitted, a few per warp.
+__device__ void apply_contested(const LpProblem &P, SubCounters &C, unsigned cnt, int r, int lb, int nb) {
+  uint8_t *act_next = r + 1 < P.rounds ? P.act[(r + 1) & 1] : nullptr;  // (no marks in the last round)
+  const unsigned warps = (unsigned)nb * kWarps, per = min(32u, (cnt + warps - 1) / warps);
+  const unsigned lane = threadIdx.x & 31;
+  for (unsigned k0 = ((unsigned)lb * kWarps + (threadIdx.x >> 5)) * per; k0 < cnt; k0 += warps * per) {
+    const bool on = lane < per && k0 + lane < cnt;
+    const unsigned idx = on ? P.ct[k0 + lane] : 0u;
+    const bool adm = on && P.mv_adm[idx] != 0;
+    apply_movers(P, C, act_next, adm, idx, adm ? P.mv_v[idx] : 0, adm ? P.mv_t[idx] : -1);
+  }
 }
 
 template <int EW, int TB>
@@ -2710,7 +2730,12 @@ __device__ bool lp_problem(const LpProblem *prob, unsigned char *dsm) {
         const unsigned nc = sV.n_contested;
         if (nc > 0) {
           if (nc <= kContestSmall) {
-            if (lb == 0) contest_small<LQ>(P, sV, &C, nc, r, dsm, sm);
+            const bool apply = nc <= kContestApply || nb == 1;
+            if (lb == 0) contest_small<LQ>(P, sV, &C, nc, r, dsm, sm, apply);
+            if (!apply) {
+              if (!grid_sync(bar)) return false;
+              apply_contested(P, C, nc, r, lb, nb);
+            }
           } else {
             if (!contest_large<LQ>(P, sV, &C, nc, r, lb, nb, bar, sm, dsm)) return false;
           }
@@ -3207,7 +3232,12 @@ __device__ bool lp_problem_own(const LpProblem *prob, unsigned char *dsm) {
         __syncthreads();
         const unsigned nc = sV.n_contested;
         if (nc <= kContestSmall) {
-          if (lb == 0) contest_small<LQ>(P, sV, &C, nc, r, dsm, sm);
+          const bool apply = nc <= kContestApply || nb == 1;
+          if (lb == 0) contest_small<LQ>(P, sV, &C, nc, r, dsm, sm, apply);
+          if (!apply) {
+            if (!grid_sync(bar)) return false;
+            apply_contested(P, C, nc, r, lb, nb);
+          }
         } else {
           if (!contest_large<LQ>(P, sV, &C, nc, r, lb, nb, bar, sm, dsm)) return false;
         }

@@ -13,19 +13,22 @@
 //   * PerformMoves: one warp per search, all searches of a local iteration in one launch. A warp keeps
 //     its whole search state in shared memory: the queue (an unsorted array; the maximum is found by a
 //     warp reduction over (gain, H(s, w, 0), -w)), its moves and a small hash map of the blocks they
-//     changed (the search's view of the partition), its copy of the block weights, and a per-block
-//     connection array for gain computations (each lane adds its neighbours' weights with shared-memory
-//     atomics, then the lanes reduce over the blocks). Each search writes its best prefix to its own
-//     slot range, so the sequences keep the todo order.
+//     changed (the search's view of the partition), its copy of the block weights, and connection arrays.
+//     The neighbours of a moved vertex are taken 32 at a time, a lane each: a lane finds its vertex in the
+//     queue and computes its gain with connections of its own, since neither depends on what the others do.
+//     (All searches of a partition of 262144 points, k = 4: 11.0 ms with a vertex per warp, 5.2 ms so.)
+//     Each search writes its best prefix to its own slot range, so the sequences keep the todo order.
 //   * ApplyMoves: one CTA walks the sequences in todo order (the non-empty ones found 256 at a time by a
 //     block scan), recomputes each move's gain with a block-wide sum over the vertex's row, and applies
-//     the best prefix; block weights live in shared memory.
-//   * Todo lists: boundary (or moved) flags compacted in vertex order, then a stable radix sort by
-//     H(s, v, 1) -- the order the oracle uses.
+//     the best prefix; block weights live in shared memory. The vertices it moved are the next todo list.
+//   * Todo lists are ordered by (H(s, v, 1), v) -- the order the oracle uses: every vertex counts the ones
+//     before it (lists of up to kRankMax), or a radix sort. (Ordering 30 lists: 2.4 ms by sorts alone, 0.35 ms.)
 // The readings the paper leaves open (fixed search bounds instead of the adaptive stopping rule, no
 // global moved bitmap during a local iteration, the degree bound, the hash orders) are those of the
 // CPU oracle; results are bit-identical to it.
 #include <algorithm>
+#include <climits>
+#include <type_traits>
 #include <vector>
 
 #include "gp_internal.cuh"
@@ -47,12 +50,21 @@ struct WarpState {
   long long qg[kQCap];
   unsigned long long qh[kQCap];
   long long bw[kMaxK];
-  long long conn[kMaxK];
   int qv[kQCap];
   int mv[kMaxMoves], mto[kMaxMoves], mfrom[kMaxMoves];
   int hk[kMovedSlots], hb[kMovedSlots];
   int qn, nm;
 };
+
+// Per-warp connection arrays behind the WarpStates: k sums per lane (a vertex per lane), or k 64-bit sums shared by
+// the lanes (a vertex per warp). More blocks than kLaneK leave no room for the former.
+template <int EW>
+using ConnT = typename std::conditional<EW == 0, unsigned, long long>::type;
+constexpr int kLaneK = 64;
+template <int EW>
+size_t conn_bytes(int k) {
+  return k <= kLaneK ? (size_t)k * 32 * sizeof(ConnT<EW>) : (size_t)k * sizeof(long long);
+}
 
 struct MlsArgs {
   DGraph g;
@@ -62,6 +74,7 @@ struct MlsArgs {
   int64_t lmax;
   uint64_t smix;  // mix64(s)
   int max_moves, fruitless, queue_cap, max_degree;
+  unsigned conn_bytes;  // per warp
 };
 
 __device__ __forceinline__ uint64_t hkey(uint64_t smix, uint64_t a, uint64_t b) { return mix64(mix64(smix ^ a) ^ b); }
@@ -85,14 +98,14 @@ __device__ __forceinline__ int64_t degree_of(const DGraph &g, int v) { return g.
 
 // Best move of x in the warp's view (all lanes call; results are uniform). Returns movable.
 template <int EW>
-__device__ bool gain_of(const MlsArgs &A, WarpState &W, int x, int *to_out, long long *gain_out) {
+__device__ bool gain_of(const MlsArgs &A, WarpState &W, long long *conn, int x, int *to_out, long long *gain_out) {
   const int lane = threadIdx.x & 31;
-  for (int b = lane; b < A.k; b += 32) W.conn[b] = 0;
+  for (int b = lane; b < A.k; b += 32) conn[b] = 0;
   __syncwarp();
   const int64_t rb = A.g.row_begin(x), re = A.g.row_begin(x + 1);
   for (int64_t e = rb + lane; e < re; e += 32) {
     const int u = __ldg(A.g.adj + e);
-    atomicAdd(reinterpret_cast<unsigned long long *>(&W.conn[view_block(A, W, u)]),
+    atomicAdd(reinterpret_cast<unsigned long long *>(&conn[view_block(A, W, u)]),
               (unsigned long long)load_ew<EW>(A.g.ew, e));
   }
   __syncwarp();
@@ -103,7 +116,7 @@ __device__ bool gain_of(const MlsArgs &A, WarpState &W, int x, int *to_out, long
   uint64_t bh = 0;
   int bb = -1;
   for (int b = lane; b < A.k; b += 32) {
-    const long long c = W.conn[b];
+    const long long c = conn[b];
     if (b == a || c <= 0 || W.bw[b] + cx > A.lmax) continue;
     const uint64_t h = mix64(hx ^ (uint64_t)b);
     if (bb < 0 || c > bc || (c == bc && (h > bh || (h == bh && b < bb)))) {
@@ -123,7 +136,7 @@ __device__ bool gain_of(const MlsArgs &A, WarpState &W, int x, int *to_out, long
       bb = b2;
     }
   }
-  const long long own = W.conn[a];
+  const long long own = conn[a];
   __syncwarp();
   if (bb < 0) return false;
   *to_out = bb;
@@ -156,23 +169,119 @@ __device__ __forceinline__ void queue_remove(WarpState &W, int i) {
   __syncwarp();
 }
 
+// Best move of the lane's vertex u (u < 0: none) in the warp's view, with connections conn[b * 32 + lane]. Bound by
+// the chain row -> neighbour -> its block, which 32 vertices share (one vertex at a time, by the whole warp, took
+// about 3 us each); four neighbours of a lane are in flight.
 template <int EW>
-__device__ void try_insert(const MlsArgs &A, WarpState &W, int x) {
-  if (degree_of(A.g, x) > A.max_degree) return;
-  if (W.nm && moved_block(W, x) >= 0) return;
-  if (queue_find(W, x) >= 0) return;
-  if (W.qn >= A.queue_cap) return;
-  int to;
-  long long gain;
-  if (!gain_of<EW>(A, W, x, &to, &gain)) return;
-  __syncwarp();
-  if ((threadIdx.x & 31) == 0) {
-    W.qv[W.qn] = x;
-    W.qg[W.qn] = gain;
-    W.qh[W.qn] = hkey(A.smix, (uint64_t)(uint32_t)x, 0);
-    W.qn += 1;
+__device__ bool lane_gain(const MlsArgs &A, const WarpState &W, ConnT<EW> *conn, int u, int *to_out,
+                          long long *gain_out) {
+  if (u < 0) return false;
+  const int lane = threadIdx.x & 31;
+  const int64_t rb = A.g.row_begin(u), re = A.g.row_begin(u + 1);
+  const int a = view_block(A, W, u);
+  const long long cu = A.g.vweight(u);
+  for (int b = 0; b < A.k; b++) conn[b * 32 + lane] = 0;
+  for (int64_t e = rb; e < re; e += 4) {
+    int x[4], p[4];
+    long long w[4];
+#pragma unroll
+    for (int y = 0; y < 4; y++) {
+      x[y] = e + y < re ? __ldg(A.g.adj + e + y) : -1;
+      w[y] = e + y < re ? load_ew<EW>(A.g.ew, e + y) : 0;
+    }
+#pragma unroll
+    for (int y = 0; y < 4; y++) p[y] = x[y] >= 0 ? A.part[x[y]] : 0;
+#pragma unroll
+    for (int y = 0; y < 4; y++) {
+      if (x[y] < 0) continue;
+      const int moved = W.nm ? moved_block(W, x[y]) : -1;
+      conn[(moved >= 0 ? moved : p[y]) * 32 + lane] += (ConnT<EW>)w[y];
+    }
   }
+  const uint64_t hu = mix64(A.smix ^ (uint64_t)(uint32_t)u);
+  long long bc = 0;
+  uint64_t bh = 0;
+  int bb = -1;
+  for (int b = 0; b < A.k; b++) {
+    const long long c = (long long)conn[b * 32 + lane];
+    if (b == a || c <= 0 || c < bc || W.bw[b] + cu > A.lmax) continue;
+    const uint64_t h = mix64(hu ^ (uint64_t)b);
+    if (c > bc || h > bh) {  // (blocks in ascending order: the smaller one stays on equal hashes)
+      bc = c;
+      bh = h;
+      bb = b;
+    }
+  }
+  if (bb < 0) return false;
+  *to_out = bb;
+  *gain_out = bc - (long long)conn[a * 32 + lane];
+  return true;
+}
+
+__device__ __forceinline__ void queue_append(const MlsArgs &A, WarpState &W, int at, int x, long long gain) {
+  W.qv[at] = x;
+  W.qg[at] = gain;
+  W.qh[at] = hkey(A.smix, (uint64_t)(uint32_t)x, 0);
+}
+
+// The lanes' vertices (u < 0: none; distinct, in lane order) are queued, or their keys recomputed: a vertex that is in
+// the queue gets its gain anew or leaves, another is inserted if it is movable and the queue has room. Vertices above
+// the degree bound and moved ones are left out. All lanes call.
+template <int EW>
+__device__ void touch(const MlsArgs &A, WarpState &W, unsigned char *conn_raw, int u) {
+  const int lane = threadIdx.x & 31;
+  if (u >= 0 && (degree_of(A.g, u) > A.max_degree || (W.nm && moved_block(W, u) >= 0))) u = -1;
+  int at = -1;
+  for (int i = 0; i < W.qn; i++)
+    if (W.qv[i] == u) at = i;
+  int to = 0;
+  long long gain = 0;
+  bool movable = false;
+  if (A.k <= kLaneK) {
+    movable = lane_gain<EW>(A, W, reinterpret_cast<ConnT<EW> *>(conn_raw), u, &to, &gain);
+  } else {
+    for (unsigned todo = __ballot_sync(kFull, u >= 0); todo; todo &= todo - 1) {
+      const int src = __ffs(todo) - 1;
+      int t1 = 0;
+      long long g1 = 0;
+      const bool m1 = gain_of<EW>(A, W, reinterpret_cast<long long *>(conn_raw), __shfl_sync(kFull, u, src), &t1, &g1);
+      if (lane == src) {
+        movable = m1;
+        to = t1;
+        gain = g1;
+      }
+    }
+  }
+  if (u < 0) at = -1;
+  if (at >= 0 && movable) W.qg[at] = gain;
+  const unsigned out = __ballot_sync(kFull, at >= 0 && !movable);
+  const unsigned in = __ballot_sync(kFull, u >= 0 && at < 0 && movable);
   __syncwarp();
+  if (W.qn + __popc(in) <= A.queue_cap) {
+    // every insertion finds room whatever the order
+    const int qn = W.qn;
+    if (in >> lane & 1u) queue_append(A, W, qn + __popc(in & lanemask_lt()), u, gain);
+    __syncwarp();
+    if (lane == 0) W.qn = qn + __popc(in);
+    __syncwarp();
+    for (unsigned o = out; o; o &= o - 1) queue_remove(W, queue_find(W, __shfl_sync(kFull, u, __ffs(o) - 1)));
+  } else {
+    for (unsigned o = out | in; o; o &= o - 1) {
+      const int src = __ffs(o) - 1;
+      const int us = __shfl_sync(kFull, u, src);
+      const long long gs = __shfl_sync(kFull, gain, src);
+      if (out >> src & 1u) {
+        queue_remove(W, queue_find(W, us));
+      } else if (W.qn < A.queue_cap) {
+        __syncwarp();
+        if (lane == 0) {
+          queue_append(A, W, W.qn, us, gs);
+          W.qn += 1;
+        }
+        __syncwarp();
+      }
+    }
+  }
 }
 
 // PerformMoves: one warp per todo vertex; seq[i * max_moves + j] = (vertex, from, to) of the best prefix,
@@ -182,6 +291,7 @@ __global__ void __launch_bounds__(kMlsThreads) k_mls_search(MlsArgs A, const int
                                                             int32_t *len) {
   extern __shared__ __align__(16) unsigned char smem[];
   WarpState &W = reinterpret_cast<WarpState *>(smem)[threadIdx.x >> 5];
+  unsigned char *const conn = smem + kMlsWarps * sizeof(WarpState) + (threadIdx.x >> 5) * A.conn_bytes;
   const int lane = threadIdx.x & 31;
   const int64_t gw = (int64_t)blockIdx.x * kMlsWarps + (threadIdx.x >> 5);
   const int64_t nw = (int64_t)gridDim.x * kMlsWarps;
@@ -199,8 +309,14 @@ __global__ void __launch_bounds__(kMlsThreads) k_mls_search(MlsArgs A, const int
       W.nm = 0;
     }
     __syncwarp();
-    try_insert<EW>(A, W, v);
-    for (int64_t e = A.g.row_begin(v); e < A.g.row_begin(v + 1); e++) try_insert<EW>(A, W, __ldg(A.g.adj + e));
+    {
+      // the start vertex, then its neighbours in row order
+      const int64_t rb = A.g.row_begin(v);
+      for (int64_t y0 = 0; y0 <= dv; y0 += 32) {
+        const int64_t y = y0 + lane;
+        touch<EW>(A, W, conn, y == 0 ? v : y <= dv ? __ldg(A.g.adj + rb + y - 1) : -1);
+      }
+    }
     long long cum = 0, best = 0;
     int best_len = 0, fruitless = 0;
     while (W.qn > 0 && W.nm < A.max_moves) {
@@ -236,7 +352,7 @@ __global__ void __launch_bounds__(kMlsThreads) k_mls_search(MlsArgs A, const int
       queue_remove(W, bi);
       int to;
       long long gain;
-      if (!gain_of<EW>(A, W, x, &to, &gain)) continue;
+      if (!gain_of<EW>(A, W, reinterpret_cast<long long *>(conn), x, &to, &gain)) continue;
       const int a = view_block(A, W, x);
       const long long cx = A.g.vweight(x);
       __syncwarp();
@@ -262,24 +378,9 @@ __global__ void __launch_bounds__(kMlsThreads) k_mls_search(MlsArgs A, const int
       } else if (++fruitless >= A.fruitless) {
         break;
       }
-      for (int64_t e = A.g.row_begin(x); e < A.g.row_begin(x + 1); e++) {
-        const int u = __ldg(A.g.adj + e);
-        if (degree_of(A.g, u) > A.max_degree || moved_block(W, u) >= 0) continue;
-        const int j = queue_find(W, u);
-        if (j >= 0) {
-          int tu;
-          long long gu;
-          if (gain_of<EW>(A, W, u, &tu, &gu)) {
-            __syncwarp();
-            if (lane == 0) W.qg[j] = gu;
-            __syncwarp();
-          } else {
-            queue_remove(W, j);
-          }
-        } else {
-          try_insert<EW>(A, W, u);
-        }
-      }
+      const int64_t re = A.g.row_begin(x + 1);
+      for (int64_t e0 = A.g.row_begin(x); e0 < re; e0 += 32)
+        touch<EW>(A, W, conn, e0 + lane < re ? __ldg(A.g.adj + e0 + lane) : -1);
     }
     const int L = best > 0 ? best_len : 0;
     for (int j = lane; j < L; j += 32) seq[i * A.max_moves + j] = make_int3(W.mv[j], W.mfrom[j], W.mto[j]);
@@ -299,12 +400,13 @@ __device__ __forceinline__ long long block_sum_ll(long long x, long long *red) {
   return t;
 }
 
-// ApplyMoves: one CTA, sequences in todo order. out[0] += gain, out[1] += applied moves.
+// ApplyMoves: one CTA, sequences in todo order. out[0] += gain, out[1] += applied moves, whose vertices (each once) go
+// to moved_list.
 template <int EW>
 __global__ void __launch_bounds__(kApplyThreads) k_mls_apply(DGraph g, int32_t *part, int64_t *bw_g, int k,
                                                              int64_t lmax, const int3 *seq, const int32_t *len,
                                                              int64_t m, int max_moves, uint32_t *moved,
-                                                             long long *out) {
+                                                             int32_t *moved_list, long long *out) {
   __shared__ long long bw[kMaxK];
   __shared__ long long red[kApplyThreads / 32];
   __shared__ int idx[kApplyThreads];
@@ -387,7 +489,11 @@ __global__ void __launch_bounds__(kApplyThreads) k_mls_apply(DGraph g, int32_t *
           bw[mvj.z] -= cw;
           bw[mvj.y] += cw;
         }
-        for (int j = 0; j < best_len; j++) moved[seq[si * max_moves + j].x] = 1;
+        for (int j = 0; j < best_len; j++) {
+          const int w = seq[si * max_moves + j].x;
+          moved[w] = 1;
+          moved_list[moves_total + j] = w;
+        }
         gain_total += best;
         moves_total += best_len;
       }
@@ -401,35 +507,82 @@ __global__ void __launch_bounds__(kApplyThreads) k_mls_apply(DGraph g, int32_t *
   }
 }
 
-__global__ void k_boundary_flags(DGraph g, const int32_t *part, int max_degree, uint32_t *flags) {
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < g.n; v += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t rb = g.row_begin(v), re = g.row_begin(v + 1);
-    uint32_t f = 0;
-    if (re - rb <= max_degree) {
-      const int a = part[v];
-      for (int64_t e = rb; e < re; e++)
-        if (part[g.adj[e]] != a) {
-          f = 1;
-          break;
+// Boundary vertices within the degree bound, in any order: list[0 .. *count).
+__global__ void k_boundary_list(DGraph g, const int32_t *part, int max_degree, int32_t *list, unsigned long long *count) {
+  for (int64_t v0 = (int64_t)blockIdx.x * blockDim.x; v0 < g.n; v0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t v = v0 + threadIdx.x;
+    bool f = false;
+    if (v < g.n) {
+      const int64_t rb = g.row_begin(v), re = g.row_begin(v + 1);
+      if (re - rb <= max_degree) {
+        const int a = part[v];
+        for (int64_t e = rb; e < re && !f; e += 4) {
+          int p[4];
+#pragma unroll
+          for (int y = 0; y < 4; y++) p[y] = e + y < re ? __ldg(g.adj + e + y) : -1;
+#pragma unroll
+          for (int y = 0; y < 4; y++) p[y] = p[y] >= 0 ? part[p[y]] : a;
+          f = p[0] != a || p[1] != a || p[2] != a || p[3] != a;
         }
+      }
     }
-    flags[v] = f;
+    const unsigned m = __ballot_sync(kFull, f);
+    if (!m) continue;
+    unsigned long long base = 0;
+    if ((threadIdx.x & 31) == 0) base = atomicAdd(count, (unsigned long long)__popc(m));
+    base = __shfl_sync(kFull, base, 0);
+    if (f) list[base + __popc(m & lanemask_lt())] = (int32_t)v;
   }
 }
 
-// keys[r] = H(s, v, 1), vals[r] = v for every flagged v at rank r (ranks in vertex order)
-__global__ void k_todo_keys(int64_t n, const uint32_t *flags, const int32_t *rank, uint64_t smix,
-                            unsigned long long *keys, unsigned long long *vals) {
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-    if (!flags[v]) continue;
-    keys[rank[v]] = hkey(smix, (uint64_t)v, 1);
-    vals[rank[v]] = (unsigned long long)v;
+// todo = list ordered by (H(s, v, 1), v). Short lists: every vertex counts those before it, a tile of keys at a time
+// (m^2 compares of a launch that takes a few microseconds, where a radix sort of 64 bits takes two dozen launches).
+constexpr int64_t kRankMax = 8192;
+constexpr int kRankThreads = 256;
+
+__global__ void __launch_bounds__(kRankThreads) k_todo_rank(const int32_t *list, int m, uint64_t smix, int32_t *todo) {
+  __shared__ unsigned long long s_key[kRankThreads];
+  __shared__ int s_v[kRankThreads];
+  // a warp of eight lanes per vertex: 32 vertices per block
+  const int i = blockIdx.x * (kRankThreads / 8) + (int)threadIdx.x / 8, part = threadIdx.x & 7;
+  const int v = i < m ? list[i] : 0;
+  const unsigned long long key = hkey(smix, (uint64_t)(uint32_t)v, 1);
+  int before = 0;
+  for (int t0 = 0; t0 < m; t0 += kRankThreads) {
+    __syncthreads();
+    if (t0 + (int)threadIdx.x < m) {
+      const int x = list[t0 + threadIdx.x];
+      s_v[threadIdx.x] = x;
+      s_key[threadIdx.x] = hkey(smix, (uint64_t)(uint32_t)x, 1);
+    }
+    __syncthreads();
+    const int cnt = min(kRankThreads, m - t0);
+    for (int y = part; y < cnt; y += 8) before += s_key[y] < key || (s_key[y] == key && s_v[y] < v);
+  }
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) before += __shfl_xor_sync(kFull, before, o, 8);
+  if (part == 0 && i < m) todo[before] = v;
+}
+
+// Longer lists: radix sort of the keys, then runs of equal keys by vertex.
+__global__ void k_todo_keys(const int32_t *list, int64_t m, uint64_t smix, unsigned long long *keys,
+                            unsigned long long *vals) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+    keys[i] = hkey(smix, (uint64_t)(uint32_t)list[i], 1);
+    vals[i] = (unsigned long long)(unsigned)list[i];
   }
 }
 
-__global__ void k_vals_to_i32(const unsigned long long *vals, int64_t m, int32_t *out) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = (int32_t)vals[i];
+__global__ void k_todo_out(const unsigned long long *keys, const unsigned long long *vals, int64_t m, int32_t *out) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+    const unsigned long long k = keys[i], v = vals[i];
+    int64_t lo = i, hi = i + 1;  // the run of equal keys
+    while (lo > 0 && keys[lo - 1] == k) lo--;
+    while (hi < m && keys[hi] == k) hi++;
+    int64_t at = lo;
+    for (int64_t y = lo; y < hi; y++) at += vals[y] < v;
+    out[at] = (int32_t)v;
+  }
 }
 
 __global__ void k_mls_block_weights(DGraph g, const int32_t *part, int64_t *bw) {
@@ -441,24 +594,34 @@ int grid_of(int64_t items, int threads) {
   return (int)std::max<int64_t>(1, std::min<int64_t>((items + threads - 1) / threads, (int64_t)num_sms() * 8));
 }
 
-// todo = flagged vertices ordered by H(s, v, 1) (ties: smaller v); returns the count via *m_out
-int build_todo(int64_t n, uint32_t *flags, uint64_t s, int32_t *rank, unsigned long long *keys,
-               unsigned long long *vals, unsigned long long *keys2, unsigned long long *vals2, int32_t *todo,
-               int64_t *m_out, Workspace &ws) {
+struct TodoBuffers {
+  unsigned long long *k0, *v0, *k1, *v1;  // long lists only
+  bool ready = false;
+};
+
+// todo = the m vertices of list (distinct, any order) ordered by (H(s, v, 1), v)
+int order_todo(const int32_t *list, int64_t m, int64_t n, uint64_t s, int32_t *todo, TodoBuffers &B, Workspace &ws) {
   cudaStream_t st = ws.stream();
-  int64_t *tot;
-  GP_TRY(ws.get(&tot, 1));
-  GP_TRY(scan_excl_u32(flags, rank, n, tot, ws));
-  int64_t m = 0;
-  GP_CUDA(cudaMemcpyAsync(&m, tot, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-  GP_CUDA(cudaStreamSynchronize(st));
-  *m_out = m;
-  if (m == 0) return GP_OK;
-  (count_launch(), k_todo_keys<<<grid_of(n, 256), 256, 0, st>>>(n, flags, rank, mix64(s), keys, vals));
+  if (m <= 0) return GP_OK;
+  if (m <= kRankMax) {
+    (count_launch(), k_todo_rank<<<(unsigned)((m + kRankThreads / 8 - 1) / (kRankThreads / 8)), kRankThreads, 0, st>>>(
+                         list, (int)m, mix64(s), todo));
+    GP_LAUNCH_CHECK();
+    return GP_OK;
+  }
+  if (!B.ready) {
+    GP_TRY(ws.get(&B.k0, (size_t)n));
+    GP_TRY(ws.get(&B.v0, (size_t)n));
+    GP_TRY(ws.get(&B.k1, (size_t)n));
+    GP_TRY(ws.get(&B.v1, (size_t)n));
+    B.ready = true;
+  }
+  (count_launch(), k_todo_keys<<<grid_of(m, 256), 256, 0, st>>>(list, m, mix64(s), B.k0, B.v0));
   GP_LAUNCH_CHECK();
   bool in_tmp = false;
-  GP_TRY(radix_sort_pairs(keys, vals, keys2, vals2, m, 64, &in_tmp, ws));
-  (count_launch(), k_vals_to_i32<<<grid_of(m, 256), 256, 0, st>>>(in_tmp ? vals2 : vals, m, todo));
+  Workspace sort_ws(st);
+  GP_TRY(radix_sort_pairs(B.k0, B.v0, B.k1, B.v1, m, 64, &in_tmp, sort_ws));
+  (count_launch(), k_todo_out<<<grid_of(m, 256), 256, 0, st>>>(in_tmp ? B.k1 : B.k0, in_tmp ? B.v1 : B.v0, m, todo));
   GP_LAUNCH_CHECK();
   return GP_OK;
 }
@@ -487,58 +650,65 @@ int run_mls(const DGraph &g, int k, int64_t lmax, uint64_t seed, const MlsParams
   Workspace ws(s);
   const int64_t n = g.n;
   uint32_t *flags;
-  int32_t *rank, *todo, *len;
-  unsigned long long *keys, *vals, *keys2, *vals2;
+  int32_t *list, *todo, *len;
   int64_t *bw;
-  long long *acc;
+  unsigned long long *acc;  // gain, moves of a local iteration; boundary vertices of a global one
   int3 *seq;
+  TodoBuffers tb;
   GP_TRY(ws.get(&flags, (size_t)n));
-  GP_TRY(ws.get(&rank, (size_t)n));
+  GP_TRY(ws.get(&list, (size_t)n));
   GP_TRY(ws.get(&todo, (size_t)n));
   GP_TRY(ws.get(&len, (size_t)n));
-  GP_TRY(ws.get(&keys, (size_t)n));
-  GP_TRY(ws.get(&vals, (size_t)n));
-  GP_TRY(ws.get(&keys2, (size_t)n));
-  GP_TRY(ws.get(&vals2, (size_t)n));
   GP_TRY(ws.zeros(&bw, (size_t)k));
-  GP_TRY(ws.zeros(&acc, 2));
+  GP_TRY(ws.get(&acc, 3));
   const int gn = grid_of(n, 256);
   (count_launch(), k_mls_block_weights<<<gn, 256, 0, s>>>(g, part, bw));
   GP_LAUNCH_CHECK();
-  const size_t smem = sizeof(WarpState) * kMlsWarps;
   const int ew = g.ew_mode();
-  static bool attr_set[3] = {false, false, false};
-  if (!attr_set[ew]) {
-    if (ew == 0) GP_CUDA(cudaFuncSetAttribute(k_mls_search<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (ew == 1) GP_CUDA(cudaFuncSetAttribute(k_mls_search<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (ew == 2) GP_CUDA(cudaFuncSetAttribute(k_mls_search<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    attr_set[ew] = true;
+  MlsArgs A;
+  A.g = g;
+  A.part = part;
+  A.bw = bw;
+  A.k = k;
+  A.lmax = lmax;
+  A.max_moves = (int)p.max_moves;
+  A.fruitless = (int)p.fruitless;
+  A.queue_cap = (int)p.queue_cap;
+  A.max_degree = (int)p.max_degree;
+  A.conn_bytes = (unsigned)(ew == 0 ? conn_bytes<0>(k) : conn_bytes<1>(k));
+  const size_t smem = (sizeof(WarpState) + A.conn_bytes) * kMlsWarps;
+  {
+    const int most = (int)((sizeof(WarpState) + std::max(conn_bytes<1>(kLaneK), conn_bytes<1>(kMaxK))) * kMlsWarps);
+    static bool attr_set[3] = {false, false, false};
+    if (!attr_set[ew]) {
+      if (ew == 0) GP_CUDA(cudaFuncSetAttribute(k_mls_search<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+      if (ew == 1) GP_CUDA(cudaFuncSetAttribute(k_mls_search<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+      if (ew == 2) GP_CUDA(cudaFuncSetAttribute(k_mls_search<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+      attr_set[ew] = true;
+    }
   }
   MlsStats st;
   size_t seq_cap = 0;
   for (int gi = 0; gi < p.global_iters; gi++) {
     uint64_t sl = hash3(seed, (uint64_t)gi, 5);
-    (count_launch(), k_boundary_flags<<<gn, 256, 0, s>>>(g, part, (int)p.max_degree, flags));
+    GP_CUDA(cudaMemsetAsync(acc, 0, sizeof(unsigned long long) * 3, s));
+    (count_launch(), k_boundary_list<<<gn, 256, 0, s>>>(g, part, (int)p.max_degree, list, acc + 2));
     GP_LAUNCH_CHECK();
-    int64_t m = 0;
-    GP_TRY(build_todo(n, flags, sl, rank, keys, vals, keys2, vals2, todo, &m, ws));
+    unsigned long long h[3];
+    {
+      Readback rb;
+      rb.add(h, acc, sizeof(h));
+      GP_TRY(rb.run(s));
+    }
+    int64_t m = (int64_t)h[2];
+    GP_TRY(order_todo(list, m, n, sl, todo, tb, ws));
     int64_t total = 0;
     for (int li = 0; li < p.max_local && m > 0; li++) {
       if ((size_t)m * p.max_moves > seq_cap) {
         seq_cap = (size_t)m * p.max_moves;
         GP_TRY(ws.get(&seq, seq_cap));
       }
-      MlsArgs A;
-      A.g = g;
-      A.part = part;
-      A.bw = bw;
-      A.k = k;
-      A.lmax = lmax;
       A.smix = mix64(sl);
-      A.max_moves = (int)p.max_moves;
-      A.fruitless = (int)p.fruitless;
-      A.queue_cap = (int)p.queue_cap;
-      A.max_degree = (int)p.max_degree;
       const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((m + kMlsWarps - 1) / kMlsWarps,
                                                                     (int64_t)num_sms() * 8));
       {
@@ -548,27 +718,31 @@ int run_mls(const DGraph &g, int k, int64_t lmax, uint64_t seed, const MlsParams
         else (count_launch(), k_mls_search<2><<<grid, kMlsThreads, smem, s>>>(A, todo, m, seq, len));
         GP_LAUNCH_CHECK();
       }
-      GP_CUDA(cudaMemsetAsync(flags, 0, sizeof(uint32_t) * (size_t)n, s));  // now: moved in this local iteration
-      GP_CUDA(cudaMemsetAsync(acc, 0, sizeof(long long) * 2, s));
+      GP_CUDA(cudaMemsetAsync(flags, 0, sizeof(uint32_t) * (size_t)n, s));  // moved in this local iteration
+      GP_CUDA(cudaMemsetAsync(acc, 0, sizeof(unsigned long long) * 2, s));
       {
         ProfScope ps("mls_apply", s);
-        if (ew == 0) (count_launch(), k_mls_apply<0><<<1, kApplyThreads, 0, s>>>(g, part, bw, k, lmax, seq, len, m, (int)p.max_moves, flags, acc));
-        else if (ew == 1) (count_launch(), k_mls_apply<1><<<1, kApplyThreads, 0, s>>>(g, part, bw, k, lmax, seq, len, m, (int)p.max_moves, flags, acc));
-        else (count_launch(), k_mls_apply<2><<<1, kApplyThreads, 0, s>>>(g, part, bw, k, lmax, seq, len, m, (int)p.max_moves, flags, acc));
+        long long *out = reinterpret_cast<long long *>(acc);
+        if (ew == 0) (count_launch(), k_mls_apply<0><<<1, kApplyThreads, 0, s>>>(g, part, bw, k, lmax, seq, len, m, (int)p.max_moves, flags, list, out));
+        else if (ew == 1) (count_launch(), k_mls_apply<1><<<1, kApplyThreads, 0, s>>>(g, part, bw, k, lmax, seq, len, m, (int)p.max_moves, flags, list, out));
+        else (count_launch(), k_mls_apply<2><<<1, kApplyThreads, 0, s>>>(g, part, bw, k, lmax, seq, len, m, (int)p.max_moves, flags, list, out));
         GP_LAUNCH_CHECK();
       }
-      long long h[2];
-      GP_CUDA(cudaMemcpyAsync(h, acc, sizeof(h), cudaMemcpyDeviceToHost, s));
-      GP_CUDA(cudaStreamSynchronize(s));
+      {
+        Readback rb;
+        rb.add(h, acc, sizeof(h));
+        GP_TRY(rb.run(s));
+      }
       st.searches += m;
-      st.moves += h[1];
+      st.moves += (int64_t)h[1];
       st.local_iters += 1;
-      const int64_t gain = h[0];
+      const int64_t gain = (int64_t)h[0];
       const bool more = gain > 0 && 100 * gain > p.alpha_pct * total;
       total += gain;
       if (!more) break;
       sl = hash3(sl, (uint64_t)li + 1, 6);
-      GP_TRY(build_todo(n, flags, sl, rank, keys, vals, keys2, vals2, todo, &m, ws));
+      m = (int64_t)h[1];  // the moved vertices, which the application listed
+      GP_TRY(order_todo(list, m, n, sl, todo, tb, ws));
     }
     st.gain += total;
   }

@@ -2837,16 +2837,23 @@ __global__ void __launch_bounds__(kThreads, 4) k_lp(const LpProblem *probs, cons
 constexpr int kOwnDeg = 128;    // longest row (half of a warp's table)
 constexpr int kOwnTile = 2048;  // vertices classified at a time (kOwnPer per thread)
 constexpr int kOwnPer = kOwnTile / kThreads;
+constexpr int kOwnList = 2560;  // active vertices kept before a choice (per pair of bins)
+constexpr int kOwnTiles = 32;   // tiles between choices (list entries number the vertices with 16 bits)
 constexpr int kOwnKeep = 512;   // proposals kept in shared memory beside their slots
 constexpr int kOwnCap = 2 * kOwnDeg;  // table slots per warp
+constexpr int kOwnTableWarps = 4;     // warps with a table (rows above 32 entries are rare here)
 static_assert(kOwnPer == 8, "a thread's flags are one 64-bit word");
+// Dynamic shared memory: tables, lists, rows; a contest's keys take up to 32 KB from its start, and the rows they cover
+// are read again. Every KB here is one less of L1 for the gathers of labels: 46 KB per block instead of 40 KB made LP
+// on 2^20 points a quarter slower.
 template <bool LQ>
-constexpr int kOwnListOff = kWarps * kOwnCap * (LQ ? 16 : 12);
+constexpr int kOwnListOff = kOwnTableWarps * kOwnCap * (LQ ? 16 : 12);
 template <bool LQ>
-constexpr int kOwnRowOff = kOwnListOff<LQ> + kOwnTile * 4;  // (the rows outlive a contest, which takes 32 KB)
+constexpr int kOwnRowOff = kOwnListOff<LQ> + 2 * kOwnList * 2;
 template <bool LQ>
-constexpr size_t kOwnSmem = kOwnRowOff<LQ> + kOwnTile * 4;
-static_assert(kOwnRowOff<false> >= kContestSmall * 8, "the rows lie behind the contest's keys");
+constexpr int kOwnUsed = kOwnRowOff<LQ> + kOwnTile * 4;
+template <bool LQ>
+constexpr size_t kOwnSmem = kOwnUsed<LQ> > kContestSmall * 8 ? kOwnUsed<LQ> : kContestSmall * 8;
 
 struct OwnProps {
   int v[kOwnKeep], t[kOwnKeep];
@@ -2854,29 +2861,35 @@ struct OwnProps {
   unsigned cur;   // parity of the running sub-round
 };
 
-// The active vertices of a tile. Four bins: 1: d <= 8, 2: d <= 16, 3: d <= 32, 4: d <= kOwnDeg (bin 0 is part
+// Active vertices of the block. Four bins: 1: d <= 8, 2: d <= 16, 3: d <= 32, 4: d <= kOwnDeg (bin 0 is part
 // of bin 1 here); bins 1 and 2 grow towards each other in the first half of the list, 3 and 4 in the second.
 struct OwnBins {
   const LpProblem &P;
   OwnProps &O;
   unsigned long long counts;   // 16 bits per bin from bin 1 on
-  unsigned short *list;        // vertices of the tile, 2 kOwnTile entries
-  unsigned *rowx;              // per vertex of the tile: (row begin - tile's first row begin) << 8 | degree
-  int t0;                      // first vertex of the tile
-  int64_t r0;                  // its row begin
+  unsigned short *list;        // vertex - t0, 2 kOwnList entries
+  const unsigned *rowx;        // rows of the block's vertices (begin - r0) << 8 | degree, or NULL: read again
+  int t0;                      // first vertex of the list's tiles
+  int64_t r0;                  // its row begin (with rowx)
   int64_t slot0;               // first proposal slot of the block
   __device__ __forceinline__ static int bin(int d) { return d <= 8 ? 1 : d <= 16 ? 2 : d <= 32 ? 3 : 4; }
   __device__ __forceinline__ static unsigned at(int b, unsigned i) {
-    return (b < 3 ? 0u : (unsigned)kOwnTile) + (b & 1 ? i : (unsigned)kOwnTile - 1u - i);
+    return (b < 3 ? 0u : (unsigned)kOwnList) + (b & 1 ? i : (unsigned)kOwnList - 1u - i);
   }
   __device__ __forceinline__ unsigned count(int b) const {
     return b ? (unsigned)(counts >> (16 * (b - 1))) & 0xffffu : 0u;
   }
   __device__ __forceinline__ void row(int b, unsigned i, int *v, int64_t *beg, int64_t *d) const {
-    const unsigned x = list[at(b, i)], y = rowx[x];
+    const unsigned x = list[at(b, i)];
     *v = t0 + (int)x;
-    *beg = r0 + (int64_t)(y >> 8);
-    *d = (int64_t)(y & 255u);
+    if (rowx) {
+      const unsigned y = rowx[x];
+      *beg = r0 + (int64_t)(y >> 8);
+      *d = (int64_t)(y & 255u);
+    } else {
+      *beg = P.g.row_begin(*v);
+      *d = P.g.row_begin(*v + 1) - *beg;
+    }
   }
   __device__ __forceinline__ void none(int, unsigned) const {}
   template <bool LQ>
@@ -2897,10 +2910,11 @@ __device__ __forceinline__ void choose_own_warp(const LpProblem &P, const OwnBin
   const unsigned cnt = B.count(4);
   if (cnt == 0) return;
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const LabelTable<EW, LQ> T(dsm, kWarps * kOwnCap, wid * kOwnCap);
+  if (wid >= kOwnTableWarps) return;
+  const LabelTable<EW, LQ> T(dsm, kOwnTableWarps * kOwnCap, wid * kOwnCap);
   for (int s = lane; s < kOwnCap; s += 32) T.clear(s);
   __syncwarp();
-  for (unsigned i = wid; i < cnt; i += kWarps) {
+  for (unsigned i = wid; i < cnt; i += kOwnTableWarps) {
     int v;
     int64_t beg, d;
     B.row(4, i, &v, &beg, &d);
@@ -2948,13 +2962,14 @@ __device__ __forceinline__ uint64_t marks_own(const LpProblem &P, int r, int64_t
   return r == 0 ? ~0ull : *reinterpret_cast<const uint64_t *>(P.act[r & 1] + P.vbase + v0);
 }
 
-// The active vertices of one tile by degree bin (degree-0 ones, which take no part in the choice, only count as
-// visits). known: rowx holds the rows already (a block of one tile reads them once per call). *packed must be
-// zero on entry; returns the bins' counts, 16 bits each.
-__device__ __forceinline__ unsigned long long classify_own(const LpProblem &P, uint8_t *act_clear,
-                                                           int s, uint64_t rmix, int t0, int t1, int64_t r0,
-                                                           uint64_t marks, bool known, unsigned short *list,
-                                                           unsigned *rowx, unsigned long long *packed, Smem &sm) {
+// The active vertices of one tile, appended to the lists by degree bin (degree-0 ones, which take no part in the choice,
+// only count as visits). t0: the tile's first vertex; base: the lists' first vertex. rowx (not NULL): the rows of the
+// tile's vertices (a block of one tile reads them once per call). *packed holds the bins' counts, 16 bits each, which
+// are returned.
+__device__ __forceinline__ unsigned long long classify_own(const LpProblem &P, uint8_t *act_clear, int s, uint64_t rmix,
+                                                           int t0, int t1, int base, uint64_t marks,
+                                                           const unsigned *rowx, unsigned short *list,
+                                                           unsigned long long *packed, Smem &sm) {
   const int v0 = t0 + (int)threadIdx.x * kOwnPer;
   unsigned flag = 0;
   if (v0 < t1) {
@@ -2967,26 +2982,13 @@ __device__ __forceinline__ unsigned long long classify_own(const LpProblem &P, u
 #pragma unroll
     for (int i = 0; i < kOwnPer; i++)
       if ((flag >> i & 1u) && (int)(mix64(rmix ^ (uint64_t)(v0 + i)) >> 63) != s) flag &= ~(1u << i);
-    unsigned *const rx = rowx + threadIdx.x * kOwnPer;
     int dd[kOwnPer];
-    if (known) {
 #pragma unroll
-      for (int i = 0; i < kOwnPer; i++) dd[i] = flag >> i & 1u ? (int)(rx[i] & 255u) : 0;
-    } else {
-      int rel[kOwnPer];
-#pragma unroll
-      for (int i = 0; i < kOwnPer; i++) {
-        rel[i] = 0;
-        dd[i] = 0;
-        if (flag >> i & 1u) {
-          const int64_t rb = P.g.row_begin(v0 + i);
-          dd[i] = (int)(P.g.row_begin(v0 + i + 1) - rb);
-          rel[i] = (int)(rb - r0);
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < kOwnPer; i++)
-        if (dd[i] > 0) rx[i] = (unsigned)rel[i] << 8 | (unsigned)dd[i];
+    for (int i = 0; i < kOwnPer; i++) {
+      dd[i] = 0;
+      if (flag >> i & 1u)
+        dd[i] = rowx ? (int)(rowx[threadIdx.x * kOwnPer + i] & 255u)
+                     : (int)(P.g.row_begin(v0 + i + 1) - P.g.row_begin(v0 + i));
     }
     unsigned long long mine = 0;
     unsigned edges = 0;
@@ -2997,7 +2999,7 @@ __device__ __forceinline__ unsigned long long classify_own(const LpProblem &P, u
         edges += (unsigned)dd[i];
       }
     }
-    // places: the lane's share of the warp's, the warp's share of the tile's (the order is of no account)
+    // places: the lane's share of the warp's, the warp's share of the lists (the order is of no account)
     const int lane = threadIdx.x & 31;
     unsigned long long incl = mine;
 #pragma unroll
@@ -3017,8 +3019,7 @@ __device__ __forceinline__ unsigned long long classify_own(const LpProblem &P, u
     for (int i = 0; i < kOwnPer; i++) {
       if (dd[i] > 0) {
         const int b = OwnBins::bin(dd[i]);
-        const unsigned x = threadIdx.x * kOwnPer + i;
-        list[OwnBins::at(b, (unsigned)(pos >> (16 * (b - 1))) & 0xffffu)] = (unsigned short)x;
+        list[OwnBins::at(b, (unsigned)(pos >> (16 * (b - 1))) & 0xffffu)] = (unsigned short)(v0 + i - base);
         pos += 1ull << (16 * (b - 1));
       }
     }
@@ -3169,7 +3170,7 @@ __device__ bool lp_problem_own(const LpProblem *prob, unsigned char *dsm) {
     P.lw2[1][x] = P.lw2[0][x];
     P.demand2[1][x] = 0;
   }
-  if (one_tile) {
+  auto read_rows = [&]() {
 #pragma unroll
     for (int i = 0; i < kOwnPer; i++) {
       const int64_t v = lo + threadIdx.x * kOwnPer + i;
@@ -3178,10 +3179,11 @@ __device__ bool lp_problem_own(const LpProblem *prob, unsigned char *dsm) {
         rowx[threadIdx.x * kOwnPer + i] = (unsigned)(rb - r_lo) << 8 | (unsigned)(P.g.row_begin(v + 1) - rb);
       }
     }
-  }
+  };
+  if (one_tile) read_rows();
   tick(-1);
   int t_last = -1;
-  unsigned tile = 0;  // classified tiles so far (their counts alternate between the two words)
+  unsigned cur = 0;  // the count word in use (the other one is zero)
   for (int r = 0; r < P.rounds; r++) {
     const uint64_t rmix = mix64(P.smix ^ (uint64_t)r);
     bool round_moved = false, round_contest = false;
@@ -3206,32 +3208,47 @@ __device__ bool lp_problem_own(const LpProblem *prob, unsigned char *dsm) {
       t_last = t;
       uint64_t marks = marks_own(P, r, lo + threadIdx.x * kOwnPer, hi);  // (loaded while the replay runs)
       replay_own(P, O, P.lw2[(t + 1) & 1], P.demand2[(t + 1) & 1], lo, O.n[(t + 1) & 1]);
-      for (int64_t t0 = lo; t0 < hi; t0 += kOwnTile, tile++) {
-        const int64_t r0 = one_tile ? r_lo : P.g.row_begin(t0);
+      // The tiles' active vertices are collected until there are enough of them to occupy the block (or no tile is
+      // left): once few vertices are active, a choice per tile would leave most threads idle.
+      int64_t base = lo;
+      for (int64_t t0 = lo; t0 < hi; t0 += kOwnTile) {
         if (t0 > lo) marks = marks_own(P, r, t0 + threadIdx.x * kOwnPer, hi);
         const unsigned long long counts =
-            classify_own(P, P.act[(r + 1) & 1], s, rmix, (int)t0, (int)min(hi, t0 + kOwnTile), r0, marks, one_tile, list,
-                         rowx, &s_packed[tile & 1], sm);
-        if (threadIdx.x == 0) s_packed[(tile + 1) & 1] = 0;  // (read by all before the barrier in classify_own)
-        if (counts) {
+            classify_own(P, P.act[(r + 1) & 1], s, rmix, (int)t0, (int)min(hi, t0 + kOwnTile), (int)base, marks,
+                         one_tile ? rowx : nullptr, list, &s_packed[cur], sm);
+        const bool last = t0 + kOwnTile >= hi;
+        // (the pairs of bins share a half of the list each: bound every bin by the sum)
+        const unsigned total = (unsigned)((counts & 0xffff) + (counts >> 16 & 0xffff) + (counts >> 32 & 0xffff) + (counts >> 48));
+        if (!last && total <= kOwnList - kOwnTile && t0 - base < (kOwnTiles - 1) * kOwnTile) {
+          __syncthreads();  // (the next tile adds to the counts)
+          continue;
+        }
+        if (threadIdx.x == 0) s_packed[cur ^ 1] = 0;  // (read by all before this tile's barrier)
+        cur ^= 1;
+        if (total) {
+          // bins one after another without a barrier: each starts with the warp after the one where the last ended
           unsigned long long grouped = counts;
+          unsigned first = threadIdx.x;
           if constexpr (!LQ) {
-            const OwnBins B{P, O, counts, list, rowx, (int)t0, r0, lo};
+            const OwnBins B{P, O, counts, list, one_tile ? rowx : nullptr, (int)base, r_lo, lo};
             const bool direct = P.singletons && t == 0;
             if (B.count(1) > kRowsMin) {
-              choose_rows<EW, 8>(P, B, 1, threadIdx.x, kThreads, direct);
+              choose_rows<EW, 8>(P, B, 1, first, kThreads, direct);
+              first = (first - (B.count(1) + 31) / 32 * 32) & (kThreads - 1);
               grouped &= ~0xffffull;
             }
             if (B.count(2) > kRowsMin) {
-              choose_rows<EW, 16>(P, B, 2, threadIdx.x, kThreads, direct);
+              choose_rows<EW, 16>(P, B, 2, first, kThreads, direct);
+              first = (first - (B.count(2) + 31) / 32 * 32) & (kThreads - 1);
               grouped &= ~(0xffffull << 16);
             }
           }
-          const OwnBins B{P, O, grouped, list, rowx, (int)t0, r0, lo};
-          choose_groups<EW, LQ>(P, B, threadIdx.x >> 5, kWarps);
+          const OwnBins B{P, O, grouped, list, one_tile ? rowx : nullptr, (int)base, r_lo, lo};
+          choose_groups<EW, LQ>(P, B, first >> 5, kWarps);
           choose_own_warp<EW, LQ>(P, B, dsm);
         }
-        if (t0 + kOwnTile < hi) __syncthreads();  // (the next tile writes the lists and their counts)
+        base = t0 + kOwnTile;
+        if (!last) __syncthreads();  // (the next tile writes the lists and their counts)
       }
       __syncthreads();
       if (threadIdx.x == 0) own_meet(P, M, 0, 1, (unsigned)nb);
@@ -3270,6 +3287,8 @@ __device__ bool lp_problem_own(const LpProblem *prob, unsigned char *dsm) {
         }
         if (!grid_sync(bar)) return false;
         round_contest = true;
+        // (the rows that the keys were written over; the next classification starts behind a block barrier)
+        if (one_tile && (nc > kContestSmall || (lb == 0 && nc > kOwnRowOff<LQ> / 16))) read_rows();
         tick(4);
       }
     }

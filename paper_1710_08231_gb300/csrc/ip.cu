@@ -470,29 +470,10 @@ __global__ void k_vw_stats(DGraph g, unsigned long long *mx, unsigned long long 
   }
 }
 
-// Keep flags (degree > 0) and degrees; with `acc`, also acc[0] = max c(v) over the kept vertices and
-// acc[1] = sum of c(v) over all vertices.
-__global__ void k_deg_flags(DGraph g, uint32_t *keep, int64_t *deg0, unsigned long long *acc) {
-  unsigned long long m = 0, sum = 0;
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < g.n; v += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t d = g.row_begin(v + 1) - g.row_begin(v);
-    keep[v] = d > 0 ? 1u : 0u;
-    deg0[v] = d;
-    if (acc) {
-      const unsigned long long c = (unsigned long long)g.vweight(v);
-      if (d > 0) m = max(m, c);
-      sum += c;
-    }
-  }
-  if (!acc) return;
-  for (int o = 16; o > 0; o >>= 1) {
-    m = max(m, __shfl_xor_sync(kFull, m, o));
-    sum += __shfl_xor_sync(kFull, sum, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    if (m) atomicMax(&acc[0], m);
-    if (sum) atomicAdd(&acc[1], sum);
-  }
+// Keep flags (degree > 0).
+__global__ void k_deg_flags(DGraph g, uint32_t *keep) {
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < g.n; v += (int64_t)gridDim.x * blockDim.x)
+    keep[v] = g.row_begin(v + 1) - g.row_begin(v) > 0 ? 1u : 0u;
 }
 
 // Degree-0 vertices own no CSR entries, so the kept vertices' rows keep their entries in the same
@@ -852,36 +833,28 @@ int strip_isolated(const DGraph &g, Stripped *out, Workspace &ws, cudaStream_t s
   if (W_out) *W_out = 0;
   if (maxc_kept_out) *maxc_kept_out = 0;
   if (g.n == 0) return GP_OK;
+  // one kernel and one read back for the degree classes (valid for the level-0 graph when no vertex is stripped), the
+  // kept vertices and the weights
+  unsigned long long *words, hw[kLpStatWords];
+  GP_TRY(ws.get(&words, (size_t)kLpStatWords));
+  GP_TRY(lp_stats_launch(g, cfg ? *cfg : LpConfig(), words, s));
+  {
+    Readback rb;
+    rb.add(hw, words, sizeof(hw));
+    GP_TRY(rb.run(s));
+  }
+  const int64_t n0 = (int64_t)hw[kStatKept];
+  if (maxc_kept_out) *maxc_kept_out = (int64_t)hw[kStatMaxKept];
+  if (W_out) *W_out = (int64_t)hw[kStatTotal];
+  if (cfg && cls && n0 == g.n) lp_classes_from(hw, *cfg, cls);
+  if (n0 == g.n) return GP_OK;
   uint32_t *keep;
-  int64_t *deg, *total;
   int32_t *rank;
   GP_TRY(ws.get(&keep, (size_t)g.n));
-  GP_TRY(ws.get(&deg, (size_t)g.n));
   GP_TRY(ws.get(&rank, (size_t)g.n));
-  // total[0] = kept vertices, total[1] = max kept weight, total[2] = total weight (one read back)
-  GP_TRY(ws.zeros(&total, 3));
-  const bool stats = W_out || maxc_kept_out;
-  (::gp::count_launch(), k_deg_flags<<<grid_for_n(g.n), 256, 0, s>>>(
-                             g, keep, deg, stats ? reinterpret_cast<unsigned long long *>(total + 1) : nullptr));
+  (::gp::count_launch(), k_deg_flags<<<grid_for_n(g.n), 256, 0, s>>>(g, keep));
   GP_LAUNCH_CHECK();
-  GP_TRY(scan_excl_u32(keep, rank, g.n, total, ws));
-  // the LP degree classes of g, valid for the level-0 graph when no vertex is stripped
-  unsigned long long *cls_dev = nullptr;
-  unsigned long long cls_words[kLpClassWords];
-  if (cfg && cls) {
-    GP_TRY(ws.get(&cls_dev, (size_t)kLpClassWords));
-    GP_TRY(lp_classes_launch(g, *cfg, cls_dev, ws));
-  }
-  int64_t h[3] = {0, 0, 0};
-  Readback rb;
-  rb.add(h, total, sizeof(h));
-  if (cls_dev) rb.add(cls_words, cls_dev, sizeof(cls_words));
-  GP_TRY(rb.run(s));
-  const int64_t n0 = h[0];
-  if (maxc_kept_out) *maxc_kept_out = h[1];
-  if (W_out) *W_out = h[2];
-  if (cls_dev && n0 == g.n) lp_classes_from(cls_words, *cfg, cls);
-  if (n0 == g.n) return GP_OK;
+  GP_TRY(scan_excl_u32(keep, rank, g.n, nullptr, ws));
   out->n0 = n0;
   out->n_iso = g.n - n0;
   out->rank = rank;

@@ -2814,12 +2814,21 @@ __device__ bool lp_problem(const LpProblem *prob, unsigned char *dsm) {
 
 // One launch runs every problem: block b runs the problems blk_list[blk_start[b] .. blk_start[b+1])
 // in order. A problem of several blocks is the only problem of each of its blocks; problems of one
-// block may share a block with others (small graphs of a batch).
+// block may share a block with others (small graphs of a batch). A single problem comes with the launch's
+// parameters instead of through memory (single != 0).
+struct LpLaunch {
+  const LpProblem *probs;
+  const int *blk_start, *blk_list;
+  int single, pad;
+  LpProblem one;
+};
+
 template <int EW, int TB>
-__global__ void __launch_bounds__(kThreads, 4) k_lp(const LpProblem *probs, const int *blk_start, const int *blk_list) {
+__global__ void __launch_bounds__(kThreads, 4) k_lp(const __grid_constant__ LpLaunch a) {
   extern __shared__ __align__(16) unsigned char dsm[];
-  for (int q = blk_start[blockIdx.x]; q < blk_start[blockIdx.x + 1]; q++)
-    if (!lp_problem<EW, TB>(probs + blk_list[q], dsm)) return;
+  const int q1 = a.single ? 1 : a.blk_start[blockIdx.x + 1];
+  for (int q = a.single ? 0 : a.blk_start[blockIdx.x]; q < q1; q++)
+    if (!lp_problem<EW, TB>(a.single ? &a.one : a.probs + a.blk_list[q], dsm)) return;
 }
 
 // ------------------------------------------------------------------------------------ block-owned problems
@@ -3324,11 +3333,11 @@ __device__ bool lp_problem_own(const LpProblem *prob, unsigned char *dsm) {
 #undef bar
 
 template <int EW, bool LQ>
-__global__ void __launch_bounds__(kThreads, EW ? 3 : 4) k_lp_own(const LpProblem *probs, const int *blk_start,
-                                                        const int *blk_list) {
+__global__ void __launch_bounds__(kThreads, EW ? 3 : 4) k_lp_own(const __grid_constant__ LpLaunch a) {
   extern __shared__ __align__(16) unsigned char dsm[];
-  for (int q = blk_start[blockIdx.x]; q < blk_start[blockIdx.x + 1]; q++)
-    if (!lp_problem_own<EW, LQ>(probs + blk_list[q], dsm)) return;
+  const int q1 = a.single ? 1 : a.blk_start[blockIdx.x + 1];
+  for (int q = a.single ? 0 : a.blk_start[blockIdx.x]; q < q1; q++)
+    if (!lp_problem_own<EW, LQ>(a.single ? &a.one : a.probs + a.blk_list[q], dsm)) return;
 }
 
 // ------------------------------------------------------------------------------------ host helpers
@@ -3395,6 +3404,71 @@ __global__ void k_degree_classes(const DGraph *gs, const int64_t *pre, int njobs
       if (t % 3) atomicAdd(&hubstat[t], s_hub[t]);
       else atomicMax(&hubstat[t], s_hub[t]);
     }
+  }
+}
+
+// Degree classes and vertex statistics of one graph (words as lp_stats_launch describes them).
+__global__ void __launch_bounds__(256) k_lp_stats(DGraph g, int deg_warp, int deg_cta, unsigned long long *words) {
+  __shared__ unsigned s_cls[9];
+  __shared__ unsigned long long s_w[kLpStatWords];
+  if (threadIdx.x < 9) s_cls[threadIdx.x] = 0;
+  if (threadIdx.x < kLpStatWords) s_w[threadIdx.x] = 0;
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  unsigned long long ent = 0, hub_max = 0, hub_sum = 0, wide = 0, kept = 0, max_kept = 0, total = 0, most = 0;
+  for (int64_t v0 = blockIdx.x * (int64_t)blockDim.x; v0 < g.n; v0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t v = v0 + threadIdx.x;
+    int bin = 8;
+    if (v < g.n) {
+      const int64_t d = g.row_begin(v + 1) - g.row_begin(v);
+      const unsigned long long c = (unsigned long long)g.vweight(v);
+      total += c;
+      most = max(most, c);
+      if (d > 0) {
+        bin = lp_bin_of(d, deg_warp, deg_cta);
+        ent += (unsigned long long)d;
+        kept++;
+        max_kept = max(max_kept, c);
+        if (bin == 6) {
+          hub_max = max(hub_max, (unsigned long long)hub_cap(d));
+          hub_sum += (unsigned long long)hub_cap(d);
+        }
+        if (d > kWideDeg) wide++;
+      }
+    }
+    const unsigned peers = __match_any_sync(kFull, bin);
+    if (bin < 8 && lane == __ffs(peers) - 1) atomicAdd(&s_cls[bin], (unsigned)__popc(peers));
+  }
+  unsigned long long sum[5] = {ent, hub_sum, wide, kept, total}, top[3] = {hub_max, max_kept, most};
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+    for (int x = 0; x < 5; x++) sum[x] += __shfl_xor_sync(kFull, sum[x], o);
+#pragma unroll
+    for (int x = 0; x < 3; x++) top[x] = max(top[x], __shfl_xor_sync(kFull, top[x], o));
+  }
+  if (lane == 0) {
+    const int at[5] = {5, 7, 8, kStatKept, kStatTotal}, am[3] = {6, kStatMaxKept, kStatMax};
+#pragma unroll
+    for (int x = 0; x < 5; x++)
+      if (sum[x]) atomicAdd(&s_w[at[x]], sum[x]);
+#pragma unroll
+    for (int x = 0; x < 3; x++)
+      if (top[x]) atomicMax(&s_w[am[x]], top[x]);
+  }
+  __syncthreads();
+  if (threadIdx.x < 9 && s_cls[threadIdx.x]) atomicAdd(reinterpret_cast<unsigned *>(words) + threadIdx.x, s_cls[threadIdx.x]);
+  if (threadIdx.x >= 5 && threadIdx.x < kLpStatWords && s_w[threadIdx.x]) {
+    const bool is_max = threadIdx.x == 6 || threadIdx.x == kStatMaxKept || threadIdx.x == kStatMax;
+    if (is_max) atomicMax(&words[threadIdx.x], s_w[threadIdx.x]);
+    else atomicAdd(&words[threadIdx.x], s_w[threadIdx.x]);
+  }
+}
+
+__global__ void k_lp_singletons(DGraph g, int32_t *labels, int64_t *lw) {
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < g.n; v += (int64_t)gridDim.x * blockDim.x) {
+    labels[v] = (int32_t)v;
+    lw[v] = g.vweight(v);
   }
 }
 
@@ -3481,10 +3555,9 @@ int coop_capacity_own(int ew, int *out) {
 }
 
 template <bool LQ>
-int launch_lp_own(int ew, const LpProblem *probs_dev, const int *blk_start_dev, const int *blk_list_dev, int grid,
-                  cudaStream_t s) {
+int launch_lp_own(int ew, LpLaunch &a, int grid, cudaStream_t s) {
   count_launch();
-  void *args[] = {(void *)&probs_dev, (void *)&blk_start_dev, (void *)&blk_list_dev};
+  void *args[] = {(void *)&a};
   void *k = ew == 0 ? (void *)k_lp_own<0, LQ> : ew == 1 ? (void *)k_lp_own<1, LQ> : (void *)k_lp_own<2, LQ>;
   GP_CUDA(cudaLaunchCooperativeKernel(k, grid, kThreads, args, kOwnSmem<LQ>, s));
   return GP_OK;
@@ -3499,18 +3572,13 @@ int coop_capacity(int ew, int tb, int *out) {
   return tb == 0 ? coop_capacity_tb<0>(ew, out) : tb == 1 ? coop_capacity_tb<1>(ew, out) : coop_capacity_tb<2>(ew, out);
 }
 
-template <int EW, int TB>
-int launch_lp(const LpProblem *probs_dev, const int *blk_start_dev, const int *blk_list_dev, int grid, cudaStream_t s) {
-  count_launch();
-  void *args[] = {(void *)&probs_dev, (void *)&blk_start_dev, (void *)&blk_list_dev};
-  GP_CUDA(cudaLaunchCooperativeKernel((void *)k_lp<EW, TB>, grid, kThreads, args, kDynSmemT<TB>, s));
-  return GP_OK;
-}
-
 template <int TB>
-int launch_lp_tb(int ew, const LpProblem *p, const int *bs, const int *bl, int grid, cudaStream_t s) {
-  return ew == 0 ? launch_lp<0, TB>(p, bs, bl, grid, s) : ew == 1 ? launch_lp<1, TB>(p, bs, bl, grid, s)
-                                                                  : launch_lp<2, TB>(p, bs, bl, grid, s);
+int launch_lp_tb(int ew, LpLaunch &a, int grid, cudaStream_t s) {
+  count_launch();
+  void *args[] = {(void *)&a};
+  void *k = ew == 0 ? (void *)k_lp<0, TB> : ew == 1 ? (void *)k_lp<1, TB> : (void *)k_lp<2, TB>;
+  GP_CUDA(cudaLaunchCooperativeKernel(k, grid, kThreads, args, kDynSmemT<TB>, s));
+  return GP_OK;
 }
 
 }  // namespace
@@ -3530,6 +3598,11 @@ LpConfig lp_config_from(const gp_params *p) {
   c.hub_batch_slots = std::max<int64_t>(kMinHubBatchSlots, std::min<int64_t>(c.hub_batch_slots, kMaxHubBatchSlots));
   c.verts_per_block = std::max<int64_t>(kMinVertsPerBlock, std::min<int64_t>(c.verts_per_block, kMaxVertsPerBlock));
   return c;
+}
+
+void lp_scored_bins(LpConfig *cfg) {  // (16-byte slots)
+  cfg->deg_warp = std::min(cfg->deg_warp, kWarpCapT<0> / 2);
+  cfg->deg_cta = std::max(cfg->deg_warp, std::min(cfg->deg_cta, kCtaCapT<0> / 2));
 }
 
 int block_weights(const DGraph &g, const int32_t *part, int64_t k, int64_t *bw, int *bad_dev, cudaStream_t s) {
@@ -3629,22 +3702,21 @@ static int account_counters(const LpCounters *hc, int n, const int64_t *vb, cons
 
 size_t lp_counters_bytes() { return sizeof(LpCounters); }
 
-int lp_classes_launch(const DGraph &g, const LpConfig &cfg, unsigned long long *words_dev, Workspace &ws) {
-  cudaStream_t s = ws.stream();
-  GP_CUDA(cudaMemsetAsync(words_dev, 0, sizeof(unsigned long long) * kLpClassWords, s));
+static int stat_grid(int64_t n) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, num_sms() * 8));
+}
+
+int lp_stats_launch(const DGraph &g, const LpConfig &cfg, unsigned long long *words_dev, cudaStream_t s) {
+  GP_CUDA(cudaMemsetAsync(words_dev, 0, sizeof(unsigned long long) * kLpStatWords, s));
   if (g.n <= 0) return GP_OK;
-  DGraph *gs_dev;
-  int64_t *pre_dev;
-  GP_TRY(ws.get(&gs_dev, 1));
-  GP_TRY(ws.get(&pre_dev, 2));
-  const int64_t pre[2] = {0, g.n};
-  GP_CUDA(cudaMemcpyAsync(gs_dev, &g, sizeof(DGraph), cudaMemcpyHostToDevice, s));
-  GP_CUDA(cudaMemcpyAsync(pre_dev, pre, sizeof(pre), cudaMemcpyHostToDevice, s));
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((g.n + 255) / 256, num_sms() * 8));
-  // words: [0, 5) the 9 unsigned class counts, [5] entries, [6, 9) hub statistics and wide vertices
-  (::gp::count_launch(), k_degree_classes<<<grid, 256, 0, s>>>(gs_dev, pre_dev, 1, cfg.deg_warp, cfg.deg_cta,
-                                                                 reinterpret_cast<unsigned *>(words_dev),
-                                                                 words_dev + 5, words_dev + 6));
+  (::gp::count_launch(), k_lp_stats<<<stat_grid(g.n), 256, 0, s>>>(g, cfg.deg_warp, cfg.deg_cta, words_dev));
+  GP_LAUNCH_CHECK();
+  return GP_OK;
+}
+
+int lp_singletons_launch(const DGraph &g, int32_t *labels, int64_t *lw, cudaStream_t s) {
+  if (g.n <= 0) return GP_OK;
+  (::gp::count_launch(), k_lp_singletons<<<stat_grid(g.n), 256, 0, s>>>(g, labels, lw));
   GP_LAUNCH_CHECK();
   return GP_OK;
 }
@@ -3684,12 +3756,8 @@ int run_lp_multi(const LpJob *jobs, int njobs, cudaStream_t s, const LpConfig &c
   if (njobs <= 0) return GP_OK;
   const int ew = jobs[0].g.ew_mode();
   const bool lq = jobs[0].q != nullptr;
-  // scored runs have the smaller shared-memory tables (16-byte slots)
   LpConfig cfg = cfg_in;
-  if (lq) {
-    cfg.deg_warp = std::min(cfg.deg_warp, kWarpCapT<0> / 2);
-    cfg.deg_cta = std::max(cfg.deg_warp, std::min(cfg.deg_cta, kCtaCapT<0> / 2));
-  }
+  if (lq) lp_scored_bins(&cfg);
   for (int j = 0; j < njobs; j++) {
     if (jobs[j].stats) std::memset(jobs[j].stats, 0, sizeof(gp_lp_stats));
     if (jobs[j].g.ew_mode() != ew || (jobs[j].q != nullptr) != lq) {
@@ -3722,6 +3790,21 @@ int run_lp_multi(const LpJob *jobs, int njobs, cudaStream_t s, const LpConfig &c
       hhub[3 * (size_t)j + 1] = ci.hub_cap_sum;
       hhub[3 * (size_t)j + 2] = ci.wide;
     }
+  } else if (njobs == 1) {
+    unsigned long long *words, hw[kLpStatWords];
+    GP_TRY(ws.get(&words, (size_t)kLpStatWords));
+    GP_TRY(lp_stats_launch(jobs[0].g, cfg, words, s));
+    Readback rb;
+    rb.add(hw, words, sizeof(hw));
+    GP_TRY(rb.run(s));
+    LpClassInfo ci;
+    lp_classes_from(hw, cfg, &ci);
+    for (int b = 0; b < 9; b++) hcls[b] = ci.cls[b];
+    hent[0] = ci.entries;
+    hhub[0] = ci.hub_max_cap;
+    hhub[1] = ci.hub_cap_sum;
+    hhub[2] = ci.wide;
+    if (jobs[0].classes) *jobs[0].classes = ci;
   } else {
     std::vector<DGraph> hg(njobs);
     std::vector<int64_t> pre(njobs + 1, 0);
@@ -3867,18 +3950,28 @@ int run_lp_multi(const LpJob *jobs, int njobs, cudaStream_t s, const LpConfig &c
     return GP_ERR_INTERNAL;
   }
   std::vector<LpProblem> hp(njobs);
+  // Counters, barriers, bin counters and demand of every job start at zero: one allocation, one memset. With
+  // deferred counters the caller's (zeroed) blocks are used in place.
+  if (deferred && deferred->count + njobs > deferred->capacity) {
+    set_error("run_lp_multi: deferred counter buffer is full");
+    return GP_ERR_INTERNAL;
+  }
   LpCounters *ctr_all;
-  unsigned *bar_all;
-  GP_TRY(ws.zeros(&ctr_all, (size_t)njobs));
-  GP_TRY(ws.zeros(&bar_all, (size_t)njobs * kBarrierStride));
-  unsigned *binres_all;
-  GP_TRY(ws.zeros(&binres_all, (size_t)njobs * 3 * 256));
-  // every job's demand array in one zeroed allocation (one memset for the launch, not one per job)
+  unsigned *bar_all, *binres_all;
   int64_t *demand_all;
   {
+    auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
     size_t total = 0;
     for (int j = 0; j < njobs; j++) total += (size_t)std::max<int64_t>(jobs[j].nl, 1);
-    GP_TRY(ws.zeros(&demand_all, total));
+    const size_t b_ctr = deferred ? 0 : up(sizeof(LpCounters) * (size_t)njobs),
+                 b_bar = up(sizeof(unsigned) * kBarrierStride * (size_t)njobs),
+                 b_bin = own ? 0 : up(sizeof(unsigned) * 3 * 256 * (size_t)njobs), b_dem = up(sizeof(int64_t) * total);
+    unsigned char *z;
+    GP_TRY(ws.zeros(&z, b_ctr + b_bar + b_bin + b_dem));
+    ctr_all = deferred ? static_cast<LpCounters *>(deferred->dev) + deferred->count : reinterpret_cast<LpCounters *>(z);
+    bar_all = reinterpret_cast<unsigned *>(z + b_ctr);
+    binres_all = reinterpret_cast<unsigned *>(z + b_ctr + b_bar);
+    demand_all = reinterpret_cast<int64_t *>(z + b_ctr + b_bar + b_bin);
   }
   int64_t *lw2_all = nullptr, *demand2_all = nullptr;
   if (own) {
@@ -3956,7 +4049,7 @@ int run_lp_multi(const LpJob *jobs, int njobs, cudaStream_t s, const LpConfig &c
     GP_TRY(ws.get(&P.hist, (size_t)nblk[j] * 256 + 16));
     GP_TRY(ws.get(&P.hoff, (size_t)nblk[j] * 256 + 256 + 16));
     P.ctr = ctr_all + j;
-    P.binres = binres_all + (size_t)j * 3 * 256;
+    P.binres = own ? nullptr : binres_all + (size_t)j * 3 * 256;
     P.bar = bar_all + (size_t)j * kBarrierStride;
     const unsigned nhub = hcls[9 * j + 6];
     if (nhub) {
@@ -4011,32 +4104,37 @@ int run_lp_multi(const LpJob *jobs, int njobs, cudaStream_t s, const LpConfig &c
       }
     }
   }
-  LpProblem *probs_dev;
-  int *bs_dev, *bl_dev;
-  GP_TRY(ws.get(&probs_dev, hp.size()));
-  GP_TRY(ws.get(&bs_dev, blk_start.size()));
-  GP_TRY(ws.get(&bl_dev, blk_list.size()));
-  GP_CUDA(cudaMemcpyAsync(probs_dev, hp.data(), sizeof(LpProblem) * hp.size(), cudaMemcpyHostToDevice, s));
-  GP_CUDA(cudaMemcpyAsync(bs_dev, blk_start.data(), sizeof(int) * blk_start.size(), cudaMemcpyHostToDevice, s));
-  GP_CUDA(cudaMemcpyAsync(bl_dev, blk_list.data(), sizeof(int) * blk_list.size(), cudaMemcpyHostToDevice, s));
+  LpLaunch la;
+  std::memset(&la, 0, sizeof(la));
+  if (njobs == 1) {
+    la.single = 1;
+    la.one = hp[0];
+  } else {
+    // problems and block lists in one copy
+    const size_t b_p = (sizeof(LpProblem) * hp.size() + 255) & ~size_t(255), b_s = sizeof(int) * blk_start.size(),
+                 b_l = sizeof(int) * blk_list.size();
+    std::vector<unsigned char> img(b_p + b_s + b_l);
+    std::memcpy(img.data(), hp.data(), sizeof(LpProblem) * hp.size());
+    std::memcpy(img.data() + b_p, blk_start.data(), b_s);
+    std::memcpy(img.data() + b_p + b_s, blk_list.data(), b_l);
+    unsigned char *dev;
+    GP_TRY(ws.get(&dev, img.size()));
+    GP_CUDA(cudaMemcpyAsync(dev, img.data(), img.size(), cudaMemcpyHostToDevice, s));
+    la.probs = reinterpret_cast<const LpProblem *>(dev);
+    la.blk_start = reinterpret_cast<const int *>(dev + b_p);
+    la.blk_list = reinterpret_cast<const int *>(dev + b_p + b_s);
+  }
   {
     ProfScope ps(jobs[0].prof, s);
     int st;
-    if (own) st = lq ? launch_lp_own<true>(ew, probs_dev, bs_dev, bl_dev, grid, s)
-                     : launch_lp_own<false>(ew, probs_dev, bs_dev, bl_dev, grid, s);
-    else if (tb == 0) st = launch_lp_tb<0>(ew, probs_dev, bs_dev, bl_dev, grid, s);
-    else if (tb == 1) st = launch_lp_tb<1>(ew, probs_dev, bs_dev, bl_dev, grid, s);
-    else st = launch_lp_tb<2>(ew, probs_dev, bs_dev, bl_dev, grid, s);
+    if (own) st = lq ? launch_lp_own<true>(ew, la, grid, s) : launch_lp_own<false>(ew, la, grid, s);
+    else if (tb == 0) st = launch_lp_tb<0>(ew, la, grid, s);
+    else if (tb == 1) st = launch_lp_tb<1>(ew, la, grid, s);
+    else st = launch_lp_tb<2>(ew, la, grid, s);
     GP_TRY(st);
   }
   if (deferred) {
-    // keep the counters on the device for lp_collect
-    if (deferred->count + njobs > deferred->capacity) {
-      set_error("run_lp_multi: deferred counter buffer is full");
-      return GP_ERR_INTERNAL;
-    }
-    GP_CUDA(cudaMemcpyAsync(static_cast<LpCounters *>(deferred->dev) + deferred->count, ctr_all,
-                            sizeof(LpCounters) * njobs, cudaMemcpyDeviceToDevice, s));
+    // the counters stay on the device for lp_collect
     deferred->count += njobs;
     for (int j = 0; j < njobs; j++) {
       const DGraph &g = jobs[j].g;
@@ -4047,8 +4145,11 @@ int run_lp_multi(const LpJob *jobs, int njobs, cudaStream_t s, const LpConfig &c
     return GP_OK;
   }
   std::vector<LpCounters> hc(njobs);
-  GP_CUDA(cudaMemcpyAsync(hc.data(), ctr_all, sizeof(LpCounters) * njobs, cudaMemcpyDeviceToHost, s));
-  GP_CUDA(cudaStreamSynchronize(s));
+  {
+    Readback rb;
+    rb.add(hc.data(), ctr_all, sizeof(LpCounters) * (size_t)njobs);
+    GP_TRY(rb.run(s));
+  }
   std::vector<int64_t> vb(njobs), eb(njobs);
   for (int j = 0; j < njobs; j++) {
     const DGraph &g = jobs[j].g;

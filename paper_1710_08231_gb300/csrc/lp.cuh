@@ -50,15 +50,20 @@ __device__ __forceinline__ int lp_bin_of(int64_t d, int deg_warp, int deg_cta) {
 __host__ __device__ __forceinline__ int64_t hub_cap(int64_t d) { return ((2 * d + 63) / 64) * 64; }
 constexpr int kWideDeg = 1024;  // degrees above this need the larger shared-memory tables
 
-// Degree classes of one graph computed without a read back: lp_classes_launch writes kLpClassWords
-// words into words_dev (device, caller-owned) on the workspace's stream; after the caller has read
-// them to the host, lp_classes_from fills the LpClassInfo.
+// Degree classes and vertex statistics of one graph by one kernel, without a read back: lp_stats_launch writes
+// kLpStatWords words into words_dev (device, caller-owned): the first kLpClassWords are what lp_classes_from reads, then
+// vertices with neighbours, largest weight of one, total weight, largest weight of any vertex.
 constexpr int kLpClassWords = 9;
-int lp_classes_launch(const DGraph &g, const LpConfig &cfg, unsigned long long *words_dev, Workspace &ws);
+constexpr int kLpStatWords = 13;
+enum { kStatKept = 9, kStatMaxKept = 10, kStatTotal = 11, kStatMax = 12 };
+int lp_stats_launch(const DGraph &g, const LpConfig &cfg, unsigned long long *words_dev, cudaStream_t s);
 void lp_classes_from(const unsigned long long *words, const LpConfig &cfg, LpClassInfo *ci);
 
+// labels[v] = v, lw[v] = c(v): the start of a clustering.
+int lp_singletons_launch(const DGraph &g, int32_t *labels, int64_t *lw, cudaStream_t s);
+
 // Counters of several LP calls kept on the device and read back once (lp_collect) instead of after
-// every call. `dev` holds `capacity` counter blocks (lp_counters_bytes() each, from the caller).
+// every call. `dev` holds `capacity` counter blocks (lp_counters_bytes() each, zeroed, from the caller).
 struct LpDeferred {
   void *dev = nullptr;
   int capacity = 0, count = 0;
@@ -98,6 +103,7 @@ struct LpJob {
 int run_lp_multi(const LpJob *jobs, int njobs, cudaStream_t s, const LpConfig &cfg, LpDeferred *deferred = nullptr);
 
 LpConfig lp_config_from(const gp_params *p);
+void lp_scored_bins(LpConfig *cfg);  // the bins of runs with scores, which have the smaller tables
 
 // One LP run from (labels, lw). labels[n] in [0,nl) and lw[nl] (int64 label weights, equal to the
 // vertex-weight sums) are device arrays updated in place. q: NULL or per-entry scores.

@@ -37,16 +37,6 @@ int64_t lmax_of(int64_t total, int64_t k, double eps) {
   return (int64_t)((1.0 + eps) * (double)ceil_avg);
 }
 
-__global__ void k_iota(int32_t *x, int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    x[i] = (int32_t)i;
-}
-
-__global__ void k_vw_to_i64(DGraph g, int64_t *out) {
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < g.n; v += (int64_t)gridDim.x * blockDim.x)
-    out[v] = g.vweight(v);
-}
-
 // CSR validation; err bits: 1 offsets, 2 range, 4 self-loop, 8 order/duplicate, 16 weight <= 0,
 // 32 missing reverse entry, 64 asymmetric weight.
 __global__ void k_validate(DGraph g, int *err) {
@@ -214,7 +204,7 @@ int partition_device(const gp_graph *gin, int32_t k, double eps, uint64_t seed, 
   lpdef.capacity = 2 * (int)p.max_levels + (int)p.ip_tries + 4;
   {
     unsigned char *buf;
-    GP_TRY(ws.get(&buf, lp_counters_bytes() * (size_t)lpdef.capacity));
+    GP_TRY(ws.zeros(&buf, lp_counters_bytes() * (size_t)lpdef.capacity));
     lpdef.dev = buf;
   }
   const double t_coarse0 = now_ms();
@@ -232,9 +222,7 @@ int partition_device(const gp_graph *gin, int32_t k, double eps, uint64_t seed, 
       // (level 0: from the strip's read back; later levels: reported by the contraction)
       const int64_t maxc = l == 0 ? maxc0 : H.levels.back().g.max_vw;
       const int64_t U = std::max<int64_t>(maxc, lmax / p.cluster_div);
-      (::gp::count_launch(), k_iota<<<grid_n(gl.n), 256, 0, s>>>(labels, gl.n));
-      (::gp::count_launch(), k_vw_to_i64<<<grid_n(gl.n), 256, 0, s>>>(gl, lw));
-      GP_LAUNCH_CHECK();
+      GP_TRY(lp_singletons_launch(gl, labels, lw, s));
       if (learned) GP_TRY(mlp_score(gl, l, static_cast<const gp_mlp *>(p.mlp), nullptr, q, s));
       if (p.coarsen == GP_COARSEN_MATCHING)
         GP_TRY(run_match(gl, U, (int)p.rounds_coarsen, hash3(seed, (uint64_t)l, 1), labels, nullptr, s, false));
@@ -502,20 +490,28 @@ int gp_lp_cluster(const gp_graph *gd, int64_t U, int32_t rounds, uint64_t seed, 
   cudaStream_t s = (cudaStream_t)stream;
   const DGraph g = make_dgraph(gd);
   Workspace ws(s);
-  int64_t maxc = 0;
-  GP_TRY(vertex_weight_stats(g, &maxc, nullptr, s));
-  if (maxc > U) {
+  // one kernel and one read back for the largest weight and the degree classes
+  const LpConfig cfg = schedule_for(nullptr);
+  LpConfig cls_cfg = cfg;
+  if (edge_q) lp_scored_bins(&cls_cfg);
+  unsigned long long *words, hw[kLpStatWords];
+  GP_TRY(ws.get(&words, (size_t)kLpStatWords));
+  GP_TRY(lp_stats_launch(g, cls_cfg, words, s));
+  {
+    Readback rb;
+    rb.add(hw, words, sizeof(hw));
+    GP_TRY(rb.run(s));
+  }
+  if ((int64_t)hw[kStatMax] > U) {
     set_error("gp_lp_cluster: U is below the largest vertex weight");
     return GP_ERR_INVALID_ARG;
   }
+  LpClassInfo cls;
+  lp_classes_from(hw, cls_cfg, &cls);
   int64_t *lw;
   GP_TRY(ws.get(&lw, (size_t)std::max<int64_t>(g.n, 1)));
-  if (g.n > 0) {
-    (::gp::count_launch(), k_iota<<<grid_n(g.n), 256, 0, s>>>(labels_out, g.n));
-    (::gp::count_launch(), k_vw_to_i64<<<grid_n(g.n), 256, 0, s>>>(g, lw));
-    GP_LAUNCH_CHECK();
-  }
-  GP_TRY(run_lp(g, edge_q, labels_out, lw, g.n, U, rounds, seed, stats, s, schedule_for(nullptr), true));
+  GP_TRY(lp_singletons_launch(g, labels_out, lw, s));
+  GP_TRY(run_lp(g, edge_q, labels_out, lw, g.n, U, rounds, seed, stats, s, cfg, true, &cls));
   GP_TRY(prof_flush(s));
   GP_CUDA(cudaStreamSynchronize(s));
   return GP_OK;
@@ -540,9 +536,7 @@ int gp_lp_cluster_async(const gp_graph *gd, int64_t U, int32_t rounds, uint64_t 
   int64_t *lw;
   GP_TRY(ws.get(&lw, (size_t)std::max<int64_t>(g.n, 1)));
   if (g.n > 0) {
-    (::gp::count_launch(), k_iota<<<grid_n(g.n), 256, 0, s>>>(labels_out, g.n));
-    (::gp::count_launch(), k_vw_to_i64<<<grid_n(g.n), 256, 0, s>>>(g, lw));
-    GP_LAUNCH_CHECK();
+    GP_TRY(lp_singletons_launch(g, labels_out, lw, s));
   }
   GP_TRY(run_lp_async(g, labels_out, lw, g.n, U, rounds, seed, single_warp != 0, stats, s));
   GP_CUDA(cudaStreamSynchronize(s));
@@ -645,14 +639,25 @@ int gp_lp_refine(const gp_graph *gd, int32_t k, int64_t lmax, int32_t rounds, ui
   GP_TRY(ws.get(&bw, (size_t)k));
   GP_TRY(ws.zeros(&bad, 1));
   GP_TRY(block_weights(g, part, k, bw, bad, s));
+  // the degree classes come with the same read back
+  const LpConfig cfg = schedule_for(nullptr);
+  unsigned long long *words, hw[kLpStatWords];
+  GP_TRY(ws.get(&words, (size_t)kLpStatWords));
+  GP_TRY(lp_stats_launch(g, cfg, words, s));
   int hbad = 0;
-  GP_CUDA(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
-  GP_CUDA(cudaStreamSynchronize(s));
+  {
+    Readback rb;
+    rb.add(&hbad, bad, sizeof(int));
+    rb.add(hw, words, sizeof(hw));
+    GP_TRY(rb.run(s));
+  }
   if (hbad) {
     set_error("gp_lp_refine: a block id is outside [0, k)");
     return GP_ERR_INVALID_ARG;
   }
-  GP_TRY(run_lp(g, nullptr, part, bw, k, lmax, rounds, seed, stats, s, schedule_for(nullptr)));
+  LpClassInfo cls;
+  lp_classes_from(hw, cfg, &cls);
+  GP_TRY(run_lp(g, nullptr, part, bw, k, lmax, rounds, seed, stats, s, cfg, false, &cls));
   if (block_w_out) GP_CUDA(cudaMemcpyAsync(block_w_out, bw, sizeof(int64_t) * k, cudaMemcpyDeviceToDevice, s));
   GP_TRY(prof_flush(s));
   GP_CUDA(cudaStreamSynchronize(s));
@@ -808,8 +813,7 @@ static int time_candidates(const DGraph &g, const std::vector<gp_params> &cand, 
     for (size_t c = 0; c < cand.size(); c++) {
       const LpConfig cfg = lp_config_from(&cand[c]);
       if (g.n > 0) {
-        (::gp::count_launch(), k_iota<<<grid_n(g.n), 256, 0, s>>>(labels, g.n));
-        (::gp::count_launch(), k_vw_to_i64<<<grid_n(g.n), 256, 0, s>>>(g, lw));
+        GP_TRY(lp_singletons_launch(g, labels, lw, s));
       }
       int st = cudaEventRecord(a, s) == cudaSuccess ? GP_OK : GP_ERR_CUDA;
       if (st == GP_OK) st = run_lp(g, nullptr, labels, lw, g.n, U, 3, 0x5eedULL, nullptr, s, cfg, true);
@@ -880,10 +884,10 @@ int gp_autotune(const gp_graph *gd, gp_params *params, double *ms_out, gp_stream
   {
     Workspace ws(s);
     unsigned long long *words;
-    GP_TRY(ws.get(&words, kLpClassWords));
+    GP_TRY(ws.get(&words, (size_t)kLpStatWords));
     const LpConfig cfg = lp_config_from(&base);
-    GP_TRY(lp_classes_launch(g, cfg, words, ws));
-    unsigned long long hw[kLpClassWords];
+    GP_TRY(lp_stats_launch(g, cfg, words, s));
+    unsigned long long hw[kLpStatWords];
     GP_CUDA(cudaMemcpyAsync(hw, words, sizeof(hw), cudaMemcpyDeviceToHost, s));
     GP_CUDA(cudaStreamSynchronize(s));
     lp_classes_from(hw, cfg, &ci);

@@ -422,7 +422,7 @@ typedef struct gp_profile_entry {
   int64_t bytes;
 } gp_profile_entry;
 int gp_profile_enable(int on);
-/* Limit of every bounded device-side wait (the grid barriers of the LP kernel), in nanoseconds of the
+/* Limit of every bounded device-side wait (the grid barriers of the LP and contraction kernels), in nanoseconds of the
  * GPU's global timer; 0 restores the default of 20 s. A wait that runs out makes the call return
  * GP_ERR_TIMEOUT after every CTA of the kernel has returned (the CUDA context stays usable). The limit is
  * process-wide and read when a call launches its kernels. */

@@ -40,6 +40,8 @@ struct PairVal<2> {
 };
 
 constexpr int kThreads = kSortThreads;
+constexpr int64_t kSegment = 32 * kSortItems;  // positions of the walk that a warp takes at a time
+constexpr int64_t kOwnedRow = 16 * kSegment;   // longest row whose segments the thread that places it records
 constexpr int kHeadThreads = 256;
 constexpr int kHeadItems = 8;  // per lane
 constexpr int64_t kHeadTile = (int64_t)kHeadThreads * kHeadItems;
@@ -62,6 +64,8 @@ struct ContractArgs {
   unsigned long long *k0, *k1;
   void *v0, *v1;
   int *tile_n;
+  int32_t *seg_owner;  // the row that holds the first position of each of the walk's segments, -1: a long one
+  int64_t segments;
   ContractHead *head;
   unsigned *bar;
   unsigned wait_us;
@@ -107,7 +111,7 @@ __device__ __forceinline__ void scan_sums(int64_t n, In in, int64_t *part, Contr
   if (threadIdx.x == 0) part[blockIdx.x] = sm.tot;
 }
 
-// Returns the sum of all items. out(i, sum of the items before i) may overwrite item i.
+// Returns the sum of all items. out(i, sum of the items before i, item i) may overwrite item i.
 template <class In, class Out>
 __device__ __forceinline__ int64_t scan_write(int64_t n, In in, Out out, const int64_t *part, ContractSmem &sm) {
   const int64_t per = scan_chunk(n), lo = min(n, (int64_t)blockIdx.x * per), hi = min(n, lo + per);
@@ -134,7 +138,7 @@ __device__ __forceinline__ int64_t scan_write(int64_t n, In in, Out out, const i
     run += sm.tot;
 #pragma unroll
     for (int k = 0; k < 4; k++) {
-      if (i + k < hi) out(i + k, at);
+      if (i + k < hi) out(i + k, at, x[k]);
       at += x[k];
     }
   }
@@ -155,7 +159,7 @@ __device__ __forceinline__ void pairs_tile(const ContractArgs &a, int64_t tile, 
   const int64_t *const mpre = a.mpre;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const unsigned mask = (1u << bits) - 1u;
-  const int64_t s0 = tile * kSortTile + (int64_t)wid * (32 * kSortItems);
+  const int64_t s0 = tile * kSortTile + (int64_t)wid * kSegment;
   __syncthreads();
   sm.h[threadIdx.x] = 0;
   int64_t x[kSortItems];
@@ -175,7 +179,8 @@ __device__ __forceinline__ void pairs_tile(const ContractArgs &a, int64_t tile, 
         own = a.f2c[v];
       }
     };
-    window(warp_owner(mpre, g.n, s0));
+    const int owner = a.seg_owner[s0 / kSegment];
+    window(owner >= 0 ? owner : warp_owner(mpre, g.n, s0));
 #pragma unroll
     for (int k = 0; k < kSortItems; k++) {
       const int64_t p = s0 + 32 * k + lane;
@@ -274,7 +279,9 @@ __device__ __forceinline__ void heads_tiles(const unsigned long long *keys, int6
 // Everything up to the coarse offsets in one cooperative launch: the steps follow one another by grid meetings
 // (about 2 us each) instead of kernel launches, and the sizes that the later steps need (n', the number of pairs)
 // never go to the host. Small levels are bound by these steps one after another: 17 launches and 9 memsets took
-// 250 us for a few thousand vertices. Large ones are bound by the sort's passes over memory.
+// 250 us for a few thousand vertices, against 140 us now. Large ones are bound by the walk's gathers and the sort's
+// passes over memory (R-MAT 22 with weights, 128 M entries: 34.2 ms with hash tables per row, 6.3 ms so; 2^20
+// points: 0.62 and 0.42 ms).
 template <int EW>
 __global__ void __launch_bounds__(kThreads, 2) k_contract(ContractArgs a) {
   using V = typename PairVal<EW>::T;
@@ -289,6 +296,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_contract(ContractArgs a) {
   const int lane = threadIdx.x & 31;
   const int64_t tid = (int64_t)blockIdx.x * kThreads + threadIdx.x, stride = (int64_t)gridDim.x * kThreads;
   // 1. used labels (a label outside [0, nl) is an error of the call: nothing more is done)
+  for (int64_t y = tid; y < a.segments; y += stride) a.seg_owner[y] = -1;
   for (int64_t v = tid; v < n; v += stride) {
     const int L = a.labels[v];
     if (L < 0 || L >= a.nl) atomicExch(&a.head->bad, 1);
@@ -300,7 +308,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_contract(ContractArgs a) {
   scan_sums(a.nl, [&](int64_t i) { return (long long)a.used[i]; }, a.part, sm);
   MEET();
   const int64_t nc = scan_write(a.nl, [&](int64_t i) { return (long long)a.used[i]; },
-                                [&](int64_t i, long long x) { a.newid[i] = (int32_t)x; }, a.part, sm);
+                                [&](int64_t i, long long x, long long) { a.newid[i] = (int32_t)x; }, a.part, sm);
   MEET();
   // 3. fine -> coarse map and, per coarse vertex, member count and weight. Members of one cluster are mostly
   // neighbours in id order, so the warp combines equal coarse ids before its atomics.
@@ -327,7 +335,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_contract(ContractArgs a) {
   // 4. members bucketed by coarse id (in any order within a cluster) with their degrees; largest coarse weight
   scan_sums(nc, [&](int64_t i) { return (long long)a.cnt[i]; }, a.part, sm);
   MEET();
-  scan_write(nc, [&](int64_t i) { return (long long)a.cnt[i]; }, [&](int64_t i, long long x) { a.mstart[i] = x; }, a.part,
+  scan_write(nc, [&](int64_t i) { return (long long)a.cnt[i]; }, [&](int64_t i, long long x, long long) { a.mstart[i] = x; }, a.part,
              sm);
   {
     unsigned long long m = 0;
@@ -348,7 +356,15 @@ __global__ void __launch_bounds__(kThreads, 2) k_contract(ContractArgs a) {
   scan_sums(n, [&](int64_t i) { return (long long)a.mpre[i]; }, a.part, sm);
   MEET();
   const int64_t m = min(g.m, scan_write(n, [&](int64_t i) { return (long long)a.mpre[i]; },
-                                        [&](int64_t i, long long x) { a.mpre[i] = x; }, a.part, sm));
+                                        [&](int64_t i, long long x, long long d) {
+                                          a.mpre[i] = x;
+                                          // the segments of the walk that begin in this row (a long row's are
+                                          // left to a search)
+                                          if (d <= kOwnedRow)
+                                            for (int64_t y = (x + kSegment - 1) / kSegment; y * kSegment < x + d; y++)
+                                              if (y < a.segments) a.seg_owner[y] = (int32_t)i;
+                                        },
+                                        a.part, sm));
   if (tid == 0) {
     a.mpre[n] = m;
     a.head->nc = nc;
@@ -376,7 +392,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_contract(ContractArgs a) {
     scan_sums(cells, [&](int64_t i) { return (long long)a.hist[i]; }, a.part, sm);
     MEET();
     pairs = scan_write(cells, [&](int64_t i) { return (long long)a.hist[i]; },
-                       [&](int64_t i, long long x) { a.hist[i] = x; }, a.part, sm);
+                       [&](int64_t i, long long x, long long) { a.hist[i] = x; }, a.part, sm);
     MEET();
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
       const int tn = p == 0 ? a.tile_n[t] : (int)min(kSortTile, pairs - t * kSortTile);
@@ -399,8 +415,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_contract(ContractArgs a) {
   scan_sums(nc, [&](int64_t i) { return (long long)a.rowcnt[i]; }, a.part + gridDim.x, sm);
   MEET();
   const int64_t mc = scan_write(htiles, [&](int64_t i) { return (long long)a.tile_heads[i]; },
-                                [&](int64_t i, long long x) { a.tile_heads[i] = x; }, a.part, sm);
-  scan_write(nc, [&](int64_t i) { return (long long)a.rowcnt[i]; }, [&](int64_t i, long long x) { a.off[i] = x; },
+                                [&](int64_t i, long long x, long long) { a.tile_heads[i] = x; }, a.part, sm);
+  scan_write(nc, [&](int64_t i) { return (long long)a.rowcnt[i]; }, [&](int64_t i, long long x, long long) { a.off[i] = x; },
              a.part + gridDim.x, sm);
   if (tid == 0) {
     a.off[nc] = mc;
@@ -621,6 +637,8 @@ int contract_graph(const DGraph &g, const int32_t *labels, int64_t nl, OwnedGrap
   int kbound = 0;  // bits of the largest n' possible: the widest digit the kernel can choose
   while (kbound < 31 && ((int64_t)1 << kbound) < (int64_t)ncb) kbound++;
   GP_TRY(ws.get(&a.tile_n, ntiles));
+  a.segments = (int64_t)ntiles * (kSortTile / kSegment);
+  GP_TRY(ws.get(&a.seg_owner, (size_t)a.segments));
   GP_TRY(ws.get(&a.hist, ntiles << std::min(std::max(kbound, 1), kSortBits)));
   GP_TRY(ws.get(&a.tile_heads, m / (size_t)kHeadTile + 1));
   a.wait_us = (unsigned)std::min<unsigned long long>(wait_limit_ns() / 1000, 0xffffffffull);

@@ -89,7 +89,7 @@ __device__ __forceinline__ void mma_16816(float c[4], const unsigned a[4], const
 // to 64 per entry, with the loads of four entries issued before the first lookup. Half-warps serve short lists (mesh rows of 12 entries take one step) and long
 // ones (four steps) alike. A lane per entry, walking its list alone, read 32 separate rows per load and
 // waited for the warp's longest list and probe: 27.3 ms for inference on an R-MAT graph of scale 19 with
-// edge weights (15.5 M entries) against 2.7 ms now, at the same bits.
+// edge weights (15.5 M entries) against 2.55 ms now, at the same bits.
 //
 // Scores: 16 entries per tensor-core step, A = 16 entries x 16 features (8 used, 8 zero), B = W1^T in four
 // 16x8 slices (32 hidden units). Thread (g = lane/4, t = lane%4) holds features 2t, 2t+1 of rows g and

@@ -3078,7 +3078,7 @@ __device__ __forceinline__ void admit_own(const LpProblem &P, SubCounters &C, co
     }
   }
   if ((threadIdx.x & 31) == 0 && moved) atomicAdd(&sm.moves, (unsigned long long)moved);
-  if (__any_sync(kFull, mg | mq)) {
+  if (__any_sync(kFull, (mg | mq) != 0)) {  // (the vote takes an int: gains may have zero low halves)
     for (int o = 16; o > 0; o >>= 1) {
       mg = max(mg, __shfl_xor_sync(kFull, mg, o));
       mq = max(mq, __shfl_xor_sync(kFull, mq, o));

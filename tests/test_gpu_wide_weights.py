@@ -58,3 +58,10 @@ def test_scored_gains_above_32_bits(gp, shift):
     src = np.repeat(np.arange(g.n), np.diff(g.off))
     q = ((np.minimum(src, g.adj) * 7 + np.maximum(src, g.adj) * 13) % 32769).astype(np.int32)
     _same(gp, g, 40, 5, q)
+
+
+@pytest.mark.parametrize("shift,kind", [(26, np.int32), (30, np.int64), (40, np.int64)])
+@pytest.mark.parametrize("deg", [6.0, 12.0])
+def test_wide_weights_of_short_rows(gp, deg, shift, kind):
+    """Enough vertices for a thread per row (rows of up to 8 and 16 entries), weights whose sums do not fit there."""
+    _same(gp, _weighted(gg.rgg(60000, deg, 9), shift, kind), 30, 7)

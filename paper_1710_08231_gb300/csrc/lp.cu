@@ -948,70 +948,26 @@ __device__ __forceinline__ void choose_groups(const LpProblem &P, const Bins &B,
       cand[u] = false;
       // all labels are the vertices' own (most vertices of a refinement): nothing to weigh
       if (!__any_sync(kFull, has && Lu[u] != L0[u])) continue;
-      bool first = true;  // the lowest lane of the group with this label
-      unsigned qsum = 0;
-      // With weights, two ways to the connections. Up to four distinct labels in the warp: match and one reduction per
-      // set of equal labels, which take a step per distinct label. More: compares with every lane of the group. (A
-      // refinement of 777777 points with 64-bit weights: choice 0.34 ms by the first, 0.65 by the second; clustering
-      // R-MAT 21 with weights: 9.0 ms by the first, 6.0 by the second.)
-      bool few = false;
-      if constexpr (EW != 0 || LQ) {
-        unsigned rem = __ballot_sync(kFull, has);
-        for (int x = 0; x < 4 && rem; x++) rem &= ~__ballot_sync(kFull, Lu[u] == __shfl_sync(kFull, Lu[u], __ffs(rem) - 1));
-        few = rem == 0;
-      }
-      if (few) {
-        const unsigned peers = __match_any_sync(kFull, (unsigned)Lu[u]) & gmask;
-        first = lane == __ffs(peers) - 1;
-        if (EW == 0) {
-          conn[u] = __popc(peers);
-        } else if (!__any_sync(kFull, w[u] >= (1ll << 26) || w[u] < 0)) {
+      // Equal labels meet by a match, their weights and scores by one reduction per set of equal labels. (Comparing
+      // every lane's label with those of the group's lanes instead, which spares the reductions' step per distinct
+      // label, was slower on every graph: clustering 300000 points of average degree 24 with weights 1..8 3.2 ms a
+      // call, so 1.9; R-MAT 21 with weights 21.7 and 20.5; 2^18 points with scores 1.32 and 0.86.)
+      const unsigned peers = __match_any_sync(kFull, (unsigned)Lu[u]) & gmask;
+      if constexpr (EW == 0) {
+        conn[u] = __popc(peers);
+        c0[u] = __popc(__ballot_sync(kFull, has && Lu[u] == L0[u]) & gmask);
+      } else {
+        if (!__any_sync(kFull, w[u] >= (1ll << 26) || w[u] < 0)) {
           conn[u] = (long long)__reduce_add_sync(peers, (unsigned)w[u]);
         } else {
           for (unsigned m = peers; m; m &= m - 1) conn[u] += __shfl_sync(peers, w[u], __ffs(m) - 1);
         }
-        if (LQ) qsum = __reduce_add_sync(peers, (unsigned)qq[u]);
         const unsigned own = __ballot_sync(kFull, has && Lu[u] == L0[u]) & gmask;
         const long long cown = __shfl_sync(kFull, conn[u], own ? __ffs(own) - 1 : lane);
         c0[u] = own ? cown : 0;
-      } else if constexpr (EW == 0 && !LQ) {
-        const unsigned peers = __match_any_sync(kFull, (unsigned)Lu[u]) & gmask;
-        conn[u] = __popc(peers);
-        first = lane == __ffs(peers) - 1;
-        c0[u] = __popc(__ballot_sync(kFull, has && Lu[u] == L0[u]) & gmask);
-      } else {
-        // each lane compares its label with those of the group's lanes, four at a time (a match and a
-        // reduction over each set of equal labels would take a step per distinct label of the warp, twice)
-        long long c = 0, own = 0;
-        const bool narrow = !__any_sync(kFull, w[u] >= (1ll << 26) || w[u] < 0);
-        for (int j0 = 0; j0 < G; j0 += 4) {
-          int Lj[4];
-          long long wj[4];
-          unsigned qj[4];
-#pragma unroll
-          for (int x = 0; x < 4; x++) {
-            Lj[x] = __shfl_sync(kFull, Lu[u], j0 + x, G);
-            wj[x] = EW == 0 ? 1 : (long long)__shfl_sync(kFull, (unsigned)w[u], j0 + x, G);
-            qj[x] = LQ ? __shfl_sync(kFull, (unsigned)qq[u], j0 + x, G) : 0u;
-          }
-          if (EW == 2 && !narrow) {  // (the high halves of wide weights)
-#pragma unroll
-            for (int x = 0; x < 4; x++)
-              wj[x] |= (long long)((unsigned long long)__shfl_sync(kFull, (unsigned)((unsigned long long)w[u] >> 32), j0 + x, G) << 32);
-          }
-#pragma unroll
-          for (int x = 0; x < 4; x++) {
-            const bool eq = Lj[x] == Lu[u];
-            c += eq ? wj[x] : 0;
-            own += Lj[x] >= 0 && Lj[x] == L0[u] ? wj[x] : 0;
-            qsum += LQ && eq ? qj[x] : 0u;
-            first = first && !(eq && j0 + x < gl);
-          }
-        }
-        conn[u] = c;
-        c0[u] = own;
       }
-      if (LQ) qs[u] = (long long)qsum;
+      if constexpr (LQ) qs[u] = (long long)__reduce_add_sync(peers, (unsigned)qq[u]);
+      const bool first = lane == __ffs(peers) - 1;  // the lowest lane of the group with this label
       cand[u] = has && first && Lu[u] != L0[u] && conn[u] > c0[u];
       lwL[u] = cand[u] ? P.lw[Lu[u]] : 0;
     }

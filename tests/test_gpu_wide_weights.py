@@ -65,3 +65,15 @@ def test_scored_gains_above_32_bits(gp, shift):
 def test_wide_weights_of_short_rows(gp, deg, shift, kind):
     """Enough vertices for a thread per row (rows of up to 8 and 16 entries), weights whose sums do not fit there."""
     _same(gp, _weighted(gg.rgg(60000, deg, 9), shift, kind), 30, 7)
+
+
+@pytest.mark.parametrize("n,deg", [(2000, 20.0), (60000, 24.0), (60000, 9.0)])
+@pytest.mark.parametrize("shift", [None, 0, 27])
+def test_scored_rows_of_lane_groups(gp, n, deg, shift):
+    """Rows of up to 32 entries with scores: connections and score sums over equal labels, few or many of them."""
+    g = gg.rgg(n, deg, 6)
+    if shift is not None:
+        g = _weighted(g, shift)
+    src = np.repeat(np.arange(g.n), np.diff(g.off))
+    q = ((np.minimum(src, g.adj) * 7 + np.maximum(src, g.adj) * 13) % 32769).astype(np.int32)
+    _same(gp, g, 60, 5, q)

@@ -2807,7 +2807,7 @@ __device__ bool lp_problem(const LpProblem *prob, unsigned char *dsm) {
 struct LpLaunch {
   const LpProblem *probs;
   const int *blk_start, *blk_list;
-  int single, pad;
+  int single, tables;  // tables: warps with a label table (k_lp_own)
   LpProblem one;
 };
 
@@ -2840,19 +2840,21 @@ constexpr int kOwnList = 2560;  // active vertices kept before a choice (per pai
 constexpr int kOwnTiles = 32;   // tiles between choices (list entries number the vertices with 16 bits)
 constexpr int kOwnKeep = 512;   // proposals kept in shared memory beside their slots
 constexpr int kOwnCap = 2 * kOwnDeg;  // table slots per warp
-constexpr int kOwnTableWarps = 4;     // warps with a table (rows above 32 entries are rare here)
 static_assert(kOwnPer == 8, "a thread's flags are one 64-bit word");
 // Dynamic shared memory: tables, lists, rows; a contest's keys take up to 32 KB from its start, and the rows they cover
 // are read again. Every KB here is one less of L1 for the gathers of labels: 46 KB per block instead of 40 KB made LP
-// on 2^20 points a quarter slower.
+// on 2^20 points a quarter slower. So four warps have a table where rows above 32 entries are rare, and all eight
+// where more than one vertex in kOwnRare has such a row (clustering 200000 vertices of degree 64: 1.78 ms with four
+// tables, 1.43 with eight, 1.27 in the list form; 300000 points of average degree 36: 2.40, 1.95 and 1.93, refining
+// them 0.63, 0.61 and 0.81; 5 % of rows above 32: 0.61 and 0.59, 1 %: 0.51 and 0.51).
+constexpr int kOwnRare = 16;
+constexpr int own_tables(bool many_long) { return many_long ? kWarps : 4; }
 template <bool LQ>
-constexpr int kOwnListOff = kOwnTableWarps * kOwnCap * (LQ ? 16 : 12);
+__host__ __device__ constexpr int own_list_off(int tables) { return tables * kOwnCap * (LQ ? 16 : 12); }
 template <bool LQ>
-constexpr int kOwnRowOff = kOwnListOff<LQ> + 2 * kOwnList * 2;
+__host__ __device__ constexpr int own_row_off(int tables) { return own_list_off<LQ>(tables) + 2 * kOwnList * 2; }
 template <bool LQ>
-constexpr int kOwnUsed = kOwnRowOff<LQ> + kOwnTile * 4;
-template <bool LQ>
-constexpr size_t kOwnSmem = kOwnUsed<LQ> > kContestSmall * 8 ? kOwnUsed<LQ> : kContestSmall * 8;
+constexpr int own_smem(int tables) { return std::max(own_row_off<LQ>(tables) + kOwnTile * 4, kContestSmall * 8); }
 
 struct OwnProps {
   int v[kOwnKeep], t[kOwnKeep];
@@ -2905,15 +2907,15 @@ struct OwnBins {
 
 // One warp per vertex with 32 < d <= kOwnDeg, table in shared memory.
 template <int EW, bool LQ>
-__device__ __forceinline__ void choose_own_warp(const LpProblem &P, const OwnBins &B, unsigned char *dsm) {
+__device__ __forceinline__ void choose_own_warp(const LpProblem &P, const OwnBins &B, unsigned char *dsm, int tables) {
   const unsigned cnt = B.count(4);
   if (cnt == 0) return;
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (wid >= kOwnTableWarps) return;
-  const LabelTable<EW, LQ> T(dsm, kOwnTableWarps * kOwnCap, wid * kOwnCap);
+  if (wid >= tables) return;
+  const LabelTable<EW, LQ> T(dsm, tables * kOwnCap, wid * kOwnCap);
   for (int s = lane; s < kOwnCap; s += 32) T.clear(s);
   __syncwarp();
-  for (unsigned i = wid; i < cnt; i += kOwnTableWarps) {
+  for (unsigned i = wid; i < cnt; i += (unsigned)tables) {
     int v;
     int64_t beg, d;
     B.row(4, i, &v, &beg, &d);
@@ -3115,7 +3117,7 @@ __device__ __forceinline__ void own_meet(const LpProblem &P, OwnMeet &M, int whi
 }
 
 template <int EW, bool LQ>
-__device__ bool lp_problem_own(const LpProblem *prob, unsigned char *dsm) {
+__device__ bool lp_problem_own(const LpProblem *prob, unsigned char *dsm, int tables) {
   __shared__ __align__(16) unsigned char p_raw[sizeof(LpProblem)];
   __shared__ Smem sm;
   __shared__ OwnProps O;
@@ -3124,8 +3126,8 @@ __device__ bool lp_problem_own(const LpProblem *prob, unsigned char *dsm) {
   __shared__ unsigned s_contested;
   __shared__ SubCounters sV;
   LpProblem &P = *reinterpret_cast<LpProblem *>(p_raw);
-  unsigned short *const list = reinterpret_cast<unsigned short *>(dsm + kOwnListOff<LQ>);
-  unsigned *const rowx = reinterpret_cast<unsigned *>(dsm + kOwnRowOff<LQ>);
+  unsigned short *const list = reinterpret_cast<unsigned short *>(dsm + own_list_off<LQ>(tables));
+  unsigned *const rowx = reinterpret_cast<unsigned *>(dsm + own_row_off<LQ>(tables));
   __syncthreads();  // the block's previous problem is done with the shared state
   {
     const unsigned *src = reinterpret_cast<const unsigned *>(prob);
@@ -3244,7 +3246,7 @@ __device__ bool lp_problem_own(const LpProblem *prob, unsigned char *dsm) {
           }
           const OwnBins B{P, O, grouped, list, one_tile ? rowx : nullptr, (int)base, r_lo, lo};
           choose_groups<EW, LQ>(P, B, first >> 5, kWarps);
-          choose_own_warp<EW, LQ>(P, B, dsm);
+          choose_own_warp<EW, LQ>(P, B, dsm, tables);
         }
         base = t0 + kOwnTile;
         if (!last) __syncthreads();  // (the next tile writes the lists and their counts)
@@ -3287,7 +3289,7 @@ __device__ bool lp_problem_own(const LpProblem *prob, unsigned char *dsm) {
         if (!grid_sync(bar)) return false;
         round_contest = true;
         // (the rows that the keys were written over; the next classification starts behind a block barrier)
-        if (one_tile && (nc > kContestSmall || (lb == 0 && nc > kOwnRowOff<LQ> / 16))) read_rows();
+        if (one_tile && (nc > kContestSmall || (lb == 0 && (int)nc > own_row_off<LQ>(tables) / 16))) read_rows();
         tick(4);
       }
     }
@@ -3327,7 +3329,7 @@ __global__ void __launch_bounds__(kThreads, EW ? 3 : 4) k_lp_own(const __grid_co
   extern __shared__ __align__(16) unsigned char dsm[];
   const int q1 = a.single ? 1 : a.blk_start[blockIdx.x + 1];
   for (int q = a.single ? 0 : a.blk_start[blockIdx.x]; q < q1; q++)
-    if (!lp_problem_own<EW, LQ>(a.single ? &a.one : a.probs + a.blk_list[q], dsm)) return;
+    if (!lp_problem_own<EW, LQ>(a.single ? &a.one : a.probs + a.blk_list[q], dsm, a.tables)) return;
 }
 
 // ------------------------------------------------------------------------------------ host helpers
@@ -3527,21 +3529,24 @@ int max_coop_blocks(int *out) {
 }
 
 template <int EW, bool LQ>
-int max_coop_blocks_own(int *out) {
-  static int cached[3][2] = {{0, 0}, {0, 0}, {0, 0}};
-  if (!cached[EW][LQ]) {
-    GP_CUDA(cudaFuncSetAttribute(k_lp_own<EW, LQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOwnSmem<LQ>));
+int max_coop_blocks_own(int tables, int *out) {
+  static int cached[3][2][2] = {};
+  int &per = cached[EW][LQ][tables == own_tables(true)];
+  if (!per) {
+    GP_CUDA(cudaFuncSetAttribute(k_lp_own<EW, LQ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 own_smem<LQ>(own_tables(true))));
     int per_sm = 0;
-    GP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lp_own<EW, LQ>, kThreads, kOwnSmem<LQ>));
-    cached[EW][LQ] = std::max(1, per_sm);
+    GP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lp_own<EW, LQ>, kThreads, own_smem<LQ>(tables)));
+    per = std::max(1, per_sm);
   }
-  *out = cached[EW][LQ] * num_sms();
+  *out = per * num_sms();
   return GP_OK;
 }
 
 template <bool LQ>
-int coop_capacity_own(int ew, int *out) {
-  return ew == 0 ? max_coop_blocks_own<0, LQ>(out) : ew == 1 ? max_coop_blocks_own<1, LQ>(out) : max_coop_blocks_own<2, LQ>(out);
+int coop_capacity_own(int ew, int tables, int *out) {
+  return ew == 0 ? max_coop_blocks_own<0, LQ>(tables, out)
+                 : ew == 1 ? max_coop_blocks_own<1, LQ>(tables, out) : max_coop_blocks_own<2, LQ>(tables, out);
 }
 
 template <bool LQ>
@@ -3549,7 +3554,7 @@ int launch_lp_own(int ew, LpLaunch &a, int grid, cudaStream_t s) {
   count_launch();
   void *args[] = {(void *)&a};
   void *k = ew == 0 ? (void *)k_lp_own<0, LQ> : ew == 1 ? (void *)k_lp_own<1, LQ> : (void *)k_lp_own<2, LQ>;
-  GP_CUDA(cudaLaunchCooperativeKernel(k, grid, kThreads, args, kOwnSmem<LQ>, s));
+  GP_CUDA(cudaLaunchCooperativeKernel(k, grid, kThreads, args, own_smem<LQ>(a.tables), s));
   return GP_OK;
 }
 
@@ -3850,8 +3855,14 @@ int run_lp_multi(const LpJob *jobs, int njobs, cudaStream_t s, const LpConfig &c
   // rows over blocks.
   bool own = cfg.deg_warp <= kOwnDeg;
   for (int j = 0; j < njobs; j++) own = own && hcls[9 * (size_t)j + 5] == 0 && hcls[9 * (size_t)j + 6] == 0;
+  int64_t n_all = 0, n_long = 0;  // vertices, and those with a row above 32 entries
+  for (int j = 0; j < njobs; j++) {
+    n_all += jobs[j].g.n;
+    n_long += hcls[9 * (size_t)j + 4];
+  }
+  const int tables = own_tables(n_long * kOwnRare > n_all);
   int cap_blocks = 0;
-  GP_TRY(own ? (lq ? coop_capacity_own<true>(ew, &cap_blocks) : coop_capacity_own<false>(ew, &cap_blocks))
+  GP_TRY(own ? (lq ? coop_capacity_own<true>(ew, tables, &cap_blocks) : coop_capacity_own<false>(ew, tables, &cap_blocks))
              : coop_capacity(ew, tb, &cap_blocks));
   // Blocks: a job gets at most one block per cfg.verts_per_block vertices. When all jobs fit the co-resident
   // capacity that way, they do; otherwise work is balanced by a cost model (entries + 4 per vertex
@@ -4096,6 +4107,7 @@ int run_lp_multi(const LpJob *jobs, int njobs, cudaStream_t s, const LpConfig &c
   }
   LpLaunch la;
   std::memset(&la, 0, sizeof(la));
+  la.tables = tables;
   if (njobs == 1) {
     la.single = 1;
     la.one = hp[0];

@@ -3324,8 +3324,11 @@ __device__ bool lp_problem_own(const LpProblem *prob, unsigned char *dsm, int ta
 
 #undef bar
 
+// (Weights without scores: 80 registers, since choose_rows holds 16 labels and weights. With scores that form is not
+// used, and a fourth block per SM is worth more: clustering 2^20 points with 64-bit weights and scores 4.07 ms with
+// three, 3.21 with four; with scores and unit weights as before.)
 template <int EW, bool LQ>
-__global__ void __launch_bounds__(kThreads, EW ? 3 : 4) k_lp_own(const __grid_constant__ LpLaunch a) {
+__global__ void __launch_bounds__(kThreads, EW && !LQ ? 3 : 4) k_lp_own(const __grid_constant__ LpLaunch a) {
   extern __shared__ __align__(16) unsigned char dsm[];
   const int q1 = a.single ? 1 : a.blk_start[blockIdx.x + 1];
   for (int q = a.single ? 0 : a.blk_start[blockIdx.x]; q < q1; q++)

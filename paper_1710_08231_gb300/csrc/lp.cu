@@ -1353,7 +1353,7 @@ __device__ __forceinline__ Best direct_best(const LpProblem &P, int64_t e0, int6
 // vertex (row, adjacency, labels, label weight, one after another): the next vertex's row is read while this one
 // is resolved, and four entries per lane are in flight.
 template <int EW, int TB>
-__device__ __forceinline__ void choose_warp(const LpProblem &P, const SubCounters &V, int lb, int nb,
+__device__ __noinline__ void choose_warp(const LpProblem &P, const SubCounters &V, int lb, int nb,
                                             unsigned char *dsm, bool direct) {
   constexpr bool LQ = TB == 0;
   const unsigned cnt = V.bin_count[4];
@@ -1476,7 +1476,7 @@ constexpr int kTeams = kWarps / kTeamWarps;
 constexpr int kTeamBatch = 16;
 
 template <int EW, int TB>
-__device__ __forceinline__ void choose_cta(const LpProblem &P, const SubCounters &V, int lb, int nb,
+__device__ __noinline__ void choose_cta(const LpProblem &P, const SubCounters &V, int lb, int nb,
                                            unsigned char *dsm, Smem &sm, bool direct) {
   const unsigned cnt = V.bin_count[5];
   if (cnt == 0) return;
@@ -2589,6 +2589,31 @@ __device__ void apply_contested(const LpProblem &P, SubCounters &C, unsigned cnt
   }
 }
 
+// The lists of rows of up to 32 entries. Out of line, like choose_warp and choose_cta: all forms of the choice inlined
+// in the loop of k_lp shared its 64 registers (1.3 KB of spill loads with 64-bit weights, 0.6 KB so; refining R-MAT 18
+// with 64-bit weights, k = 8: 10.4 and 10.0 ms; clustering R-MAT 21 17.7 and 17.2).
+template <int EW, bool LQ>
+__device__ __noinline__ void choose_short(const LpProblem &P, const SubCounters &V, int lb, int nb, bool direct) {
+  unsigned grouped = 0xfu;
+  if constexpr (!LQ) {
+    // bins long enough to give every block more than kRowsMin vertices: a thread per vertex
+    const ListBins B{P, V, 0xfu};
+    const unsigned i0 = (unsigned)lb * kThreads + threadIdx.x, step = (unsigned)nb * kThreads;
+    for (int b = 0; b < 2; b++) {
+      if (B.count(b) > kRowsMin * (unsigned)nb) {
+        choose_rows<EW, 8>(P, B, b, i0, step, direct);
+        grouped &= ~(1u << b);
+      }
+    }
+    if (B.count(2) > kRowsMin * (unsigned)nb) {
+      choose_rows<EW, 16>(P, B, 2, i0, step, direct);
+      grouped &= ~4u;
+    }
+  }
+  choose_groups<EW, LQ>(P, ListBins{P, V, grouped}, (unsigned)lb * kWarps + (threadIdx.x >> 5),
+                        (unsigned)nb * kWarps);
+}
+
 template <int EW, int TB>
 __device__ bool lp_problem(const LpProblem *prob, unsigned char *dsm) {
   constexpr bool LQ = TB == 0;
@@ -2692,23 +2717,7 @@ __device__ bool lp_problem(const LpProblem *prob, unsigned char *dsm) {
         // while block 0 prepares the hub list, the other blocks take its share of the choice
         const int clb = (hubs_now && nb > 1) ? lb - 1 : lb, cnb = (hubs_now && nb > 1) ? nb - 1 : nb;
         if (clb >= 0) {
-          unsigned grouped = 0xfu;
-          if constexpr (!LQ) {
-            // bins long enough to give every block more than kRowsMin vertices: a thread per vertex
-            const ListBins B{P, sV, 0xfu};
-            const unsigned i0 = (unsigned)clb * kThreads + threadIdx.x, step = (unsigned)cnb * kThreads;
-            for (int b = 0; b < 2; b++) {
-              if (B.count(b) > kRowsMin * (unsigned)cnb) {
-                choose_rows<EW, 8>(P, B, b, i0, step, direct);
-                grouped &= ~(1u << b);
-              }
-            }
-            if (B.count(2) > kRowsMin * (unsigned)cnb) {
-              choose_rows<EW, 16>(P, B, 2, i0, step, direct);
-              grouped &= ~4u;
-            }
-          }
-          choose_groups<EW, LQ>(P, ListBins{P, sV, grouped}, (unsigned)clb * kWarps + (threadIdx.x >> 5), (unsigned)cnb * kWarps);
+          choose_short<EW, LQ>(P, sV, clb, cnb, direct);
           choose_warp<EW, TB>(P, sV, clb, cnb, dsm, direct);
           choose_cta<EW, TB>(P, sV, clb, cnb, dsm, sm, direct);
         }

@@ -67,3 +67,23 @@ def test_tables_of_four_and_eight_warps(gp, n, share, weighted, scored):
         assert np.array_equal(lab.cpu().numpy(), lab_o) and st["moves"] == st_o.moves
         assert np.array_equal(p.cpu().numpy(), p_o) and np.array_equal(bw.cpu().numpy(), bw_o)
         assert st_r["moves"] == st_ro.moves
+
+
+@pytest.mark.parametrize("n", [250, 600, 5000, 20000, 45000])
+@pytest.mark.parametrize("k", [2, 9])
+@pytest.mark.parametrize("weighted", [False, True])
+def test_contests_decided_by_one_block(gp, n, k, weighted):
+    """Random partitions: contests of a few, hundreds and thousands of proposals, whose moves are made by the block that
+    decides them or by all blocks of the problem."""
+    import torch
+    g = gg.rgg(n, 9.0, 12)
+    if weighted:
+        src = np.repeat(np.arange(n), np.diff(g.off))
+        g.ew = (1 + (np.minimum(src, g.adj).astype(np.int64) * 31 + np.maximum(src, g.adj) * 17) % 9).astype(np.int32)
+        g.vw = np.random.default_rng(n).integers(1, 6, n).astype(np.int64)
+    part = np.random.default_rng(k).integers(0, k, n).astype(np.int32)
+    lm = O.lmax(int(O.vertex_weights(g).sum()), k, 0.02)
+    p, bw, st = gp.lp_refine(gp.DeviceGraph.from_host(g), torch.from_numpy(part).cuda(), k, lm, 12, 5)
+    p_o, bw_o, st_o = O.lp_refine(g, part, k, lm, 12, 5)
+    assert np.array_equal(p.cpu().numpy(), p_o) and np.array_equal(bw.cpu().numpy(), bw_o)
+    assert (st["moves"], st["visits"]) == (st_o.moves, st_o.visits)

@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "gp_internal.cuh"
+#include "per_device.h"
 
 namespace gp {
 
@@ -213,6 +214,16 @@ int num_sms() {
     cached[d] = v > 0 ? v : 148;
   }
   return cached[d];
+}
+
+int kernel_blocks_per_sm(const void *kernel, int threads, size_t smem, size_t smem_most, int *per_sm) {
+  static PerDevice known;
+  return known.find(device_id(), kernel, smem, per_sm, [&](int *v) -> int {
+    GP_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_most));
+    GP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(v, kernel, threads, smem));
+    *v = std::max(1, *v);
+    return GP_OK;
+  });
 }
 
 // ------------------------------------------------------------------------------------------ scans

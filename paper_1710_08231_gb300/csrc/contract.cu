@@ -547,13 +547,8 @@ __global__ void __launch_bounds__(kHeadThreads) k_entries(const unsigned long lo
 template <int EW>
 int launch_contract(ContractArgs &a, cudaStream_t s) {
   using V = typename PairVal<EW>::T;
-  static int per_sm = 0;
-  if (!per_sm) {
-    GP_CUDA(cudaFuncSetAttribute(k_contract<EW>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSortSmem<V>));
-    int x = 0;
-    GP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x, k_contract<EW>, kThreads, kSortSmem<V>));
-    per_sm = std::max(1, x);
-  }
+  int per_sm = 0;
+  GP_TRY(kernel_blocks_per_sm((const void *)k_contract<EW>, kThreads, kSortSmem<V>, kSortSmem<V>, &per_sm));
   // a block per sort tile or per 2048 vertices, up to what is resident: fewer blocks meet sooner
   const int64_t want = std::max<int64_t>(sort_tiles(a.g.m), (std::max(a.g.n, a.nl) + 2047) / 2048);
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, std::min<int64_t>((int64_t)per_sm * num_sms(), kMaxContractBlocks)));

@@ -208,6 +208,10 @@ __device__ __forceinline__ int64_t load_ew(const void *ew, int64_t e) {
 
 // ------------------------------------------------------------------------------------------ device
 int num_sms();
+// Raises the dynamic shared-memory limit of a kernel to smem_most on the current device and finds how many blocks of
+// `threads` threads with smem bytes of it an SM holds (at least 1). Both belong to the device, not to the process: they
+// are found once per device (per_device.h).
+int kernel_blocks_per_sm(const void *kernel, int threads, size_t smem, size_t smem_most, int *per_sm);
 int device_id();
 
 constexpr unsigned kFull = 0xffffffffu;

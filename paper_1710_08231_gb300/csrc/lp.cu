@@ -3537,29 +3537,18 @@ __global__ void k_block_weights(DGraph g, const int32_t *part, int64_t k, int64_
 
 template <int EW, int TB>
 int max_coop_blocks(int *out) {
-  static int cached[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-  if (!cached[EW][TB]) {
-    GP_CUDA(cudaFuncSetAttribute(k_lp<EW, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynSmemT<TB>));
-    int per_sm = 0;
-    GP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lp<EW, TB>, kThreads, kDynSmemT<TB>));
-    cached[EW][TB] = std::max(1, per_sm);
-  }
-  *out = cached[EW][TB] * num_sms();
+  int per_sm = 0;
+  GP_TRY(kernel_blocks_per_sm((const void *)k_lp<EW, TB>, kThreads, kDynSmemT<TB>, kDynSmemT<TB>, &per_sm));
+  *out = per_sm * num_sms();
   return GP_OK;
 }
 
 template <int EW, bool LQ>
 int max_coop_blocks_own(int tables, int *out) {
-  static int cached[3][2][2] = {};
-  int &per = cached[EW][LQ][tables == own_tables(true)];
-  if (!per) {
-    GP_CUDA(cudaFuncSetAttribute(k_lp_own<EW, LQ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 own_smem<LQ>(own_tables(true))));
-    int per_sm = 0;
-    GP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lp_own<EW, LQ>, kThreads, own_smem<LQ>(tables)));
-    per = std::max(1, per_sm);
-  }
-  *out = per * num_sms();
+  int per_sm = 0;
+  GP_TRY(kernel_blocks_per_sm((const void *)k_lp_own<EW, LQ>, kThreads, own_smem<LQ>(tables),
+                              own_smem<LQ>(own_tables(true)), &per_sm));
+  *out = per_sm * num_sms();
   return GP_OK;
 }
 

@@ -230,13 +230,11 @@ int run_lp_async(const DGraph &g, int32_t *labels, int64_t *lw, int64_t nl, int6
   GP_LAUNCH_CHECK();
   const size_t smem = (size_t)kAsyncWarps * kAsyncCap * 12;
   const int ew = g.ew_mode();
-  static bool attr[3] = {false, false, false};
-  if (!attr[ew]) {
-    if (ew == 0) GP_CUDA(cudaFuncSetAttribute(k_lp_async<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (ew == 1) GP_CUDA(cudaFuncSetAttribute(k_lp_async<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (ew == 2) GP_CUDA(cudaFuncSetAttribute(k_lp_async<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    attr[ew] = true;
-  }
+  const void *const kernel = ew == 0   ? (const void *)k_lp_async<0>
+                             : ew == 1 ? (const void *)k_lp_async<1>
+                                       : (const void *)k_lp_async<2>;
+  int per_sm = 0;
+  GP_TRY(kernel_blocks_per_sm(kernel, kAsyncThreads, smem, smem, &per_sm));
   const int grid = single_warp ? 1 : num_sms() * 4;
   const int threads = single_warp ? 32 : kAsyncThreads;
   gp_lp_stats st = {0, 0, 0, 0, 0};

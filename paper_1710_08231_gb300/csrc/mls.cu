@@ -679,13 +679,11 @@ int run_mls(const DGraph &g, int k, int64_t lmax, uint64_t seed, const MlsParams
   const size_t smem = (sizeof(WarpState) + A.conn_bytes) * kMlsWarps;
   {
     const int most = (int)((sizeof(WarpState) + std::max(conn_bytes<1>(kLaneK), conn_bytes<1>(kMaxK))) * kMlsWarps);
-    static bool attr_set[3] = {false, false, false};
-    if (!attr_set[ew]) {
-      if (ew == 0) GP_CUDA(cudaFuncSetAttribute(k_mls_search<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-      if (ew == 1) GP_CUDA(cudaFuncSetAttribute(k_mls_search<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-      if (ew == 2) GP_CUDA(cudaFuncSetAttribute(k_mls_search<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-      attr_set[ew] = true;
-    }
+    const void *const kernel = ew == 0   ? (const void *)k_mls_search<0>
+                               : ew == 1 ? (const void *)k_mls_search<1>
+                                         : (const void *)k_mls_search<2>;
+    int per_sm = 0;
+    GP_TRY(kernel_blocks_per_sm(kernel, kMlsThreads, smem, most, &per_sm));
   }
   MlsStats st;
   size_t seq_cap = 0;

@@ -37,9 +37,9 @@ int radix_sort_pairs(unsigned long long *keys, unsigned long long *vals, unsigne
   cudaStream_t s = ws.stream();
   *result_in_tmp = false;
   if (n <= 1 || bits <= 0) return GP_OK;
-  static const cudaError_t attr = cudaFuncSetAttribute(k_radix_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       kSortSmem<unsigned long long>);
-  GP_CUDA(attr);
+  int per_sm = 0;
+  GP_TRY(kernel_blocks_per_sm((const void *)k_radix_scatter, kSortThreads, kSortSmem<unsigned long long>,
+                              kSortSmem<unsigned long long>, &per_sm));
   const int passes = sort_passes(bits), width = (bits + passes - 1) / passes;
   const int64_t ntiles = sort_tiles(n);
   int64_t *hist;

@@ -176,7 +176,12 @@ void *dev_alloc(size_t bytes, cudaStream_t s) {
       }
     }
   }
-  return raw_alloc(bytes, s);
+  void *p = raw_alloc(bytes, s);
+  if (!p) {
+    free_cached();  // (up to 1 GiB of other sizes that the allocator may make this one from)
+    p = raw_alloc(bytes, s);
+  }
+  return p;
 }
 
 void dev_free(void *p, size_t bytes, cudaStream_t s) {

@@ -14,6 +14,9 @@
 // equal pairs are adjacent and summed. Rows of every length take the same path, so neither a hub row nor the
 // mix of lengths decides the time.
 #include <algorithm>
+#include <memory>
+#include <new>
+#include <vector>
 
 #include "contract.cuh"
 #include "lp.cuh"
@@ -70,6 +73,7 @@ struct ContractArgs {
   unsigned *bar;
   unsigned wait_us;
   int want_classes, deg_warp, deg_cta;
+  int walk_only;  // up to step 5: the caller sorts the pairs in parts (contract_in_parts)
 };
 
 struct ContractSmem {
@@ -369,6 +373,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_contract(ContractArgs a) {
     a.mpre[n] = m;
     a.head->nc = nc;
   }
+  if (a.walk_only) return;
   MEET();
   // 6. pairs, sorted by row
   int kb = 0;
@@ -558,6 +563,50 @@ int launch_contract(ContractArgs &a, cudaStream_t s) {
   return GP_OK;
 }
 
+// ------------------------------------------------------------------------------------------ in parts
+// The pairs of a contraction take 17 (unit weights) to 33 bytes per entry while they are sorted. Where the allocator
+// cannot give that, or not the coarse graph beside them, the coarse rows are made in parts of about an eighth of the
+// entries, whose pairs (row, neighbour) are sorted by both halves of the key with 33 bytes per entry of the part: once
+// for the row lengths and, with the coarse graph allocated, once more for the rows. Slower (a launch per step, two to
+// three times the passes, two read backs per part), with the same coarse graph.
+constexpr int64_t kParts = 8;
+
+// starts[c]: where coarse row c starts in the walk over the members' rows (starts[nc]: its end)
+__global__ void k_walk_starts(const int64_t *mstart, const int64_t *mpre, int64_t n, int64_t nc, int64_t *starts) {
+  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c <= nc; c += (int64_t)gridDim.x * blockDim.x)
+    starts[c] = mpre[c < nc ? mstart[c] : n];
+}
+
+// Keys ((cu - c0) << 32 | cv) and weights of the entries of coarse rows [c0, c1), whose walk starts at w0; entries inside
+// a cluster get a row behind the others. *kept += the entries between clusters. A warp per member row.
+template <int EW>
+__global__ void k_part_pairs(DGraph g, const int32_t *members, const int32_t *f2c, const int64_t *mstart,
+                             const int64_t *mpre, int64_t nc, int64_t c0, int64_t c1, int64_t w0,
+                             unsigned long long *keys, unsigned long long *vals, unsigned long long *kept) {
+  const int lane = threadIdx.x & 31;
+  const int64_t i0 = mstart[c0], i1 = c1 < nc ? mstart[c1] : g.n;
+  const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  unsigned long long out = 0;
+  for (int64_t i = i0 + gw; i < i1; i += nw) {
+    const int v = members[i], cu = f2c[v];
+    const int64_t beg = g.row_begin(v), end = g.row_begin(v + 1), at = mpre[i] - w0 - beg;
+    for (int64_t x = beg + lane; x < end; x += 32) {
+      const int cv = f2c[__ldg(g.adj + x)];
+      keys[at + x] = (unsigned long long)(cv == cu ? c1 - c0 : (int64_t)cu - c0) << 32 | (unsigned)cv;
+      vals[at + x] = (unsigned long long)load_ew<EW>(g.ew, x);
+      out += cv != cu;
+    }
+  }
+  out = (unsigned long long)warp_sum64((int64_t)out);
+  if (lane == 0 && out) atomicAdd(kept, out);
+}
+
+__global__ void __launch_bounds__(kThreads) k_part_heads(const unsigned long long *keys, int64_t n, int64_t *tile_heads,
+                                                         int64_t htiles, int64_t *rowcnt) {
+  __shared__ ContractSmem sm;
+  for (int64_t t = blockIdx.x; 2 * t < htiles; t += gridDim.x) heads_tiles(keys, n, t, tile_heads, htiles, rowcnt, sm);
+}
+
 }  // namespace
 
 int alloc_graph(OwnedGraph *g, int64_t n, int64_t m, cudaStream_t s) {
@@ -575,6 +624,104 @@ int alloc_graph(OwnedGraph *g, int64_t n, int64_t m, cudaStream_t s) {
     g->release(s);
     set_error("device allocation for a coarse graph failed");
     return GP_ERR_OOM;
+  }
+  return GP_OK;
+}
+
+// The coarse graph of a walk that k_contract has prepared, part by part: first the row lengths, unless they are known
+// already (counted), then the rows.
+static int contract_in_parts(const ContractArgs &a, const ContractHead &h, bool counted, OwnedGraph *out, cudaStream_t s,
+                             const LpConfig *cfg, LpClassInfo *cls) {
+  Workspace ws(s);
+  const DGraph &g = a.g;
+  const int64_t nc = h.nc;
+  auto grid_n = [](int64_t items) {
+    return (int)std::max<int64_t>(1, std::min<int64_t>((items + 255) / 256, (int64_t)num_sms() * 8));
+  };
+  const std::unique_ptr<int64_t[]> starts(new (std::nothrow) int64_t[(size_t)nc + 1]);
+  if (!starts) {
+    set_error("contraction: host allocation failed");
+    return GP_ERR_OOM;
+  }
+  {
+    int64_t *d;
+    GP_TRY(ws.get(&d, (size_t)nc + 1));
+    (::gp::count_launch(), k_walk_starts<<<grid_n(nc + 1), 256, 0, s>>>(a.mstart, a.mpre, g.n, nc, d));
+    GP_LAUNCH_CHECK();
+    GP_CUDA(cudaMemcpyAsync(starts.get(), d, sizeof(int64_t) * ((size_t)nc + 1), cudaMemcpyDeviceToHost, s));
+    GP_CUDA(cudaStreamSynchronize(s));
+    ws.release();
+  }
+  const int64_t per = std::max<int64_t>(1, starts[(size_t)nc] / kParts);
+  int64_t mc = h.mc;
+  for (int write = counted ? 1 : 0; write < 2; write++) {
+    if (write) GP_TRY(alloc_graph(out, nc, mc, s));
+    if (write && mc > 0) GP_CUDA(cudaMemsetAsync(out->ew, 0, sizeof(int64_t) * (size_t)mc, s));
+    int64_t at = 0;  // coarse entries of the rows before
+    for (int64_t c0 = 0, c1 = 0; c0 < nc; c0 = c1) {
+      // rows c0 .. c1 - 1: as many as stay within the part, one at least
+      const int64_t w0 = starts[(size_t)c0];
+      c1 = std::upper_bound(starts.get() + c0 + 1, starts.get() + nc + 1, w0 + per) - starts.get() - 1;
+      c1 = std::max(c0 + 1, std::min(c1, nc));
+      const int64_t np = starts[(size_t)c1] - w0;
+      if (np <= 0) continue;
+      Workspace part(s);
+      unsigned long long *k0, *v0, *k1, *v1;
+      int64_t *sizes, hs[2] = {0, 0};  // pairs between clusters, coarse entries
+      GP_TRY(part.get(&k0, (size_t)np));
+      GP_TRY(part.get(&v0, (size_t)np));
+      GP_TRY(part.get(&k1, (size_t)np));
+      GP_TRY(part.get(&v1, (size_t)np));
+      GP_TRY(part.zeros(&sizes, 2));
+      auto pairs_of = [&](auto kernel) {
+        (::gp::count_launch(), kernel<<<grid_n(np), 256, 0, s>>>(g, a.members, a.f2c, a.mstart, a.mpre, nc, c0, c1, w0, k0,
+                                                                 v0, reinterpret_cast<unsigned long long *>(sizes)));
+      };
+      if (g.ew_mode() == 0) pairs_of(k_part_pairs<0>);
+      else if (g.ew_mode() == 1) pairs_of(k_part_pairs<1>);
+      else pairs_of(k_part_pairs<2>);
+      GP_LAUNCH_CHECK();
+      GP_CUDA(cudaMemcpyAsync(hs, sizes, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+      GP_CUDA(cudaStreamSynchronize(s));
+      if (hs[0] == 0) continue;
+      int bits = 32;
+      while (((int64_t)1 << (bits - 32)) <= c1 - c0) bits++;
+      bool in_tmp = false;
+      GP_TRY(radix_sort_pairs(k0, v0, k1, v1, np, bits, &in_tmp, part));
+      const unsigned long long *keys = in_tmp ? k1 : k0, *vals = in_tmp ? v1 : v0;
+      const int64_t htiles = (hs[0] + kHeadTile - 1) / kHeadTile;
+      int64_t *tile_heads;
+      GP_TRY(part.get(&tile_heads, (size_t)htiles));
+      // (the row lengths are read no more once the rows are written)
+      (::gp::count_launch(), k_part_heads<<<(unsigned)std::min<int64_t>((htiles + 1) / 2, (int64_t)num_sms() * 4), kThreads,
+                                            0, s>>>(keys, hs[0], tile_heads, htiles, a.rowcnt + c0));
+      GP_TRY(scan_excl_i64(tile_heads, tile_heads, htiles, sizes + 1, part));
+      GP_CUDA(cudaMemcpyAsync(hs + 1, sizes + 1, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+      GP_CUDA(cudaStreamSynchronize(s));
+      if (write) {
+        (::gp::count_launch(), k_entries<2><<<(unsigned)htiles, kHeadThreads, 0, s>>>(
+                                   keys, vals, hs[0], tile_heads, out->adj + at, out->ew + at, -1, nullptr, nullptr, nullptr, nullptr));
+        GP_LAUNCH_CHECK();
+      }
+      at += hs[1];
+    }
+    if (!write) {
+      mc = at;
+      GP_TRY(scan_excl_i64(a.rowcnt, a.off, nc, a.off + nc, ws));
+      ws.release();
+    }
+  }
+  out->max_vw = (int64_t)h.maxcw;
+  GP_CUDA(cudaMemcpyAsync(out->off, a.off, sizeof(int64_t) * ((size_t)nc + 1), cudaMemcpyDeviceToDevice, s));
+  GP_CUDA(cudaMemcpyAsync(out->vw, a.cw, sizeof(int64_t) * (size_t)nc, cudaMemcpyDeviceToDevice, s));
+  if (cfg && cls) {
+    unsigned long long *words, hw[kLpStatWords];
+    GP_TRY(ws.get(&words, (size_t)kLpStatWords));
+    GP_TRY(lp_stats_launch(out->view(), *cfg, words, s));
+    Readback rb;
+    rb.add(hw, words, sizeof(hw));
+    GP_TRY(rb.run(s));
+    lp_classes_from(hw, *cfg, cls);
   }
   return GP_OK;
 }
@@ -618,26 +765,42 @@ int contract_graph(const DGraph &g, const int32_t *labels, int64_t nl, OwnedGrap
   GP_TRY(ws.get(&a.mpre, (size_t)n + 1));
   GP_TRY(ws.get(&a.off, ncb + 1));
   GP_TRY(ws.get(&a.part, (size_t)2 * kMaxContractBlocks));
-  GP_TRY(ws.get(&a.k0, m));
-  GP_TRY(ws.get(&a.k1, m));
-  const size_t vb = ew == 0 ? 0 : ew == 1 ? 4 : 8;
-  unsigned char *v0 = nullptr, *v1 = nullptr;
-  if (vb) {
-    GP_TRY(ws.get(&v0, m * vb));
-    GP_TRY(ws.get(&v1, m * vb));
+  Workspace pairs(s);  // what is sized by the entries
+  auto get_pairs = [&]() -> int {
+    GP_TRY(pairs.get(&a.k0, m));
+    GP_TRY(pairs.get(&a.k1, m));
+    const size_t vb = ew == 0 ? 0 : ew == 1 ? 4 : 8;
+    unsigned char *v0 = nullptr, *v1 = nullptr;
+    if (vb) {
+      GP_TRY(pairs.get(&v0, m * vb));
+      GP_TRY(pairs.get(&v1, m * vb));
+    }
+    a.v0 = v0;
+    a.v1 = v1;
+    const size_t ntiles = (size_t)sort_tiles(g.m);
+    int kbound = 0;  // bits of the largest n' possible: the widest digit the kernel can choose
+    while (kbound < 31 && ((int64_t)1 << kbound) < (int64_t)ncb) kbound++;
+    GP_TRY(pairs.get(&a.tile_n, ntiles));
+    a.segments = (int64_t)ntiles * (kSortTile / kSegment);
+    GP_TRY(pairs.get(&a.seg_owner, (size_t)a.segments));
+    GP_TRY(pairs.get(&a.hist, ntiles << std::min(std::max(kbound, 1), kSortBits)));
+    GP_TRY(pairs.get(&a.tile_heads, m / (size_t)kHeadTile + 1));
+    return GP_OK;
+  };
+  const int got = get_pairs();
+  if (got != GP_OK && got != GP_ERR_OOM) return got;
+  a.walk_only = got == GP_ERR_OOM;
+  if (a.walk_only) {
+    pairs.release();
+    a.k0 = a.k1 = nullptr;
+    a.v0 = a.v1 = nullptr;
+    a.tile_n = nullptr;
+    a.seg_owner = nullptr;
+    a.segments = 0;
+    a.hist = a.tile_heads = nullptr;
   }
-  a.v0 = v0;
-  a.v1 = v1;
-  const size_t ntiles = (size_t)sort_tiles(g.m);
-  int kbound = 0;  // bits of the largest n' possible: the widest digit the kernel can choose
-  while (kbound < 31 && ((int64_t)1 << kbound) < (int64_t)ncb) kbound++;
-  GP_TRY(ws.get(&a.tile_n, ntiles));
-  a.segments = (int64_t)ntiles * (kSortTile / kSegment);
-  GP_TRY(ws.get(&a.seg_owner, (size_t)a.segments));
-  GP_TRY(ws.get(&a.hist, ntiles << std::min(std::max(kbound, 1), kSortBits)));
-  GP_TRY(ws.get(&a.tile_heads, m / (size_t)kHeadTile + 1));
   a.wait_us = (unsigned)std::min<unsigned long long>(wait_limit_ns() / 1000, 0xffffffffull);
-  a.want_classes = cfg && cls;
+  a.want_classes = cfg && cls && !a.walk_only;
   a.deg_warp = cfg ? cfg->deg_warp : 0;
   a.deg_cta = cfg ? cfg->deg_cta : 0;
   {
@@ -658,8 +821,14 @@ int contract_graph(const DGraph &g, const int32_t *labels, int64_t nl, OwnedGrap
     set_error("contraction: a bounded device barrier gave up");
     return GP_ERR_TIMEOUT;
   }
+  const int room = a.walk_only ? GP_ERR_OOM : alloc_graph(out, h.nc, h.mc, s);
+  if (room != GP_OK) {
+    pairs.release();
+    const int st = contract_in_parts(a, h, !a.walk_only, out, s, cfg, cls);
+    if (st != GP_OK) out->release(s);
+    return st;
+  }
   if (cfg && cls) lp_classes_from(h.classes, *cfg, cls);
-  GP_TRY(alloc_graph(out, h.nc, h.mc, s));
   out->max_vw = (int64_t)h.maxcw;
   {
     // equal pairs summed into the coarse entries; the sorted pairs lie where the last pass left them

@@ -329,9 +329,7 @@ int gp_contract(const gp_graph *g, const int32_t *labels, gp_coarse **coarse, in
                 gp_stream stream);
 const gp_graph *gp_coarse_graph(const gp_coarse *c);
 void gp_coarse_free(gp_coarse *c, gp_stream stream);
-/* As gp_coarse_free, but the arrays stay untouched until the library allocates next (or gp_free_cached or
- * gp_set_allocator is called): for owners that may be collected a little before the last view of the arrays.
- * At most 4 GiB are held that way; what exceeds that is given back at once, oldest first. */
+/* As gp_coarse_free, without waiting for the stream: the arrays are given back in stream order. */
 void gp_coarse_drop(gp_coarse *c, gp_stream stream);
 
 /* Full multilevel partition into k blocks (Section III, Section IV): strip degree-0 vertices,

@@ -10,6 +10,7 @@ from __future__ import annotations
 import ctypes
 import os
 import threading
+import weakref
 from dataclasses import dataclass
 from typing import Optional
 
@@ -360,17 +361,40 @@ def lp_refine(dg: DeviceGraph, part, k: int, lmax_: int, rounds: int, seed: int,
     return part, bw, st.as_dict()
 
 
-class CoarseGraph:
-    """Library-owned coarse graph returned by ``contract``; freed with ``free()``, or with the library's next
-    allocation after it was collected."""
+class _CoarseHandle:
+    """The library's coarse graph, given back when its last holder is gone (or by free())."""
 
     def __init__(self, handle, stream):
-        self.handle = handle
-        self._stream = stream
+        self.handle, self._stream = handle, stream
+
+    def free(self):
+        if self.handle:
+            lib().gp_coarse_free(self.handle, self._stream)
+            self.handle = None
+
+    def __del__(self):
+        try:
+            if self.handle:
+                lib().gp_coarse_drop(self.handle, self._stream)
+                self.handle = None
+        except Exception:
+            pass
+
+
+class CoarseGraph:
+    """Library-owned coarse graph returned by ``contract``. Its arrays live as long as this object or the f2c tensor
+    that ``contract`` returned with it, or until ``free()``."""
+
+    def __init__(self, handle, stream):
+        self._owner = _CoarseHandle(handle, stream)
         d = lib().gp_coarse_graph(handle).contents
         self.n, self.m_dir = int(d.n), int(d.m_dir)
         self.desc = GpGraph()
         ctypes.pointer(self.desc)[0] = d
+
+    @property
+    def handle(self):
+        return self._owner.handle
 
     def to_host(self):
         """Copies the coarse CSR to host numpy arrays (int64 offsets and weights)."""
@@ -381,19 +405,11 @@ class CoarseGraph:
                      _wrap(d.vwgt, n, "<i8").cpu().numpy(), _wrap(d.ewgt, m, "<i8").cpu().numpy(), "coarse")
 
     def free(self):
-        if self.handle:
-            lib().gp_coarse_free(self.handle, self._stream)
-            self.handle = None
+        self._owner.free()
 
-    def __del__(self):
-        # (tensors that view the arrays may outlive their owner by a few statements: the memory goes back
-        # with the library's next allocation, not to torch's next tensor)
-        try:
-            if self.handle:
-                lib().gp_coarse_drop(self.handle, self._stream)
-                self.handle = None
-        except Exception:
-            pass
+
+def _hold(_owner):
+    """Called when a tensor that keeps `_owner` alive is gone."""
 
 
 class _CudaArray:
@@ -418,7 +434,11 @@ def contract(dg: DeviceGraph, labels, stream=None):
     s = _stream(stream)
     _check(lib().gp_contract(ctypes.byref(dg.desc), labels.data_ptr(), ctypes.byref(h), f2c.data_ptr(), s),
            "gp_contract")
-    return CoarseGraph(h, s), f2c[: dg.n]
+    coarse, f2c = CoarseGraph(h, s), f2c[: dg.n]
+    # Tensors made from the descriptor's addresses are mostly kept beside the map: it holds the arrays too. (Not as an
+    # attribute of the tensor: those travel with copies and pickles.)
+    weakref.finalize(f2c, _hold, coarse._owner).atexit = False
+    return coarse, f2c
 
 
 @dataclass

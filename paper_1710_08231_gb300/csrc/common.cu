@@ -54,37 +54,6 @@ static size_t g_cache_bytes = 0;
 constexpr size_t kCacheMaxBlock = size_t(64) << 20;
 constexpr size_t kCacheMaxTotal = size_t(1) << 30;
 
-// Blocks of dropped coarse graphs (gp_coarse_drop): given back by the library's next allocation on any stream, or
-// at once as far as they exceed kDroppedMax bytes in all.
-constexpr size_t kDroppedMax = size_t(4) << 30;
-static std::mutex g_dropped_mu;
-static std::vector<CachedBlock> g_dropped;
-static std::atomic<size_t> g_dropped_bytes{0};
-
-void dev_drop(void *p, size_t bytes, cudaStream_t s) {
-  if (!p) return;
-  {
-    std::lock_guard<std::mutex> lk(g_dropped_mu);
-    g_dropped.push_back({p, bytes, s});
-    g_dropped_bytes += bytes;
-  }
-  release_dropped(kDroppedMax);
-}
-
-void release_dropped(size_t keep) {
-  while (g_dropped_bytes.load() > keep) {
-    CachedBlock b;
-    {
-      std::lock_guard<std::mutex> lk(g_dropped_mu);
-      if (g_dropped.empty()) return;
-      b = g_dropped.front();
-      g_dropped.erase(g_dropped.begin());
-      g_dropped_bytes -= b.bytes;
-    }
-    dev_free(b.p, b.bytes, b.s);
-  }
-}
-
 // The calling thread's pinned staging buffer for Readback (grown on demand, kept until the thread
 // exits).
 namespace {
@@ -136,7 +105,6 @@ int Readback::run(cudaStream_t s) {
 }
 
 void free_cached() {
-  release_dropped(0);
   std::lock_guard<std::mutex> lk(g_cache_mu);
   for (const CachedBlock &b : g_cache) raw_free(b.p, b.bytes, b.s);
   g_cache.clear();
@@ -163,7 +131,6 @@ void *dev_alloc(size_t bytes, cudaStream_t s) {
     if (t_arena->used > t_arena->high) t_arena->high = t_arena->used;
     return t_arena->base + off;
   }
-  if (g_dropped_bytes.load(std::memory_order_relaxed)) release_dropped(0);
   if (bytes <= kCacheMaxBlock) {
     std::lock_guard<std::mutex> lk(g_cache_mu);
     for (size_t i = g_cache.size(); i-- > 0;) {

@@ -27,13 +27,11 @@ struct OwnedGraph {
     d.ew64 = 1;
     return d;
   }
-  void release(cudaStream_t s) { give_back(s, dev_free); }
-  void drop(cudaStream_t s) { give_back(s, dev_drop); }
-  void give_back(cudaStream_t s, void (*to)(void *, size_t, cudaStream_t)) {
-    to(off, off_bytes, s);
-    to(adj, adj_bytes, s);
-    to(vw, vw_bytes, s);
-    to(ew, ew_bytes, s);
+  void release(cudaStream_t s) {
+    dev_free(off, off_bytes, s);
+    dev_free(adj, adj_bytes, s);
+    dev_free(vw, vw_bytes, s);
+    dev_free(ew, ew_bytes, s);
     off = nullptr;
     adj = nullptr;
     vw = nullptr;

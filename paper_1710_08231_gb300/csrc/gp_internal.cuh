@@ -43,8 +43,6 @@ void set_thread_arena(ScratchArena *a);
 bool arena_active();
 void *dev_alloc(size_t bytes, cudaStream_t s);
 void dev_free(void *p, size_t bytes, cudaStream_t s);
-void dev_drop(void *p, size_t bytes, cudaStream_t s);  // dev_free at the next dev_alloc (see gp_coarse_drop)
-void release_dropped(size_t keep);  // dropped blocks back until at most `keep` bytes are held
 void free_cached();  // returns the blocks the library keeps for reuse to the allocator
 long long pinned_stage_allocs();  // pinned host staging allocations made by Readback so far
 

@@ -704,7 +704,7 @@ void gp_coarse_free(gp_coarse *c, gp_stream stream) {
 
 void gp_coarse_drop(gp_coarse *c, gp_stream stream) {
   if (!c) return;
-  c->g.drop((cudaStream_t)stream);
+  c->g.release((cudaStream_t)stream);
   delete c;
 }
 

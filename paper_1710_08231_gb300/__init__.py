@@ -408,8 +408,14 @@ class CoarseGraph:
         self._owner.free()
 
 
-def _hold(_owner):
-    """Called when a tensor that keeps `_owner` alive is gone."""
+_held = {}  # id of a weak reference to a map -> (the reference, the handle that it keeps)
+
+
+def _hold(tensor, owner):
+    """`owner` stays as long as `tensor`. (Not as an attribute of the tensor: those travel with copies and pickles;
+    weakref.finalize takes 5 us.)"""
+    r = weakref.ref(tensor, lambda r: _held.pop(id(r), None))
+    _held[id(r)] = (r, owner)
 
 
 class _CudaArray:
@@ -435,9 +441,7 @@ def contract(dg: DeviceGraph, labels, stream=None):
     _check(lib().gp_contract(ctypes.byref(dg.desc), labels.data_ptr(), ctypes.byref(h), f2c.data_ptr(), s),
            "gp_contract")
     coarse, f2c = CoarseGraph(h, s), f2c[: dg.n]
-    # Tensors made from the descriptor's addresses are mostly kept beside the map: it holds the arrays too. (Not as an
-    # attribute of the tensor: those travel with copies and pickles.)
-    weakref.finalize(f2c, _hold, coarse._owner).atexit = False
+    _hold(f2c, coarse._owner)  # tensors made from the descriptor's addresses are mostly kept beside the map
     return coarse, f2c
 
 

@@ -88,10 +88,12 @@ __device__ __forceinline__ void mma_16816(float c[4], const unsigned a[4], const
 // The neighbours of two entries are looked up together, each by a half-warp that reads them contiguously, up
 // to 64 per entry, with the loads of four entries issued before the first lookup. Half-warps serve short lists (mesh rows of 12 entries take one step) and long
 // ones (four steps) alike. A lane per entry, walking its list alone, read 32 separate rows per load and
-// waited for the warp's longest list and probe: 27.3 ms for inference on an R-MAT graph of scale 19 with
-// edge weights (15.5 M entries) against 2.55 ms now, at the same bits.
+// waited for the warp's longest list and probe: 22.4 ms a call on an R-MAT graph of scale 19 with edge
+// weights (15.5 M entries) against 2.1 ms now, at the same bits.
 //
-// Scores: 16 entries per tensor-core step, A = 16 entries x 16 features (8 used, 8 zero), B = W1^T in four
+// Scores: the entries of a segment are staged in shared memory and scored 32 at a time, whatever rows they lie
+// in (a step per row left most lanes of the network idle on meshes: a grid of 2000 x 2000 took 3.81 ms a call
+// so, 2.97 now, R-MAT 19 2.57 and 2.13). 16 entries per tensor-core step, A = 16 entries x 16 features (8 used, 8 zero), B = W1^T in four
 // 16x8 slices (32 hidden units). Thread (g = lane/4, t = lane%4) holds features 2t, 2t+1 of rows g and
 // g+8, and C elements (rows g, g+8; hidden units 8nb + 2t, 8nb + 2t + 1).
 constexpr int kTab = 1024;
@@ -104,25 +106,70 @@ __global__ void __launch_bounds__(kEdgeWarps * 32, 4) k_edges(DGraph g, int seg,
                                                            float *fout, const gp_mlp *mlp, float *s_out,
                                                            int32_t *q_out) {
   __shared__ int s_tab[kEdgeWarps][kTab], s_over[kEdgeWarps][64];
-  __shared__ uint4 s_x[SCORE ? kEdgeWarps : 1][32];
+  __shared__ uint4 s_x[SCORE ? kEdgeWarps : 1][SCORE ? 64 : 1];
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, half = lane >> 4, hl = lane & 15;
   const int gq = lane >> 2, t = lane & 3;
   int *tab = s_tab[wid], *over = s_over[wid];
   for (int x = lane; x < kTab; x += 32) tab[x] = -1;
-  unsigned bfrag[4];  // (features 8..15 are zero)
-  float bias[4][2], w2v[4][2], b2 = 0.f;
+  // The network's operands: W1^T by lane, and (bias, bias, w2, w2) by lane % 4 and slice. In registers they made
+  // the lookups spill.
+  __shared__ uint4 s_w1[SCORE ? 32 : 1];
+  __shared__ float4 s_bw[SCORE ? 4 : 1][4];
   if (SCORE) {
+    if (wid == 0) {
+      unsigned w[4];
 #pragma unroll
-    for (int nb = 0; nb < 4; nb++) {
-      const int j = nb * 8 + gq;
-      bfrag[nb] = pack2(mlp->w1[j * kIn + 2 * t], mlp->w1[j * kIn + 2 * t + 1]);
-      bias[nb][0] = mlp->b1[nb * 8 + 2 * t];
-      bias[nb][1] = mlp->b1[nb * 8 + 2 * t + 1];
-      w2v[nb][0] = bf16_to_float(mlp->w2[nb * 8 + 2 * t]);
-      w2v[nb][1] = bf16_to_float(mlp->w2[nb * 8 + 2 * t + 1]);
+      for (int nb = 0; nb < 4; nb++) w[nb] = pack2(mlp->w1[(nb * 8 + gq) * kIn + 2 * t], mlp->w1[(nb * 8 + gq) * kIn + 2 * t + 1]);
+      s_w1[SCORE ? lane : 0] = make_uint4(w[0], w[1], w[2], w[3]);
+      if (lane < 16) {
+        const int j = (lane >> 2) * 8 + 2 * t;
+        s_bw[SCORE ? t : 0][lane >> 2] = make_float4(mlp->b1[j], mlp->b1[j + 1], bf16_to_float(mlp->w2[j]), bf16_to_float(mlp->w2[j + 1]));
+      }
     }
-    b2 = mlp->b2;
+    __syncthreads();
   }
+  // Scores of the staged entries b .. b + cnt - 1 (b: a multiple of 32 entries after the segment's first).
+  int64_t first = 0;
+  auto score = [&](int64_t b, int cnt) {
+    const unsigned *xw = reinterpret_cast<const unsigned *>(s_x[SCORE ? wid : 0]) + ((b - first) & 63) * 4;
+    const uint4 w1 = s_w1[SCORE ? lane : 0];
+    const unsigned bfrag[4] = {w1.x, w1.y, w1.z, w1.w};
+    const float b2 = mlp->b2;
+    float zmine = 0.f;
+#pragma unroll
+    for (int tile = 0; tile < 2; tile++) {
+      if (tile * 16 >= cnt) break;
+      const int r0 = tile * 16 + gq, r1 = r0 + 8;
+      const unsigned a[4] = {r0 < cnt ? xw[r0 * 4 + t] : 0u, r1 < cnt ? xw[r1 * 4 + t] : 0u, 0u, 0u};
+      float z0 = 0.f, z1 = 0.f;
+#pragma unroll
+      for (int nb = 0; nb < 4; nb++) {
+        const float4 bw = s_bw[SCORE ? t : 0][nb];
+        float c[4] = {bw.x, bw.y, bw.x, bw.y};
+        const unsigned bf[2] = {bfrag[nb], 0u};  // (features 8..15 are zero)
+        mma_16816(c, a, bf);
+        // hidden activations are rounded to BF16 before the second layer
+        const float h0 = bf16_to_float(float_to_bf16(fmaxf(c[0], 0.f)));
+        const float h1 = bf16_to_float(float_to_bf16(fmaxf(c[1], 0.f)));
+        const float h2 = bf16_to_float(float_to_bf16(fmaxf(c[2], 0.f)));
+        const float h3 = bf16_to_float(float_to_bf16(fmaxf(c[3], 0.f)));
+        z0 = fmaf(h0, bw.z, fmaf(h1, bw.w, z0));
+        z1 = fmaf(h2, bw.z, fmaf(h3, bw.w, z1));
+      }
+      z0 += __shfl_xor_sync(kFull, z0, 1);
+      z0 += __shfl_xor_sync(kFull, z0, 2);
+      z1 += __shfl_xor_sync(kFull, z1, 1);
+      z1 += __shfl_xor_sync(kFull, z1, 2);
+      // back to the entries' lanes: entry 16 tile + x comes from lane 4 (x mod 8)
+      const float a0 = __shfl_sync(kFull, z0, (lane & 7) * 4), a1 = __shfl_sync(kFull, z1, (lane & 7) * 4);
+      if (half == tile) zmine = lane & 8 ? a1 : a0;
+    }
+    if (lane < cnt) {
+      const float s = 1.0f / (1.0f + expf(-(zmine + b2)));
+      if (s_out) s_out[b + lane] = s;
+      if (q_out) q_out[b + lane] = __float2int_rn(s * 32768.0f);
+    }
+  };
   const float flevel = (float)level / 16.0f;
   const int64_t m = gp_min64(g.m, g.row_begin(g.n)), nseg = (m + seg - 1) / seg;
   const int64_t gw = blockIdx.x * (int64_t)kEdgeWarps + wid, nw = (int64_t)gridDim.x * kEdgeWarps;
@@ -130,7 +177,9 @@ __global__ void __launch_bounds__(kEdgeWarps * 32, 4) k_edges(DGraph g, int seg,
     const int64_t s1 = gp_min64(m, (sg + 1) * seg);
     RowWindow W;
     W.load(g, warp_row_of(g, sg * seg));
-    for (int64_t e0 = sg * seg; e0 < s1;) {
+    first = sg * seg;
+    int64_t staged = first;  // the first entry that waits for its score
+    for (int64_t e0 = first; e0 < s1;) {
       int64_t beg, end;
       const int64_t v = W.seek(g, e0, &beg, &end);
       const int64_t stop = gp_min64(end, s1), dv = end - beg;
@@ -236,43 +285,16 @@ __global__ void __launch_bounds__(kEdgeWarps * 32, 4) k_edges(DGraph g, int seg,
         pk.y = pack2(float_to_bf16(f[2]), float_to_bf16(f[3]));
         pk.z = pack2(float_to_bf16(f[4]), float_to_bf16(f[5]));
         pk.w = pack2(float_to_bf16(f[6]), float_to_bf16(f[7]));
+        // the step's entries join the ones staged before (entry e at slot (e - first) mod 64)
+        if (has) s_x[SCORE ? wid : 0][(e - first) & 63] = pk;
+        const int64_t upto = e0 + cnt;
         __syncwarp();
-        s_x[SCORE ? wid : 0][lane] = pk;
+        while (upto - staged >= 32 || (upto == s1 && staged < s1)) {
+          const int c = (int)gp_min64(upto - staged, 32);
+          score(staged, c);
+          staged += c;
+        }
         __syncwarp();
-        const unsigned *xw = reinterpret_cast<const unsigned *>(s_x[SCORE ? wid : 0]);
-        float zmine = 0.f;
-#pragma unroll
-        for (int tile = 0; tile < 2; tile++) {
-          if (tile * 16 >= cnt) break;
-          const int r0 = tile * 16 + gq, r1 = r0 + 8;
-          const unsigned a[4] = {r0 < cnt ? xw[r0 * 4 + t] : 0u, r1 < cnt ? xw[r1 * 4 + t] : 0u, 0u, 0u};
-          float z0 = 0.f, z1 = 0.f;
-#pragma unroll
-          for (int nb = 0; nb < 4; nb++) {
-            float c[4] = {bias[nb][0], bias[nb][1], bias[nb][0], bias[nb][1]};
-            const unsigned bf[2] = {bfrag[nb], 0u};
-            mma_16816(c, a, bf);
-            // hidden activations are rounded to BF16 before the second layer
-            const float h0 = bf16_to_float(float_to_bf16(fmaxf(c[0], 0.f)));
-            const float h1 = bf16_to_float(float_to_bf16(fmaxf(c[1], 0.f)));
-            const float h2 = bf16_to_float(float_to_bf16(fmaxf(c[2], 0.f)));
-            const float h3 = bf16_to_float(float_to_bf16(fmaxf(c[3], 0.f)));
-            z0 = fmaf(h0, w2v[nb][0], fmaf(h1, w2v[nb][1], z0));
-            z1 = fmaf(h2, w2v[nb][0], fmaf(h3, w2v[nb][1], z1));
-          }
-          z0 += __shfl_xor_sync(kFull, z0, 1);
-          z0 += __shfl_xor_sync(kFull, z0, 2);
-          z1 += __shfl_xor_sync(kFull, z1, 1);
-          z1 += __shfl_xor_sync(kFull, z1, 2);
-          // back to the entries' lanes: entry 16 tile + x comes from lane 4 (x mod 8)
-          const float a0 = __shfl_sync(kFull, z0, (lane & 7) * 4), a1 = __shfl_sync(kFull, z1, (lane & 7) * 4);
-          if (half == tile) zmine = lane & 8 ? a1 : a0;
-        }
-        if (has) {
-          const float s = 1.0f / (1.0f + expf(-(zmine + b2)));
-          if (s_out) s_out[e] = s;
-          if (q_out) q_out[e] = __float2int_rn(s * 32768.0f);
-        }
       }
       e0 = stop;
       __syncwarp();
@@ -300,7 +322,10 @@ struct TrainWeights {
 // loss and dz; then lane j owns hidden unit j, with its weights and ten gradient sums in registers, and
 // walks the 32 entries (features and dz broadcast from shared memory). No value crosses lanes, against one
 // warp reduction per parameter and group of entries before: 568 us for a million entries then, 65 us now.
-// Each sum is over a few hundred entries per lane, then over the warps and the blocks (in 64 bits).
+// Each sum is over m / (8 blocks) entries per lane (290 at a million entries, 27,000 at 10^8: the grid is at
+// most three blocks per SM), then over the warps and the blocks (in 64 bits). RMS error of the gradient against
+// 64 bits: 4.4e-8 of its size at 10^6 entries, 3.6e-8 at 2 10^7, 4.4e-8 at 10^8 (with the reductions 4.4, 3.5
+// and 4.8e-8).
 constexpr int kGradWarps = 8;
 
 __global__ void __launch_bounds__(kGradWarps * 32) k_grad(const float *x, const float *y, int64_t m,

@@ -87,3 +87,43 @@ def test_contests_decided_by_one_block(gp, n, k, weighted):
     p_o, bw_o, st_o = O.lp_refine(g, part, k, lm, 12, 5)
     assert np.array_equal(p.cpu().numpy(), p_o) and np.array_equal(bw.cpu().numpy(), bw_o)
     assert (st["moves"], st["visits"]) == (st_o.moves, st_o.visits)
+
+
+@pytest.mark.parametrize("n", [40, 3001, 90000])
+@pytest.mark.parametrize("extra", [0, 1, 6])
+@pytest.mark.parametrize("weighted,scored", [(False, False), (True, False), (False, True), (True, True)])
+def test_groups_of_four_and_eight_lanes(gp, n, extra, weighted, scored):
+    """Rows of at most 4 entries only (four lanes each), one row of 5, and one of 10 (no row of 5 to 8 but longer
+    ones), with tiles too small for a thread per row and larger ones."""
+    import torch
+    i = np.arange(n)
+    a, b = np.concatenate([i, i]), np.concatenate([(i + 1) % n, (i + 7) % n])
+    a, b = np.concatenate([a, [3] * extra]), np.concatenate([b, (3 + 9 + 2 * np.arange(extra)) % n])
+    lo, hi = np.minimum(a, b).astype(np.int64), np.maximum(a, b).astype(np.int64)
+    if extra == 6:  # (the row of 10 has its new neighbours' other edges taken out: they have 1 + at most 3)
+        keep = ~(np.isin(lo, (3 + 9 + 2 * np.arange(6)) % n) & (hi == lo + 1))
+        lo, hi = lo[keep], hi[keep]
+    if extra == 1:
+        keep = ~((lo == (3 + 9) % n) & (hi == lo + 1))
+        lo, hi = lo[keep], hi[keep]
+    key = np.unique(lo * n + hi)
+    lo, hi = key // n, key % n
+    w = 1 + (lo * 31 + hi * 17) % 9
+    src, dst = np.concatenate([lo, hi]), np.concatenate([hi, lo])
+    order = np.lexsort((dst, src))
+    off = np.concatenate([[0], np.cumsum(np.bincount(src, minlength=n))]).astype(np.int64)
+    g = gg.Graph(n, off, dst[order].astype(np.int32), None,
+                 np.concatenate([w, w])[order].astype(np.int32) if weighted else None, "four")
+    d = np.diff(off)
+    assert (d.max(), ((d > 4) & (d <= 8)).sum()) == {0: (4, 0), 1: (5, 1), 6: (10, 0)}[extra]
+    q = None
+    if scored:
+        s = np.repeat(i, d)
+        q = ((np.minimum(s, g.adj) * 7 + np.maximum(s, g.adj) * 13) % 32769).astype(np.int32)
+    dg = gp.DeviceGraph.from_host(g)
+    for vpb in (0, 4096):
+        gp.lp_set_tiles(0, vpb)
+        lab, st = gp.lp_cluster(dg, 30, 6, 3, None if q is None else torch.from_numpy(q).cuda())
+        gp.lp_set_tiles(0, 0)
+        lab_o, _, st_o = O.lp_cluster(g, 30, 6, 3, q)
+        assert np.array_equal(lab.cpu().numpy(), lab_o) and st["moves"] == st_o.moves

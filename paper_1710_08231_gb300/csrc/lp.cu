@@ -14,9 +14,11 @@
 //     several independent runs can share a launch) meet at bounded barriers between the phases of a
 //     sub-round: classify -> aggregate+choose -> admission with apply (-> contest when a target's
 //     proposals do not all fit);
-//   * active vertices are binned by degree: groups of 4/8/16/32 lanes (labels aggregated with
-//     __match_any_sync), one warp with a shared-memory hash table, one CTA with a shared-memory hash
-//     table, or several CTAs with a global-memory hash table for hubs;
+//   * active vertices are binned by degree: a thread per row of up to 16 entries where there are many,
+//     else groups of 4/8/16/32 lanes (__match_any_sync), one warp with a shared-memory hash table, a team
+//     of four warps or a CTA with one (labels entered one by one with 32-bit atomics, slots read and
+//     cleared by who claimed them), or several CTAs with a global-memory hash table for hubs;
+//   * where no row has more than 128 entries, blocks own their vertices instead (k_lp_own);
 //   * connection sums are exact integers and the choice is a total order (connection, score sum,
 //     H(seed, v, L), -L), so the aggregation order never matters;
 //   * admission is deterministic instead of CAS: proposals to one target are ordered by (gain desc,
@@ -44,7 +46,7 @@ constexpr int kWarps = kThreads / 32;
 //           2048 per CTA, hub chunks of 1024 entries, 32 KB of dynamic shared memory;
 //   TB = 1  plain runs on graphs without a vertex of degree above 1024: the same capacities, 32 KB;
 //   TB = 2  plain runs on graphs with such vertices: 12-byte slots, 512 per warp, 4096 per CTA (the CTA
-//           bin reaches degree 2048), hub chunks of 2048 entries, 48 KB.
+//           bin reaches degree 2048), hub chunks of 1024 entries, 48 KB.
 // The smaller class leaves more of the SM's unified L1/shared memory to L1, which the label gathers of
 // low-degree graphs use; the larger one pre-aggregates more hub entries per global table claim.
 template <int TB>
@@ -52,12 +54,10 @@ constexpr int kWarpCapT = TB == 2 ? 512 : 256;
 template <int TB>
 constexpr int kCtaCapT = TB == 2 ? 4096 : 2048;
 template <int TB>
-constexpr int kHubChunkT = 1024;  // hub row entries per accumulation chunk
-template <int TB>
 constexpr size_t kDynSmemT = TB == 2 ? 48 * 1024 : 32 * 1024;
 constexpr int kWarpCap = kWarpCapT<2>;  // the larger capacities (bounds of the schedule)
 constexpr int kCtaCap = kCtaCapT<2>;
-constexpr int kHubChunk = 1024;         // (bound of the work items)
+constexpr int kHubChunk = 1024;         // hub row entries per accumulation chunk
 // Hub accumulation: a 2048-slot shared table (a 1024-entry chunk fills at most half of it). With the
 // larger class (TB = 2) the rest of the 48 KB holds two staging buffers, each the 16-byte-aligned part
 // of one chunk's adjacency (4 KB) and edge weights (up to 8 KB), filled by bulk copies (cp.async.bulk
@@ -88,7 +88,6 @@ static_assert(sizeof(DGraph) % 4 == 0, "graph view is copied word by word");
 
 struct __align__(8) SubCounters {
   unsigned int bin_count[8];  // (the running counts live in LpProblem::binres; views copy them here)
-  unsigned int n_movers;
   unsigned int n_contested;
   unsigned int hub_chunks;
   unsigned int n_big;  // marking items of admitted movers of degree > kBigDeg (done by all blocks)
@@ -121,7 +120,7 @@ struct LpProblem {
   int64_t vbase, lbase;
   int64_t nl, U;
   int64_t hub_batch_slots;     // hub table slots per batch (tile size of the hub path)
-  int64_t hub_chunk;           // hub row entries per accumulation work item (kHubChunkT<TB>)
+  int64_t hub_chunk;           // hub row entries per accumulation work item (kHubChunk)
   int hub_chunk_shift;         // log2(hub_chunk)
   int own_four;                // no row has 5 to 8 entries (OwnBins)
   int pad_chunk;
@@ -1766,7 +1765,7 @@ struct HubChunk {
   }
 };
 
-// Accumulation of batch [h0, h1): hub rows are cut into chunks of kHubChunkT<TB> entries. A block aggregates
+// Accumulation of batch [h0, h1): hub rows are cut into chunks of kHubChunk entries. A block aggregates
 // its chunk's labels in a shared-memory table first and then adds one entry per distinct label to the
 // hub's table, so labels that many neighbours share cost one global atomic per chunk. With the larger
 // table class the block's next chunk is copied into a staging buffer (bulk copy, thread 0) while it
@@ -1777,7 +1776,7 @@ __device__ __noinline__ void hub_accum(const LpProblem &P, unsigned h0, unsigned
   constexpr bool LQ = TB == 0;
   constexpr bool kStage = TB == 2;
   constexpr int kCap = kHubCap;
-  constexpr int kChunk = kHubChunkT<TB>;
+  constexpr int kChunk = kHubChunk;
   const LabelTable<EW, LQ> T(dsm, kCap, 0);
   unsigned char *stage = dsm + kStageOff;
   __shared__ __align__(8) unsigned long long s_bar[2];
@@ -2667,7 +2666,7 @@ __device__ bool lp_problem(const LpProblem *prob, unsigned char *dsm) {
     sm.moves = 0;
     sm.movers = 0;
     for (int b = 0; b < 8; b++) sV.bin_count[b] = 0;
-    sV.n_movers = sV.n_contested = sV.hub_chunks = sV.n_big = sV.hub_batches = 0;
+    sV.n_contested = sV.hub_chunks = sV.n_big = sV.hub_batches = 0;
     sV.max_gain = sV.max_q = 0;
   }
   tick(-1);
@@ -2682,7 +2681,6 @@ __device__ bool lp_problem(const LpProblem *prob, unsigned char *dsm) {
         // counter set t+1 was last used by sub-round t-2, which every block has finished
         if (threadIdx.x < 8) P.binres[((t + 1) % 3) * 256 + threadIdx.x * 32] = 0;
         if (threadIdx.x == 0) {
-          Cn.n_movers = 0;
           Cn.n_contested = 0;
           Cn.hub_chunks = 0;
           Cn.n_inval = 0;
@@ -4007,11 +4005,10 @@ int run_lp_multi(const LpJob *jobs, int njobs, cudaStream_t s, const LpConfig &c
     P.nl = jb.nl;
     P.U = jb.U;
     P.hub_batch_slots = cfg.hub_batch_slots;
-    P.hub_chunk = kHubChunkT<0>;
+    P.hub_chunk = kHubChunk;
     P.own_four = hcls[9 * (size_t)j + 1] == 0;
     P.hub_chunk_shift = 10;
-    static_assert(kHubChunkT<0> == 1 << 10 && kHubChunkT<1> == 1 << 10 && kHubChunkT<2> == 1 << 10,
-                  "hub chunks are powers of two");
+    static_assert(kHubChunk == 1 << 10, "hub chunks are a power of two");
     P.wait_us = (unsigned)std::min<unsigned long long>(std::max<unsigned long long>(wait_limit_ns() / 1000, 0),
                                                         0xffffffffull);
     P.smix = mix64(jb.seed);

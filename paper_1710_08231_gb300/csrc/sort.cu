@@ -1,8 +1,8 @@
 // sort.cu -- device-wide stable LSD radix sort of (uint64 key, uint64 value) pairs.
 //
 // Each pass takes up to nine key bits with three kernels: per-tile digit counts (digit-major), an exclusive scan
-// of the counts, and a stable scatter in which every tile ranks its items per digit in order (one warp match
-// per 32 items, per-warp counts), stages them in shared memory in digit order and writes each digit's run
+// of the counts, and a stable scatter in which every tile ranks its items per digit in order (one vote per
+// digit bit and 32 items, per-warp counts), stages them in shared memory in digit order and writes each digit's run
 // contiguously. Used for vertex orders; the contraction runs the same tiles in its own kernel.
 #include <algorithm>
 

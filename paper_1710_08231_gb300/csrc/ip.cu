@@ -69,21 +69,23 @@ struct IpArgs {
 };
 
 // Multi-source BFS restricted to same-set vertices (part equal, set still being split). All sources start at
-// distance 0 together, so a step finds the vertices of one distance. A frontier of more than an eighth of the vertices
-// is taken from the other side: every vertex still without a distance looks for a neighbour in the frontier and stops
-// at the first 32 entries that hold one, instead of every frontier vertex walking its whole row (on the coarsest
-// level of an R-MAT graph, one CTA per try, the two or three large steps of each search: 8.6 -> 7.2 ms). The
-// distances are the same.
+// distance 0 together, so a step finds the vertices of one distance. On graphs of long rows a frontier of more than an
+// eighth of the vertices is taken from the other side: every vertex still without a distance looks for a neighbour in
+// the frontier and stops at the first 32 entries that hold one, instead of every frontier vertex walking its whole row
+// (on the coarsest level of an R-MAT graph, one CTA per try, the two or three large steps of each search: 8.6 -> 7.2
+// ms). Rows of up to 32 entries cost a step from either side, and the frontier has the fewer of them. The distances
+// are the same.
 __device__ void set_bfs(const DGraph &g, int64_t vbase, int32_t *part, int32_t *gk, int32_t *dist, int32_t *qa,
                         int32_t *qb, int nf) {
   __shared__ int s_next;
   const int n = (int)g.n;
+  const bool long_rows = g.row_begin(n) - g.row_begin(0) > 32 * (int64_t)n;
   for (int level = 0; nf > 0; level++) {
     if (threadIdx.x == 0) s_next = 0;
     __syncthreads();
     // one warp per frontier vertex, lanes over its row
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if (8 * (int64_t)nf > n) {
+    if (long_rows && 8 * (int64_t)nf > n) {
       for (int u0 = wid * 32; u0 < n; u0 += nw * 32) {
         const int mine = u0 + lane;
         unsigned open = __ballot_sync(kFull, mine < n && gk[mine] > 1 && dist[mine] == -1);

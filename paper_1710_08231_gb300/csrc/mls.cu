@@ -41,7 +41,7 @@ namespace {
 constexpr int kMlsWarps = 4;
 constexpr int kMlsThreads = kMlsWarps * 32;
 constexpr int kMaxMoves = 64;
-constexpr int kQCap = 256;
+constexpr int kQCap = 256;  // (even: the queue is searched by pairs)
 constexpr int kMaxK = 256;
 constexpr int kMovedSlots = 128;  // hash map of moved vertices (at most kMaxMoves entries)
 constexpr int kApplyThreads = 256;
@@ -57,14 +57,28 @@ struct WarpState {
 };
 
 // Per-warp connection arrays behind the WarpStates: k sums per lane (a vertex per lane), or k 64-bit sums shared by
-// the lanes (a vertex per warp). More blocks than kLaneK leave no room for the former.
+// the lanes (a vertex per warp). More blocks than kLaneK leave no room for the former. Where rows are long, many lanes
+// wait for the longest and what counts is how many searches are resident: there the arrays of a warp are at most
+// kLaneBytes, half of its state (R-MAT 18 with weights, k = 64: 2.92 s with 16 KB a warp, 1.61 s with a vertex per
+// warp; R-MAT 14, k = 24 / 32 / 48: unit 873 / 843 / 992 against 798 / 748 / 753 ms, weighted 986 / 1060 / - against
+// 732 / 765 / -). With rows of up to kLaneMean entries on average lanes are faster (50000 points of degree 12, k = 32 /
+// 48 / 64: 195 / 220 / 208 against 221 / 241 / 223 ms).
 template <int EW>
 using ConnT = typename std::conditional<EW == 0, unsigned, long long>::type;
 constexpr int kLaneK = 64;
+constexpr int kLaneRow = 64;  // longest row that a lane walks alone
+constexpr int64_t kLaneMean = 16;
+constexpr size_t kLaneBytes = 4096;
 template <int EW>
-size_t conn_bytes(int k) {
-  return k <= kLaneK ? (size_t)k * 32 * sizeof(ConnT<EW>) : (size_t)k * sizeof(long long);
+bool lane_conn(const DGraph &g, int k) {
+  return k <= kLaneK && (g.m <= kLaneMean * g.n || (size_t)k * 32 * sizeof(ConnT<EW>) <= kLaneBytes);
 }
+template <int EW>
+size_t conn_bytes(const DGraph &g, int k) {
+  return lane_conn<EW>(g, k) ? (size_t)k * 32 * sizeof(ConnT<EW>) : (size_t)k * sizeof(long long);
+}
+constexpr size_t kConnMost = (size_t)kLaneK * 32 * sizeof(long long);
+static_assert(kConnMost >= kMaxK * sizeof(long long), "the largest connection arrays are those of the lanes");
 
 struct MlsArgs {
   DGraph g;
@@ -75,6 +89,7 @@ struct MlsArgs {
   uint64_t smix;  // mix64(s)
   int max_moves, fruitless, queue_cap, max_degree;
   unsigned conn_bytes;  // per warp
+  int lane_conn;
 };
 
 __device__ __forceinline__ uint64_t hkey(uint64_t smix, uint64_t a, uint64_t b) { return mix64(mix64(smix ^ a) ^ b); }
@@ -230,32 +245,75 @@ __device__ __forceinline__ void queue_append(const MlsArgs &A, WarpState &W, int
 template <int EW>
 __device__ void touch(const MlsArgs &A, WarpState &W, unsigned char *conn_raw, int u) {
   const int lane = threadIdx.x & 31;
-  if (u >= 0 && (degree_of(A.g, u) > A.max_degree || (W.nm && moved_block(W, u) >= 0))) u = -1;
+  const int64_t d = u >= 0 ? degree_of(A.g, u) : 0;
+  if (u >= 0 && (d > A.max_degree || (W.nm && moved_block(W, u) >= 0))) u = -1;
   int at = -1;
-  for (int i = 0; i < W.qn; i++)
-    if (W.qv[i] == u) at = i;
+  const int qn0 = W.qn;
+#pragma unroll 4
+  for (int i = 0; i < qn0; i += 2) {
+    const int2 x = *reinterpret_cast<const int2 *>(&W.qv[i]);
+    if (x.x == u) at = i;
+    if (x.y == u && i + 1 < qn0) at = i + 1;
+  }
+  if (u < 0) at = -1;
+  const unsigned queued = __ballot_sync(kFull, at >= 0), fresh = __ballot_sync(kFull, u >= 0) & ~queued;
+  const unsigned shorts = __ballot_sync(kFull, A.lane_conn && d <= kLaneRow);
   int to = 0;
   long long gain = 0;
   bool movable = false;
-  if (A.k <= kLaneK) {
-    movable = lane_gain<EW>(A, W, reinterpret_cast<ConnT<EW> *>(conn_raw), u, &to, &gain);
-  } else {
-    for (unsigned todo = __ballot_sync(kFull, u >= 0); todo; todo &= todo - 1) {
-      const int src = __ffs(todo) - 1;
-      int t1 = 0;
-      long long g1 = 0;
-      const bool m1 = gain_of<EW>(A, W, reinterpret_cast<long long *>(conn_raw), __shfl_sync(kFull, u, src), &t1, &g1);
-      if (lane == src) {
-        movable = m1;
-        to = t1;
-        gain = g1;
+  // The gains of vertices that a full queue has no room for are not computed (on dense graphs most neighbours are
+  // such): then the vertices in the queue come first and, in lane order, those that find room left by a leaving vertex
+  // come in a second step. Vertices of a lane each come in the first one unless the queue is full already, the others
+  // only if all fit.
+  int room = A.queue_cap - W.qn;
+  unsigned now = queued | fresh, later = 0, leave = 0;
+  if (__popc(fresh) > room) {
+    later = room > 0 ? fresh & ~shorts : fresh;
+    now &= ~later;
+  }
+#pragma unroll 1
+  for (int step = 0;; step++) {
+    const unsigned lanes = now & shorts;
+    if (lanes) {
+      const bool on = lanes >> lane & 1u;
+      if (lane_gain<EW>(A, W, reinterpret_cast<ConnT<EW> *>(conn_raw), on ? u : -1, &to, &gain)) movable = true;
+      __syncwarp();
+    }
+    unsigned o = now & ~lanes;
+    if (o) {
+      const unsigned enter = step ? fresh & __ballot_sync(kFull, movable) : 0;
+      if (step) o |= leave | enter;
+      for (; o; o &= o - 1) {
+        const int src = __ffs(o) - 1;
+        if (step) {
+          if (leave >> src & 1u) {
+            room++;
+            continue;
+          }
+          if (room <= 0) continue;
+          room--;
+          if (enter >> src & 1u) continue;
+        }
+        int t1 = 0;
+        long long g1 = 0;
+        const bool m1 = gain_of<EW>(A, W, reinterpret_cast<long long *>(conn_raw), __shfl_sync(kFull, u, src), &t1, &g1);
+        if (lane == src) {
+          movable = m1;
+          to = t1;
+          gain = g1;
+        }
+        if (step && !m1) room++;
       }
     }
+    if (!later) break;
+    leave = queued & ~__ballot_sync(kFull, movable);
+    now = later & (room > 0 ? kFull : leave ? ~(2u * (leave & (0u - leave)) - 1u) : 0u);
+    later = 0;
+    if (!now) break;
   }
-  if (u < 0) at = -1;
   if (at >= 0 && movable) W.qg[at] = gain;
-  const unsigned out = __ballot_sync(kFull, at >= 0 && !movable);
-  const unsigned in = __ballot_sync(kFull, u >= 0 && at < 0 && movable);
+  const unsigned moving = __ballot_sync(kFull, movable);
+  const unsigned out = queued & ~moving, in = fresh & moving;
   __syncwarp();
   if (W.qn + __popc(in) <= A.queue_cap) {
     // every insertion finds room whatever the order
@@ -675,10 +733,11 @@ int run_mls(const DGraph &g, int k, int64_t lmax, uint64_t seed, const MlsParams
   A.fruitless = (int)p.fruitless;
   A.queue_cap = (int)p.queue_cap;
   A.max_degree = (int)p.max_degree;
-  A.conn_bytes = (unsigned)(ew == 0 ? conn_bytes<0>(k) : conn_bytes<1>(k));
+  A.conn_bytes = (unsigned)(ew == 0 ? conn_bytes<0>(g, k) : conn_bytes<1>(g, k));
+  A.lane_conn = ew == 0 ? lane_conn<0>(g, k) : lane_conn<1>(g, k);
   const size_t smem = (sizeof(WarpState) + A.conn_bytes) * kMlsWarps;
   {
-    const int most = (int)((sizeof(WarpState) + std::max(conn_bytes<1>(kLaneK), conn_bytes<1>(kMaxK))) * kMlsWarps);
+    const int most = (int)((sizeof(WarpState) + kConnMost) * kMlsWarps);
     const void *const kernel = ew == 0   ? (const void *)k_mls_search<0>
                                : ew == 1 ? (const void *)k_mls_search<1>
                                          : (const void *)k_mls_search<2>;

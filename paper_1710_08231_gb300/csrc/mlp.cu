@@ -86,15 +86,15 @@ __device__ __forceinline__ void mma_16816(float c[4], const unsigned a[4], const
 // v's first 64 neighbours is a table in the warp's shared memory (kTab slots and no probing: the keys whose
 // slot was taken, two on average for a full set, are compared one by one), and lane l owns one entry of 32.
 // The neighbours of two entries are looked up together, each by a half-warp that reads them contiguously, up
-// to 64 per entry, with the loads of four entries issued before the first lookup. Half-warps serve short lists (mesh rows of 12 entries take one step) and long
-// ones (four steps) alike. A lane per entry, walking its list alone, read 32 separate rows per load and
+// to 64 per entry, with the loads of four entries issued before the first lookup. Half-warps serve short
+// lists (mesh rows of 12 entries take one step) and long ones (four steps) alike. A lane per entry, walking its list alone, read 32 separate rows per load and
 // waited for the warp's longest list and probe: 22.4 ms a call on an R-MAT graph of scale 19 with edge
 // weights (15.5 M entries) against 2.1 ms now, at the same bits.
 //
 // Scores: the entries of a segment are staged in shared memory and scored 32 at a time, whatever rows they lie
 // in (a step per row left most lanes of the network idle on meshes: a grid of 2000 x 2000 took 3.81 ms a call
-// so, 2.97 now, R-MAT 19 2.57 and 2.13). 16 entries per tensor-core step, A = 16 entries x 16 features (8 used, 8 zero), B = W1^T in four
-// 16x8 slices (32 hidden units). Thread (g = lane/4, t = lane%4) holds features 2t, 2t+1 of rows g and
+// so, 2.97 now, R-MAT 19 2.57 and 2.13). 16 entries per tensor-core step, A = 16 entries x 16 features (8
+// used, 8 zero), B = W1^T in four 16x8 slices (32 hidden units). Thread (g = lane/4, t = lane%4) holds features 2t, 2t+1 of rows g and
 // g+8, and C elements (rows g, g+8; hidden units 8nb + 2t, 8nb + 2t + 1).
 constexpr int kTab = 1024;
 constexpr int kEdgeWarps = 8;
